@@ -79,7 +79,7 @@ typedef struct {
     int32_t queue_capacity; /* BnB queue entries per window (default 8192)               */
     int32_t band_rows;      /* rows of the shared-memory IWE tile (default: from W)      */
     int32_t threads;        /* threads per block of the IWE kernels, a multiple of 32    */
-                            /* up to 512 (default 512)                                    */
+                            /* up to 512 (default 512; above 480 a block works with 480)  */
     int32_t max_rounds;     /* BnB round limit, DD_ERR_TIMEOUT beyond (default 1<<20)    */
     int32_t host_loop;      /* 0: each solve's rounds run as one CUDA graph with a       */
                             /*    conditional loop (no host round trips); 1: the host    */
@@ -496,7 +496,7 @@ double dd_serve_clock(void);
  * every case dd_contrast rejects (the same descriptor and domain checks), or
  * if the events are not device pointers; DD_ERR_NO_DEVICE; DD_ERR_CUDA. */
 #define DD_NOALLOC_MAX_EVENTS (1 << 20)
-#define DD_NOALLOC_SCRATCH_BYTES 25224704
+#define DD_NOALLOC_SCRATCH_BYTES 16836096
 int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_y, const dd_events* ev, const float* D,
                         int32_t nD, dd_i128* K, void* stream);
 

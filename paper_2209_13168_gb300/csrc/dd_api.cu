@@ -22,9 +22,8 @@ struct dd_ctx {
     int eval_blocks = 0;          // resident blocks of the evaluation grid
     cudaStream_t own = nullptr, stream = nullptr;
 
-    // events: sorted and reciprocals for all windows of a call
+    // events: sorted, for all windows of a call
     dd::Ev* ev = nullptr;
-    float2* rcp = nullptr;
     int64_t ev_cap = 0;
     int16_t *in_x = nullptr, *in_y = nullptr;   // staging of host-array inputs
     float* in_t = nullptr;
@@ -159,7 +158,6 @@ void drop_graph(dd_ctx* c) {
 dd::EvalArgs eval_args(dd_ctx* c, uint32_t* iwe_out, bool single) {
     dd::EvalArgs a{};
     a.ev = c->ev;
-    a.rcp = c->rcp;
     a.row_off = c->row_off;
     a.wins = c->wins;
     a.tasks = c->tasks;
@@ -274,11 +272,9 @@ int ingest(dd_ctx* c, const dd_events* evs, int nw) {
     if (total > c->ev_cap) {
         drop_graph(c);
         release(c->ev);
-        release(c->rcp);
         c->ev_cap = 0;
         const int64_t nc = total < 1024 ? 1024 : total + total / 4;
         DD_TRY(cudaMalloc((void**)&c->ev, sizeof(dd::Ev) * nc));
-        DD_TRY(cudaMalloc((void**)&c->rcp, sizeof(float2) * nc));
         c->ev_cap = nc;
     }
     rc = ensure_staging(c, host_total);
@@ -328,7 +324,7 @@ int ingest(dd_ctx* c, const dd_events* evs, int nw) {
     DD_TRY(copy(c, c->wins, c->h_wins, sizeof(dd::WinIn) * nw, cudaMemcpyHostToDevice));
     if (ch) DD_TRY(copy(c, c->chunk_win, c->h_chunks, sizeof(int32_t) * ch, cudaMemcpyHostToDevice));
     c->n_chunks = ch;
-    DD_TRY(dd::launch_ingest(c->g, c->wins, nw, c->chunk_win, ch, c->ev, c->rcp, c->row_count, c->row_off,
+    DD_TRY(dd::launch_ingest(c->g, c->wins, nw, c->chunk_win, ch, c->ev, c->row_count, c->row_off,
                              c->cursor, c->err, c->stream));
     c->stats.kernel_launches += ch ? 3 : 1;
     return DD_OK;
@@ -657,7 +653,6 @@ void dd_destroy(dd_ctx* c) {
     if (!c) return;
     drop_graph(c);
     release(c->ev);
-    release(c->rcp);
     release(c->in_x);
     release(c->in_y);
     release(c->in_t);
@@ -727,6 +722,7 @@ int dd_create(int32_t W, int32_t H, float foe_x, float foe_y, const dd_config* c
     c->device = dev;
     c->cfg = k;
     c->threads = k.threads ? k.threads : 512;
+    if (c->threads > dd::EVAL_THREADS) c->threads = dd::EVAL_THREADS;
     c->g.W = W;
     c->g.H = H;
     c->g.fx = foe_x;

@@ -25,11 +25,11 @@ struct NvtxRange {
 };
 
 // One event after ingest: its offsets from the FOE as the warp uses them
-// (binary32 x - FOE_x and y - FOE_y) and its time since t0 (binary32
-// t - t0); one 16-byte load.
+// (binary32 x - FOE_x and y - FOE_y), its time since t0 (binary32 t - t0) and
+// the correctly rounded reciprocal of its larger offset (ties: dx), which a
+// bound's cell walk divides by; one 16-byte load.
 struct __align__(16) Ev {
-    float dx, dy, t;
-    int32_t pad;
+    float dx, dy, t, rm;
 };
 
 enum TaskKind : int32_t { TASK_POINT = 0, TASK_BOUND = 1 };
@@ -88,6 +88,9 @@ struct __align__(16) TraceRec {
 
 enum Phase : int32_t { PH_INIT = 0, PH_RUN = 1, PH_DONE = 2 };
 
+// Working threads of an evaluation block, at most (one more warp prepares
+// their units): two full blocks of an SM then have 64 registers a thread.
+constexpr int EVAL_THREADS = 480;
 constexpr int MAX_POP = 64;
 constexpr int MAX_TASKS = 3 * MAX_POP;   // tasks of one window in one round
 constexpr int CHUNK = 8192;              // events per ingest block
@@ -181,7 +184,7 @@ __host__ __device__ inline float warp_tref(const Geom& g, float tau) { return g.
 // typical offset from the FOE, (W + H)/4.  Bounds of at least DENSE_CELLS are
 // dense (their tiles are summed in one pass) and are the ones worth
 // splitting over several blocks.  A schedule estimate only (the threshold
-// and the per-lane walk limit in bound_pass were set by measurement).
+// was set by measurement).
 constexpr float DENSE_CELLS = 2.0f;
 // Split bands of bounds below SPLIT_ROWS_CELLS are divided by rows, longer
 // ones by events (see eval_unit).
@@ -262,7 +265,6 @@ struct CtlArgs {
 // Everything an evaluation launch reads or writes.
 struct EvalArgs {
     const Ev* ev;
-    const float2* rcp;
     const int32_t* row_off;        // per window: bins_of(g) + 1 entries
     const WinIn* wins;
     const Task* tasks;             // per window: task_stride entries
@@ -279,7 +281,7 @@ struct EvalArgs {
 
 // Kernel launches (dd_kernels.cu).  All asynchronous on `s`.
 cudaError_t launch_ingest(const Geom& g, const WinIn* wins_dev, int32_t n_windows, const int32_t* chunk_win_dev,
-                          int32_t n_chunks, Ev* out, float2* rcp, int32_t* row_count, int32_t* row_off,
+                          int32_t n_chunks, Ev* out, int32_t* row_count, int32_t* row_off,
                           int32_t* cursor, int32_t* err, cudaStream_t s);
 cudaError_t launch_eval(const Geom& g, const EvalArgs& a, int threads, int grid_blocks, cudaStream_t s);
 int eval_resident_blocks(const Geom& g, int threads);

@@ -20,6 +20,7 @@
 #include "../../include/dd.h"
 
 #include <cfloat>
+#include <math_constants.h>
 #include <mutex>
 
 namespace dd {
@@ -38,6 +39,61 @@ __device__ __forceinline__ int cell_of(float foe, float d, float s) {
 }
 __device__ __forceinline__ float fmin_t(float a, float b) { return a < b ? a : b; }
 __device__ __forceinline__ float fmax_t(float a, float b) { return a < b ? b : a; }
+
+// --------------------------------------------------- paired binary32 arithmetic
+
+// Two binary32 values in one 64-bit register pair.  sm_103a adds and
+// multiplies both halves in one instruction (add/mul.f32x2), each half
+// rounded as the scalar operation is, so a warp's pair of offsets, scales or
+// cells costs one issue slot instead of two; k_eval is bound by issue slots.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pair(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo_of(f32x2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi_of(f32x2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+// A product as a fused multiply-add onto +0, which rounds once, to the
+// product (a product of -0 becomes +0; no cell depends on that sign).  The
+// plain mul.rn.f32x2 will not do: the assembler contracts it with a following
+// add.rn.f32x2 into one rounding (measured: 39% of FOE + d s differ from the
+// two scalar operations; none with this form).
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(0ull));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// Biased cells: for |v| < 2^22, v + 1.5 x 2^23 rounded towards minus infinity
+// is floor(v) + 1.5 x 2^23 exactly, whose bit pattern is CELL0 + floor(v).
+// Cells stay below 2^22 in magnitude: scales are at most 65 (D tau >= -64)
+// and 4 (D tau <= 3/4), offsets at most 4096.  The conversion instruction
+// this replaces runs at a sixteenth of the add's rate.
+constexpr uint32_t CELL0 = 0x4B400000u;
+__device__ constexpr float CELL0_F = 12582912.0f;
+__device__ __forceinline__ f32x2 floor2(f32x2 v) {
+    f32x2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(v), "l"(pair(CELL0_F, CELL0_F)));
+    return r;
+}
+// Eq. (12): floor((foe + d s) + 1/2), biased, of one coordinate and of a pair.
+__device__ __forceinline__ uint32_t cell1(float foe, float d, float s) {
+    return __float_as_uint(__fadd_rd(__fadd_rn(__fadd_rn(foe, __fmul_rn(d, s)), 0.5f), CELL0_F));
+}
+__device__ __forceinline__ f32x2 cells2(f32x2 foe, f32x2 d, f32x2 s) {
+    return floor2(add2(add2(foe, mul2(d, s)), pair(0.5f, 0.5f)));
+}
+// An event's biased pixel (x, y) at scale s.
+__device__ __forceinline__ uint2 pixel_of(f32x2 foe, f32x2 d, float s) {
+    const f32x2 c = cells2(foe, d, pair(s, s));
+    return make_uint2((uint32_t)c, (uint32_t)(c >> 32));
+}
 
 // Relative widening of the per-event scale range (binary32 s(D) is monotone
 // in D only up to a few ulps; 2^-19 covers the error for D*tau <= 3/4).
@@ -68,6 +124,15 @@ __device__ __forceinline__ bool dd_in(long long i, long long n, unsigned bit) {
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
+}
+
+// Warp sum of 64-bit values as three 32-bit warp reductions (20, 20 and 24
+// bits per part: 32 of each add up within 32 bits).
+__device__ __forceinline__ unsigned long long warp_total(unsigned long long v) {
+    const uint32_t a = __reduce_add_sync(0xffffffffu, (uint32_t)v & 0xFFFFFu);
+    const uint32_t b = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 20) & 0xFFFFFu);
+    const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 40));
+    return (unsigned long long)a + ((unsigned long long)b << 20) + ((unsigned long long)c << 40);
 }
 
 // Inclusive prefix sum over the warp.
@@ -189,12 +254,11 @@ __global__ void __launch_bounds__(1024) k_row_scan(int bins, const int32_t* row_
 
 // Scatter each valid event of the block's sub-chunk to its bin (offsets
 // within the window); a block reserves one range per bin, so the global
-// atomics are per (block, bin).  Also stores the reciprocals of the event's
-// offsets from the FOE (used by the bound's cell walk).
+// atomics are per (block, bin).  Also stores the reciprocal of the event's
+// larger offset from the FOE (used by the bound's cell walk).
 __global__ void __launch_bounds__(INGEST_THREADS) k_row_scatter(Geom g, const WinIn* __restrict__ wins,
                                                                 const int32_t* __restrict__ chunk_win,
-                                                                int32_t* cursor, Ev* __restrict__ out,
-                                                                float2* __restrict__ rcp) {
+                                                                int32_t* cursor, Ev* __restrict__ out) {
     __shared__ int32_t h[MAX_BINS];
     __shared__ int32_t base[MAX_BINS];
     const int chunk = blockIdx.x / INGEST_SUB;
@@ -206,7 +270,6 @@ __global__ void __launch_bounds__(INGEST_THREADS) k_row_scatter(Geom g, const Wi
     sub_chunk(win, chunk, blockIdx.x % INGEST_SUB, i0, i1);
     int32_t* cur = cursor + (size_t)w * bins;
     Ev* o = out + win.ev_off;
-    float2* rc = rcp + win.ev_off;
     for (int r = threadIdx.x; r < bins; r += blockDim.x) h[r] = 0;
     __syncthreads();
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
@@ -234,14 +297,13 @@ __global__ void __launch_bounds__(INGEST_THREADS) k_row_scatter(Geom g, const Wi
         e.dx = __fsub_rn((float)xi, g.fx);
         e.dy = __fsub_rn((float)yi, g.fy);
         e.t = tr;
-        e.pad = 0;
+        e.rm = __frcp_rn(fabsf(e.dx) >= fabsf(e.dy) ? e.dx : e.dy);
         o[pos] = e;
-        rc[pos] = make_float2(__frcp_rn(e.dx), __frcp_rn(e.dy));
     }
 }
 
 cudaError_t launch_ingest(const Geom& g, const WinIn* wins_dev, int32_t n_windows, const int32_t* chunk_win_dev,
-                          int32_t n_chunks, Ev* out, float2* rcp, int32_t* row_count, int32_t* row_off,
+                          int32_t n_chunks, Ev* out, int32_t* row_count, int32_t* row_off,
                           int32_t* cursor, int32_t* err, cudaStream_t s) {
     const int bins = bins_of(g);
     if (n_windows <= 0) return cudaSuccess;
@@ -252,7 +314,7 @@ cudaError_t launch_ingest(const Geom& g, const WinIn* wins_dev, int32_t n_window
     const unsigned blocks = (unsigned)n_chunks * INGEST_SUB;
     if (n_chunks > 0) k_row_hist<<<blocks, INGEST_THREADS, 0, s>>>(g, wins_dev, chunk_win_dev, row_count, err);
     k_row_scan<<<n_windows, 1024, 0, s>>>(bins, row_count, row_off, cursor);
-    if (n_chunks > 0) k_row_scatter<<<blocks, INGEST_THREADS, 0, s>>>(g, wins_dev, chunk_win_dev, cursor, out, rcp);
+    if (n_chunks > 0) k_row_scatter<<<blocks, INGEST_THREADS, 0, s>>>(g, wins_dev, chunk_win_dev, cursor, out);
     return cudaGetLastError();
 }
 
@@ -305,803 +367,812 @@ __device__ void bucket_event_range(const Geom& g, const int32_t* row_off, float 
     e1 = row_off[b * g.H + rhi + 1];
 }
 
-// Eq. (16) for one event restricted to tile rows [y0, y1).  The segment is
-// walked along its major axis (larger |offset| from the FOE, ties to x): for
-// major cell k, the s-range where the major coordinate rounds to k (widened
-// by 2^-8 px, clipped to [s_a, s_b]) gives a run of minor cells.  The walk is
-// split into a set-up (seg_range: which major cells can reach the tile) and
-// the per-major-cell work (seg_cell), so that a warp can spread the major
-// cells of its events over its lanes.  The per-cell arithmetic is that of a
-// whole-frame walk; the tile only skips major cells whose runs cannot reach
-// its rows.
-enum SegMode : int { SEG_NONE = 0, SEG_ONE = 1, SEG_X = 2, SEG_Y = 3 };
+// A unit's candidate events: one run of consecutive events per time bucket,
+// taken in chunks of 32 (a run's last chunk may be partial), so that a warp
+// works on one run at a time and finds it with a uniform test.  Run b holds
+// chunks [next of run b - 1, next of run b); chunk c's events are
+// 32 c + first + lane, below end.
+constexpr int MAX_TB = 8;         // time buckets of the event sort
 
-struct Seg {
-    int mode, k0, count, addr;   // addr: the tile cell of SEG_ONE
-    float dn, rm, sa, sb;        // minor offset, 1/major offset, scale range
+struct __align__(16) Run {
+    int first, end, next, pad;
 };
+constexpr Run NO_RUN = {0, INT32_MIN, INT32_MAX, 0};   // after the last run: chunks without events
 
-__device__ __forceinline__ Seg seg_range(const Geom& g, float dx, float dy, float rdx, float rdy, float sa,
-                                         float sb, int xa, int ya, int xb, int yb, int y0, int y1) {
-    Seg s;
-    s.mode = SEG_NONE;
-    s.k0 = s.count = s.addr = 0;
-    s.dn = s.rm = 0.0f;
-    s.sa = sa;
-    s.sb = sb;
-    const int W = g.W, H = g.H;
-    if (dx == 0.0f && dy == 0.0f) {               // on the FOE: one pixel for every D
-        if (xa >= 0 && xa < W && ya >= y0 && ya < y1) {
-            s.mode = SEG_ONE;
-            s.count = 1;
-            s.addr = (ya - y0) * tile_pitch(g) + xa;
-        }
-        return s;
-    }
-    if (fabsf(dx) >= fabsf(dy)) {
-        int k0 = max(min(xa, xb), 0), k1 = min(max(xa, xb), W - 1);
-        if (dy == 0.0f) {
-            if (ya < y0 || ya >= y1) return s;
-        } else {
-            const float r = rdy;
-            const float e0 = __fsub_rn(__fsub_rn((float)y0, g.fy), HALF_PLUS);
-            const float e1 = __fadd_rn(__fsub_rn((float)(y1 - 1), g.fy), HALF_PLUS);
-            const float b0 = __fmul_rn(e0, r), b1 = __fmul_rn(e1, r);
-            const float lo = fmax_t(fmin_t(b0, b1), sa), hi = fmin_t(fmax_t(b0, b1), sb);
-            if (lo > hi) return s;
-            const int c0 = cell_of(g.fx, dx, lo), c1 = cell_of(g.fx, dx, hi);
-            k0 = max(k0, min(c0, c1) - 2);
-            k1 = min(k1, max(c0, c1) + 2);
-        }
-        if (k1 < k0) return s;
-        s.mode = SEG_X;
-        s.k0 = k0;
-        s.count = k1 - k0 + 1;
-        s.dn = dy;
-        s.rm = rdx;
-    } else {
-        const int k0 = max(max(min(ya, yb), 0), y0), k1 = min(min(max(ya, yb), H - 1), y1 - 1);
-        if (k1 < k0) return s;
-        s.mode = SEG_Y;
-        s.k0 = k0;
-        s.count = k1 - k0 + 1;
-        s.dn = dx;
-        s.rm = rdy;
-    }
-    return s;
-}
+// One unit -- a job's row band -- as warp 0 prepares it in shared memory for
+// the block: everything that is the same for all threads is worked out once.
+enum UnitKind : int { UNIT_NONE = 0, UNIT_POINT, UNIT_BOUND, UNIT_DENSE, UNIT_FUSED };
 
-// One increment of a tile cell.  Sparse images (at most a few increments per
-// cell): the sum of squares grows by 2v + 1 from the cell's previous count v
-// and C counts increments (32 bits: callers fold it into 64 bits often
-// enough that it cannot wrap).  Dense images (many increments per cell): the
-// increment alone, the sums taken from the tile afterwards.  Undo: the
-// decrement that takes back an earlier sparse increment of the same cell.
-enum BumpMode : int { BUMP_SPARSE = 0, BUMP_DENSE = 1, BUMP_UNDO = 2 };
-template <int MODE>
-__device__ __forceinline__ void bump(uint32_t* cell, unsigned long long& S, uint32_t& C) {
-    if (MODE == BUMP_DENSE) {
-        atomicAdd(cell, 1u);
-    } else if (MODE == BUMP_UNDO) {
-        atomicSub(cell, 1u);
-    } else {
-        const uint32_t v = atomicAdd(cell, 1u);
-        S += 2u * v + 1u;
-        C++;
-    }
-}
-
-template <int MODE>
-__device__ __forceinline__ void seg_cell(const Geom& g, int mode, int k, float dn, float rm, float sa, float sb,
-                                         int addr, int y0, int y1, uint32_t* tile, unsigned long long& S,
-                                         uint32_t& C) {
-    if (mode == SEG_ONE) {
-        if (DD_IN(addr, (y1 - y0) * tile_pitch(g), 2u)) bump<MODE>(&tile[addr], S, C);
-        return;
-    }
-    const bool major_x = mode == SEG_X;
-    const float fm = major_x ? g.fx : g.fy, fn = major_x ? g.fy : g.fx;
-    const float e = __fsub_rn((float)k, fm);
-    const float b1 = __fmul_rn(__fsub_rn(e, HALF_PLUS), rm), b2 = __fmul_rn(__fadd_rn(e, HALF_PLUS), rm);
-    float lo = b1 < b2 ? b1 : b2, hi = b1 < b2 ? b2 : b1;
-    if (lo < sa) lo = sa;
-    if (hi > sb) hi = sb;
-    if (lo > hi) return;
-    const int j1 = cell_of(fn, dn, lo), j2 = cell_of(fn, dn, hi);
-    if (major_x) {
-        const int j0 = max(max(min(j1, j2), 0), y0), jn = min(min(max(j1, j2), g.H - 1), y1 - 1);
-        for (int j = j0; j <= jn; j++)
-            if (DD_IN((j - y0) * tile_pitch(g) + k, (y1 - y0) * tile_pitch(g), 2u))
-                bump<MODE>(&tile[(j - y0) * tile_pitch(g) + k], S, C);
-    } else {
-        const int j0 = max(min(j1, j2), 0), jn = min(max(j1, j2), g.W - 1);
-        uint32_t* row = tile + (k - y0) * tile_pitch(g);
-        for (int j = j0; j <= jn; j++)
-            if (DD_IN((k - y0) * tile_pitch(g) + j, (y1 - y0) * tile_pitch(g), 2u)) bump<MODE>(&row[j], S, C);
-    }
-}
-
-// Position-to-event cursor over a unit's candidate runs (erange: first
-// event of each bucket's run, then each run's offset in the concatenation).
-// Each thread visits increasing positions, so the cursor (the first
-// position of the next run and the current run's offset from positions to
-// event indices) only moves forward; positions stay below
-// erange[MAX_TB + n_tb].
-constexpr int MAX_TB = 8;    // time buckets of the event sort
-
-struct Cursor {
-    const int* erange;
-    int cur_b, next_f, delta;
-    __device__ __forceinline__ Cursor(const int* er, int) : erange(er), cur_b(0) {
-        next_f = er[MAX_TB + 1];
-        delta = er[0] - er[MAX_TB];
-    }
-    __device__ __forceinline__ int at(int f) {
-        while (f >= next_f) {
-            cur_b++;
-            delta = erange[cur_b] - erange[MAX_TB + cur_b];
-            next_f = erange[MAX_TB + cur_b + 1];
-        }
-        return f + delta;
-    }
-};
-
-
-
-constexpr int QUEUE = 64;    // queued long-segment events per warp (a power of two, >= 63)
-constexpr int MAX_WARPS = 16;   // warps of a k_eval block (at most 512 threads)
-
-// Where one unit reads and writes.
-struct UnitPtrs {
-    const Ev* ev;                 // the window's sorted events
-    const float2* rcp;
-    const int32_t* row_off;       // the window's bin offsets
-    Partial* part;                // the task's sums (atomic accumulation over its row bands)
-    uint32_t* out;                // nullable: the task's image [H][W]
-    uint32_t* acc;                // event-split jobs: the task's accumulator [H][W]
-    int32_t* done;                // event-split jobs: finished splits per tile
-    Partial* sums;                // event-split jobs: sums of the splits per tile
+struct __align__(16) Unit {
+    Run run[MAX_TB + 1];     // candidate events (an event split: its share of them), then NO_RUN
+    int chunks;              // of all runs
+    int kind;
+    int y0, rows;            // tile rows [y0, y0 + rows) of the frame
+    float D_lo, D_hi, D_c, tau;  // D_c: a fused job's centre
+    int win, task, left;     // left: a fused job's left half
+    int tile;                // the job's band over both planes, and its plane
+    int plane;
+    int split, splits;       // event splits (1: none; a split by rows is a unit of its own rows)
+    const Ev* ev;            // the window's sorted events
 #ifdef DD_CHECKED
-    int64_t n_ev;                 // the window's event count
+    int64_t n_ev;            // the window's event count
 #endif
 };
 
-// Dense bound images (bound_cells >= DENSE_CELLS): their increments skip the
-// returned count and the tile's sums are taken in one pass afterwards.
-
-// Eqs. (16) and (19) for the unit's share of events, positions [f_begin,
-// total): Hbar into the tile, N_full into `full`, and (sparse) S and C.
-// Per-warp rings of queued long segments (see bound_pass): QUEUE records of
-// five words (event, s_a, s_b, both end cells' x, both end cells' y) per warp
-// of the block, in dynamic shared memory after the tile (so a block's ring
-// memory grows with its warps: 1,280 bytes per warp).
-constexpr int QREC = 5;
-struct SegQueue {
-    int* rec;       // [warps * QUEUE][QREC]
-    int cap;        // warps * QUEUE records
+// Chunk-to-event cursor of one warp; visited chunks increase.
+struct Cursor {
+    const Run* at;
+    Run r;
+    __device__ __forceinline__ explicit Cursor(const Unit& u) : at(u.run), r(u.run[0]) {}
+    __device__ __forceinline__ int event(int chunk, int lane) {   // the lane's event; none if >= r.end
+        while (chunk >= r.next) r = *++at;
+        return 32 * chunk + r.first + lane;
+    }
 };
 
-// Dynamic shared memory of a k_eval block: the band tile (rounded up to 16
-// bytes) and the segment rings of its warps.
-__host__ __device__ inline int eval_tile_words(const Geom& g) { return (g.band_rows * tile_pitch(g) + 3) & ~3; }
-__host__ __device__ inline size_t eval_smem_bytes(const Geom& g, int threads);
-
-template <int MODE>
-__device__ __forceinline__ void bound_pass(const Geom& g, const UnitPtrs& p, const Task& tk, float tau, uint32_t* tile,
-                                           SegQueue queue, int y0, int y1, int f_begin, int total, Cursor& cur,
-                                           unsigned long long& S, unsigned long long& C, unsigned long long& full) {
-    const int W = g.W, P = tile_pitch(g), rows = y1 - y0;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const float tref = warp_tref(g, tau);
-    const float Dl = tk.D_lo, Dh = tk.D_hi, gl = warp_g(Dl, tref), gh = warp_g(Dh, tref);
-    // The cells of up to 32 queued segments, one event per lane (`valid`,
-    // with the end scales and end cells computed when it was queued): short
-    // runs walked by their own lane, long runs spread over the warp as
-    // (event, major cell) pairs.
-    auto walk = [&](int e, bool valid, float sa, float sb, int xa, int ya, int xb, int yb) {
-        uint32_t Ci = 0;
-        Seg sg;
-        sg.mode = SEG_NONE;
-        sg.k0 = sg.count = sg.addr = 0;
-        sg.dn = sg.rm = sg.sa = sg.sb = 0.0f;
-        if (valid) {
-            const Ev v = p.ev[e];
-            const float2 r = p.rcp[e];
-            sg = seg_range(g, v.dx, v.dy, r.x, r.y, sa, sb, xa, ya, xb, yb, y0, y1);
-        }
-        const int cmax = __reduce_max_sync(0xffffffffu, (unsigned)sg.count);
-        if (cmax <= 4) {                       // short runs: each lane walks its own
-            for (int i = 0; i < sg.count; i++)
-                seg_cell<MODE>(g, sg.mode, sg.k0 + i, sg.dn, sg.rm, sg.sa, sg.sb, sg.addr, y0, y1, tile, S, Ci);
-            C += Ci;
-            return;
-        }
-        const int incl = warp_incl_scan(sg.count), excl = incl - sg.count;
-        const int tot = __shfl_sync(0xffffffffu, incl, 31);
-        for (int c0 = 0; c0 < tot; c0 += 32) {
-            const int gi = c0 + lane;
-            int o = 0;                            // owner: first lane whose inclusive sum exceeds gi
-            for (int step = 16; step > 0; step >>= 1) {
-                const int probe = __shfl_sync(0xffffffffu, incl, o + step - 1);
-                if (probe <= gi) o += step;
-            }
-            const int om = __shfl_sync(0xffffffffu, sg.mode, o);
-            const int ok = __shfl_sync(0xffffffffu, sg.k0 - excl, o);
-            const int oa = __shfl_sync(0xffffffffu, sg.addr, o);
-            const float odn = __shfl_sync(0xffffffffu, sg.dn, o);
-            const float orm = __shfl_sync(0xffffffffu, sg.rm, o);
-            const float osa = __shfl_sync(0xffffffffu, sg.sa, o);
-            const float osb = __shfl_sync(0xffffffffu, sg.sb, o);
-            if (gi < tot) seg_cell<MODE>(g, om, ok + gi, odn, orm, osa, osb, oa, y0, y1, tile, S, Ci);
-        }
-        C += Ci;
-    };
-    // Warps take 32 positions at a time, one event per lane.  A segment
-    // within one pixel is counted at once; an event whose segment spans more
-    // pixels is queued with its end scales and end cells (a ring of 64 entries
-    // per warp; cells packed as two 16-bit halves, their range being under
-    // 2^15 in magnitude), and every 32 queued events are walked together, so
-    // the walk runs on full warps.
-    const int qb = wid * QUEUE;
-    int q_head = 0, q_tail = 0;
-    auto take = [&](int i, int& e, float& sa, float& sb, int& xa, int& ya, int& xb, int& yb) {
-        const int* r = queue.rec + QREC * (qb + (i & (QUEUE - 1)));
-        e = r[0];
-        sa = __int_as_float(r[1]);
-        sb = __int_as_float(r[2]);
-        const int px = r[3], py = r[4];
-        xa = (int)(short)(px & 0xFFFF);
-        xb = px >> 16;
-        ya = (int)(short)(py & 0xFFFF);
-        yb = py >> 16;
-    };
-    for (int base = f_begin + wid * 32; base < total; base += nw * 32) {
-        const int f = base + lane;
-        bool pend = false;
-        int e = 0, xa = 0, xb = 0, ya = 0, yb = 0;
-        float sa = 0.0f, sb = 0.0f;
-        if (f < total) {
-            e = cur.at(f);
-            if (!DD_IN(e, p.n_ev, 4u)) e = 0;
-            const Ev v = p.ev[e];
-            const float dy = v.dy;
-            const float sl = warp_s(Dl, v.t, gl), sh = warp_s(Dh, v.t, gh);
-            sa = __fmul_rn(sl < sh ? sl : sh, WIDEN_DN);
-            sb = __fmul_rn(sl < sh ? sh : sl, WIDEN_UP);
-            ya = cell_of(g.fy, dy, sa);
-            yb = cell_of(g.fy, dy, sb);
-            // Every covered cell lies between the rows of the two end cells
-            // (each cell coordinate is monotone in s).
-            if (max(ya, yb) >= y0 && min(ya, yb) < y1) {
-                const float dx = v.dx;
-                xa = cell_of(g.fx, dx, sa);
-                xb = cell_of(g.fx, dx, sb);
-                const bool ya_here = (unsigned)(ya - y0) < (unsigned)rows;
-                // Eq. (19): both end cells in the frame; counted by the tile of row ya.
-                if ((unsigned)xa < (unsigned)W && (unsigned)xb < (unsigned)W && (unsigned)yb < (unsigned)g.H &&
-                    ya_here)
-                    full++;
-                if (xa == xb && ya == yb) {
-                    // Both ends in one pixel: each cell coordinate is monotone
-                    // in s, so the segment covers that pixel only.
-                    if ((unsigned)xa < (unsigned)W && ya_here) {
-                        uint32_t Ci = 0;
-                        if (DD_IN((ya - y0) * P + xa, rows * P, 1u)) bump<MODE>(&tile[(ya - y0) * P + xa], S, Ci);
-                        C += Ci;
-                    }
-                } else if ((xa == xb && abs(ya - yb) == 1) || (ya == yb && abs(xa - xb) == 1)) {
-                    // End cells side by side: one coordinate is constant and
-                    // the other takes two adjacent values, so the segment
-                    // covers exactly those two pixels (each counted where it
-                    // lies in the frame and in this band).
-                    uint32_t Ci = 0;
-                    if ((unsigned)xa < (unsigned)W && ya_here && DD_IN((ya - y0) * P + xa, rows * P, 1u))
-                        bump<MODE>(&tile[(ya - y0) * P + xa], S, Ci);
-                    if ((unsigned)xb < (unsigned)W && (unsigned)(yb - y0) < (unsigned)rows &&
-                        DD_IN((yb - y0) * P + xb, rows * P, 1u))
-                        bump<MODE>(&tile[(yb - y0) * P + xb], S, Ci);
-                    C += Ci;
-                } else {
-                    pend = true;
-                }
-            }
-        }
-        const unsigned pm = __ballot_sync(0xffffffffu, pend);
-        if (pend) {
-            int* r = queue.rec + QREC * (qb + ((q_tail + __popc(pm & ((1u << lane) - 1u))) & (QUEUE - 1)));
-            r[0] = e;
-            r[1] = __float_as_int(sa);
-            r[2] = __float_as_int(sb);
-            r[3] = (xa & 0xFFFF) | (xb << 16);
-            r[4] = (ya & 0xFFFF) | (yb << 16);
-        }
-        q_tail += __popc(pm);
-        if (q_tail - q_head >= 32) {
-            __syncwarp();                         // the queued entries are visible to the warp
-            take(q_head + lane, e, sa, sb, xa, ya, xb, yb);
-            __syncwarp();                         // read before the next pass may overwrite
-            q_head += 32;
-            walk(e, true, sa, sb, xa, ya, xb, yb);
-        }
-    }
-    while (q_tail > q_head) {                     // the rest of the queue
-        const int n = min(32, q_tail - q_head);
-        int e = 0, xa = 0, xb = 0, ya = 0, yb = 0;
-        float sa = 0.0f, sb = 0.0f;
-        __syncwarp();
-        if (lane < n) take(q_head + lane, e, sa, sb, xa, ya, xb, yb);
-        __syncwarp();
-        q_head += n;
-        walk(e, lane < n, sa, sb, xa, ya, xb, yb);
-    }
-}
-
-// One unit: split `split` of `splits` of one task's row band `ti`.  The block
-// scatters the events that can reach its rows into the shared tile.  Sparse
-// images: each increment returns the cell's previous count v and the band's
-// sum of squares grows by (v + 1)^2 - v^2 = 2v + 1, so the tile is only
-// cleared afterwards; dense bound images: one pass over the tile takes S and
-// C and clears it.  A split band is divided by rows when its bound's segments
-// are short (bound_cells below SPLIT_ROWS_CELLS): split s owns rows
-// [y0 + R s/splits, y0 + R (s + 1)/splits) of the band's R rows and counts the
-// events that reach them in its own rows of the tile, so the splits share no
-// cell.  With long segments (where every thin slice would read nearly all of
-// the band's candidates) the band is divided by events instead: split s
-// takes its share of the band's candidates, adds its tile into the L2
-// accumulator, and each addition of u onto a count w adds (w + u)^2 - w^2 to
-// S, so the splits' sums add up to the band's; the last split to finish
-// clears the accumulated band.  The tile arrives zeroed and leaves zeroed.
-__device__ __forceinline__ void eval_unit(const Geom& g, const UnitPtrs& p, const Task& tk, int ti, int split,
-                                          int splits, float tau, uint32_t* tile, unsigned long long (*red)[32],
-                                          int* erange, int* s_last, SegQueue queue) {
-    // Unit ti is row band `band` of polarity plane `plane`: the plane's own
-    // run of sorted events, its own image and its own counts.
-    const int plane = ti >= g.plane_tiles ? 1 : 0, band = ti - plane * g.plane_tiles;
-    const bool by_rows = splits > 1 && (!p.acc || bound_cells(g, tk.D_lo, tk.D_hi, tau) < SPLIT_ROWS_CELLS);
-    const int b0 = band * g.band_rows, R = min(b0 + g.band_rows, g.H) - b0;
-    const int y0 = by_rows ? b0 + (int)((long long)R * split / splits) : b0;
-    const int y1 = by_rows ? b0 + (int)((long long)R * (split + 1) / splits) : b0 + R;
-    const int32_t* row_off = p.row_off + (size_t)plane * g.n_tb * g.H;
-    const size_t plane_off = (size_t)plane * g.W * g.H;
-    const int W = g.W, P = tile_pitch(g), rows = y1 - y0;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-
-    // erange[b] = first event of bucket b's candidate run; erange[MAX_TB + b] =
-    // the run's offset in the concatenation of all runs (MAX_TB + n_tb: total).
-    if (threadIdx.x < 32) {
-        int e0 = 0, e1 = 0;
-        if (lane < g.n_tb && y1 > y0)
-            bucket_event_range(g, row_off, tk.D_lo, tk.D_hi, tau, __fdiv_rn((float)g.n_tb, tau), lane, y0, y1, e0,
-                               e1);
-        const int len = e1 - e0, incl = warp_incl_scan(len);
-        if (lane < g.n_tb) {
-            erange[lane] = e0;
-            erange[MAX_TB + lane] = incl - len;
-        }
-        if (lane == g.n_tb - 1) erange[MAX_TB + g.n_tb] = incl;
-    }
-    __syncthreads();
-    unsigned long long full = 0;
-    const int all = erange[MAX_TB + g.n_tb];
-    const int f_begin = by_rows ? 0 : (int)((long long)all * split / splits);
-    const int total = by_rows ? all : (int)((long long)all * (split + 1) / splits);
-    Cursor cur(erange, MAX_TB);
-
-    unsigned long long S = 0, C = 0;
-    bool dense = false;
-    if (tk.kind == TASK_POINT) {
-        const float D = tk.D_lo, gg = warp_g(D, warp_tref(g, tau));
-        uint32_t Ct = 0;                          // at most one increment per event
-#pragma unroll 4
-        for (int f = f_begin + threadIdx.x; f < total; f += blockDim.x) {
-            const int e = cur.at(f);
-            if (!DD_IN(e, p.n_ev, 4u)) continue;
-            const Ev v = p.ev[e];
-            const float s = warp_s(D, v.t, gg);
-            const int uy = cell_of(g.fy, v.dy, s);
-            if ((unsigned)(uy - y0) >= (unsigned)rows) continue;
-            const int ux = cell_of(g.fx, v.dx, s);
-            if ((unsigned)ux < (unsigned)W && DD_IN((uy - y0) * P + ux, rows * P, 1u))
-                bump<BUMP_SPARSE>(&tile[(uy - y0) * P + ux], S, Ct);
-        }
-        C = Ct;
-    } else {
-        dense = bound_cells(g, tk.D_lo, tk.D_hi, tau) >= DENSE_CELLS;
-        if (dense)
-            bound_pass<BUMP_DENSE>(g, p, tk, tau, tile, queue, y0, y1, f_begin, total, cur, S, C, full);
-        else
-            bound_pass<BUMP_SPARSE>(g, p, tk, tau, tile, queue, y0, y1, f_begin, total, cur, S, C, full);
-    }
-    __syncthreads();
-
-    uint32_t* out = p.out ? p.out + plane_off + (size_t)y0 * W : nullptr;
-    unsigned long long Cl = C;
-    // Tile rows have pitch P (odd), frame rows pitch W: warps take rows, lanes
-    // take columns.
-    if (splits == 1 || by_rows) {
-        if (out) {
-            if (dense) S = Cl = 0;
-            for (int r = wid; r < rows; r += nw)
-                for (int c = lane; c < W; c += 32) {
-                    const uint32_t v = tile[r * P + c];
-                    if (DD_IN(r * W + c, rows * W, 16u)) out[r * W + c] = v;
-                    tile[r * P + c] = 0u;
-                    if (dense) {
-                        S += (unsigned long long)v * v;
-                        Cl += v;
-                    }
-                }
-        } else {
-            // The band's rows are contiguous in the tile (the padding column
-            // of an odd pitch stays zero): 16-byte words, then the tail.
-            const int words = rows * P, quads = words >> 2;
-            uint4* t4 = reinterpret_cast<uint4*>(tile);
-            if (dense) {
-                S = Cl = 0;
-                for (int i = threadIdx.x; i < quads; i += blockDim.x) {
-                    const uint4 v = t4[i];
-                    t4[i] = make_uint4(0u, 0u, 0u, 0u);
-                    S += (unsigned long long)v.x * v.x + (unsigned long long)v.y * v.y +
-                         (unsigned long long)v.z * v.z + (unsigned long long)v.w * v.w;
-                    Cl += (unsigned long long)v.x + v.y + v.z + v.w;
-                }
-                for (int i = 4 * quads + threadIdx.x; i < words; i += blockDim.x) {
-                    const uint32_t v = tile[i];
-                    tile[i] = 0u;
-                    S += (unsigned long long)v * v;
-                    Cl += v;
-                }
-            } else {
-                for (int i = threadIdx.x; i < quads; i += blockDim.x) t4[i] = make_uint4(0u, 0u, 0u, 0u);
-                for (int i = 4 * quads + threadIdx.x; i < words; i += blockDim.x) tile[i] = 0u;
-            }
-        }
-    } else {
-        uint32_t* acc = p.acc + plane_off + (size_t)y0 * W;
-        // Splits of one band finish together: each starts its pass at its own
-        // row so that they add into different words at a time.
-        const int rot = (int)((long long)rows * split / splits);
-        S = Cl = 0;
-        // Four columns per lane at a time: their additions are issued
-        // before any returned count is used, so the L2 round trips overlap.
-        constexpr int MERGE_COLS = 4;
-        for (int q = wid; q < rows; q += nw) {
-            const int r = q + rot < rows ? q + rot : q + rot - rows;
-            for (int c0 = lane; c0 < W; c0 += 32 * MERGE_COLS) {
-                uint32_t v[MERGE_COLS], w[MERGE_COLS];
-#pragma unroll
-                for (int k = 0; k < MERGE_COLS; k++) {
-                    const int c = c0 + 32 * k;
-                    v[k] = c < W ? tile[r * P + c] : 0u;
-                }
-#pragma unroll
-                for (int k = 0; k < MERGE_COLS; k++) {
-                    const int c = c0 + 32 * k;
-                    w[k] = 0u;
-                    if (v[k]) {
-                        tile[r * P + c] = 0u;
-                        if (DD_IN(r * W + c, rows * W, 16u)) w[k] = atomicAdd(&acc[r * W + c], v[k]);
-                        else v[k] = 0u;
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < MERGE_COLS; k++) {
-                    S += (2ull * w[k] + v[k]) * v[k];
-                    Cl += v[k];
-                }
-            }
-        }
-        __threadfence();                          // this thread's additions, before the count below
-        S = warp_sum(S);
-        Cl = warp_sum(Cl);
-        full = warp_sum(full);
-        if (lane == 0) {
-            red[0][wid] = S;
-            red[1][wid] = Cl;
-            red[2][wid] = full;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long a = 0, b = 0, f = 0;
-            for (int w = 0; w < nw; w++) {
-                a += red[0][w];
-                b += red[1][w];
-                f += red[2][w];
-            }
-            atomicAdd(&p.sums[ti].S, a);
-            atomicAdd(&p.sums[ti].cells[0], b);
-            if (f) atomicAdd(&p.sums[ti].full[0], f);
-            __threadfence();
-            *s_last = atomicAdd(&p.done[ti], 1) == splits - 1;
-        }
-        __syncthreads();
-        if (!*s_last) return;                     // another split finishes the band
-        __threadfence();                          // every split's additions are visible now
-        for (int i = threadIdx.x; i < rows * W; i += blockDim.x) {
-            if (out) out[i] = __ldcg(&acc[i]);
-            acc[i] = 0u;
-        }
-        if (threadIdx.x == 0) {
-            const unsigned long long qS = atomicExch(&p.sums[ti].S, 0ull);
-            const unsigned long long qC = atomicExch(&p.sums[ti].cells[0], 0ull);
-            const unsigned long long qF = atomicExch(&p.sums[ti].full[0], 0ull);
-            p.done[ti] = 0;
-            if (qS) atomicAdd(&p.part->S, qS);
-            if (qC) atomicAdd(&p.part->cells[plane], qC);
-            if (qF) atomicAdd(&p.part->full[plane], qF);
-        }
+// Prepares unit `id` (job id / n_tiles, band id % n_tiles) in `un`: one warp,
+// one time bucket per lane.  The jobs' rows or events are divided here, so no
+// other thread divides.
+__device__ __forceinline__ void prepare_unit(const Geom& g, const EvalArgs& a, const Job* jobs, int id, int n_units,
+                                             Unit& un) {
+    const int lane = threadIdx.x & 31;
+    if (id >= n_units) {
+        if (lane == 0) un.kind = UNIT_NONE;
         return;
     }
-    // Each warp adds its share of the band's sums to the task's.
-    S = warp_sum(S);
-    const unsigned long long C64 = warp_sum(Cl);
-    full = warp_sum(full);
+    const int j = id / g.n_tiles, ti = id - j * g.n_tiles;
+    const Job jb = jobs[j];
+    const WinIn* win = a.wins + jb.win;
+    const int64_t ev_off = win->ev_off;
+    const float tau = win->tau;
+    const Task* wt = a.tasks + (size_t)jb.win * a.task_stride;
+    const Task tk = wt[jb.task];
+    const bool fused = jb.splits < 0;             // one expanded interval: its three tasks together
+    const float Dl = fused ? wt[jb.split].D_lo : tk.D_lo, Dh = fused ? wt[jb.split + 1].D_hi : tk.D_hi;
+    const float cells = bound_cells(g, Dl, Dh, tau);
+    const int kind = fused ? UNIT_FUSED : (tk.kind == TASK_POINT ? UNIT_POINT
+                                                                 : (cells >= DENSE_CELLS ? UNIT_DENSE : UNIT_BOUND));
+    const int plane = ti >= g.plane_tiles ? 1 : 0, band = ti - plane * g.plane_tiles;
+    int splits = fused ? 1 : max(1, jb.splits);
+    int y0 = band * g.band_rows, rows = min(g.band_rows, g.H - y0);
+    if (splits > 1 && (!a.mg.acc || cells < SPLIT_ROWS_CELLS)) {    // split by rows: its own rows
+        const int r0 = (int)((uint32_t)(rows * jb.split) / (uint32_t)splits);
+        rows = (int)((uint32_t)(rows * (jb.split + 1)) / (uint32_t)splits) - r0;
+        y0 += r0;
+        splits = 1;
+    }
+    const int32_t* row_off = a.row_off + (size_t)jb.win * (bins_of(g) + 1) + (size_t)plane * g.n_tb * g.H;
+    int e0 = 0, e1 = 0;
+    if (lane < g.n_tb && rows > 0)
+        bucket_event_range(g, row_off, Dl, Dh, tau, __fdiv_rn((float)g.n_tb, tau), lane, y0, y0 + rows, e0, e1);
+    int n = (e1 - e0 + 31) >> 5, incl = warp_incl_scan(n);
+    if (splits > 1) {                             // this split's share of the chunks of all runs
+        const uint32_t all = (uint32_t)__shfl_sync(0xffffffffu, incl, 31);
+        const int c0 = (int)(all * (uint32_t)jb.split / (uint32_t)splits);
+        const int c1 = (int)(all * (uint32_t)(jb.split + 1) / (uint32_t)splits);
+        const int a0 = incl - n, b0 = max(a0, c0), b1 = min(incl, c1);
+        e1 = min(e1, e0 + 32 * (b1 - a0));
+        e0 += 32 * (b0 - a0);
+        n = max(b1 - b0, 0);
+        incl = warp_incl_scan(n);
+    }
+    if (lane <= g.n_tb) {
+        Run r = NO_RUN;
+        if (lane < g.n_tb) {
+            r.first = e0 - 32 * (incl - n);
+            r.end = e1;
+            r.next = incl;
+        }
+        un.run[lane] = r;
+    }
+    const int chunks = __shfl_sync(0xffffffffu, incl, 31);
     if (lane == 0) {
-        if (S) atomicAdd(&p.part->S, S);
-        if (C64) atomicAdd(&p.part->cells[plane], C64);
-        if (full) atomicAdd(&p.part->full[plane], full);
+        un.chunks = chunks;
+        un.kind = kind;
+        un.y0 = y0;
+        un.rows = rows;
+        un.D_lo = Dl;
+        un.D_hi = Dh;
+        un.D_c = tk.D_lo;
+        un.tau = tau;
+        un.win = jb.win;
+        un.task = jb.task;
+        un.left = jb.split;
+        un.tile = ti;
+        un.plane = plane;
+        un.split = jb.split;
+        un.splits = splits;
+        un.ev = a.ev + ev_off;
+#ifdef DD_CHECKED
+        un.n_ev = win->n;
+#endif
     }
 }
 
-// The bound's work for one event (Eqs. 16 and 19 restricted to the tile rows
-// [y0, y1)), as bound_pass does it, with the event's own lane walking its
-// segment: from its offsets (dx, dy) and its binary32 scales at the
-// interval's ends (sl, sh), the widened scale range, the end cells, N_full
-// into F and the covered cells.  BUMP_UNDO takes back exactly the increments
-// an earlier BUMP_SPARSE call made for the same event and interval.
-template <int MODE>
-__device__ __forceinline__ void bound_event(const Geom& g, const UnitPtrs& p, int e, float dx, float dy, float sl,
-                                            float sh, int y0, int y1, uint32_t* tile, unsigned long long& S,
-                                            uint32_t& C, uint32_t& F) {
-    const int W = g.W, P = tile_pitch(g), rows = y1 - y0;
-    const float sa = __fmul_rn(sl < sh ? sl : sh, WIDEN_DN);
-    const float sb = __fmul_rn(sl < sh ? sh : sl, WIDEN_UP);
-    const int ya = cell_of(g.fy, dy, sa), yb = cell_of(g.fy, dy, sb);
-    if (max(ya, yb) < y0 || min(ya, yb) >= y1) return;
-    const int xa = cell_of(g.fx, dx, sa), xb = cell_of(g.fx, dx, sb);
-    const bool ya_here = (unsigned)(ya - y0) < (unsigned)rows;
-    if (MODE != BUMP_UNDO && (unsigned)xa < (unsigned)W && (unsigned)xb < (unsigned)W && (unsigned)yb < (unsigned)g.H &&
-        ya_here)
-        F++;
-    if (xa == xb && ya == yb) {
-        if ((unsigned)xa < (unsigned)W && ya_here && DD_IN((ya - y0) * P + xa, rows * P, 1u))
-            bump<MODE>(&tile[(ya - y0) * P + xa], S, C);
-    } else if ((xa == xb && abs(ya - yb) == 1) || (ya == yb && abs(xa - xb) == 1)) {
-        if ((unsigned)xa < (unsigned)W && ya_here && DD_IN((ya - y0) * P + xa, rows * P, 1u))
-            bump<MODE>(&tile[(ya - y0) * P + xa], S, C);
-        if ((unsigned)xb < (unsigned)W && (unsigned)(yb - y0) < (unsigned)rows && DD_IN((yb - y0) * P + xb, rows * P, 1u))
-            bump<MODE>(&tile[(yb - y0) * P + xb], S, C);
+// ----------------------------------------------------- passes over the events
+
+constexpr int MAX_WARPS = 16;     // working warps of a k_eval block (at most 512 threads)
+// A block of k_eval: working warps and one more that prepares their units.
+__device__ __forceinline__ int work_threads() { return (int)blockDim.x - 32; }
+__device__ __forceinline__ int work_warps() { return ((int)blockDim.x >> 5) - 1; }
+__device__ __forceinline__ void work_sync() {     // a barrier of the working warps
+    asm volatile("bar.sync 1, %0;" : : "r"(work_threads()) : "memory");
+}
+
+// Shared scratch of one working warp (WARP_WORDS words of dynamic shared
+// memory after the tile): the ring of a sparse bound's queued events, the
+// segment descriptors of a dense bound's walks, or the warp's list of a fused
+// unit's unstable events.
+constexpr int WARP_WORDS = 320;
+constexpr int RUN = 7;            // major cells of a segment that one lane walks at a time (odd)
+constexpr int RING = 64;          // queued events per warp (a power of two, >= 63)
+
+// Dynamic shared memory of a k_eval block: the band tile (rounded up to 16
+// bytes) and its warps' scratch.
+__host__ __device__ inline int eval_tile_words(const Geom& g) { return (g.band_rows * tile_pitch(g) + 3) & ~3; }
+__host__ __device__ inline size_t eval_smem_bytes(const Geom& g, int threads) {
+    return sizeof(uint32_t) * ((size_t)eval_tile_words(g) + (size_t)WARP_WORDS * (threads / 32));
+}
+
+// The block's tile and what every pass needs of the unit: rows [row0, row0 +
+// rows) of the frame (biased), pitch P.
+struct Tile {
+    uint32_t* cell;
+    uint32_t base;           // shared-memory address of biased pixel (0, 0) if the tile reached it
+    uint32_t pitch;          // bytes
+    uint32_t idle;           // shared-memory address of the lane's own word outside the tile
+    uint32_t row0, rows, W;
+    __device__ __forceinline__ uint32_t first() const {           // address of the tile's first cell
+        return base + row0 * pitch + 4u * CELL0;
+    }
+};
+
+// Increments of a tile cell.  Sparse images: the sum of squares grows by
+// 2v + 1 from the cell's previous count v, so S = 2 sum(v) + (increments).
+// Dense images (many increments per cell) add without an answer; their sums
+// are taken from the tile afterwards.  A fused unit keeps the images of its
+// three tasks in three 10-bit fields of one cell.
+enum Field : int { FIELD_P = 0, FIELD_L = 10, FIELD_R = 20, FIELD_ALL = 30, WHOLE = 32, DENSE = 33 };
+constexpr uint32_t FIELD_MAX = 1023;
+
+template <int F>
+__device__ __forceinline__ uint32_t field_inc() {
+    return F >= WHOLE ? 1u : (F == FIELD_ALL ? 0x00100401u : 1u << (F & 31));
+}
+// The previous count in an atomic's answer (0 if it was not issued): into V,
+// and into top, their maximum (a field that held FIELD_MAX has run over into
+// the next one).
+template <int F>
+__device__ __forceinline__ void take(uint32_t old, unsigned long long& V, uint32_t& top) {
+    if (F == WHOLE) {
+        V += old;
+    } else if (F != DENSE) {
+        const uint32_t v = (old >> (F == FIELD_ALL ? 0 : F & 31)) & FIELD_MAX;
+        V += v;
+        top = max(top, v);
+    }
+}
+
+// One atomic increment at shared-memory address `at`; a lane that has none
+// (`here` false) adds to a word of its own instead.  A predicated atomic is
+// compiled to a branch around it (measured: about five control instructions
+// per atomic, a third of a wide bound's instructions); an address that is
+// always valid takes none.
+template <int F>
+__device__ __forceinline__ void bump(const Tile& T, uint32_t at, bool here, unsigned long long& V, uint32_t& top) {
+    const uint32_t to = here ? at : T.idle;
+    if (F == DENSE) {
+        asm volatile("red.shared.add.u32 [%0], 1;" : : "r"(to) : "memory");
     } else {
-        const float2 r = p.rcp[e];
-        const Seg sg = seg_range(g, dx, dy, r.x, r.y, sa, sb, xa, ya, xb, yb, y0, y1);
-        for (int i = 0; i < sg.count; i++)
-            seg_cell<MODE>(g, sg.mode, sg.k0 + i, sg.dn, sg.rm, sg.sa, sg.sb, sg.addr, y0, y1, tile, S, C);
+        uint32_t old;
+        asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(to), "r"(field_inc<F>()) : "memory");
+        take<F>(here ? old : 0u, V, top);
     }
 }
 
-// The contrast's work for one event (Eqs. 11-12) restricted to the tile rows,
-// from its offsets and its binary32 scale.
-template <int MODE>
-__device__ __forceinline__ void point_event(const Geom& g, float dx, float dy, float sc, int y0, int y1,
-                                            uint32_t* tile, unsigned long long& S, uint32_t& C) {
-    const int rows = y1 - y0, P = tile_pitch(g);
-    const int uy = cell_of(g.fy, dy, sc);
-    if ((unsigned)(uy - y0) >= (unsigned)rows) return;
-    const int ux = cell_of(g.fx, dx, sc);
-    if ((unsigned)ux < (unsigned)g.W && DD_IN((uy - y0) * P + ux, rows * P, 1u))
-        bump<MODE>(&tile[(uy - y0) * P + ux], S, C);
+// Adds one to the field of biased pixel c if it is in the tile (and `also`
+// holds); n counts the increments.
+template <int F>
+__device__ __forceinline__ void bump_pixel(const Tile& T, uint2 c, unsigned long long& V, uint32_t& n, uint32_t& top,
+                                           bool also = true) {
+    const uint32_t r = c.y - T.row0, x = c.x - CELL0, at = T.base + c.y * T.pitch + 4u * c.x;
+    bool here = (r < T.rows) & (x < T.W) & also;
+#ifdef DD_CHECKED
+    here = here && DD_IN((int)(at - T.first()), T.rows * T.pitch, 1u);
+#endif
+    bump<F>(T, at, here, V, top);
+    n += here;
 }
 
+// An event's widened scale range over an interval and its end pixels (biased).
+struct Span {
+    float sa, sb;
+    uint2 a, b;
+};
+__device__ __forceinline__ Span span_of(f32x2 foe, f32x2 d, float s1, float s2, f32x2 widen) {
+    const f32x2 w = mul2(pair(fminf(s1, s2), fmaxf(s1, s2)), widen);
+    Span s;
+    s.sa = lo_of(w);
+    s.sb = hi_of(w);
+    s.a = pixel_of(foe, d, s.sa);
+    s.b = pixel_of(foe, d, s.sb);
+    return s;
+}
+// Both scales of an event at time t: (1 - D t) g for the pair of D.
+__device__ __forceinline__ f32x2 scales2(f32x2 minus_D, f32x2 gg, float t) {
+    return mul2(add2(pair(1.0f, 1.0f), mul2(minus_D, pair(t, t))), gg);
+}
+// Every covered cell lies between the end pixels (each coordinate is monotone
+// in s): does that box meet the tile?
+__device__ __forceinline__ bool meets(const Tile& T, const Span& s) {
+    return max(s.a.y, s.b.y) >= T.row0 && min(s.a.y, s.b.y) < T.row0 + T.rows && max(s.a.x, s.b.x) >= CELL0 &&
+           min(s.a.x, s.b.x) < CELL0 + T.W;
+}
+// Eq. (19): both end pixels in the frame; counted by the tile of row a.y.
+__device__ __forceinline__ bool counts_full(const Geom& g, const Tile& T, const Span& s) {
+    return s.a.x - CELL0 < T.W && s.b.x - CELL0 < T.W && s.b.y - CELL0 < (uint32_t)g.H && s.a.y - T.row0 < T.rows;
+}
+// End pixels side by side: one coordinate is constant and the other takes two
+// adjacent values, so the segment covers exactly those two pixels.
+__device__ __forceinline__ bool adjacent(const Span& s) {
+    return abs((int)(s.a.x - s.b.x)) + abs((int)(s.a.y - s.b.y)) == 1;
+}
+
+// Eq. (16), the cells of one longer segment.  It is walked along its major
+// axis (the larger offset from the FOE, ties to x): major cell k takes the
+// s-range in which the major coordinate rounds to k, widened by 2^-8 px and
+// clipped to [s_a, s_b], and covers the minor cells between the ends of that
+// range.  walk_range gives the major cells whose runs can reach the tile (a
+// superset: the runs are cut to the tile's rows and the frame's columns);
+// their number can be negative.  Major y: the rows in the tile.  Major x: the
+// columns at the scales at which the minor coordinate is within the tile's
+// rows (half a pixel and the margin beyond, which exceeds the error of the
+// approximate reciprocal, 2^-22 of at most 4096 px), 2^-6 px farther than the
+// event's own positions there (a column's s-range reaches 2^-8 px beyond it,
+// rounding far less).  A minor offset of 0 makes those scales infinite or not
+// a number, which the minimum and maximum ignore: any scale will do.  One
+// straight line of code: a warp has events of both axes.
+__device__ __forceinline__ int walk_range(const Geom& g, const Tile& T, float4 v, const Span& s, bool major_x,
+                                          uint32_t& k) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v.y));
+    const float y0 = __uint_as_float(T.row0) - CELL0_F, y1 = __uint_as_float(T.row0 + T.rows - 1) - CELL0_F;
+    const float b0 = __fmul_rn(__fsub_rn(__fsub_rn(y0, g.fy), HALF_PLUS), r);
+    const float b1 = __fmul_rn(__fadd_rn(__fsub_rn(y1, g.fy), HALF_PLUS), r);
+    const float lo = fmaxf(fminf(b0, b1), s.sa), hi = fminf(fmaxf(b0, b1), s.sb);
+    const float x0 = __fadd_rn(g.fx, __fmul_rn(v.x, lo)), x1 = __fadd_rn(g.fx, __fmul_rn(v.x, hi));
+    const uint32_t c0 = __float_as_uint(__fadd_rd(__fadd_rn(fminf(x0, x1), 0.5f - 0x1p-6f), CELL0_F));
+    const uint32_t c1 = __float_as_uint(__fadd_rd(__fadd_rn(fmaxf(x0, x1), 0.5f + 0x1p-6f), CELL0_F));
+    const uint32_t ea = major_x ? s.a.x : s.a.y, eb = major_x ? s.b.x : s.b.y;
+    const uint32_t a = max(min(ea, eb), major_x ? max(c0, CELL0) : T.row0);
+    const uint32_t b = min(max(ea, eb), major_x ? min(c1, CELL0 + T.W - 1) : T.row0 + T.rows - 1);
+    k = a;
+    return major_x && lo > hi ? 0 : (int)(b - a) + 1;
+}
+
+// `n` consecutive major cells of a segment from k (biased) on, by one lane:
+// each covers the run of minor cells between the ends of its s-range, cut to
+// the tile's rows and the frame's columns.  dn, rm: the minor offset and the
+// major one's reciprocal.  A run has at most three cells: its s-range spans
+// 1.008 major cells and the slope is at most 1.
+template <int F>
+__device__ __forceinline__ void walk_cells(const Geom& g, const Tile& T, bool mx, uint32_t k, int n, float dn, float rm,
+                                           float sa, float sb, unsigned long long& V, uint32_t& C, uint32_t& top) {
+    const float fm = mx ? g.fx : g.fy, fn = mx ? g.fy : g.fx;
+    const float h = copysignf(HALF_PLUS, rm);     // so that lo is the smaller end
+    const uint32_t jmin = mx ? T.row0 : CELL0, jmax = mx ? T.row0 + T.rows - 1 : CELL0 + T.W - 1;
+    const uint32_t sk = mx ? 4u : T.pitch, sj = mx ? T.pitch : 4u;
+    uint32_t at_k = T.base + k * sk;
+    float kf = __fsub_rn(__uint_as_float(k), CELL0_F);
+#pragma unroll 2
+    for (; n > 0; n--) {
+        const float e = __fsub_rn(kf, fm);
+        const float lo = fmaxf(__fmul_rn(__fsub_rn(e, h), rm), sa), hi = fminf(__fmul_rn(__fadd_rn(e, h), rm), sb);
+        const uint32_t c0 = cell1(fn, dn, lo), c1 = cell1(fn, dn, hi);
+        const uint32_t j0 = max(min(c0, c1), jmin), jn = min(max(c0, c1), jmax);
+        const uint32_t at = at_k + j0 * sj;
+        bool some = lo <= hi;                     // an empty s-range covers nothing
+#ifdef DD_CHECKED
+        if (some && j0 <= jn)
+            some = DD_IN(jn - j0, 3, 2u) && DD_IN((int)(at - T.first()), T.rows * T.pitch, 2u) &&
+                   DD_IN((int)(at + (jn - j0) * sj - T.first()), T.rows * T.pitch, 2u);
+#endif
+        bump<F>(T, at, some & (j0 <= jn), V, top);
+        bump<F>(T, at + sj, some & (j0 < jn), V, top);
+        if (some & (j0 + 1 < jn)) bump<F>(T, at + 2 * sj, true, V, top);     // rare: slopes near 1
+        if (F != DENSE) C += some & (j0 <= jn) ? jn - j0 + 1 : 0u;
+        kf = __fadd_rn(kf, 1.0f);
+        at_k += sk;
+    }
+}
+
+// A short segment walked by its own lane.
+template <int F>
+__device__ __forceinline__ void walk_lane(const Geom& g, const Tile& T, float4 v, const Span& s,
+                                          unsigned long long& V, uint32_t& C, uint32_t& top) {
+    const bool mx = fabsf(v.x) >= fabsf(v.y);
+    uint32_t k;
+    const int n = walk_range(g, T, v, s, mx, k);
+    walk_cells<F>(g, T, mx, k, n, mx ? v.y : v.x, v.w, s.sa, s.sb, V, C, top);
+}
+
+// The segments of a warp's events (`here`: the lane has one that meets the
+// tile).  If none has more than RUN major cells in the tile, each lane walks
+// its own; otherwise they are cut into runs of RUN cells that are spread over
+// the lanes: the segments put their descriptors in shared memory in lane
+// order, and 32 runs at a time find their owners from the bit mask of the
+// segments whose runs start among them.  RUN is odd, so that the runs of one
+// segment lie in different shared-memory banks.
+template <int F>
+__device__ __forceinline__ void walk_warp(const Geom& g, const Tile& T, float4 v, const Span& s, bool here,
+                                          uint32_t* scratch, unsigned long long& V, uint32_t& C, uint32_t& top) {
+    const int lane = threadIdx.x & 31;
+    const bool mx = fabsf(v.x) >= fabsf(v.y);
+    uint32_t k;
+    const int cells = walk_range(g, T, v, s, mx, k), n = here ? max(cells, 0) : 0;
+    const int longest = __reduce_max_sync(0xffffffffu, n);
+    if (longest == 0) return;
+    const float dn = mx ? v.y : v.x;
+    if (longest <= RUN) {
+        walk_cells<F>(g, T, mx, k, n, dn, v.w, s.sa, s.sb, V, C, top);
+        return;
+    }
+    float4* desc = reinterpret_cast<float4*>(scratch);            // [32] rm, dn, s_a, s_b
+    uint2* key = reinterpret_cast<uint2*>(scratch + 128);         // [32] first cell (top bit: major y), cells << 16 | first run
+    const int runs = (n + RUN - 1) / RUN, incl = warp_incl_scan(runs), excl = incl - runs;
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned act = __ballot_sync(0xffffffffu, n > 0);
+    if (n > 0) {
+        const int r = __popc(act & ((1u << lane) - 1u));
+        desc[r] = make_float4(v.w, dn, s.sa, s.sb);
+        key[r] = make_uint2(k | (mx ? 0u : 0x80000000u), (uint32_t)n << 16 | (uint32_t)excl);
+    }
+    __syncwarp();
+    const unsigned upto = 0xffffffffu >> (31 - lane);             // lanes 0..lane
+    int seen = -1;
+    for (int c0 = 0; c0 < total; c0 += 32) {
+        const uint32_t rel = (uint32_t)(excl - c0);
+        const unsigned starts = __reduce_or_sync(0xffffffffu, n > 0 && rel < 32u ? 1u << rel : 0u);
+        const int r = seen + __popc(starts & upto);
+        seen += __popc(starts);
+        if (c0 + lane < total) {
+            const float4 q = desc[r];
+            const uint2 w = key[r];
+            const int i = RUN * (c0 + lane - (int)(w.y & 0xffffu));
+            walk_cells<F>(g, T, (int)w.x >= 0, (w.x & 0x7fffffffu) + (uint32_t)i, min(RUN, (int)(w.y >> 16) - i), q.y, q.x,
+                          q.z, q.w, V, C, top);
+        }
+    }
+    __syncwarp();                                 // read before the scratch is written again
+}
+
+__device__ __forceinline__ float4 load_event(const float4* ev, int e) {
+    return __ldg(ev + e);                         // dx, dy, t, 1/major offset
+}
+// The lane's event of a chunk; a lane without one gets offsets that are not
+// numbers, whose biased pixel lies in no tile and at every scale is the same.
+__device__ __forceinline__ float4 chunk_event(const Unit& un, const float4* ev, Cursor& cur, int chunk, int lane,
+                                              int& e) {
+    e = cur.event(chunk, lane);
+    float4 v = make_float4(CUDART_NAN_F, CUDART_NAN_F, 0.0f, 0.0f);
+    if (e < cur.r.end && DD_IN(e, un.n_ev, 4u)) v = load_event(ev, e);
+    return v;
+}
+
+// Eqs. (11)-(12) at D: each event of the unit's chunks into the tile.  V and
+// C collect the previous counts and the increments.  Four chunks are loaded
+// before any is used, so that a warp waits for one L2 round trip per 128
+// events.
+__device__ __forceinline__ void point_pass(const Geom& g, const Unit& un, const Tile& T, float D,
+                                           unsigned long long& V, unsigned long long& C) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31, nw = work_warps(), chunks = un.chunks;
+    const float4* ev = reinterpret_cast<const float4*>(un.ev);
+    const float gg = warp_g(D, warp_tref(g, un.tau));
+    const f32x2 foe = pair(g.fx, g.fy);
+    uint32_t n = 0, top = 0;                      // increments: at most one per event
+    Cursor cur(un);
+    for (int ch = (int)(threadIdx.x >> 5); ch < chunks; ch += U * nw) {
+        float4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            int e;
+            v[u] = chunk_event(un, ev, cur, ch + u * nw, lane, e);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            bump_pixel<WHOLE>(T, pixel_of(foe, pair(v[u].x, v[u].y), warp_s(D, v[u].z, gg)), V, n, top);
+    }
+    C += n;
+}
+
+// Eqs. (16) and (19) over [Dl, Dh] for the unit's chunks: Hbar into the tile,
+// N_full into F, and (sparse) the previous counts and increments into V and C.
+// An event whose end pixels coincide covers that pixel only.  Sparse bounds
+// (few such segments are longer) queue the others, so that full warps handle
+// them; dense bounds walk them at once, chunk by chunk.
+template <bool IS_DENSE>
+__device__ __forceinline__ void bound_pass(const Geom& g, const Unit& un, const Tile& T, float Dl, float Dh,
+                                           uint32_t* scratch, unsigned long long& V, unsigned long long& C,
+                                           unsigned long long& F) {
+    constexpr int U = IS_DENSE ? 1 : 2;
+    const int lane = threadIdx.x & 31, nw = work_warps(), chunks = un.chunks;
+    const float4* ev = reinterpret_cast<const float4*>(un.ev);
+    const float tref = warp_tref(g, un.tau);
+    const f32x2 foe = pair(g.fx, g.fy), minus_D = pair(-Dl, -Dh), gg = pair(warp_g(Dl, tref), warp_g(Dh, tref));
+    const f32x2 widen = pair(WIDEN_DN, WIDEN_UP);
+    uint32_t one = 0, more = 0, full = 0, top = 0;
+    int head = 0, tail = 0;
+    auto span = [&](float4 v) {
+        const f32x2 s2 = scales2(minus_D, gg, v.z);
+        return span_of(foe, pair(v.x, v.y), lo_of(s2), hi_of(s2), widen);
+    };
+    auto queued = [&](bool valid) {               // up to 32 queued events, one per lane
+        __syncwarp();                             // the queued events are visible to the warp
+        float4 v = make_float4(CUDART_NAN_F, CUDART_NAN_F, 0.0f, 0.0f);
+        if (valid) v = load_event(ev, (int)scratch[(head + lane) & (RING - 1)]);
+        __syncwarp();                             // read before the next chunk overwrites them
+        const Span s = span(v);
+        full += (uint32_t)(valid & counts_full(g, T, s));
+        const bool two = adjacent(s);
+        bump_pixel<WHOLE>(T, s.a, V, more, top, two);
+        bump_pixel<WHOLE>(T, s.b, V, more, top, two);
+        walk_warp<WHOLE>(g, T, v, s, valid & !two & meets(T, s), scratch + RING, V, more, top);
+    };
+    Cursor cur(un);
+    for (int ch = (int)(threadIdx.x >> 5); ch < chunks; ch += U * nw) {
+        float4 v[U];
+        int e[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) v[u] = chunk_event(un, ev, cur, ch + u * nw, lane, e[u]);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const Span s = span(v[u]);
+            const bool single = s.a.x == s.b.x && s.a.y == s.b.y;
+            bump_pixel<IS_DENSE ? DENSE : WHOLE>(T, s.a, V, one, top, single);
+            const unsigned m = __ballot_sync(0xffffffffu, !single);
+            if (!m) continue;
+            if (IS_DENSE) {
+                const bool here = !single && meets(T, s);
+                full += (uint32_t)(here & counts_full(g, T, s));
+                walk_warp<DENSE>(g, T, v[u], s, here, scratch, V, more, top);
+            } else {
+                if (!single) scratch[(tail + __popc(m & ((1u << lane) - 1u))) & (RING - 1)] = (uint32_t)e[u];
+                tail += __popc(m);
+                if (tail - head >= 32) {
+                    queued(true);
+                    head += 32;
+                }
+            }
+        }
+    }
+    if (!IS_DENSE) queued(lane < tail - head);
+    C += (unsigned long long)one + more;
+    F += (unsigned long long)one + full;
+}
 
 // One fused unit: the three tasks of one expanded interval [lo, hi] with
 // centre c -- the contrast at c (Eqs. 11-13) and the bounds over [lo, c] and
-// [c, hi] (Eqs. 14-19) -- on one row band, with one pass over the events.
-// Per event, the range [RN(min(s_lo, s_c, s_hi)(1 - 2^-19)),
-// RN(max(s_lo, s_c, s_hi)(1 + 2^-19))] of its binary32 scales at lo, c and hi
-// (computed as the tasks compute them) contains every scale the three tasks
-// use: s_c itself and the widened ends of both halves (rounding is
-// monotone).  Each cell coordinate is monotone in s, so when both ends of
-// that range fall in one pixel, every task puts the event in that pixel and
-// nowhere else: a stable event, counted once into the tile for all three (its
-// increments give a common sum of squares S_C and count N_C, which is also
-// each bound's N_full share).  The other events are listed as unstable; each
-// task in turn adds its own increments for them on top of the common counts,
-// each increment returning the cell's previous count v, so that the task's
-// sum of squares is S_C + sum(2v + 1); the centre's and the left half's
-// increments are taken back before the next task.  The sums, and so the keys,
-// are those of three separate passes.  A band with more unstable events than
-// the list holds runs as three ordinary units instead.
-__device__ void eval_fused_unit(const Geom& g, const UnitPtrs& p, const Task& tp, const Task& tl, const Task& tr,
-                                Partial* part_p, Partial* part_l, Partial* part_r, int ti, float tau, uint32_t* tile,
-                                unsigned long long (*red)[32], int* erange, int* s_n, int* s_last, SegQueue queue) {
-    const int plane = ti >= g.plane_tiles ? 1 : 0, band = ti - plane * g.plane_tiles;
-    const int y0 = band * g.band_rows, y1 = min(y0 + g.band_rows, g.H);
-    const int32_t* row_off = p.row_off + (size_t)plane * g.n_tb * g.H;
-    const int W = g.W, P = tile_pitch(g), rows = y1 - y0;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const float lo = tl.D_lo, c = tp.D_lo, hi = tr.D_hi;
-    if (threadIdx.x < 32) {
-        int e0 = 0, e1 = 0;
-        if (lane < g.n_tb)
-            bucket_event_range(g, row_off, lo, hi, tau, __fdiv_rn((float)g.n_tb, tau), lane, y0, y1, e0, e1);
-        const int len = e1 - e0, incl = warp_incl_scan(len);
-        if (lane < g.n_tb) {
-            erange[lane] = e0;
-            erange[MAX_TB + lane] = incl - len;
-        }
-        if (lane == g.n_tb - 1) erange[MAX_TB + g.n_tb] = incl;
-        if (lane == 0) *s_n = 0;
-    }
-    __syncthreads();
-    const int total = erange[MAX_TB + g.n_tb];
-    Cursor cur(erange, MAX_TB);
-    const float tref = warp_tref(g, tau);
-    const float glo = warp_g(lo, tref), gc = warp_g(c, tref), ghi = warp_g(hi, tref);
-    int* list = queue.rec;                        // unstable events (the segment rings' memory)
-    const int list_cap = QREC * queue.cap;
+// [c, hi] (Eqs. 14-19) -- with one pass over the events.  Per event, the
+// range [min(s_lo, s_hi)(1 - 2^-18), max(s_lo, s_hi)(1 + 2^-18)] contains
+// every scale the three tasks use: the binary32 scale at any D of the
+// interval is within 2^-19 of the range of its end scales, so s_c and the
+// halves' ends, widened by 2^-19, are within 2^-18.  Each cell coordinate is
+// monotone in s, so when both ends of that range fall in one pixel, every
+// task puts the event in that pixel and nowhere else: a stable event, added
+// to the cell's three fields at once (its previous count, the same in all
+// three, goes to V[0]).  Each warp lists the others, and once every stable
+// event is in, each task adds the listed events to its own field (V[1..3]):
+// one pass instead of five (with the increments of two tasks taken back
+// between them) and one barrier instead of five.  The sums of squares, 2 sum(v) + increments,
+// are those of three separate passes.  Returns false if the list or a field
+// overflowed: then the tile holds nothing of use.
+struct FusedSums {
+    unsigned long long V[4];                      // previous counts: stable, centre, left, right
+    uint32_t n, C[3], F[2];                       // stable increments; each task's own; the halves' N_full
+};
 
-    // Pass over the candidates: stable events into the tile, the rest listed.
-    unsigned long long SC = 0;
-    uint32_t NC = 0;
-    for (int base = wid * 32; base < total; base += nw * 32) {
-        const int f = base + lane;
-        bool uns = false;
-        int e = 0;
-        if (f < total) {
-            e = cur.at(f);
-            if (!DD_IN(e, p.n_ev, 4u)) e = 0;
-            const Ev v = p.ev[e];
-            const float a = warp_s(lo, v.t, glo), b = warp_s(c, v.t, gc), d = warp_s(hi, v.t, ghi);
-            const float wa = __fmul_rn(fmin_t(fmin_t(a, b), d), WIDEN_DN);
-            const float wb = __fmul_rn(fmax_t(fmax_t(a, b), d), WIDEN_UP);
-            const int ya = cell_of(g.fy, v.dy, wa), yb = cell_of(g.fy, v.dy, wb);
-            if (max(ya, yb) >= y0 && min(ya, yb) < y1) {
-                const int xa = cell_of(g.fx, v.dx, wa), xb = cell_of(g.fx, v.dx, wb);
-                if (xa == xb && ya == yb) {
-                    if ((unsigned)xa < (unsigned)W && DD_IN((ya - y0) * P + xa, rows * P, 1u))
-                        bump<BUMP_SPARSE>(&tile[(ya - y0) * P + xa], SC, NC);
-                } else {
-                    uns = true;
+template <int F>
+__device__ __forceinline__ void fused_half(const Geom& g, const Tile& T, float4 v, f32x2 foe, float s1, float s2,
+                                           unsigned long long& V, uint32_t& C, uint32_t& full, uint32_t& top) {
+    const Span s = span_of(foe, pair(v.x, v.y), s1, s2, pair(WIDEN_DN, WIDEN_UP));
+    full += counts_full(g, T, s);
+    const bool single = s.a.x == s.b.x && s.a.y == s.b.y, two = adjacent(s);
+    bump_pixel<F>(T, s.a, V, C, top, single | two);
+    bump_pixel<F>(T, s.b, V, C, top, two);
+    if (!single && !two && meets(T, s)) walk_lane<F>(g, T, v, s, V, C, top);
+}
+
+__device__ __forceinline__ bool fused_pass(const Geom& g, const Unit& un, const Tile& T, uint32_t* list,
+                                           int* s_over, FusedSums& q) {
+    constexpr int U = 2;
+    const int lane = threadIdx.x & 31, nw = work_warps(), chunks = un.chunks;
+    const float4* ev = reinterpret_cast<const float4*>(un.ev);
+    const float tref = warp_tref(g, un.tau), lo = un.D_lo, hi = un.D_hi;
+    const f32x2 foe = pair(g.fx, g.fy), minus_D = pair(-lo, -hi), gg = pair(warp_g(lo, tref), warp_g(hi, tref));
+    const f32x2 widen = pair(1.0f - 0x1p-18f, 1.0f + 0x1p-18f);
+    uint32_t top = 0;
+    int listed = 0;
+    Cursor cur(un);
+    for (int ch = (int)(threadIdx.x >> 5); ch < chunks; ch += U * nw) {
+        float4 v[U];
+        int e[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) v[u] = chunk_event(un, ev, cur, ch + u * nw, lane, e[u]);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const f32x2 s2 = scales2(minus_D, gg, v[u].z);
+            const Span s = span_of(foe, pair(v[u].x, v[u].y), lo_of(s2), hi_of(s2), widen);
+            const bool single = s.a.x == s.b.x && s.a.y == s.b.y;
+            bump_pixel<FIELD_ALL>(T, s.a, q.V[0], q.n, top, single);
+            const unsigned m = __ballot_sync(0xffffffffu, !single);
+            const int at = listed + __popc(m & ((1u << lane) - 1u));
+            if (!single && at < WARP_WORDS) list[at] = (uint32_t)e[u];
+            listed += __popc(m);
+        }
+    }
+    if (top >= FIELD_MAX || listed > WARP_WORDS) *s_over = 1;
+    work_sync();
+    if (*s_over) return false;
+    const float c = un.D_c, gc = warp_g(c, tref);
+    for (int k = lane; k < listed; k += 32) {
+        const float4 v = load_event(ev, (int)list[k]);
+        const f32x2 s2 = scales2(minus_D, gg, v.z);
+        const float sc = warp_s(c, v.z, gc);
+        bump_pixel<FIELD_P>(T, pixel_of(foe, pair(v.x, v.y), sc), q.V[1], q.C[0], top);
+        fused_half<FIELD_L>(g, T, v, foe, lo_of(s2), sc, q.V[2], q.C[1], q.F[0], top);
+        fused_half<FIELD_R>(g, T, v, foe, sc, hi_of(s2), q.V[3], q.C[2], q.F[1], top);
+    }
+    if (top >= FIELD_MAX) *s_over = 1;
+    work_sync();
+    return !*s_over;
+}
+
+// ------------------------------------------------------------------- units
+
+// Zeroes the tile: one instruction of one thread (bulk store of zeros),
+// ordered by the block's next barrier like any store of that thread.
+__device__ __forceinline__ void clear_tile(uint32_t* tile, int words) {
+    asm volatile("st.bulk.weak.shared::cta [%0], %1, 0;"
+                 :
+                 : "r"((uint32_t)__cvta_generic_to_shared(tile)), "l"((unsigned long long)words * 4ull)
+                 : "memory");
+}
+
+// A band of a bound split by events: this split's tile added into the band's
+// L2 accumulator (each addition of u onto a count w adds (w + u)^2 - w^2 to S,
+// so the splits' sums add up to the band's), the tile zeroed on the way; the
+// last split to finish copies the image, clears the accumulated band and adds
+// the band's sums to the task's.
+__device__ __noinline__ void merge_split(const Geom& g, const EvalArgs& a, const Unit& un, const Tile& T, Partial* part,
+                                         uint32_t* out, unsigned long long F, unsigned long long (*red)[MAX_WARPS],
+                                         int* s_last) {
+    const size_t task_cells = (size_t)g.planes * g.W * g.H, plane_off = (size_t)un.plane * g.W * g.H;
+    const int W = g.W, P = tile_pitch(g), rows = un.rows;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = work_warps();
+    uint32_t* acc = a.mg.acc + (size_t)un.task * task_cells + plane_off + (size_t)un.y0 * W;
+    const size_t ti = (size_t)un.task * g.n_tiles + un.tile;
+    Partial* sums = a.mg.sums + ti;
+    // Splits of one band finish together: each starts its pass at its own row
+    // so that they add into different words at a time.
+    const int rot = (int)((uint32_t)(rows * un.split) / (uint32_t)un.splits);
+    unsigned long long S = 0, C = 0;
+    // Four columns per lane at a time: their additions are issued before any
+    // returned count is used, so the L2 round trips overlap.
+    constexpr int MERGE_COLS = 4;
+    for (int q = wid; q < rows; q += nw) {
+        const int r = q + rot < rows ? q + rot : q + rot - rows;
+        for (int c0 = lane; c0 < W; c0 += 32 * MERGE_COLS) {
+            uint32_t v[MERGE_COLS], w[MERGE_COLS];
+#pragma unroll
+            for (int k = 0; k < MERGE_COLS; k++) {
+                const int c = c0 + 32 * k;
+                v[k] = c < W ? T.cell[r * P + c] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < MERGE_COLS; k++) {
+                const int c = c0 + 32 * k;
+                w[k] = 0u;
+                if (v[k]) {
+                    T.cell[r * P + c] = 0u;
+                    if (DD_IN(r * W + c, rows * W, 16u)) w[k] = atomicAdd(&acc[r * W + c], v[k]);
+                    else v[k] = 0u;
                 }
             }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, uns);
-        if (m) {
-            int at = 0;
-            if (lane == 0) at = atomicAdd(s_n, __popc(m));
-            at = __shfl_sync(0xffffffffu, at, 0);
-            const int pos = at + __popc(m & ((1u << lane) - 1u));
-            if (uns && pos < list_cap) list[pos] = e;
+#pragma unroll
+            for (int k = 0; k < MERGE_COLS; k++) {
+                S += (2ull * w[k] + v[k]) * v[k];
+                C += v[k];
+            }
         }
     }
-    __syncthreads();
-    const int n = *s_n;
-    if (n > list_cap) {                           // too many unstable events: three ordinary units
-        const int words = rows * P;
-        for (int i = threadIdx.x; i < words; i += blockDim.x) tile[i] = 0u;
-        __syncthreads();
-        for (int k = 0; k < 3; k++) {
-            UnitPtrs q = p;
-            q.part = k == 0 ? part_p : (k == 1 ? part_l : part_r);
-            const Task tk = k == 0 ? tp : (k == 1 ? tl : tr);
-            eval_unit(g, q, tk, ti, 0, 1, tau, tile, red, erange, s_last, queue);
-            __syncthreads();
+    __threadfence();                              // this thread's additions, before the count below
+    S = warp_total(S);
+    C = warp_total(C);
+    F = warp_total(F);
+    if (lane == 0) {
+        red[0][wid] = S;
+        red[1][wid] = C;
+        red[2][wid] = F;
+    }
+    work_sync();
+    if (threadIdx.x == 0) {
+        S = C = F = 0;
+        for (int w = 0; w < nw; w++) {
+            S += red[0][w];
+            C += red[1][w];
+            F += red[2][w];
         }
-        return;
+        atomicAdd(&sums->S, S);
+        atomicAdd(&sums->cells[0], C);
+        if (F) atomicAdd(&sums->full[0], F);
+        __threadfence();
+        *s_last = atomicAdd(&a.mg.done[ti], 1) == un.splits - 1;
     }
-    // Each task's own increments for the unstable events, on top of the
-    // common counts: the centre, then the left half, then the right half.  A
-    // thread's first listed event stays in registers (offsets and its three
-    // scales) through the five passes; further ones are read again.
-    unsigned long long Sp = 0, Sl = 0, Sr = 0, Sx = 0;
-    uint32_t Cp = 0, Cl = 0, Cr = 0, Fl = 0, Fr = 0, Cx = 0, Fx = 0;
-    int e1 = -1;
-    float ex = 0.0f, ey = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
-    if ((int)threadIdx.x < n) {
-        e1 = list[threadIdx.x];
-        const Ev v = p.ev[e1];
-        ex = v.dx;
-        ey = v.dy;
-        s1 = warp_s(lo, v.t, glo);
-        s2 = warp_s(c, v.t, gc);
-        s3 = warp_s(hi, v.t, ghi);
+    work_sync();
+    if (!*s_last) return;                         // another split finishes the band
+    __threadfence();                              // every split's additions are visible now
+    for (int i = threadIdx.x; i < rows * W; i += work_threads()) {
+        if (out) out[i] = __ldcg(&acc[i]);
+        acc[i] = 0u;
     }
-    auto each = [&](auto&& f) {
-        if (e1 >= 0) f(e1, ex, ey, s1, s2, s3);
-        for (int i = threadIdx.x + blockDim.x; i < n; i += blockDim.x) {
-            const int e = list[i];
-            const Ev v = p.ev[e];
-            f(e, v.dx, v.dy, warp_s(lo, v.t, glo), warp_s(c, v.t, gc), warp_s(hi, v.t, ghi));
-        }
-    };
-    each([&](int, float dx, float dy, float, float b, float) {
-        point_event<BUMP_SPARSE>(g, dx, dy, b, y0, y1, tile, Sp, Cp);
-    });
-    __syncthreads();
-    each([&](int, float dx, float dy, float, float b, float) {
-        point_event<BUMP_UNDO>(g, dx, dy, b, y0, y1, tile, Sx, Cx);
-    });
-    __syncthreads();
-    each([&](int e, float dx, float dy, float a, float b, float) {
-        bound_event<BUMP_SPARSE>(g, p, e, dx, dy, a, b, y0, y1, tile, Sl, Cl, Fl);
-    });
-    __syncthreads();
-    each([&](int e, float dx, float dy, float a, float b, float) {
-        bound_event<BUMP_UNDO>(g, p, e, dx, dy, a, b, y0, y1, tile, Sx, Cx, Fx);
-    });
-    __syncthreads();
-    each([&](int e, float dx, float dy, float, float b, float d) {
-        bound_event<BUMP_SPARSE>(g, p, e, dx, dy, b, d, y0, y1, tile, Sr, Cr, Fr);
-    });
-    __syncthreads();
-
-    // The tile leaves zeroed (its padding column stays zero): 16-byte words,
-    // then the tail.
-    {
-        const int words = rows * P, quads = words >> 2;
-        uint4* t4 = reinterpret_cast<uint4*>(tile);
-        for (int i = threadIdx.x; i < quads; i += blockDim.x) t4[i] = make_uint4(0u, 0u, 0u, 0u);
-        for (int i = 4 * quads + threadIdx.x; i < words; i += blockDim.x) tile[i] = 0u;
-    }
-    // Sums of the three tasks: per warp, then per block (in the list's memory).
-    unsigned long long* wsum = reinterpret_cast<unsigned long long*>(queue.rec);   // [8][MAX_WARPS]
-    auto put = [&](int k, unsigned long long x) {
-        x = warp_sum(x);
-        if (lane == 0) wsum[k * MAX_WARPS + wid] = x;
-    };
-    put(0, SC + Sp);
-    put(1, (unsigned long long)NC + Cp);
-    put(2, SC + Sl);
-    put(3, (unsigned long long)NC + Cl);
-    put(4, (unsigned long long)NC + Fl);
-    put(5, SC + Sr);
-    put(6, (unsigned long long)NC + Cr);
-    put(7, (unsigned long long)NC + Fr);
-    __syncthreads();
-    if (threadIdx.x < 8) {
-        const int k = threadIdx.x;
-        unsigned long long t = 0;
-        for (int w = 0; w < nw; w++) t += wsum[k * MAX_WARPS + w];
-        // k: 0 centre S, 1 centre N_in, then S, cells, N_full of the left (2-4) and right (5-7) halves
-        Partial* q = k < 2 ? part_p : (k < 5 ? part_l : part_r);
-        const int f = k < 2 ? k : (k < 5 ? k - 2 : k - 5);
-        unsigned long long* dst = f == 0 ? &q->S : (f == 1 ? &q->cells[plane] : &q->full[plane]);
-        if (t) atomicAdd(dst, t);
+    if (threadIdx.x == 0) {
+        S = atomicExch(&sums->S, 0ull);
+        C = atomicExch(&sums->cells[0], 0ull);
+        F = atomicExch(&sums->full[0], 0ull);
+        a.mg.done[ti] = 0;
+        if (S) atomicAdd(&part->S, S);
+        if (C) atomicAdd(&part->cells[un.plane], C);
+        if (F) atomicAdd(&part->full[un.plane], F);
     }
 }
 
-constexpr int Q_STAGE = 256;   // queued intervals staged in shared memory for the merge
+// A unit's sums in shared memory, one entry per warp: [0..2] S, cells and
+// N_full of the point, the bound or a fused unit's centre, [3..5] and [6..8]
+// of its left and right halves.
+constexpr int UNIT_SUMS = 9;
 
-// Shared memory of one control step (one block of k_control per window).
-struct __align__(16) CtlShared {
-    SolveState s;
-    i128 key[3 * MAX_POP];
-    unsigned long long cells[3 * MAX_POP];
-    Node kids[2 * MAX_POP + 1];
-    Node sorted_kids[2 * MAX_POP + 1];
-    Node q_stage[Q_STAGE];
-    Node q_head[MAX_POP];               // the merged queue's first entries, for the dequeue
-    float2 bound_iv[3 * MAX_POP];       // the next round's bound tasks' intervals
-    int16_t t_fuse[3 * MAX_POP];        // per next-round task: 0 own jobs, -1 part of a fused
-                                        // job, k > 0 the centre of a fused job (left half k - 1)
-    int8_t t_dense[3 * MAX_POP];        // per next-round task: a dense bound that may be split
-    int16_t t_jobs[3 * MAX_POP];        // per next-round task, in job order: its number of jobs
-    int s_nk, s_stop;
-};
+// One warp adds n of the warps' sums (rows 0.. of `red`) to the tasks' sums
+// k0.. (per plane).
+__device__ __forceinline__ void add_sums(const EvalArgs& a, const Unit& un, unsigned long long (*red)[MAX_WARPS],
+                                         int n, int k0 = 0) {
+    const int lane = threadIdx.x & 31, nw = work_warps();
+    Partial* wp = a.part + (size_t)un.win * a.task_stride;
+    for (int k = k0; k < k0 + n; k++) {
+        const unsigned long long t = warp_total(lane < nw ? red[k - k0][lane] : 0ull);
+        if (lane == 0 && t) {
+            Partial* q = wp + (k < 3 ? un.task : un.left + (k >= 6));
+            const int f = k % 3;
+            atomicAdd(f == 0 ? &q->S : (f == 1 ? &q->cells[un.plane] : &q->full[un.plane]), t);
+        }
+    }
+}
 
+// The pass of a point or bound unit and its warps' sums.  Images and dense
+// sums are read from the finished tile.  Ends before the barrier after which
+// the sums may be read and the tile cleared.
+__device__ __forceinline__ void single_unit(const Geom& g, const EvalArgs& a, const Unit& un, const Tile& T, int kind,
+                                            float Dl, float Dh, uint32_t* scratch, uint32_t* out,
+                                            unsigned long long (*red)[MAX_WARPS], int* s_last) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = work_warps();
+    unsigned long long V = 0, C = 0, F = 0, S;
+    if (kind == UNIT_POINT) point_pass(g, un, T, Dl, V, C);
+    else if (kind == UNIT_DENSE) bound_pass<true>(g, un, T, Dl, Dh, scratch, V, C, F);
+    else bound_pass<false>(g, un, T, Dl, Dh, scratch, V, C, F);
+    S = 2 * V + C;
+    if (un.splits > 1) {
+        work_sync();
+        merge_split(g, a, un, T, a.part + (size_t)un.win * a.task_stride + un.task, out, F, red, s_last);
+        return;
+    }
+    if (out) {
+        // Tile rows have pitch P, frame rows pitch W: warps take rows, lanes
+        // take columns.
+        work_sync();
+        for (int r = wid; r < un.rows; r += nw)
+            for (int c = lane; c < g.W; c += 32)
+                if (DD_IN(r * g.W + c, un.rows * g.W, 16u)) out[r * g.W + c] = T.cell[r * tile_pitch(g) + c];
+    }
+    if (kind == UNIT_DENSE) {
+        // The band's rows are contiguous in the tile (the padding column of an
+        // odd pitch stays zero): 16-byte words, then the tail.
+        work_sync();
+        const int words = un.rows * tile_pitch(g), quads = words >> 2;
+        const uint4* t4 = reinterpret_cast<const uint4*>(T.cell);
+        S = C = 0;
+        for (int i = threadIdx.x; i < quads; i += work_threads()) {
+            const uint4 v = t4[i];
+            S += (unsigned long long)v.x * v.x + (unsigned long long)v.y * v.y + (unsigned long long)v.z * v.z +
+                 (unsigned long long)v.w * v.w;
+            C += (unsigned long long)v.x + v.y + v.z + v.w;
+        }
+        for (int i = 4 * quads + threadIdx.x; i < words; i += work_threads()) {
+            const uint32_t v = T.cell[i];
+            S += (unsigned long long)v * v;
+            C += v;
+        }
+    }
+    S = warp_total(S);
+    C = kind == UNIT_DENSE || un.chunks > (1 << 20) ? warp_total(C) : __reduce_add_sync(0xffffffffu, (uint32_t)C);
+    if (kind != UNIT_POINT) F = __reduce_add_sync(0xffffffffu, (uint32_t)F);
+    if (lane == 0) {
+        red[0][wid] = S;
+        red[1][wid] = C;
+        red[2][wid] = F;
+    }
+}
 
-__host__ __device__ inline size_t eval_smem_bytes(const Geom& g, int threads) {
-    return sizeof(uint32_t) * (size_t)eval_tile_words(g) + sizeof(int) * (size_t)QREC * QUEUE * (threads / 32);
+// A fused unit and its warps' sums; if its list or a field overflows, its
+// three tasks run as ordinary units over the same candidates.  Returns the
+// number of sums left in `red`.
+__device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, const Unit& un, const Tile& T,
+                                          int tile_words, uint32_t* scratch, unsigned long long (*red)[MAX_WARPS],
+                                          int* s_over, int* s_last) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    FusedSums q = {};
+    if (fused_pass(g, un, T, scratch, s_over, q)) {
+        const unsigned long long S0 = 2 * q.V[0] + q.n;
+        auto put = [&](int k, unsigned long long x) {
+            x = warp_total(x);
+            if (lane == 0) red[k][wid] = x;
+        };
+        auto put32 = [&](int k, uint32_t x) {
+            x = __reduce_add_sync(0xffffffffu, x);
+            if (lane == 0) red[k][wid] = x;
+        };
+        put(0, S0 + 2 * q.V[1] + q.C[0]);
+        put32(1, q.n + q.C[0]);
+        if (lane == 0) red[2][wid] = 0;
+        put(3, S0 + 2 * q.V[2] + q.C[1]);
+        put32(4, q.n + q.C[1]);
+        put32(5, q.n + q.F[0]);
+        put(6, S0 + 2 * q.V[3] + q.C[2]);
+        put32(7, q.n + q.C[2]);
+        put32(8, q.n + q.F[1]);
+        return 9;
+    }
+    const int kind = bound_cells(g, un.D_lo, un.D_hi, un.tau) >= DENSE_CELLS ? UNIT_DENSE : UNIT_BOUND;
+    for (int k = 0; k < 3; k++) {
+        work_sync();
+        if (threadIdx.x == 0) clear_tile(T.cell, tile_words);
+        work_sync();
+        single_unit(g, a, un, T, k == 0 ? UNIT_POINT : kind, k == 1 ? un.D_lo : un.D_c, k == 1 ? un.D_c : un.D_hi,
+                    scratch, nullptr, red, s_last);
+        work_sync();
+        if (wid == 0) add_sums(a, un, red, 3, 3 * k);
+    }
+    return 0;
 }
 
 // IWE evaluation of the round's job list.  A grid of resident blocks takes
-// units (job, row band) from a counter; block 0 clears the other parity's
-// list and counter for the control blocks of this round.
-__global__ void __launch_bounds__(512, 3) k_eval(Geom g, EvalArgs a) {
+// units (job, row band).  The last warp of a block only prepares units, one
+// ahead of the others: a unit's preparation is a chain of dependent L2 loads
+// (its number, job, task, bin offsets) that takes longer than a small unit's
+// pass over its events.  Per unit there is one barrier of the whole block
+// (the unit is prepared, the tile is clear) and one of the working warps (the
+// pass is done), after which the sums go to the tasks and the tile is cleared
+// by different warps.  Block b starts with unit b; later units come from a
+// counter, which numbers them from gridDim.x on.  Block 0 clears the other
+// parity's list and counter for the control blocks of this round.
+//
+// What bounds it: with many units, issue slots (60 bounds of 100,000 events:
+// 70-84% of the cycles issue, DRAM under 1%), so the passes are written for
+// few instructions per event and cell; with few units, the latency of a unit
+// (its preparation 2.7 us, two barriers, one L2 round trip per four chunks).
+// Two blocks of 480 + 32 threads per SM with 64 registers a thread and tiles
+// of up to 96 KB: three of 256 + 32 with smaller tiles are 4% faster on
+// 640-pixel frames in late rounds but 29% slower on 1280-pixel ones, where
+// the lower tile re-reads more events.  Against one thread deciding each
+// unit's split, candidates and sums in every warp (512 threads, 3 blocks of 40
+// registers): 129 points of 100,000 events 74 -> 50 us, 60 bounds of width
+// 1/2 569 -> 340 us, of width 1/32 124 -> 90 us; 256 uneven windows 97.8 ->
+// 64.2 ms, 96 windows of a 1280x720 stream 112.0 -> 66.2 ms.
+__global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_eval(Geom g, EvalArgs a) {
     extern __shared__ __align__(16) uint32_t tile[];
-    __shared__ unsigned long long red[3][32];
-    __shared__ int erange[2 * MAX_TB + 1];
-    __shared__ int s_unit, s_last, s_n;
+    __shared__ Unit s_un[2];
+    __shared__ unsigned long long red[UNIT_SUMS][MAX_WARPS];
+    __shared__ int s_last, s_over;
+    __shared__ uint32_t s_idle[32];
     Sched* sch = a.sch;
     const int par = sch->round & 1;
     const int n_units = sch->n_jobs[par] * g.n_tiles;
@@ -1109,55 +1180,53 @@ __global__ void __launch_bounds__(512, 3) k_eval(Geom g, EvalArgs a) {
         sch->n_jobs[par ^ 1] = 0;
         sch->work[par ^ 1] = 0;
     }
-    if (n_units == 0) return;
-    int32_t* work = &sch->work[par];
-    const Job* jobs = a.jobs + (size_t)par * a.job_stride;
-    const int tile_words = g.band_rows * tile_pitch(g);
-    SegQueue queue;
-    queue.rec = reinterpret_cast<int*>(tile + eval_tile_words(g));
-    queue.cap = (int)(blockDim.x >> 5) * QUEUE;
-    const int bins1 = bins_of(g) + 1;
-    const size_t task_cells = (size_t)g.planes * g.W * g.H;
-    // Block b starts with unit b; later units come from the counter, which
-    // numbers them from gridDim.x on.  The counter is asked when a unit
-    // starts and its answer stored only when the unit ends, so no warp waits
-    // for it; the unit's own barriers order every thread's read of s_unit
-    // before that store.
-    if (threadIdx.x == 0) s_unit = blockIdx.x;
-    for (int i = threadIdx.x; i < tile_words; i += blockDim.x) tile[i] = 0u;
-    __syncthreads();
-    for (;;) {
-        const int u = s_unit;
-        if (u >= n_units) break;
-        int next = 0;
-        if (threadIdx.x == 0) next = atomicAdd(work, 1);
-        const int j = u / g.n_tiles, ti = u - j * g.n_tiles;
-        const Job jb = jobs[j];
-        const int64_t ev_off = a.wins[jb.win].ev_off;
-        const float tau = a.wins[jb.win].tau;
-        const Task* wt = a.tasks + (size_t)jb.win * a.task_stride;
-        const Task tk = wt[jb.task];
-        UnitPtrs p;
-        p.ev = a.ev + ev_off;
-        p.rcp = a.rcp + ev_off;
-#ifdef DD_CHECKED
-        p.n_ev = a.wins[jb.win].n;
-#endif
-        p.row_off = a.row_off + (size_t)jb.win * bins1;
-        p.part = a.part + ((size_t)jb.win * a.task_stride + jb.task);
-        p.out = a.iwe_out ? a.iwe_out + (size_t)jb.task * task_cells : nullptr;
-        p.acc = a.mg.acc ? a.mg.acc + (size_t)jb.task * task_cells : nullptr;
-        p.done = a.mg.done ? a.mg.done + (size_t)jb.task * g.n_tiles : nullptr;
-        p.sums = a.mg.sums ? a.mg.sums + (size_t)jb.task * g.n_tiles : nullptr;
-        if (jb.splits < 0) {                      // one expanded interval: its three tasks together
-            Partial* wp = a.part + (size_t)jb.win * a.task_stride;
-            eval_fused_unit(g, p, tk, wt[jb.split], wt[jb.split + 1], wp + jb.task, wp + jb.split,
-                            wp + jb.split + 1, ti, tau, tile, red, erange, &s_n, &s_last, queue);
-        } else {
-            eval_unit(g, p, tk, ti, jb.split, max(1, jb.splits), tau, tile, red, erange, &s_last, queue);
+    if ((int)blockIdx.x >= n_units) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = work_warps();
+    if (wid == nw) {                              // the preparing warp
+        const Job* jobs = a.jobs + (size_t)par * a.job_stride;
+        int id = blockIdx.x;
+        for (int b = 0;; b ^= 1) {
+            prepare_unit(g, a, jobs, id, n_units, s_un[b]);
+            __syncthreads();
+            if (id >= n_units) return;
+            id = n_units;
+            if (lane == 0 && n_units > (int)gridDim.x) id = (int)gridDim.x + atomicAdd(&sch->work[par], 1);
+            id = __shfl_sync(0xffffffffu, id, 0);
         }
-        if (threadIdx.x == 0) s_unit = gridDim.x + next;
-        __syncthreads();                          // the unit is done; s_unit is set
+    }
+    const int tile_words = eval_tile_words(g);
+    uint32_t* scratch = tile + tile_words + WARP_WORDS * wid;
+    if (threadIdx.x == 0) {
+        clear_tile(tile, tile_words);
+        s_over = 0;
+    }
+    for (int b = 0;; b ^= 1) {
+        __syncthreads();                          // unit b is prepared, the tile is clear
+        const Unit& un = s_un[b];
+        if (un.kind == UNIT_NONE) return;
+        Tile T;
+        T.cell = tile;
+        T.pitch = 4u * (uint32_t)tile_pitch(g);
+        T.idle = (uint32_t)__cvta_generic_to_shared(s_idle + lane);
+        T.row0 = CELL0 + (uint32_t)un.y0;
+        T.base = (uint32_t)__cvta_generic_to_shared(tile) - T.row0 * T.pitch - 4u * CELL0;
+        T.rows = (uint32_t)un.rows;
+        T.W = (uint32_t)g.W;
+        int sums = 3;
+        if (un.kind == UNIT_FUSED) {
+            sums = fused_unit(g, a, un, T, tile_words, scratch, red, &s_over, &s_last);
+        } else {
+            uint32_t* out = a.iwe_out ? a.iwe_out + ((size_t)un.task * g.planes + un.plane) * g.W * g.H + (size_t)un.y0 * g.W
+                                      : nullptr;
+            single_unit(g, a, un, T, un.kind, un.D_lo, un.D_hi, scratch, out, red, &s_last);
+            if (un.splits > 1) sums = 0;
+        }
+        work_sync();                              // the pass is done
+        if (threadIdx.x == 0) {
+            clear_tile(tile, tile_words);
+            s_over = 0;
+        }
+        if (wid == nw - 1 && sums) add_sums(a, un, red, sums);
     }
 }
 
@@ -1182,7 +1251,7 @@ cudaError_t check_flags(uint32_t* flags, int32_t* checked, bool reset) {
 int eval_resident_blocks(const Geom& g, int threads) {
     int per_sm = 0, dev = 0, sms = 0;
     const size_t smem = eval_smem_bytes(g, threads);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eval, threads, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eval, threads + 32, smem) != cudaSuccess) return 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     return per_sm * sms;
@@ -1190,7 +1259,7 @@ int eval_resident_blocks(const Geom& g, int threads) {
 
 cudaError_t launch_eval(const Geom& g, const EvalArgs& a, int threads, int grid_blocks, cudaStream_t s) {
     if (grid_blocks <= 0) return cudaErrorInvalidValue;
-    k_eval<<<grid_blocks, threads, eval_smem_bytes(g, threads), s>>>(g, a);
+    k_eval<<<grid_blocks, threads + 32, eval_smem_bytes(g, threads), s>>>(g, a);
     return cudaGetLastError();
 }
 
@@ -1216,6 +1285,25 @@ cudaError_t launch_keys(const Geom& g, const Task* tasks, int32_t n_tasks, Parti
     k_keys<<<(n_tasks + 63) / 64, 64, 0, s>>>(g, tasks, n_tasks, part, key, S, cells, full);
     return cudaGetLastError();
 }
+
+constexpr int Q_STAGE = 256;   // queued intervals staged in shared memory for the merge
+
+// Shared memory of one control step (one block of k_control per window).
+struct __align__(16) CtlShared {
+    SolveState s;
+    i128 key[3 * MAX_POP];
+    unsigned long long cells[3 * MAX_POP];
+    Node kids[2 * MAX_POP + 1];
+    Node sorted_kids[2 * MAX_POP + 1];
+    Node q_stage[Q_STAGE];
+    Node q_head[MAX_POP];               // the merged queue's first entries, for the dequeue
+    float2 bound_iv[3 * MAX_POP];       // the next round's bound tasks' intervals
+    int16_t t_fuse[3 * MAX_POP];        // per next-round task: 0 own jobs, -1 part of a fused
+                                        // job, k > 0 the centre of a fused job (left half k - 1)
+    int8_t t_dense[3 * MAX_POP];        // per next-round task: a dense bound that may be split
+    int16_t t_jobs[3 * MAX_POP];        // per next-round task, in job order: its number of jobs
+    int s_nk, s_stop;
+};
 
 __device__ __forceinline__ float centre(float lo, float hi) {
     return __fadd_rn(lo, __fmul_rn(0.5f, __fsub_rn(hi, lo)));

@@ -19,8 +19,7 @@ constexpr int NA_MAX_TILES = 1024;   // row bands of one frame (at most 683 for 
 // Byte offsets of the sub-buffers inside the static array (each 256-aligned).
 constexpr size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 constexpr size_t OFF_EV = 0;
-constexpr size_t OFF_RCP = align256(OFF_EV + sizeof(dd::Ev) * NA_MAX_EVENTS);
-constexpr size_t OFF_ROW_COUNT = align256(OFF_RCP + sizeof(float2) * NA_MAX_EVENTS);
+constexpr size_t OFF_ROW_COUNT = align256(OFF_EV + sizeof(dd::Ev) * NA_MAX_EVENTS);
 constexpr size_t OFF_ROW_OFF = align256(OFF_ROW_COUNT + sizeof(int32_t) * NA_MAX_ROWS);
 constexpr size_t OFF_CURSOR = align256(OFF_ROW_OFF + sizeof(int32_t) * (NA_MAX_ROWS + 1));
 constexpr size_t OFF_ERR = align256(OFF_CURSOR + sizeof(int32_t) * NA_MAX_ROWS);
@@ -112,7 +111,6 @@ extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_
 
     cudaStream_t s = (cudaStream_t)stream;
     dd::Ev* ev_sorted = (dd::Ev*)(base + OFF_EV);
-    float2* rcp = (float2*)(base + OFF_RCP);
     int32_t* row_count = (int32_t*)(base + OFF_ROW_COUNT);
     int32_t* row_off = (int32_t*)(base + OFF_ROW_OFF);
     int32_t* cursor = (int32_t*)(base + OFF_CURSOR);
@@ -149,12 +147,11 @@ extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_
     if (n_chunks &&
         cudaMemcpyAsync(chunk_win, h_chunks, sizeof(int32_t) * n_chunks, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return DD_ERR_CUDA;
-    if (dd::launch_ingest(g, win, 1, chunk_win, n_chunks, ev_sorted, rcp, row_count, row_off, cursor, err, s) !=
+    if (dd::launch_ingest(g, win, 1, chunk_win, n_chunks, ev_sorted, row_count, row_off, cursor, err, s) !=
         cudaSuccess)
         return DD_ERR_CUDA;
     dd::EvalArgs a{};
     a.ev = ev_sorted;
-    a.rcp = rcp;
     a.row_off = row_off;
     a.wins = win;
     a.tasks = tasks;
@@ -169,7 +166,7 @@ extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_
     dd::Sched h_sch;
     dd::i128 h_keys[NA_MAX_TASKS];
     int32_t h_err = 0;
-    const int grid = dd::eval_resident_blocks(g, 512);
+    const int grid = dd::eval_resident_blocks(g, dd::EVAL_THREADS);
     if (grid <= 0) return DD_ERR_CUDA;
     for (int32_t j0 = 0; j0 < nD || j0 == 0; j0 += NA_MAX_TASKS) {
         const int32_t m = nD - j0 < NA_MAX_TASKS ? nD - j0 : NA_MAX_TASKS;
@@ -190,7 +187,7 @@ extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_
                 cudaMemcpyAsync(sch, &h_sch, sizeof(h_sch), cudaMemcpyHostToDevice, s) != cudaSuccess)
                 return DD_ERR_CUDA;
             if (cudaMemsetAsync(part, 0, sizeof(dd::Partial) * m, s) != cudaSuccess) return DD_ERR_CUDA;
-            if (dd::launch_eval(g, a, 512, grid, s) != cudaSuccess) return DD_ERR_CUDA;
+            if (dd::launch_eval(g, a, dd::EVAL_THREADS, grid, s) != cudaSuccess) return DD_ERR_CUDA;
             if (dd::launch_keys(g, tasks, m, part, keys, S, C, F, s) != cudaSuccess) return DD_ERR_CUDA;
             if (cudaMemcpyAsync(h_keys, keys, sizeof(dd::i128) * m, cudaMemcpyDeviceToHost, s) != cudaSuccess)
                 return DD_ERR_CUDA;

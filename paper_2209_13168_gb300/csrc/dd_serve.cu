@@ -73,7 +73,6 @@ struct dd_server {
 
     // device, per slot
     dd::Ev* ev = nullptr;
-    float2* rcp = nullptr;
     int16_t *in_x = nullptr, *in_y = nullptr;
     float* in_t = nullptr;
     int8_t* in_p = nullptr;       // polarities (two planes only)
@@ -128,7 +127,6 @@ void release_host(T*& p) {
 
 void free_server(dd_server* s) {
     release(s->ev);
-    release(s->rcp);
     release(s->in_x);
     release(s->in_y);
     release(s->in_t);
@@ -162,7 +160,7 @@ void free_server(dd_server* s) {
 }
 
 size_t slot_bytes(const dd_server* s) {
-    return (size_t)s->E * (sizeof(dd::Ev) + sizeof(float2) + 2 * sizeof(int16_t) + sizeof(float) +
+    return (size_t)s->E * (sizeof(dd::Ev) + 2 * sizeof(int16_t) + sizeof(float) +
                            (s->g.planes > 1 ? sizeof(int8_t) : 0)) +
            sizeof(int32_t) * (3 * (size_t)s->bins + 1) + sizeof(dd::SolveState) +
            sizeof(dd::Node) * 2 * (size_t)s->qcap + sizeof(dd::Task) * (size_t)s->max_tasks +
@@ -179,7 +177,6 @@ int alloc_server(dd_server* s) {
     };
     const size_t S = (size_t)s->S, E = (size_t)s->E;
     A((void**)&s->ev, sizeof(dd::Ev) * S * E);
-    A((void**)&s->rcp, sizeof(float2) * S * E);
     A((void**)&s->in_x, sizeof(int16_t) * S * E);
     A((void**)&s->in_y, sizeof(int16_t) * S * E);
     A((void**)&s->in_t, sizeof(float) * S * E);
@@ -288,7 +285,7 @@ cudaError_t start_search(dd_server* s, int k, const Request& r, int sharers) {
     c = cudaMemcpyAsync(s->params + k, &q, sizeof(dd::WinParams), cudaMemcpyHostToDevice, s->stream);
     if (c != cudaSuccess) return c;
     const int32_t n_chunks = (int32_t)((e.n + dd::CHUNK - 1) / dd::CHUNK);
-    c = dd::launch_ingest(s->g, s->wins + k, 1, s->chunk_zero, n_chunks, s->ev, s->rcp,
+    c = dd::launch_ingest(s->g, s->wins + k, 1, s->chunk_zero, n_chunks, s->ev,
                           s->row_count + (size_t)k * s->bins, s->row_off + (size_t)k * (s->bins + 1),
                           s->cursor + (size_t)k * s->bins, s->err + k, s->stream);
     if (c != cudaSuccess) return c;
@@ -378,7 +375,6 @@ void loop(dd_server* s) {
     const int64_t M = (int64_t)s->g.W * s->g.H;
     dd::EvalArgs a{};
     a.ev = s->ev;
-    a.rcp = s->rcp;
     a.row_off = s->row_off;
     a.wins = s->wins;
     a.tasks = s->tasks;
