@@ -20,6 +20,7 @@ struct dd_ctx {
     int threads = 512;
     int max_tasks = 0;            // task slots per window
     int eval_blocks = 0;          // resident blocks of the evaluation grid
+    int search_blocks = 0;        // resident blocks of a one-launch search (0: not available)
     cudaStream_t own = nullptr, stream = nullptr;
 
     // events: sorted, for all windows of a call
@@ -544,9 +545,19 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
                            (int32_t)trace_cap, c->stream));
     c->stats.kernel_launches++;
     dd::TraceRec* tr_dev = trace_cap > 0 ? c->trace : nullptr;
-    const bool graph = !c->cfg.host_loop && !c->timing;
+    // One window: all rounds in one cooperative launch.  Several: one graph
+    // launch, whose control step runs one block per window at once.
+    const bool device = !c->cfg.host_loop && !c->timing;
+    const bool search = device && nw == 1 && c->search_blocks > 1 && evs[0].n <= dd::SEARCH_MAX_EVENTS;
+    const bool graph = device && !search;
     dd::NvtxRange rounds("dd rounds");
-    if (graph) {
+    if (search) {
+        const dd::CtlArgs ctl = dd::control_args(1, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err, tr_dev,
+                                                 c->jobs, c->job_stride, c->sch, 0, 0, 1, nullptr);
+        DD_TRY(dd::launch_search(c->g, eval_args(c, nullptr, true), ctl, c->threads, c->search_blocks, c->stream));
+        c->stats.kernel_launches++;
+        c->stats.eval_launches++;
+    } else if (graph) {
         // One graph launch runs every round on the device.
         if (!c->gexec || c->g_nw != nw || c->g_key[0] != (const void*)c->ev || c->g_key[1] != (const void*)tr_dev ||
             c->g_key[2] != (const void*)c->st) {
@@ -576,6 +587,14 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
     std::vector<dd::TraceRec> tr((size_t)trace_cap);
     if (trace_cap > 0) DD_TRY(copy(c, tr.data(), c->trace, sizeof(dd::TraceRec) * trace_cap, cudaMemcpyDeviceToHost));
     DD_TRY(sync(c));
+    if (search && c->h_sch->failed) {             // a wait ran out: leave the merge buffers as they must be
+        const size_t M1 = (size_t)c->g.planes * M, tiles = (size_t)c->max_tasks * c->g.n_tiles;
+        DD_TRY(cudaMemsetAsync(c->macc, 0, sizeof(uint32_t) * (size_t)c->max_tasks * M1, c->stream));
+        DD_TRY(cudaMemsetAsync(c->mdone, 0, sizeof(int32_t) * tiles, c->stream));
+        DD_TRY(cudaMemsetAsync(c->msums, 0, sizeof(dd::Partial) * tiles, c->stream));
+        DD_TRY(sync(c));
+        return DD_ERR_CUDA;
+    }
     if (graph) {                                  // every round ran one evaluation and one control launch
         c->stats.kernel_launches += 2 * (int64_t)c->h_sch->round;
         c->stats.eval_launches += c->h_sch->round;
@@ -779,7 +798,8 @@ int dd_create(int32_t W, int32_t H, float foe_x, float foe_y, const dd_config* c
     if (rc == DD_OK && cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking) != cudaSuccess) rc = DD_ERR_CUDA;
     if (rc == DD_OK && dd::eval_smem_setup(c->g) != cudaSuccess) rc = DD_ERR_CUDA;
     if (rc == DD_OK && (c->eval_blocks = dd::eval_resident_blocks(c->g, c->threads)) <= 0) rc = DD_ERR_CUDA;
-    c->g.split_target = c->eval_blocks;
+    c->g.split_target = c->eval_blocks > 1 ? c->eval_blocks - 1 : c->eval_blocks;   // a search keeps one for its control
+    if (rc == DD_OK) c->search_blocks = dd::search_resident_blocks(c->g, c->threads);
     if (rc == DD_OK) rc = ensure_windows(c, 1);
     if (rc != DD_OK) {
         dd_destroy(c);

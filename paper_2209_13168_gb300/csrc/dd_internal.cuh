@@ -155,6 +155,8 @@ struct Sched {
     int32_t n_jobs[2];
     int32_t work[2];
     int32_t ticket, active, running;
+    int32_t failed, pad;           // k_search: a block gave up waiting for the others
+    unsigned long long go;         // k_search: (next round) << 32 | its jobs
 };
 
 // Geometry of a context.  Events are sorted by (polarity plane, time
@@ -285,6 +287,13 @@ cudaError_t launch_ingest(const Geom& g, const WinIn* wins_dev, int32_t n_window
                           int32_t* cursor, int32_t* err, cudaStream_t s);
 cudaError_t launch_eval(const Geom& g, const EvalArgs& a, int threads, int grid_blocks, cudaStream_t s);
 int eval_resident_blocks(const Geom& g, int threads);
+// All rounds of one window's search in one cooperative launch of at most
+// search_resident_blocks blocks, for windows of at most SEARCH_MAX_EVENTS
+// events (a round's waits are bounded).
+constexpr int64_t SEARCH_MAX_EVENTS = 1 << 22;
+int search_resident_blocks(const Geom& g, int threads);
+cudaError_t launch_search(const Geom& g, const EvalArgs& a, const CtlArgs& c, int threads, int grid_blocks,
+                          cudaStream_t s);
 cudaError_t launch_keys(const Geom& g, const Task* tasks, int32_t n_tasks, Partial* part, i128* key,
                         unsigned long long* S, unsigned long long* cells, unsigned long long* full,
                         cudaStream_t s);

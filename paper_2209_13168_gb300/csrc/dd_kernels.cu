@@ -496,7 +496,7 @@ constexpr int MAX_WARPS = 16;     // working warps of a k_eval block (at most 51
 __device__ __forceinline__ int work_threads() { return (int)blockDim.x - 32; }
 __device__ __forceinline__ int work_warps() { return ((int)blockDim.x >> 5) - 1; }
 __device__ __forceinline__ void work_sync() {     // a barrier of the working warps
-    asm volatile("bar.sync 1, %0;" : : "r"(work_threads()) : "memory");
+    __barrier_sync_count(1, work_threads());
 }
 
 // Shared scratch of one working warp (WARP_WORDS words of dynamic shared
@@ -1152,7 +1152,7 @@ __device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, cons
 // (the unit is prepared, the tile is clear) and one of the working warps (the
 // pass is done), after which the sums go to the tasks and the tile is cleared
 // by different warps.  Block b starts with unit b; later units come from a
-// counter, which numbers them from gridDim.x on.  Block 0 clears the other
+// counter, which numbers them from the number of blocks on.  Block 0 clears the other
 // parity's list and counter for the control blocks of this round.
 //
 // What bounds it: with many units, issue slots (60 bounds of 100,000 events:
@@ -1167,12 +1167,65 @@ __device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, cons
 // registers): 129 points of 100,000 events 74 -> 50 us, 60 bounds of width
 // 1/2 569 -> 340 us, of width 1/32 124 -> 90 us; 256 uneven windows 97.8 ->
 // 64.2 ms, 96 windows of a 1280x720 stream 112.0 -> 66.2 ms.
-__global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_eval(Geom g, EvalArgs a) {
+struct EvalShared {
+    Unit un[2];
+    unsigned long long red[UNIT_SUMS][MAX_WARPS];
+    uint32_t idle[32];
+    int last, over;
+};
+
+// The share of block `block` of `blocks` in a round of n_units units.  The tile arrives clear and
+// leaves clear; ends with a barrier of the whole block.
+__device__ __forceinline__ void eval_round(const Geom& g, const EvalArgs& a, const Job* jobs, int32_t* work, int n_units,
+                                           int block, int blocks, uint32_t* tile, EvalShared& sm) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = work_warps();
+    if (wid == nw) {                              // the preparing warp
+        int id = block;
+        for (int b = 0;; b ^= 1) {
+            prepare_unit(g, a, jobs, id, n_units, sm.un[b]);
+            __syncthreads();
+            if (id >= n_units) return;
+            id = n_units;
+            if (lane == 0 && n_units > blocks) id = blocks + atomicAdd(work, 1);
+            id = __shfl_sync(0xffffffffu, id, 0);
+        }
+    }
+    const int tile_words = eval_tile_words(g);
+    uint32_t* scratch = tile + tile_words + WARP_WORDS * wid;
+    for (int b = 0;; b ^= 1) {
+        __syncthreads();                          // unit b is prepared, the tile is clear
+        const Unit& un = sm.un[b];
+        if (un.kind == UNIT_NONE) return;
+        Tile T;
+        T.cell = tile;
+        T.pitch = 4u * (uint32_t)tile_pitch(g);
+        T.idle = (uint32_t)__cvta_generic_to_shared(sm.idle + lane);
+        T.row0 = CELL0 + (uint32_t)un.y0;
+        T.base = (uint32_t)__cvta_generic_to_shared(tile) - T.row0 * T.pitch - 4u * CELL0;
+        T.rows = (uint32_t)un.rows;
+        T.W = (uint32_t)g.W;
+        int sums = 3;
+        if (un.kind == UNIT_FUSED) {
+            sums = fused_unit(g, a, un, T, tile_words, scratch, sm.red, &sm.over, &sm.last);
+        } else {
+            uint32_t* out = a.iwe_out ? a.iwe_out + ((size_t)un.task * g.planes + un.plane) * g.W * g.H + (size_t)un.y0 * g.W
+                                      : nullptr;
+            single_unit(g, a, un, T, un.kind, un.D_lo, un.D_hi, scratch, out, sm.red, &sm.last);
+            if (un.splits > 1) sums = 0;
+        }
+        work_sync();                              // the pass is done
+        if (threadIdx.x == 0) {
+            clear_tile(tile, tile_words);
+            sm.over = 0;
+        }
+        if (wid == nw - 1 && sums) add_sums(a, un, sm.red, sums);
+    }
+}
+
+__global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_eval(const __grid_constant__ Geom g,
+                                                               const __grid_constant__ EvalArgs a) {
     extern __shared__ __align__(16) uint32_t tile[];
-    __shared__ Unit s_un[2];
-    __shared__ unsigned long long red[UNIT_SUMS][MAX_WARPS];
-    __shared__ int s_last, s_over;
-    __shared__ uint32_t s_idle[32];
+    __shared__ EvalShared sm;
     Sched* sch = a.sch;
     const int par = sch->round & 1;
     const int n_units = sch->n_jobs[par] * g.n_tiles;
@@ -1181,53 +1234,11 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_eval(Geom g, EvalArgs 
         sch->work[par ^ 1] = 0;
     }
     if ((int)blockIdx.x >= n_units) return;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = work_warps();
-    if (wid == nw) {                              // the preparing warp
-        const Job* jobs = a.jobs + (size_t)par * a.job_stride;
-        int id = blockIdx.x;
-        for (int b = 0;; b ^= 1) {
-            prepare_unit(g, a, jobs, id, n_units, s_un[b]);
-            __syncthreads();
-            if (id >= n_units) return;
-            id = n_units;
-            if (lane == 0 && n_units > (int)gridDim.x) id = (int)gridDim.x + atomicAdd(&sch->work[par], 1);
-            id = __shfl_sync(0xffffffffu, id, 0);
-        }
-    }
-    const int tile_words = eval_tile_words(g);
-    uint32_t* scratch = tile + tile_words + WARP_WORDS * wid;
     if (threadIdx.x == 0) {
-        clear_tile(tile, tile_words);
-        s_over = 0;
+        clear_tile(tile, eval_tile_words(g));
+        sm.over = 0;
     }
-    for (int b = 0;; b ^= 1) {
-        __syncthreads();                          // unit b is prepared, the tile is clear
-        const Unit& un = s_un[b];
-        if (un.kind == UNIT_NONE) return;
-        Tile T;
-        T.cell = tile;
-        T.pitch = 4u * (uint32_t)tile_pitch(g);
-        T.idle = (uint32_t)__cvta_generic_to_shared(s_idle + lane);
-        T.row0 = CELL0 + (uint32_t)un.y0;
-        T.base = (uint32_t)__cvta_generic_to_shared(tile) - T.row0 * T.pitch - 4u * CELL0;
-        T.rows = (uint32_t)un.rows;
-        T.W = (uint32_t)g.W;
-        int sums = 3;
-        if (un.kind == UNIT_FUSED) {
-            sums = fused_unit(g, a, un, T, tile_words, scratch, red, &s_over, &s_last);
-        } else {
-            uint32_t* out = a.iwe_out ? a.iwe_out + ((size_t)un.task * g.planes + un.plane) * g.W * g.H + (size_t)un.y0 * g.W
-                                      : nullptr;
-            single_unit(g, a, un, T, un.kind, un.D_lo, un.D_hi, scratch, out, red, &s_last);
-            if (un.splits > 1) sums = 0;
-        }
-        work_sync();                              // the pass is done
-        if (threadIdx.x == 0) {
-            clear_tile(tile, tile_words);
-            s_over = 0;
-        }
-        if (wid == nw - 1 && sums) add_sums(a, un, red, sums);
-    }
+    eval_round(g, a, a.jobs + (size_t)par * a.job_stride, &sch->work[par], n_units, blockIdx.x, gridDim.x, tile, sm);
 }
 
 // The checked-build error word (always 0 in other builds); reset clears it.
@@ -1302,7 +1313,9 @@ struct __align__(16) CtlShared {
                                         // job, k > 0 the centre of a fused job (left half k - 1)
     int8_t t_dense[3 * MAX_POP];        // per next-round task: a dense bound that may be split
     int16_t t_jobs[3 * MAX_POP];        // per next-round task, in job order: its number of jobs
-    int s_nk, s_stop;
+    int16_t t_at[3 * MAX_POP];          // and the place of its first one in the window's jobs
+    int s_nk, s_stop, s_base;
+    int q_shared;                       // resident: the queue is in the block's shared memory
 };
 
 __device__ __forceinline__ float centre(float lo, float hi) {
@@ -1472,7 +1485,14 @@ __device__ __forceinline__ i128 warp_max_i128(i128 v) {
 // merge into the other buffer, a dequeue takes a prefix.  The last block to
 // finish counts the windows still searching, advances the round and sets the
 // graph loop condition (with one window, its block does so directly).
-__device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, int w, CtlShared& sm) {
+//
+// RESIDENT (the control block of k_search): the state stays in `sm` from round
+// to round, and so does the queue while it has at most q_cap entries (two
+// buffers of q_cap at q_mem); both reach global memory when the search ends
+// or the queue grows beyond that.
+template <bool RESIDENT>
+__device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, int w, CtlShared& sm, int par,
+                                             Node* q_mem = nullptr, int q_cap = 0) {
     SolveState& s = sm.s;
     i128* key = sm.key;
     unsigned long long* cells = sm.cells;
@@ -1484,6 +1504,7 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
     int16_t* t_fuse = sm.t_fuse;
     int8_t* t_dense = sm.t_dense;
     int16_t* t_jobs = sm.t_jobs;
+    int16_t* t_at = sm.t_at;
     int& s_nk = sm.s_nk;
     int& s_stop = sm.s_stop;
     const int32_t n_windows = c.n_windows, task_stride = c.task_stride, job_stride = c.job_stride;
@@ -1498,29 +1519,36 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
     Sched* sch = c.sch;
     int32_t* phase_out = c.phase_out;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int par = sch->round & 1;
-    const int running = sch->running;             // searches still running after the last round
+    const int running = RESIDENT ? 1 : sch->running;   // searches still running after the last round
     SolveState* st = st_all + w;
     Task* tasks = tasks_all + (size_t)w * task_stride;
     Partial* part = part_all + (size_t)w * task_stride;
     Job* jobs = jobs_all + (size_t)(par ^ 1) * job_stride;
     static_assert(sizeof(SolveState) % 16 == 0, "state is copied as int4");
-    for (int i = tid; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
-        reinterpret_cast<int4*>(&s)[i] = reinterpret_cast<const int4*>(st)[i];
-    __syncthreads();
-    if (s.phase != PH_DONE) {
+    if (!RESIDENT) {
+        for (int i = tid; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
+            reinterpret_cast<int4*>(&s)[i] = reinterpret_cast<const int4*>(st)[i];
+        __syncthreads();
+    }
+    const int phase = s.phase;                    // read before a barrier: warp 0 changes it
+    if (phase != PH_DONE) {
     Node* qa = queues + (size_t)w * 2 * s.qcap;
     Node* qb = qa + s.qcap;
     const int32_t* err = err_all + w;
     const int64_t M = s.M;
-    const int n_tasks = s.n_tasks;
+    const int n_tasks = s.n_tasks, n_points = phase == PH_INIT ? 1 : s.n_pop;   // points come first
 
-    // Each task's sums (accumulated by the evaluation over its row bands),
-    // read and cleared for the next round.
+    // Each task's sums (accumulated by the evaluation over its row bands, in
+    // L2), read and cleared for the next round.
     for (int t = tid; t < n_tasks; t += blockDim.x) {
-        const Partial q = part[t];
+        Partial q;
+        q.S = __ldcg(&part[t].S);
+        for (int k = 0; k < 2; k++) {
+            q.cells[k] = __ldcg(&part[t].cells[k]);
+            q.full[k] = __ldcg(&part[t].full[k]);
+        }
         part[t] = Partial{};
-        key[t] = partial_key(M, q, tasks[t].kind == TASK_POINT);
+        key[t] = partial_key(M, q, t < n_points);
         cells[t] = q.cells[0] + q.cells[1];
     }
     __syncthreads();
@@ -1533,7 +1561,7 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
         } else if (s.cancel) {                    // the host cancelled the search between rounds
             if (lane == 0) s.status = DD_ERR_CANCELLED;
             stop = 1;
-        } else if (s.phase == PH_INIT) {
+        } else if (phase == PH_INIT) {
             if (lane == 0) {
                 s.K_hat = key[0];
                 s.point_evals = 1;
@@ -1666,10 +1694,11 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
         // sort the new children, then merge them with the queued intervals;
         // a queue that fits is staged in shared memory first, so that the
         // children's ranks are searched there instead of in global memory
-        const Node* src = (s.q_cur ? qb : qa) + s.q_start;
-        Node* dst = s.q_cur ? qa : qb;
         const int a = s.q_n;
-        const bool staged = a <= Q_STAGE;
+        const bool in_shared = RESIDENT && sm.q_shared, to_shared = RESIDENT && a + nk <= q_cap;
+        const Node* src = (in_shared ? q_mem + (s.q_cur ? q_cap : 0) : (s.q_cur ? qb : qa)) + s.q_start;
+        Node* dst = to_shared ? q_mem + (s.q_cur ? 0 : q_cap) : (s.q_cur ? qa : qb);
+        const bool staged = !in_shared && a <= Q_STAGE;
         // A child's rank among the children (they are distinct: popped
         // intervals are disjoint) counted by `per` threads, each over every
         // per-th child, summed within the thread group.
@@ -1703,6 +1732,7 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
         if (tid == 0) {
             s.q_cur ^= 1;
             s.q_start = 0;
+            sm.q_shared = to_shared;
             s.q_n = a + nk;
             if (s.q_n > s.max_queue) s.max_queue = s.q_n;
         }
@@ -1844,43 +1874,46 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
                 const unsigned db = __ballot_sync(0xffffffffu, d);
                 const int rank = seen + __popc(db & ((1u << lane) - 1u));
                 seen += __popc(db);
-                const int c = q >= nt || t_fuse[t] < 0 ? 0 : (d ? fill_splits(g, target, units, nd, rank) : 1);
-                if (q < nt) t_jobs[q] = (int16_t)c;
-                total += __reduce_add_sync(0xffffffffu, (unsigned)c);
+                const int n = q >= nt || t_fuse[t] < 0 ? 0 : (d ? fill_splits(g, target, units, nd, rank) : 1);
+                const int incl = warp_incl_scan(n);
+                if (q < nt) {
+                    t_jobs[q] = (int16_t)n;
+                    t_at[q] = (int16_t)(total + incl - n);
+                }
+                total += __shfl_sync(0xffffffffu, incl, 31);
             }
-            int base = 0;
             if (lane == 0) {
                 if (n_windows == 1) {             // the only block: the list is its own
                     sch->n_jobs[par ^ 1] = total;
+                    sm.s_base = 0;
                 } else {
-                    base = atomicAdd(&sch->n_jobs[par ^ 1], total);
+                    sm.s_base = atomicAdd(&sch->n_jobs[par ^ 1], total);
                 }
-            }
-            base = __shfl_sync(0xffffffffu, base, 0);
-            __syncwarp();
-            int run = 0;
-            for (int c0 = 0; c0 < nt; c0 += 32) {
-                const int q = c0 + lane;
-                const int t = nt - 1 - q;
-                const int c = q < nt ? (int)t_jobs[q] : 0;
-                const int incl = warp_incl_scan(c);
-                const int fz = c > 0 ? (int)t_fuse[t] : 0;
-                for (int k = 0; k < c; k++) {
-                    Job j;
-                    j.win = w;
-                    j.task = t;
-                    j.split = fz > 0 ? fz - 1 : k;
-                    j.splits = fz > 0 ? -1 : c;
-                    jobs[base + run + incl - c + k] = j;
-                }
-                run += __shfl_sync(0xffffffffu, incl, 31);
             }
         }
     }
     __syncthreads();
-    for (int i = tid; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
-        reinterpret_cast<int4*>(st)[i] = reinterpret_cast<const int4*>(&s)[i];
+    if (s.phase != PH_DONE) {                     // the jobs, written by the whole block
+        const int nt = s.n_tasks;
+        for (int q = tid; q < nt; q += blockDim.x) {
+            const int n = t_jobs[q], t = nt - 1 - q;
+            const int fz = n > 0 ? (int)t_fuse[t] : 0;
+            Job* out = jobs + sm.s_base + t_at[q];
+            for (int k = 0; k < n; k++) {
+                Job j;
+                j.win = w;
+                j.task = t;
+                j.split = fz > 0 ? fz - 1 : k;
+                j.splits = fz > 0 ? -1 : n;
+                out[k] = j;
+            }
+        }
+    }
+    if (!RESIDENT || s.phase == PH_DONE)
+        for (int i = tid; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
+            reinterpret_cast<int4*>(st)[i] = reinterpret_cast<const int4*>(&s)[i];
     } // s.phase != PH_DONE at entry
+    if (RESIDENT) return;
     __syncthreads();
     if (tid == 0 && phase_out) phase_out[w] = s.phase;
     if (tid == 0 && n_windows == 1) {             // the only block is the last: no ticket
@@ -1905,9 +1938,114 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
 
 __global__ void __launch_bounds__(CTL_THREADS) k_control(Geom g, CtlArgs c) {
     __shared__ CtlShared sm;
-    control_body(g, c, blockIdx.x, sm);
+    control_body<false>(g, c, blockIdx.x, sm, c.sch->round & 1);
 }
 
+
+// A polled 64-bit word: the round it announces in the high half, that round's
+// jobs in the low half (none: the search has ended).
+__device__ __forceinline__ unsigned long long load_acquire(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int32_t load_acquire(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_release(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" : : "l"(p), "l"(v) : "memory");
+}
+
+// Polls before a block gives up on the others: each takes about a
+// microsecond, and rounds of at most SEARCH_MAX_EVENTS events end within a
+// fraction of a second.
+constexpr int SEARCH_POLLS = 1 << 23;
+
+// The control block of k_search: waits for the `others` evaluating blocks,
+// runs the control step and announces the next round.
+__device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, CtlShared& sm, Node* q_mem, int q_cap,
+                                            int others) {
+    Sched* sch = c.sch;
+    for (int i = threadIdx.x; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
+        reinterpret_cast<int4*>(&sm.s)[i] = reinterpret_cast<const int4*>(c.st_all)[i];
+    if (threadIdx.x == 0) sm.q_shared = 1;        // empty
+    __syncthreads();
+    for (uint32_t round = 0;; round++) {
+        if (threadIdx.x == 0) {
+            const int32_t all = (int32_t)(round + 1) * others;
+            int polls = 0;
+            while (load_acquire(&sch->ticket) != all && ++polls < SEARCH_POLLS) __nanosleep(20);
+            sm.s_stop = polls >= SEARCH_POLLS;
+        }
+        __syncthreads();
+        if (sm.s_stop) {                          // never in a sound run
+            if (threadIdx.x == 0) sch->failed = 1;
+            return;
+        }
+        __syncthreads();
+        control_body<true>(g, c, 0, sm, (int)(round & 1), q_mem, q_cap);
+        __syncthreads();                          // the round's tasks and jobs are written
+        const bool done = sm.s.phase == PH_DONE;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            store_release(&sch->go, (unsigned long long)(round + 1) << 32 |
+                                        (done ? 0u : (uint32_t)sch->n_jobs[(round & 1) ^ 1]));
+            if (done) sch->round = (int32_t)(round + 1);
+        }
+        if (done) return;
+    }
+}
+
+// All rounds of one window's search in one cooperative launch.  Block 0 runs
+// the control steps, with the search's state and queue in its shared memory;
+// the others evaluate a round's units as k_eval does, count themselves in
+// sch->ticket and poll sch->go for the next round.  A search of few events is
+// bound by the latency of its rounds, and a round of two graph nodes, the
+// loop's condition and a control step that reads and writes its state in L2
+// costs about 10 us beside the evaluation.
+__global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_constant__ Geom g,
+                                                                 const __grid_constant__ EvalArgs a,
+                                                                 const __grid_constant__ CtlArgs c, int q_cap) {
+    extern __shared__ __align__(16) uint32_t tile[];
+    __shared__ EvalShared sm;
+    __shared__ unsigned long long s_go;
+    Sched* sch = a.sch;
+    if (blockIdx.x == 0) {
+        CtlShared& ctl = *reinterpret_cast<CtlShared*>(tile);
+        control_rounds(g, c, ctl, reinterpret_cast<Node*>(&ctl + 1), q_cap, (int)gridDim.x - 1);
+        return;
+    }
+    if (threadIdx.x == 0) {
+        clear_tile(tile, eval_tile_words(g));
+        sm.over = 0;
+        s_go = (unsigned long long)(uint32_t)sch->n_jobs[0];
+    }
+    __syncthreads();
+    const int block = (int)blockIdx.x - 1, blocks = (int)gridDim.x - 1;
+    for (uint32_t round = 0;; round++) {
+        const int par = round & 1, n_units = (int)(uint32_t)s_go * g.n_tiles;
+        if (block == 0 && threadIdx.x == 0) sch->work[par ^ 1] = 0;
+        if (block < n_units)
+            eval_round(g, a, a.jobs + (size_t)par * a.job_stride, &sch->work[par], n_units, block, blocks, tile, sm);
+        __syncthreads();                          // the block's sums are on their way; s_go has been read
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(&sch->ticket, 1);
+            unsigned long long v = 0;
+            int polls = 0;
+            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < SEARCH_POLLS) __nanosleep(20);
+            if (polls >= SEARCH_POLLS) {          // never in a sound run: end the search
+                sch->failed = 1;
+                v = 0;
+            }
+            s_go = v;
+        }
+        __syncthreads();
+        if ((uint32_t)s_go == 0) return;
+    }
+}
 
 CtlArgs control_args(int32_t n_windows, SolveState* st, Node* queues, Task* tasks, int32_t task_stride, Partial* part,
                      const int32_t* err, TraceRec* trace, Job* jobs, int32_t job_stride, Sched* sch,
@@ -1941,8 +2079,41 @@ cudaError_t launch_control(const Geom& g, int32_t n_windows, SolveState* st, Nod
     return cudaGetLastError();
 }
 
+// The dynamic shared memory of a k_search block holds the tile and scratch of
+// the evaluation or, in the control block, the search's state and as much of
+// its queue (two buffers) as fits, up to SEARCH_QUEUE entries.
+constexpr int SEARCH_QUEUE = 1024;
+static size_t search_smem_bytes(const Geom& g, int threads) {
+    const size_t e = eval_smem_bytes(g, threads);
+    return e > sizeof(CtlShared) ? e : sizeof(CtlShared);
+}
+static int search_queue(const Geom& g, int threads) {
+    const size_t n = (search_smem_bytes(g, threads) - sizeof(CtlShared)) / (2 * sizeof(Node));
+    return n < SEARCH_QUEUE ? (int)n : SEARCH_QUEUE;
+}
+
+int search_resident_blocks(const Geom& g, int threads) {
+    int per_sm = 0, dev = 0, sms = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_search, threads + 32, search_smem_bytes(g, threads)) !=
+        cudaSuccess)
+        return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    return per_sm * sms;
+}
+
+cudaError_t launch_search(const Geom& g, const EvalArgs& a, const CtlArgs& c, int threads, int grid_blocks,
+                          cudaStream_t s) {
+    if (grid_blocks < 2) return cudaErrorInvalidValue;            // block 0 evaluates nothing
+    int q_cap = search_queue(g, threads);
+    void* args[] = {const_cast<Geom*>(&g), const_cast<EvalArgs*>(&a), const_cast<CtlArgs*>(&c), &q_cap};
+    return cudaLaunchCooperativeKernel((const void*)k_search, dim3(grid_blocks), dim3(threads + 32), args,
+                                       search_smem_bytes(g, threads), s);
+}
+
 // Function attributes are per device: the carveout and the dynamic
-// shared-memory limit of k_eval are set on the current device the first time
+// shared-memory limit of k_eval and k_search are set on the current device the first time
 // it is used, and the limit only ever raised, under one lock (contexts of
 // several host threads and devices share these records).
 constexpr int SMEM_MAX_DEVICES = 64;
@@ -1960,7 +2131,7 @@ cudaError_t eval_smem_setup(const Geom& g) {
         // One shared-memory carveout for every kernel of the library, so that
         // consecutive launches never wait for an L1 / shared reconfiguration.
         const void* fns[] = {(const void*)k_eval, (const void*)k_control, (const void*)k_init,
-                             (const void*)k_keys, (const void*)k_row_hist, (const void*)k_row_scan,
+                             (const void*)k_keys, (const void*)k_search, (const void*)k_row_hist, (const void*)k_row_scan,
                              (const void*)k_row_scatter};
         for (const void* f : fns) {
             e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1969,9 +2140,10 @@ cudaError_t eval_smem_setup(const Geom& g) {
         }
         g_carveout[dev] = true;
     }
-    const int bytes = (int)eval_smem_bytes(g, 32 * MAX_WARPS);   // any block size up to 512 threads
+    const int bytes = (int)search_smem_bytes(g, EVAL_THREADS);   // any block size
     if (bytes <= g_smem_bytes[dev]) return cudaSuccess;
     e = cudaFuncSetAttribute(k_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_search, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) g_smem_bytes[dev] = bytes;
     return e;
 }

@@ -1,0 +1,64 @@
+"""One window's search in one cooperative launch: a control block with the
+queue in its shared memory while it fits, evaluating blocks that poll for the
+next round.  Results, counts and traces are the oracle's whatever the queue's
+place (never, sometimes or always in shared memory), and windows beyond the
+launch's size limit go through the graph with the same result.
+"""
+import pytest
+
+import oracle as O
+from synth import make_window
+from synth.descent import serve_spec5
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+import paper_2209_13168_gb300 as dd  # noqa: E402
+
+KEYS = ("D_star", "D_end", "K_hat", "gap_K", "nodes_expanded", "point_evals", "bound_evals", "event_warps",
+        "cell_increments", "bound_increments", "rounds", "max_queue")
+
+
+# 160-pixel frames: dynamic shared memory of the block (bytes) decides how many
+# intervals fit: none, a few tens (the queue of this window reaches 98) or all
+@pytest.mark.parametrize("threads,band_rows", [(32, 4), (96, 50), (480, 90)])
+@pytest.mark.parametrize("pop_k", [1, 16, 64])
+def test_queue_in_and_out_of_shared_memory(threads, band_rows, pop_k):
+    w = make_window(160, 90, 80.0, 45.0, 16000, 444, 5333, 0.35, 0.3, seed=74)
+    want = O.solve(O.Window.of(w), -1.0, 1.0, 1e-4, 0.0, pop_k, trace_cap=4096)
+    ctx = dd.Context(160, 90, 80.0, 45.0, pop_k=pop_k, threads=threads, band_rows=band_rows)
+    for _ in range(2):
+        got = ctx.solve(dd.Events.of(w, device="cuda"), trace_cap=4096)
+        for k in KEYS:
+            assert got[k] == want[k], (k, got[k], want[k])
+        assert got["trace"] == want["trace"]
+    ctx.close()
+
+
+def test_round_and_queue_limits():
+    w = make_window(160, 90, 80.0, 45.0, 4000, 110, 1300, 0.35, 0.3, seed=75)
+    ev = dd.Events.of(w, device="cuda")
+    for kw, status in (({"max_rounds": 5}, dd.DD_ERR_TIMEOUT), ({"queue_capacity": 3}, dd.DD_ERR_QUEUE_OVERFLOW)):
+        ctx = dd.Context(160, 90, 80.0, 45.0, pop_k=4, **kw)
+        with pytest.raises(dd.DDError) as e:
+            ctx.solve(ev)
+        assert e.value.status == status
+        ctx.close()
+
+
+def test_window_beyond_the_launch_limit():
+    from synth.gpu import make_window_gpu
+    n = (1 << 22) + 33
+    spec = list(serve_spec5(0, 100))
+    spec[4], spec[5], spec[6] = n - n // 8, n // 40, n // 8
+    ev = dd.Events.of(make_window_gpu(tuple(spec)))
+    got = []
+    for kw in ({}, {"host_loop": 1}):
+        ctx = dd.Context(1280, 720, 640.0, 360.0, pop_k=16, **kw)
+        got.append(ctx.solve(ev, -1.0, 1.0, 1e-2, 0.0))
+        ctx.close()
+    for k in KEYS:
+        assert got[0][k] == got[1][k], k
