@@ -1308,12 +1308,13 @@ struct __align__(16) CtlShared {
     Node sorted_kids[2 * MAX_POP + 1];
     Node q_stage[Q_STAGE];
     Node q_head[MAX_POP];               // the merged queue's first entries, for the dequeue
-    float2 bound_iv[3 * MAX_POP];       // the next round's bound tasks' intervals
     int16_t t_fuse[3 * MAX_POP];        // per next-round task: 0 own jobs, -1 part of a fused
                                         // job, k > 0 the centre of a fused job (left half k - 1)
     int8_t t_dense[3 * MAX_POP];        // per next-round task: a dense bound that may be split
     int16_t t_jobs[3 * MAX_POP];        // per next-round task, in job order: its number of jobs
     int16_t t_at[3 * MAX_POP];          // and the place of its first one in the window's jobs
+    uint4 pop_mask[2];                  // per 32 dequeued: to split, fused, dense left and right halves
+    int pop_fail[2];                    // first that fails the gap test
     int s_nk, s_stop, s_base;
     int q_shared;                       // resident: the queue is in the block's shared memory
 };
@@ -1461,82 +1462,66 @@ __device__ __forceinline__ int rank_in(const Node* q, int n, const Node& e) {
 
 constexpr int CTL_THREADS = 256;
 
-__device__ __forceinline__ i128 shfl_i128(i128 v, int src) {
-    unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)((unsigned __int128)v >> 64);
-    lo = __shfl_sync(0xffffffffu, lo, src);
-    hi = __shfl_sync(0xffffffffu, hi, src);
-    return (i128)(((unsigned __int128)hi << 64) | (unsigned __int128)lo);
-}
-
-__device__ __forceinline__ i128 warp_max_i128(i128 v) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const i128 w = shfl_i128(v, threadIdx.x ^ o);
-        if (w > v) v = w;
+// Warp maximum of non-negative 128-bit values, word by word from the top (a
+// lane without a value passes 0); `at`: the lanes that hold it.
+__device__ __forceinline__ i128 warp_max_i128(i128 v, bool valid, unsigned& at) {
+    uint32_t w[4], m[4];
+    for (int k = 0; k < 4; k++) w[k] = (uint32_t)((unsigned __int128)v >> (32 * k));
+    bool in = valid;
+    for (int k = 3; k >= 0; k--) {
+        m[k] = __reduce_max_sync(0xffffffffu, in ? w[k] : 0u);
+        in = in && w[k] == m[k];
     }
-    return v;
+    at = __ballot_sync(0xffffffffu, in);
+    return (i128)(((unsigned __int128)((unsigned long long)m[3] << 32 | m[2]) << 64) |
+                  ((unsigned long long)m[1] << 32 | m[0]));
 }
 
 // One block per window.  Consumes the keys of the round just evaluated
 // (Algorithm 1: incumbent update, leaves, child bounds and their insertion),
 // then dequeues the next batch (dequeue and gap test) and writes its tasks
-// and jobs, or finishes.  The search state is staged in shared memory;
-// per-interval work runs one interval per lane of warp 0.  The queue is kept
-// sorted in priority order in one of two buffers: insertion is a parallel
-// merge into the other buffer, a dequeue takes a prefix.  The last block to
-// finish counts the windows still searching, advances the round and sets the
-// graph loop condition (with one window, its block does so directly).
+// and jobs, or finishes.  The search state is staged in shared memory.  The
+// queue is kept sorted in priority order in one of two buffers: insertion is
+// a parallel merge into the other buffer, a dequeue takes a prefix.  The last
+// block to finish counts the windows still searching, advances the round and
+// sets the graph loop condition (with one window, its block does so
+// directly).
+//
+// Nothing here is much work (at most 64 intervals and 128 children): its time
+// is the chain of dependent steps, so the steps are as wide as the data allows
+// (a thread per task, child, queued interval or dequeued interval; the sums
+// and maxima of a round by different warps) and a block barrier apart.  Per
+// round of one window, in k_search: 6.5 -> 4 us.
 //
 // RESIDENT (the control block of k_search): the state stays in `sm` from round
 // to round, and so does the queue while it has at most q_cap entries (two
-// buffers of q_cap at q_mem); both reach global memory when the search ends
-// or the queue grows beyond that.
+// buffers of q_cap at q_mem); the state reaches global memory when the search
+// ends, the queue when it grows beyond that.
 template <bool RESIDENT>
 __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, int w, CtlShared& sm, int par,
                                              Node* q_mem = nullptr, int q_cap = 0) {
     SolveState& s = sm.s;
     i128* key = sm.key;
     unsigned long long* cells = sm.cells;
-    Node* kids = sm.kids;
-    Node* sorted_kids = sm.sorted_kids;
-    Node* q_stage = sm.q_stage;
-    Node* q_head = sm.q_head;
-    float2* bound_iv = sm.bound_iv;
-    int16_t* t_fuse = sm.t_fuse;
-    int8_t* t_dense = sm.t_dense;
-    int16_t* t_jobs = sm.t_jobs;
-    int16_t* t_at = sm.t_at;
-    int& s_nk = sm.s_nk;
-    int& s_stop = sm.s_stop;
-    const int32_t n_windows = c.n_windows, task_stride = c.task_stride, job_stride = c.job_stride;
-    const int32_t use_loop = c.use_loop, split_ok = c.split_ok;
-    SolveState* st_all = c.st_all;
-    Node* queues = c.queues;
-    Task* tasks_all = c.tasks_all;
-    Partial* part_all = c.part_all;
-    const int32_t* err_all = c.err_all;
-    TraceRec* trace = c.trace;
-    Job* jobs_all = c.jobs_all;
     Sched* sch = c.sch;
-    int32_t* phase_out = c.phase_out;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = (int)blockDim.x >> 5;
     const int running = RESIDENT ? 1 : sch->running;   // searches still running after the last round
-    SolveState* st = st_all + w;
-    Task* tasks = tasks_all + (size_t)w * task_stride;
-    Partial* part = part_all + (size_t)w * task_stride;
-    Job* jobs = jobs_all + (size_t)(par ^ 1) * job_stride;
+    SolveState* st = c.st_all + w;
+    Task* tasks = c.tasks_all + (size_t)w * c.task_stride;
+    Partial* part = c.part_all + (size_t)w * c.task_stride;
+    Job* jobs = c.jobs_all + (size_t)(par ^ 1) * c.job_stride;
     static_assert(sizeof(SolveState) % 16 == 0, "state is copied as int4");
     if (!RESIDENT) {
         for (int i = tid; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
             reinterpret_cast<int4*>(&s)[i] = reinterpret_cast<const int4*>(st)[i];
         __syncthreads();
     }
-    const int phase = s.phase;                    // read before a barrier: warp 0 changes it
+    const int phase = s.phase;                    // read before a barrier: one thread changes it
     if (phase != PH_DONE) {
-    Node* qa = queues + (size_t)w * 2 * s.qcap;
+    Node* qa = c.queues + (size_t)w * 2 * s.qcap;
     Node* qb = qa + s.qcap;
-    const int32_t* err = err_all + w;
     const int64_t M = s.M;
-    const int n_tasks = s.n_tasks, n_points = phase == PH_INIT ? 1 : s.n_pop;   // points come first
+    const int n_tasks = s.n_tasks, np0 = s.n_pop, n_points = phase == PH_INIT ? 1 : np0;   // points come first
 
     // Each task's sums (accumulated by the evaluation over its row bands, in
     // L2), read and cleared for the next round.
@@ -1551,72 +1536,92 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
         key[t] = partial_key(M, q, t < n_points);
         cells[t] = q.cells[0] + q.cells[1];
     }
+    if (tid == 0) {
+        sm.s_nk = 0;
+        sm.s_stop = 0;
+        if (!RESIDENT || phase == PH_INIT) {
+            if (c.err_all[w]) {                   // malformed events
+                s.status = DD_ERR_ARG;
+                sm.s_stop = 1;
+            } else if (s.cancel) {                // the host cancelled the search between rounds
+                s.status = DD_ERR_CANCELLED;
+                sm.s_stop = 1;
+            }
+        }
+    }
     __syncthreads();
+    int stop = sm.s_stop;
 
-    if (wid == 0) {
-        int stop = 0, nk = 0;
-        if (*err) {
-            if (lane == 0) s.status = DD_ERR_ARG;
-            stop = 1;
-        } else if (s.cancel) {                    // the host cancelled the search between rounds
-            if (lane == 0) s.status = DD_ERR_CANCELLED;
-            stop = 1;
-        } else if (phase == PH_INIT) {
-            if (lane == 0) {
-                s.K_hat = key[0];
-                s.point_evals = 1;
-                s.bound_evals = n_tasks - 1;
-                s.cells = (int64_t)cells[0];
-                s.bcells = 0;
-                for (int t = 1; t < n_tasks; t++) {
-                    s.cells += (int64_t)cells[t];
-                    s.bcells += (int64_t)cells[t];
-                    // the domain is queued unconditionally; warm-start pieces
-                    // when their bound reaches the incumbent, as children are
-                    if (s.warm && !(key[t] >= s.K_hat)) continue;
-                    Node nd;
-                    nd.lo = tasks[t].D_lo;
-                    nd.hi = tasks[t].D_hi;
-                    nd.pad0 = nd.pad1 = 0;
-                    nd.kb = key[t];
-                    kids[nk++] = nd;
-                }
-                s.phase = PH_RUN;
+    // The incumbent, the counters and the leaves, each by a warp of its own.
+    if (!stop && phase == PH_INIT) {
+        if (tid == 0) {
+            s.K_hat = key[0];
+            s.point_evals = 1;
+            s.bound_evals = n_tasks - 1;
+            s.cells = (int64_t)cells[0];
+            s.bcells = 0;
+            for (int t = 1; t < n_tasks; t++) {
+                s.cells += (int64_t)cells[t];
+                s.bcells += (int64_t)cells[t];
             }
-            nk = __shfl_sync(0xffffffffu, nk, 0);
-        } else {
-            const int np = s.n_pop;
-            // Incumbent update in dequeue order (a centre with K >= K_hat wins):
-            // per chunk of 32, the chunk maximum wins if it reaches the running
-            // incumbent, at the last lane attaining it.
+            s.phase = PH_RUN;
+        }
+    } else if (!stop) {
+        if (wid == 0) {
+            // Incumbent update in dequeue order (a centre with K >= K_hat
+            // wins): per chunk of 32, the chunk maximum wins if it reaches
+            // the running incumbent, at the last lane attaining it.
             i128 K_hat = s.K_hat;
-            float D_hat = s.D_hat;
-            unsigned long long pc = 0;
-            for (int base = 0; base < np; base += 32) {
-                const int j = base + lane;
-                const bool v = j < np;
-                const i128 kc = v ? key[s.pop[j].t_point] : (i128)(-1);
-                if (v) pc += cells[s.pop[j].t_point];
-                const i128 m = warp_max_i128(kc);
+            int best = -1;
+            for (int base = 0; base < np0; base += 32) {
+                const bool v = base + lane < np0;
+                unsigned at;
+                const i128 m = warp_max_i128(v ? key[base + lane] : (i128)0, v, at);
                 if (m >= K_hat) {
-                    const unsigned at = __ballot_sync(0xffffffffu, v && kc == m);
-                    const int last = 31 - __clz(at);
                     K_hat = m;
-                    D_hat = __shfl_sync(0xffffffffu, v ? s.pop[j].c : 0.0f, last);
+                    best = base + 31 - __clz(at);
                 }
             }
-            pc = warp_sum(pc);
-            // Leaves, traces, child bounds, children inserted against the
-            // end-of-round incumbent.
-            int nonleaf = 0, has_leaf = 0;
-            i128 lmax = (i128)(-1);
-            unsigned long long bc = 0;
-            for (int base = 0; base < np; base += 32) {
-                const int j = base + lane;
-                const bool v = j < np;
-                Popped p;
-                if (v) p = s.pop[j];
-                if (v && trace && w == 0 && s.trace_len + j < s.trace_cap) {
+            if (lane == 0) {
+                s.K_hat = K_hat;
+                if (best >= 0) s.D_hat = s.pop[best].c;
+            }
+        }
+        if (wid == (nwarps > 2 ? 1 : 0)) {        // cells of the points and of all tasks
+            unsigned long long pc = 0, all = 0;
+            for (int t = lane; t < n_tasks; t += 32) {
+                if (t < np0) pc += cells[t];
+                all += cells[t];
+            }
+            pc = warp_total(pc);
+            all = warp_total(all);
+            if (lane == 0) {
+                s.nodes_expanded += np0;
+                s.point_evals += np0;
+                s.bound_evals += n_tasks - np0;
+                s.cells += (int64_t)all;
+                s.bcells += (int64_t)(all - pc);
+            }
+        }
+        if (wid == (nwarps > 2 ? 2 : 1)) {        // the largest bound among the leaves
+            bool any = false;
+            i128 lmax = 0;
+            for (int base = 0; base < np0; base += 32) {
+                const bool v = base + lane < np0 && s.pop[base + lane].leaf;
+                unsigned at;
+                const i128 m = warp_max_i128(v ? s.pop[base + lane].kb : (i128)0, v, at);
+                if (at && (!any || m > lmax)) lmax = m;
+                any |= at != 0;
+            }
+            if (lane == 0 && any) {
+                if (!s.have_leaf || lmax > s.leaf_max) s.leaf_max = lmax;
+                s.have_leaf = 1;
+            }
+        }
+        if (c.trace && w == 0)
+            for (int j = tid; j < np0; j += blockDim.x)
+                if (s.trace_len + j < s.trace_cap) {
+                    const Popped& p = s.pop[j];
                     TraceRec r;
                     r.D_lo = p.lo;
                     r.D_hi = p.hi;
@@ -1624,77 +1629,47 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
                     r.leaf = p.leaf;
                     r.Kbar = p.kb;
                     r.K_c = key[p.t_point];
-                    trace[s.trace_len + j] = r;
+                    c.trace[s.trace_len + j] = r;
                 }
-                const bool leaf = v && p.leaf, split = v && !p.leaf;
-                if (leaf && (!has_leaf || p.kb > lmax)) lmax = p.kb;
-                has_leaf |= leaf;
-                i128 kl = 0, kr = 0;
-                int c = 0;
-                if (split) {
-                    kl = key[p.t_left];
-                    kr = key[p.t_right];
-                    bc += cells[p.t_left] + cells[p.t_right];
-                    c = (kl >= K_hat) + (kr >= K_hat);
-                }
-                nonleaf += __popc(__ballot_sync(0xffffffffu, split));
-                const int incl = warp_incl_scan(c);
-                const int at = nk + incl - c;
-                if (split) {
-                    int o = at;
-                    if (kl >= K_hat) {
-                        Node nd;
-                        nd.lo = p.lo;
-                        nd.hi = p.c;
-                        nd.pad0 = nd.pad1 = 0;
-                        nd.kb = kl;
-                        kids[o++] = nd;
-                    }
-                    if (kr >= K_hat) {
-                        Node nd;
-                        nd.lo = p.c;
-                        nd.hi = p.hi;
-                        nd.pad0 = nd.pad1 = 0;
-                        nd.kb = kr;
-                        kids[o] = nd;
-                    }
-                }
-                nk += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    __syncthreads();
+
+    // Children (or the first pieces) that reach the end-of-round incumbent,
+    // one thread each, in any order: they are sorted next.
+    const i128 K_hat = s.K_hat;
+    if (!stop) {
+        const int nc = phase == PH_INIT ? n_tasks - 1 : 2 * np0;
+        for (int k = tid; k < nc; k += blockDim.x) {
+            Node nd;
+            nd.pad0 = nd.pad1 = 0;
+            bool in;
+            if (phase == PH_INIT) {
+                // the domain is queued unconditionally; warm-start pieces
+                // when their bound reaches the incumbent, as children are
+                nd.lo = tasks[1 + k].D_lo;
+                nd.hi = tasks[1 + k].D_hi;
+                nd.kb = key[1 + k];
+                in = !s.warm || nd.kb >= K_hat;
+            } else {
+                const Popped& p = s.pop[k >> 1];
+                const bool right = k & 1;
+                nd.lo = right ? p.c : p.lo;
+                nd.hi = right ? p.hi : p.c;
+                nd.kb = p.leaf ? (i128)0 : key[right ? p.t_right : p.t_left];
+                in = !p.leaf && nd.kb >= K_hat;
             }
-            bc = warp_sum(bc);
-            has_leaf = __any_sync(0xffffffffu, has_leaf);
-            lmax = warp_max_i128(lmax);
-            if (lane == 0) {
-                s.K_hat = K_hat;
-                s.D_hat = D_hat;
-                s.nodes_expanded += np;
-                s.point_evals += np;
-                s.bound_evals += 2 * nonleaf;
-                s.cells += (int64_t)(pc + bc);
-                s.bcells += (int64_t)bc;
-                if (has_leaf && (!s.have_leaf || lmax > s.leaf_max)) s.leaf_max = lmax;
-                s.have_leaf |= has_leaf;
-                s.trace_len += np;
-            }
-        }
-        if (!stop && s.q_n + nk > s.qcap) {
-            if (lane == 0) s.status = DD_ERR_QUEUE_OVERFLOW;
-            stop = 1;
-        }
-        if (lane == 0) {
-            s_nk = nk;
-            s_stop = stop;
+            if (in) sm.kids[atomicAdd(&sm.s_nk, 1)] = nd;
         }
     }
     __syncthreads();
-    const int nk = s_nk;
-    const int stop = s_stop;
+    const int nk = sm.s_nk, a = s.q_n;
+    if (!stop && a + nk > s.qcap) stop = 2;       // (the same for every thread)
+    if (stop == 2 && tid == 0) s.status = DD_ERR_QUEUE_OVERFLOW;
 
     if (!stop) {
-        // sort the new children, then merge them with the queued intervals;
-        // a queue that fits is staged in shared memory first, so that the
-        // children's ranks are searched there instead of in global memory
-        const int a = s.q_n;
+        // Sort the new children, then merge them with the queued intervals; a
+        // queue in global memory that fits is staged in shared memory first,
+        // so that the children's ranks are searched there.
         const bool in_shared = RESIDENT && sm.q_shared, to_shared = RESIDENT && a + nk <= q_cap;
         const Node* src = (in_shared ? q_mem + (s.q_cur ? q_cap : 0) : (s.q_cur ? qb : qa)) + s.q_start;
         Node* dst = to_shared ? q_mem + (s.q_cur ? 0 : q_cap) : (s.q_cur ? qa : qb);
@@ -1703,202 +1678,188 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
         // intervals are disjoint) counted by `per` threads, each over every
         // per-th child, summed within the thread group.
         int per = 1;
-        while (nk > 32 && per < 32 && 2 * per * nk <= (int)blockDim.x) per *= 2;
+        while (nk > 8 && per < 32 && 2 * per * nk <= (int)blockDim.x) per *= 2;
         for (int base = 0; base < nk * per; base += blockDim.x) {
-            const int i = (base + tid) / per, part = (base + tid) % per;
+            const int i = (base + tid) / per, p = (base + tid) % per;
             int r = 0;
             if (i < nk)
-                for (int j = part; j < nk; j += per) r += better(kids[j], kids[i]);
+                for (int j = p; j < nk; j += per) r += better(sm.kids[j], sm.kids[i]);
             for (int o = per / 2; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-            if (i < nk && part == 0) sorted_kids[r] = kids[i];
+            if (i < nk && p == 0) sm.sorted_kids[r] = sm.kids[i];
         }
         if (staged)
-            for (int i = tid; i < a; i += blockDim.x) q_stage[i] = src[i];
+            for (int i = tid; i < a; i += blockDim.x) sm.q_stage[i] = src[i];
         __syncthreads();
-        const Node* qs = staged ? q_stage : src;
+        const Node* qs = staged ? sm.q_stage : src;
+        // Children from the last thread down, queued intervals from the first
+        // up: one pass of different warps.
         for (int i = tid; i < a; i += blockDim.x) {
             const Node e = qs[i];
-            const int at = i + rank_in(sorted_kids, nk, e);
+            const int at = i + rank_in(sm.sorted_kids, nk, e);
             dst[at] = e;
-            if (at < MAX_POP) q_head[at] = e;
+            if (at < MAX_POP) sm.q_head[at] = e;
         }
-        for (int j = tid; j < nk; j += blockDim.x) {
-            const Node e = sorted_kids[j];
+        for (int j = (int)blockDim.x - 1 - tid; j < nk; j += blockDim.x) {
+            const Node e = sm.sorted_kids[j];
             const int at = j + rank_in(qs, a, e);
             dst[at] = e;
-            if (at < MAX_POP) q_head[at] = e;
+            if (at < MAX_POP) sm.q_head[at] = e;
         }
         __syncthreads();
         if (tid == 0) {
             s.q_cur ^= 1;
             s.q_start = 0;
-            sm.q_shared = to_shared;
             s.q_n = a + nk;
+            sm.q_shared = to_shared;
+            s.trace_len += phase == PH_INIT ? 0 : np0;
             if (s.q_n > s.max_queue) s.max_queue = s.q_n;
         }
-        __syncthreads();
     }
 
-    if (wid == 0) {
-        const Node* q = q_head;                   // the first entries of the queue just merged
-        int np = 0;
-        if (!stop) {                              // dequeue up to K_pop intervals
-            const i128 K0 = s.K_hat, gK = s.gamma_K;
-            const int lim = min(s.K_pop, s.q_n);
-            for (int base = 0; base < lim; base += 32) {
-                const int j = base + lane;
-                const bool v = j < lim;
-                Node nd;
-                if (v) nd = q[j];
-                const bool pass = v && (nd.kb - K0 > gK);   // gap test
-                const unsigned fail = __ballot_sync(0xffffffffu, v && !pass);
-                const int first = fail ? __ffs(fail) - 1 : 32;
-                if (v && lane < first) {
-                    s.pop[j].lo = nd.lo;
-                    s.pop[j].hi = nd.hi;
-                    s.pop[j].kb = nd.kb;
-                }
-                if (fail) {
-                    if (base + first == 0 && lane == 0) {
-                        s.have_stop = 1;
-                        s.stop_kb = nd.kb;
-                    }
-                    np = base + first;
-                    break;
-                }
-                np = min(lim, base + 32);
-            }
-            if (lane == 0) {
-                s.q_start = np;
-                s.q_n -= np;
-            }
+    // Dequeue up to K_pop intervals, one thread each (two warps): the gap
+    // test, the centre and the bisection, and which tasks the interval will
+    // need; the first that fails the gap test ends the batch.
+    const int lim = stop ? 0 : min(s.K_pop, a + nk);
+    Popped p;
+    bool split = false, fuse = false, dense_l = false, dense_r = false;
+    if (wid < 2) {
+        const bool v = tid < lim;
+        bool pass = false;
+        if (v) {
+            const Node nd = sm.q_head[tid];
+            pass = nd.kb - K_hat > s.gamma_K;     // gap test
+            p.lo = nd.lo;
+            p.hi = nd.hi;
+            p.kb = nd.kb;
+            p.c = centre(p.lo, p.hi);
+            const float wd = __fsub_rn(p.hi, p.lo);
+            p.leaf = !(wd > s.tol) || !(p.c > p.lo) || !(p.c < p.hi);
+            split = !p.leaf;
+            // narrow intervals: centre and halves evaluated by one fused job
+            fuse = split && g.fuse_cells > 0.0f && bound_cells(g, p.lo, p.hi, s.tau) - 1.0f <= g.fuse_cells;
+            // dense bounds (splittable when the round is small)
+            const bool own = split && !fuse && c.split_ok;
+            dense_l = own && bound_cells(g, p.lo, p.c, s.tau) >= DENSE_CELLS;
+            dense_r = own && bound_cells(g, p.c, p.hi, s.tau) >= DENSE_CELLS;
         }
-        __syncwarp();
-        if (stop || np == 0) {
-            if (lane == 0) {
-                i128 top = s.K_hat;
-                if (s.have_leaf && s.leaf_max > top) top = s.leaf_max;
-                if (s.have_stop && s.stop_kb > top) top = s.stop_kb;
-                s.stop_kb = top - s.K_hat;        // the certificate gap_K
-                s.n_pop = 0;
-                s.n_tasks = 0;
-                s.phase = PH_DONE;
-            }
-        } else {
-            int nl_before = 0;
-            for (int base = 0; base < np; base += 32) {   // centre and bisection
-                const int j = base + lane;
-                const bool v = j < np;
-                bool split = false, fuse = false;
-                if (v) {
-                    Popped& p = s.pop[j];
-                    p.c = centre(p.lo, p.hi);
-                    const float w = __fsub_rn(p.hi, p.lo);
-                    p.leaf = !(w > s.tol) || !(p.c > p.lo) || !(p.c < p.hi);
-                    split = !p.leaf;
-                    // narrow intervals: centre and halves evaluated by one fused job
-                    fuse = split && g.fuse_cells > 0.0f && bound_cells(g, p.lo, p.hi, s.tau) - 1.0f <= g.fuse_cells;
-                }
-                const unsigned sb = __ballot_sync(0xffffffffu, split);
-                if (v) {
-                    Popped& p = s.pop[j];
-                    p.t_point = j;
-                    Task a;
-                    a.D_lo = a.D_hi = p.c;
-                    a.kind = TASK_POINT;
-                    a.splits = 1;
-                    tasks[j] = a;
-                    t_fuse[j] = 0;
-                    t_dense[j] = 0;
-                    if (split) {
-                        const int t = np + 2 * (nl_before + __popc(sb & ((1u << lane) - 1u)));
-                        p.t_left = t;
-                        p.t_right = t + 1;
-                        t_fuse[j] = fuse ? (int16_t)(t + 1) : (int16_t)0;
-                        t_fuse[t] = t_fuse[t + 1] = fuse ? (int16_t)-1 : (int16_t)0;
-                        // dense bounds (splittable when the round is small), decided once here
-                        t_dense[t] = split_ok && !fuse && bound_cells(g, p.lo, p.c, s.tau) >= DENSE_CELLS;
-                        t_dense[t + 1] = split_ok && !fuse && bound_cells(g, p.c, p.hi, s.tau) >= DENSE_CELLS;
-                        Task l, r;
-                        l.D_lo = p.lo;
-                        l.D_hi = p.c;
-                        l.kind = TASK_BOUND;
-                        l.splits = 1;                 // the job builder decides (fill_splits)
-                        r.D_lo = p.c;
-                        r.D_hi = p.hi;
-                        r.kind = TASK_BOUND;
-                        r.splits = 1;
-                        tasks[t] = l;
-                        tasks[t + 1] = r;
-                        bound_iv[t] = make_float2(p.lo, p.c);
-                        bound_iv[t + 1] = make_float2(p.c, p.hi);
-                    } else {
-                        p.t_left = p.t_right = -1;
-                    }
-                }
-                nl_before += __popc(sb);
-            }
-            if (lane == 0) {
-                s.rounds++;
-                s.n_pop = np;
-                s.n_tasks = np + 2 * nl_before;
-                if (s.rounds > s.max_rounds) {
-                    s.status = DD_ERR_TIMEOUT;
-                    s.stop_kb = 0;
-                    s.n_tasks = 0;
-                    s.phase = PH_DONE;
-                }
-            }
+        const unsigned fail = __ballot_sync(0xffffffffu, v && !pass);
+        const unsigned ms = __ballot_sync(0xffffffffu, split), mf = __ballot_sync(0xffffffffu, fuse);
+        const unsigned ml = __ballot_sync(0xffffffffu, dense_l), mr = __ballot_sync(0xffffffffu, dense_r);
+        if (lane == 0) {
+            sm.pop_fail[wid] = fail ? 32 * wid + __ffs(fail) - 1 : MAX_POP;
+            sm.pop_mask[wid] = make_uint4(ms, mf, ml, mr);
         }
-        __syncwarp();
-        // Jobs of the next round, bound tasks first: a task of `splits` splits
-        // contributes that many jobs (fill_splits for the dense bounds, ranked
-        // in this loop's order; every other task has one split).
-        if (s.phase != PH_DONE) {
-            const int nt = s.n_tasks;
-            int nd = 0, nabs = 0;                 // dense bound tasks; tasks inside fused jobs
-            for (int c0 = 0; c0 < nt; c0 += 32) {
-                const int q = c0 + lane, t = nt - 1 - q;
-                nd += __popc(__ballot_sync(0xffffffffu, q < nt && t_dense[t]));
-                nabs += __popc(__ballot_sync(0xffffffffu, q < nt && t_fuse[t] < 0));
-            }
-            const int units = (nt - nabs) * g.n_tiles;   // one per job and band before any split
-            // the window's share of the grid: the searches still running
-            // after the last round share it (all of them before the first)
-            const int sharers = n_windows == 1 ? 1 : (running > 0 ? running : n_windows);
-            const int target = g.split_target / sharers;
-            int total = 0, seen = 0;
-            for (int c0 = 0; c0 < nt; c0 += 32) {     // jobs per task, counted once
-                const int q = c0 + lane, t = nt - 1 - q;
-                const bool d = q < nt && t_dense[t];
+    }
+    __syncthreads();
+    const int first = min(sm.pop_fail[0], sm.pop_fail[1]), np = min(lim, first);
+    const unsigned in0 = np >= 32 ? 0xffffffffu : (1u << np) - 1u;
+    const unsigned in1 = np >= 64 ? 0xffffffffu : (np > 32 ? (1u << (np - 32)) - 1u : 0u);
+    const uint4 m0 = sm.pop_mask[0], m1 = sm.pop_mask[1];
+    const int n_split = __popc(m0.x & in0) + __popc(m1.x & in1);
+    const int nt = np + 2 * n_split, n_fused = __popc(m0.y & in0) + __popc(m1.y & in1);
+    const int nd = __popc(m0.z & in0) + __popc(m1.z & in1) + __popc(m0.w & in0) + __popc(m1.w & in1);
+    const bool late = np > 0 && s.rounds + 1 > s.max_rounds, done = np == 0 || late;
+    if (wid < 2 && tid < np) {
+        const unsigned below = (1u << lane) - 1u;
+        p.t_point = tid;
+        p.t_left = p.t_right = -1;
+        p.pad = 0;
+        Task t;
+        t.D_lo = t.D_hi = p.c;
+        t.kind = TASK_POINT;
+        t.splits = 1;                             // the job builder decides (fill_splits)
+        tasks[tid] = t;
+        sm.t_fuse[tid] = 0;
+        sm.t_dense[tid] = 0;
+        if (split) {
+            const int l = np + 2 * (__popc((wid ? m1.x : m0.x) & below) + (wid ? __popc(m0.x) : 0));
+            p.t_left = l;
+            p.t_right = l + 1;
+            sm.t_fuse[tid] = fuse ? (int16_t)(l + 1) : (int16_t)0;
+            sm.t_fuse[l] = sm.t_fuse[l + 1] = fuse ? (int16_t)-1 : (int16_t)0;
+            sm.t_dense[l] = dense_l;
+            sm.t_dense[l + 1] = dense_r;
+            t.kind = TASK_BOUND;
+            t.D_lo = p.lo;
+            t.D_hi = p.c;
+            tasks[l] = t;
+            t.D_lo = p.c;
+            t.D_hi = p.hi;
+            tasks[l + 1] = t;
+        }
+        s.pop[tid] = p;
+    }
+    __syncthreads();                              // the state above is read, the tasks' kinds are known
+    if (tid == 0) {
+        if (!stop && first == 0 && lim > 0) {     // the search ends here
+            s.have_stop = 1;
+            s.stop_kb = sm.q_head[0].kb;
+        }
+        s.q_start = np;
+        s.q_n -= np;
+        s.n_pop = done ? 0 : np;
+        s.n_tasks = done ? 0 : nt;
+        if (np > 0) s.rounds++;
+        if (late) {
+            s.status = DD_ERR_TIMEOUT;
+            s.stop_kb = 0;
+            s.n_pop = np;
+        } else if (done) {
+            i128 top = K_hat;
+            if (s.have_leaf && s.leaf_max > top) top = s.leaf_max;
+            if (s.have_stop && s.stop_kb > top) top = s.stop_kb;
+            s.stop_kb = top - K_hat;              // the certificate gap_K
+        }
+        if (done) s.phase = PH_DONE;
+    }
+    // Jobs of the next round, bound tasks first: a task of `splits` splits
+    // contributes that many jobs (fill_splits for the dense bounds, ranked in
+    // this loop's order; every other task has one split).
+    if (wid == 0 && !done) {
+        const int units = (nt - 2 * n_fused) * g.n_tiles;    // one per job and band before any split
+        // the window's share of the grid: the searches still running after
+        // the last round share it (all of them before the first)
+        const int sharers = c.n_windows == 1 ? 1 : (running > 0 ? running : c.n_windows);
+        const int target = sharers == 1 ? g.split_target : g.split_target / sharers;
+        const bool extra = nd > 0 && target - units >= g.n_tiles;
+        int total = 0, seen = 0;
+        for (int c0 = 0; c0 < nt; c0 += 32) {     // jobs per task, counted once
+            const int q = c0 + lane, t = nt - 1 - q;
+            int n = q < nt && sm.t_fuse[t] >= 0 ? 1 : 0;
+            int before;
+            if (extra) {
+                const bool d = q < nt && sm.t_dense[t];
                 const unsigned db = __ballot_sync(0xffffffffu, d);
-                const int rank = seen + __popc(db & ((1u << lane) - 1u));
+                if (d) n = fill_splits(g, target, units, nd, seen + __popc(db & ((1u << lane) - 1u)));
                 seen += __popc(db);
-                const int n = q >= nt || t_fuse[t] < 0 ? 0 : (d ? fill_splits(g, target, units, nd, rank) : 1);
                 const int incl = warp_incl_scan(n);
-                if (q < nt) {
-                    t_jobs[q] = (int16_t)n;
-                    t_at[q] = (int16_t)(total + incl - n);
-                }
+                before = total + incl - n;
                 total += __shfl_sync(0xffffffffu, incl, 31);
+            } else {                              // one job or none each
+                const unsigned b = __ballot_sync(0xffffffffu, n);
+                before = total + __popc(b & ((1u << lane) - 1u));
+                total += __popc(b);
             }
-            if (lane == 0) {
-                if (n_windows == 1) {             // the only block: the list is its own
-                    sch->n_jobs[par ^ 1] = total;
-                    sm.s_base = 0;
-                } else {
-                    sm.s_base = atomicAdd(&sch->n_jobs[par ^ 1], total);
-                }
+            if (q < nt) {
+                sm.t_jobs[q] = (int16_t)n;
+                sm.t_at[q] = (int16_t)before;
+            }
+        }
+        if (lane == 0) {
+            if (c.n_windows == 1) {               // the only block: the list is its own
+                sch->n_jobs[par ^ 1] = total;
+                sm.s_base = 0;
+            } else {
+                sm.s_base = atomicAdd(&sch->n_jobs[par ^ 1], total);
             }
         }
     }
     __syncthreads();
-    if (s.phase != PH_DONE) {                     // the jobs, written by the whole block
-        const int nt = s.n_tasks;
+    if (!done)                                    // the jobs, written by the whole block
         for (int q = tid; q < nt; q += blockDim.x) {
-            const int n = t_jobs[q], t = nt - 1 - q;
-            const int fz = n > 0 ? (int)t_fuse[t] : 0;
-            Job* out = jobs + sm.s_base + t_at[q];
+            const int n = sm.t_jobs[q], t = nt - 1 - q;
+            const int fz = n > 0 ? (int)sm.t_fuse[t] : 0;
+            Job* out = jobs + sm.s_base + sm.t_at[q];
             for (int k = 0; k < n; k++) {
                 Job j;
                 j.win = w;
@@ -1908,30 +1869,29 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
                 out[k] = j;
             }
         }
-    }
-    if (!RESIDENT || s.phase == PH_DONE)
+    if (!RESIDENT || done)
         for (int i = tid; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
             reinterpret_cast<int4*>(st)[i] = reinterpret_cast<const int4*>(&s)[i];
-    } // s.phase != PH_DONE at entry
+    } // phase != PH_DONE at entry
     if (RESIDENT) return;
     __syncthreads();
-    if (tid == 0 && phase_out) phase_out[w] = s.phase;
-    if (tid == 0 && n_windows == 1) {             // the only block is the last: no ticket
+    if (tid == 0 && c.phase_out) c.phase_out[w] = s.phase;
+    if (tid == 0 && c.n_windows == 1) {           // the only block is the last: no ticket
         const int active = s.phase != PH_DONE ? 1 : 0;
         sch->running = active;
         sch->round += 1;
-        if (use_loop) cudaGraphSetConditional(c.loop, active ? 1u : 0u);
+        if (c.use_loop) cudaGraphSetConditional(c.loop, active ? 1u : 0u);
     } else if (tid == 0) {
         __threadfence();
         if (s.phase != PH_DONE) atomicAdd(&sch->active, 1);
-        if (atomicAdd(&sch->ticket, 1) == n_windows - 1) {    // the last block of the round
+        if (atomicAdd(&sch->ticket, 1) == c.n_windows - 1) {  // the last block of the round
             __threadfence();
             const int active = atomicAdd(&sch->active, 0);
             sch->running = active;
             sch->active = 0;
             sch->ticket = 0;
             sch->round += 1;
-            if (use_loop) cudaGraphSetConditional(c.loop, active > 0 ? 1u : 0u);
+            if (c.use_loop) cudaGraphSetConditional(c.loop, active > 0 ? 1u : 0u);
         }
     }
 }
