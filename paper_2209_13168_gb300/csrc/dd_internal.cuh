@@ -188,9 +188,15 @@ __host__ __device__ inline float warp_tref(const Geom& g, float tau) { return g.
 // splitting over several blocks.  A schedule estimate only (the threshold
 // was set by measurement).
 constexpr float DENSE_CELLS = 2.0f;
-// Split bands of bounds below SPLIT_ROWS_CELLS are divided by rows, longer
-// ones by events (see eval_unit).
+// Split bands of bounds below SPLIT_ROWS_CELLS, and of windows of fewer than
+// SPLIT_ROWS_EVENTS events, are divided by rows, others by events.  A slice of
+// rows reads nearly all of a long bound's candidates again; a share of the
+// events counts into a whole band, which is then merged cell by cell in L2.
+// By rows against by events for every long bound (searches, us): 4,000 events
+// 330 / 370, 20,000 466 / 527, 50,000 880 / 950, 100,000 865 / 882, 150,000
+// 1,597 / 1,560, 300,000 2,778 / 2,620, 600,000 5,350 / 4,980.
 constexpr float SPLIT_ROWS_CELLS = 64.0f;
+constexpr int64_t SPLIT_ROWS_EVENTS = 1 << 17;
 __host__ __device__ inline float bound_cells(const Geom& g, float D_lo, float D_hi, float tau) {
 #ifdef __CUDA_ARCH__
     // an estimate: fast reciprocals (deterministic, so every unit of a task agrees)

@@ -435,7 +435,7 @@ __device__ __forceinline__ void prepare_unit(const Geom& g, const EvalArgs& a, c
     const int plane = ti >= g.plane_tiles ? 1 : 0, band = ti - plane * g.plane_tiles;
     int splits = fused ? 1 : max(1, jb.splits);
     int y0 = band * g.band_rows, rows = min(g.band_rows, g.H - y0);
-    if (splits > 1 && (!a.mg.acc || cells < SPLIT_ROWS_CELLS)) {    // split by rows: its own rows
+    if (splits > 1 && (!a.mg.acc || cells < SPLIT_ROWS_CELLS || win->n < SPLIT_ROWS_EVENTS)) {    // split by rows: its own rows
         const int r0 = (int)((uint32_t)(rows * jb.split) / (uint32_t)splits);
         rows = (int)((uint32_t)(rows * (jb.split + 1)) / (uint32_t)splits) - r0;
         y0 += r0;
