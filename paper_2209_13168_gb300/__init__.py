@@ -317,6 +317,12 @@ class Events:
                    None if p is None else torch.from_numpy(p).to(device))
 
 
+def _i128s(K, n):
+    """The first n of an array of dd_i128 as Python integers."""
+    w = np.frombuffer(K, np.uint64)
+    return [(hi << 64) | lo for lo, hi in zip(w[0:2 * n:2].tolist(), w[1:2 * n:2].view(np.int64).tolist())]
+
+
 def dd_contrast(h, ev, D, want=("S", "N"), want_iwe=False, M=None):
     D = np.ascontiguousarray(D, dtype=np.float32)
     n = D.size
@@ -326,7 +332,7 @@ def dd_contrast(h, ev, D, want=("S", "N"), want_iwe=False, M=None):
     img = np.zeros(n * M, np.uint32) if want_iwe else None
     _check(load().dd_contrast(h, ctypes.byref(ev.c), D.ctypes.data, n, ctypes.cast(K, _VP), S.ctypes.data,
                               N.ctypes.data, img.ctypes.data if want_iwe else None), "dd_contrast")
-    return [K[i].value() for i in range(n)], S, N, img
+    return _i128s(K, n), S, N, img
 
 
 def dd_bound(h, ev, D_lo, D_hi, want_iwe=False, M=None):
@@ -339,7 +345,7 @@ def dd_bound(h, ev, D_lo, D_hi, want_iwe=False, M=None):
     img = np.zeros(n * M, np.uint32) if want_iwe else None
     _check(load().dd_bound(h, ctypes.byref(ev.c), D_lo.ctypes.data, D_hi.ctypes.data, n, ctypes.cast(K, _VP),
                            S.ctypes.data, N.ctypes.data, img.ctypes.data if want_iwe else None), "dd_bound")
-    return [K[i].value() for i in range(n)], S, N, img
+    return _i128s(K, n), S, N, img
 
 
 def dd_solve(h, ev, D_lo, D_hi, tol_D, gamma):
@@ -567,7 +573,7 @@ def dd_contrast_noalloc(W, H, foe_x, foe_y, ev, D, stream_ptr=None):
     _check(load().dd_contrast_noalloc(W, H, foe_x, foe_y, ctypes.byref(ev.c), D.ctypes.data, n,
                                       ctypes.cast(K, _VP), _VP(stream_ptr) if stream_ptr else None),
            "dd_contrast_noalloc")
-    return [K[i].value() for i in range(n)]
+    return _i128s(K, n)
 
 
 class Server:

@@ -33,17 +33,25 @@ struct dd_ctx {
 
     // per-window buffers, sized for win_cap windows
     int win_cap = 0;
-    int32_t *row_count = nullptr, *row_off = nullptr, *cursor = nullptr, *err = nullptr;
-    dd::WinIn* wins = nullptr;
-    dd::WinParams* params = nullptr;
+    int32_t *row_count = nullptr, *row_off = nullptr, *cursor = nullptr;   // row_count: zero between calls
     dd::SolveState* st = nullptr;
     dd::Node* queues = nullptr;   // per window: two buffers of queue_capacity nodes
     dd::Task* tasks = nullptr;
-    dd::Partial* part = nullptr;
+    dd::Partial* part = nullptr;  // zero between calls
     dd::Job* jobs = nullptr;      // two lists of job_stride jobs
     int job_stride = 0;
-    int32_t* chunk_win = nullptr;
-    int64_t chunk_cap = 0;
+
+    // What a call hands to the device, staged in pinned memory (h_call) and
+    // copied at once: the round bookkeeping and error words (zero), window
+    // descriptors and search parameters at fixed places, then the call's
+    // ingest chunks and, for dd_contrast and dd_bound, tasks and jobs.
+    unsigned char *call = nullptr, *h_call = nullptr;
+    size_t call_cap = 0, call_head = 0, call_used = 0;
+    dd::Sched *sch = nullptr, *h_sch = nullptr;
+    int32_t* err = nullptr;
+    dd::WinIn *wins = nullptr, *h_wins = nullptr;
+    dd::WinParams *params = nullptr, *h_params = nullptr;
+    int32_t* chunk_win = nullptr; // this call's
     int32_t n_chunks = 0;         // ingest chunks of the last call
 
     // fast mode scratch
@@ -56,14 +64,12 @@ struct dd_ctx {
     dd_mlp* warm_model = nullptr;
     int32_t* feat_counts = nullptr;   // [window][128]
     int feat_cap = 0;
-    dd::Sched* sch = nullptr;
 
     // single-window extras
     uint32_t* macc = nullptr;     // merge buffers of split jobs (zero between uses)
     int32_t* mdone = nullptr;
     dd::Partial* msums = nullptr;
-    i128* keys = nullptr;
-    unsigned long long *S = nullptr, *C = nullptr, *F = nullptr;
+    unsigned char *out = nullptr, *h_out = nullptr;   // results of up to max_tasks tasks, copied back at once
     uint32_t* iwe = nullptr;
     size_t iwe_cap = 0;
     dd::TraceRec* trace = nullptr;
@@ -84,12 +90,6 @@ struct dd_ctx {
 
     // pinned host staging
     dd::SolveState* h_st = nullptr;
-    dd::Task* h_tasks = nullptr;
-    dd::Job* h_jobs = nullptr;
-    dd::Sched* h_sch = nullptr;
-    dd::WinIn* h_wins = nullptr;
-    dd::WinParams* h_params = nullptr;
-    int32_t* h_chunks = nullptr;
     int32_t* h_err = nullptr;
 };
 
@@ -174,12 +174,12 @@ dd::EvalArgs eval_args(dd_ctx* c, uint32_t* iwe_out, bool single) {
     return a;
 }
 
-cudaError_t eval(dd_ctx* c, uint32_t* iwe, bool single) {
+cudaError_t eval(dd_ctx* c, const dd::EvalArgs& a) {
     if (c->timing) {
         cudaError_t e = record(c);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = dd::launch_eval(c->g, eval_args(c, iwe, single), c->threads, c->eval_blocks, c->stream);
+    cudaError_t e = dd::launch_eval(c->g, a, c->threads, c->eval_blocks, c->stream);
     if (e != cudaSuccess) return e;
     c->stats.kernel_launches++;
     c->stats.eval_launches++;
@@ -196,18 +196,16 @@ int ensure_windows(dd_ctx* c, int nw) {
     release(c->row_count);
     release(c->row_off);
     release(c->cursor);
-    release(c->err);
-    release(c->wins);
-    release(c->params);
     release(c->st);
     release(c->queues);
     release(c->tasks);
     release(c->part);
     release(c->jobs);
     release_host(c->h_st);
-    release_host(c->h_wins);
-    release_host(c->h_params);
     release_host(c->h_err);
+    release(c->call);
+    release_host(c->h_call);
+    c->call_cap = 0;
     c->win_cap = 0;
     const int jw = cap * dd::jobs_per_window(c->g, c->max_tasks);
     const int js = jw > c->max_tasks * c->g.max_splits ? jw : c->max_tasks * c->g.max_splits;
@@ -221,21 +219,49 @@ int ensure_windows(dd_ctx* c, int nw) {
     A((void**)&c->row_count, sizeof(int32_t) * (size_t)bins * cap);
     A((void**)&c->row_off, sizeof(int32_t) * (size_t)(bins + 1) * cap);
     A((void**)&c->cursor, sizeof(int32_t) * (size_t)bins * cap);
-    A((void**)&c->err, sizeof(int32_t) * (size_t)cap);
-    A((void**)&c->wins, sizeof(dd::WinIn) * (size_t)cap);
-    A((void**)&c->params, sizeof(dd::WinParams) * (size_t)cap);
     A((void**)&c->st, sizeof(dd::SolveState) * (size_t)cap);
     A((void**)&c->queues, sizeof(dd::Node) * 2 * (size_t)c->cfg.queue_capacity * cap);
     A((void**)&c->tasks, sizeof(dd::Task) * (size_t)c->max_tasks * cap);
     A((void**)&c->part, sizeof(dd::Partial) * (size_t)c->max_tasks * cap);
     A((void**)&c->jobs, sizeof(dd::Job) * 2 * (size_t)js);
     AH((void**)&c->h_st, sizeof(dd::SolveState) * (size_t)cap);
-    AH((void**)&c->h_wins, sizeof(dd::WinIn) * (size_t)cap);
-    AH((void**)&c->h_params, sizeof(dd::WinParams) * (size_t)cap);
     AH((void**)&c->h_err, sizeof(int32_t) * (size_t)cap);
     if (rc) return rc;
+    // on the stream that uses them: the context's own does not wait for others
+    const cudaStream_t st = c->stream ? c->stream : c->own;
+    DD_TRY(cudaMemsetAsync(c->row_count, 0, sizeof(int32_t) * (size_t)bins * cap, st));
+    DD_TRY(cudaMemsetAsync(c->part, 0, sizeof(dd::Partial) * (size_t)c->max_tasks * cap, st));
     c->job_stride = js;
     c->win_cap = cap;
+    return DD_OK;
+}
+
+size_t align64(size_t n) { return (n + 63) & ~(size_t)63; }
+
+// The call block with room for `tail` bytes after its head (which has room for
+// win_cap windows).
+int ensure_call(dd_ctx* c, size_t tail) {
+    if (c->call && c->call_head + tail <= c->call_cap) return DD_OK;
+    drop_graph(c);                                // it holds the block's addresses
+    release(c->call);
+    release_host(c->h_call);
+    c->call_cap = 0;
+    const size_t n = (size_t)c->win_cap;
+    const size_t at_err = align64(sizeof(dd::Sched)), at_win = at_err + align64(sizeof(int32_t) * n);
+    const size_t at_par = at_win + align64(sizeof(dd::WinIn) * n);
+    c->call_head = at_par + align64(sizeof(dd::WinParams) * n);
+    const size_t cap = c->call_head + tail + tail / 2;
+    DD_TRY(cudaMalloc((void**)&c->call, cap));
+    DD_TRY(cudaMallocHost((void**)&c->h_call, cap));
+    std::memset(c->h_call, 0, c->call_head);
+    c->sch = (dd::Sched*)c->call;
+    c->err = (int32_t*)(c->call + at_err);
+    c->wins = (dd::WinIn*)(c->call + at_win);
+    c->params = (dd::WinParams*)(c->call + at_par);
+    c->h_sch = (dd::Sched*)c->h_call;
+    c->h_wins = (dd::WinIn*)(c->h_call + at_win);
+    c->h_params = (dd::WinParams*)(c->h_call + at_par);
+    c->call_cap = cap;
     return DD_OK;
 }
 
@@ -257,11 +283,10 @@ int ensure_staging(dd_ctx* c, int64_t n) {
     return DD_OK;
 }
 
-// Upload (host arrays) or alias (device arrays) the events of nw windows,
-// then sort each window's events by (time bucket, row).  Sets err[w] on
-// malformed events of window w.
-int ingest(dd_ctx* c, const dd_events* evs, int nw) {
-    dd::NvtxRange range("dd ingest");
+// Upload (host arrays) or alias (device arrays) the events of nw windows and
+// stage their descriptors and ingest chunks in the call block, with room for
+// `more` further bytes at call_used.
+int stage(dd_ctx* c, const dd_events* evs, int nw, size_t more = 0) {
     int rc = ensure_windows(c, nw);
     if (rc) return rc;
     int64_t total = 0, host_total = 0, chunks = 0;
@@ -280,15 +305,13 @@ int ingest(dd_ctx* c, const dd_events* evs, int nw) {
     }
     rc = ensure_staging(c, host_total);
     if (rc) return rc;
-    if (chunks > c->chunk_cap) {
-        release(c->chunk_win);
-        release_host(c->h_chunks);
-        c->chunk_cap = 0;
-        const int64_t nc = chunks < 256 ? 256 : chunks + chunks / 2;
-        DD_TRY(cudaMalloc((void**)&c->chunk_win, sizeof(int32_t) * nc));
-        DD_TRY(cudaMallocHost((void**)&c->h_chunks, sizeof(int32_t) * nc));
-        c->chunk_cap = nc;
-    }
+    const size_t chunk_bytes = align64(sizeof(int32_t) * (size_t)chunks);
+    rc = ensure_call(c, chunk_bytes + more);
+    if (rc) return rc;
+    std::memset(c->h_sch, 0, sizeof(dd::Sched));
+    c->chunk_win = (int32_t*)(c->call + c->call_head);
+    int32_t* h_chunks = (int32_t*)(c->h_call + c->call_head);
+    c->call_used = c->call_head + chunk_bytes;
     int64_t off = 0, hoff = 0;
     int32_t ch = 0;
     for (int w = 0; w < nw; w++) {
@@ -318,16 +341,23 @@ int ingest(dd_ctx* c, const dd_events* evs, int nw) {
         wi.chunk0 = ch;
         wi.pad = 0;
         const int32_t nch = (int32_t)((e.n + dd::CHUNK - 1) / dd::CHUNK);
-        for (int32_t k = 0; k < nch; k++) c->h_chunks[ch + k] = w;
+        for (int32_t k = 0; k < nch; k++) h_chunks[ch + k] = w;
         ch += nch;
         off += e.n;
     }
-    DD_TRY(copy(c, c->wins, c->h_wins, sizeof(dd::WinIn) * nw, cudaMemcpyHostToDevice));
-    if (ch) DD_TRY(copy(c, c->chunk_win, c->h_chunks, sizeof(int32_t) * ch, cudaMemcpyHostToDevice));
     c->n_chunks = ch;
-    DD_TRY(dd::launch_ingest(c->g, c->wins, nw, c->chunk_win, ch, c->ev, c->row_count, c->row_off,
-                             c->cursor, c->err, c->stream));
-    c->stats.kernel_launches += ch ? 3 : 1;
+    return DD_OK;
+}
+
+// Copy the call block, then sort each window's events by (time bucket, row).
+// Sets err[w] on malformed events of window w.
+int ingest(dd_ctx* c, int nw) {
+    dd::NvtxRange range("dd ingest");
+    DD_TRY(copy(c, c->call, c->h_call, c->call_used, cudaMemcpyHostToDevice));
+    int launches = 0;
+    DD_TRY(dd::launch_ingest(c->g, c->wins, nw, c->chunk_win, c->n_chunks, c->ev, c->row_count, c->row_off, c->cursor,
+                             c->err, c->stream, false, &launches));
+    c->stats.kernel_launches += launches;
     return DD_OK;
 }
 
@@ -338,70 +368,99 @@ dd_i128 from_i128(i128 v) {
     return r;
 }
 
-// Evaluate n tasks (point or bound) of one window and copy keys, sums and
-// images to the host.
+// Stage up to max_tasks tasks (point or bound) of one window, and their jobs,
+// at call_used; returns the number of tasks and sets their places.
+int32_t stage_tasks(dd_ctx* c, int32_t n, int kind, const float* A, const float* B, float tau, dd::EvalArgs* a) {
+    const int32_t m = n < c->max_tasks ? n : c->max_tasks;
+    const size_t at_tasks = c->call_used, at_jobs = at_tasks + align64(sizeof(dd::Task) * (size_t)m);
+    dd::Task* tasks = (dd::Task*)(c->h_call + at_tasks);
+    dd::Job* jobs = (dd::Job*)(c->h_call + at_jobs);
+    auto dense = [&](int32_t j) {
+        return kind == dd::TASK_BOUND && dd::bound_cells(c->g, A[j], B[j], tau) >= dd::DENSE_CELLS;
+    };
+    int32_t nj = 0, n_dense = 0, rank = 0;
+    for (int32_t j = 0; j < m; j++) n_dense += dense(j);
+    for (int32_t j = 0; j < m; j++) {
+        dd::Task& t = tasks[j];
+        t.D_lo = A[j];
+        t.D_hi = B[j];
+        t.kind = kind;
+        t.splits = dense(j) ? dd::fill_splits(c->g, c->g.split_target, m * c->g.n_tiles, n_dense, rank++) : 1;
+    }
+    for (int32_t j = m - 1; j >= 0; j--)              // heavier tasks first
+        for (int32_t s = 0; s < tasks[j].splits; s++) {
+            dd::Job& jb = jobs[nj++];
+            jb.win = 0;
+            jb.task = j;
+            jb.split = s;
+            jb.splits = tasks[j].splits;
+        }
+    std::memset(c->h_sch, 0, sizeof(dd::Sched));
+    c->h_sch->n_jobs[0] = nj;
+    a->tasks = (dd::Task*)(c->call + at_tasks);
+    a->jobs = (dd::Job*)(c->call + at_jobs);
+    c->call_used = at_jobs + sizeof(dd::Job) * (size_t)nj;
+    return m;
+}
+
+// Evaluate n tasks of one window and copy keys, sums and images to the host,
+// max_tasks at a time: one copy in (with the window's descriptor the first
+// time), the evaluation and the keys, one copy out.
 int eval_tasks(dd_ctx* c, const dd_events* ev, int32_t n, int kind, const float* A, const float* B, dd_i128* K,
                uint64_t* S, int64_t* N, uint32_t* iwe) {
     const int64_t M = (int64_t)c->g.planes * c->g.W * c->g.H;     // image cells of one task
     dd::NvtxRange range(kind == dd::TASK_POINT ? "dd contrast" : "dd bound");
-    for (int32_t j0 = 0; j0 < n; j0 += c->max_tasks) {
-        const int32_t m = n - j0 < c->max_tasks ? n - j0 : c->max_tasks;
-        int32_t nj = 0;
-        int32_t n_dense = 0, rank = 0;
-        for (int32_t j = 0; j < m; j++)
-            n_dense += kind == dd::TASK_BOUND && dd::bound_cells(c->g, A[j0 + j], B[j0 + j], ev->tau) >= dd::DENSE_CELLS;
-        for (int32_t j = 0; j < m; j++) {
-            dd::Task& t = c->h_tasks[j];
-            t.D_lo = A[j0 + j];
-            t.D_hi = B[j0 + j];
-            t.kind = kind;
-            const bool dense = kind == dd::TASK_BOUND && dd::bound_cells(c->g, t.D_lo, t.D_hi, ev->tau) >= dd::DENSE_CELLS;
-            t.splits = dense ? dd::fill_splits(c->g, c->g.split_target, m * c->g.n_tiles, n_dense, rank++) : 1;
+    int rc = stage(c, ev, 1, align64(sizeof(dd::Task) * (size_t)c->max_tasks) +
+                                 sizeof(dd::Job) * (size_t)c->max_tasks * c->g.max_splits);
+    if (rc) return rc;
+    const size_t tail = c->call_used;
+    for (int32_t j0 = 0; j0 < n || j0 == 0;) {
+        dd::EvalArgs a = eval_args(c, nullptr, true);
+        int32_t m = 0;
+        c->call_used = tail;
+        if (n > 0) m = stage_tasks(c, n - j0, kind, A + j0, B + j0, ev->tau, &a);
+        if (j0 == 0) {
+            rc = ingest(c, 1);
+            if (rc) return rc;
+        } else {
+            DD_TRY(copy(c, c->sch, c->h_sch, sizeof(dd::Sched), cudaMemcpyHostToDevice));
+            DD_TRY(copy(c, c->call + tail, c->h_call + tail, c->call_used - tail, cudaMemcpyHostToDevice));
         }
-        for (int32_t j = m - 1; j >= 0; j--)              // heavier tasks first
-            for (int32_t s = 0; s < c->h_tasks[j].splits; s++) {
-                dd::Job& jb = c->h_jobs[nj++];
-                jb.win = 0;
-                jb.task = j;
-                jb.split = s;
-                jb.splits = c->h_tasks[j].splits;
+        // results: the window's error word, then keys, S, C and F
+        const size_t at_key = 16, at_S = at_key + sizeof(i128) * (size_t)m, w = sizeof(unsigned long long) * (size_t)m;
+        if (m > 0) {
+            if (iwe) {
+                const size_t need = (size_t)m * M;
+                if (need > c->iwe_cap) {
+                    release(c->iwe);
+                    c->iwe_cap = 0;
+                    DD_TRY(cudaMalloc((void**)&c->iwe, need * sizeof(uint32_t)));
+                    c->iwe_cap = need;
+                }
+                a.iwe_out = c->iwe;
             }
-        std::memset(c->h_sch, 0, sizeof(dd::Sched));
-        c->h_sch->n_jobs[0] = nj;
-        DD_TRY(copy(c, c->tasks, c->h_tasks, sizeof(dd::Task) * m, cudaMemcpyHostToDevice));
-        DD_TRY(copy(c, c->jobs, c->h_jobs, sizeof(dd::Job) * nj, cudaMemcpyHostToDevice));
-        DD_TRY(copy(c, c->sch, c->h_sch, sizeof(dd::Sched), cudaMemcpyHostToDevice));
-        DD_TRY(cudaMemsetAsync(c->part, 0, sizeof(dd::Partial) * m, c->stream));   // the tasks' sums start at zero
-        uint32_t* iw = nullptr;
-        if (iwe) {
-            size_t need = (size_t)m * M;
-            if (need > c->iwe_cap) {
-                release(c->iwe);
-                c->iwe_cap = 0;
-                DD_TRY(cudaMalloc((void**)&c->iwe, need * sizeof(uint32_t)));
-                c->iwe_cap = need;
-            }
-            iw = c->iwe;
+            DD_TRY(eval(c, a));
+            DD_TRY(dd::launch_keys(c->g, a.tasks, m, c->part, (i128*)(c->out + at_key),
+                                   (unsigned long long*)(c->out + at_S), (unsigned long long*)(c->out + at_S + w),
+                                   (unsigned long long*)(c->out + at_S + 2 * w), c->stream, c->err, (int32_t*)c->out));
+            c->stats.kernel_launches++;
+            DD_TRY(copy(c, c->h_out, c->out, at_S + 3 * w, cudaMemcpyDeviceToHost));
+            if (iwe)
+                DD_TRY(copy(c, iwe + (size_t)j0 * M, c->iwe, sizeof(uint32_t) * (size_t)m * M, cudaMemcpyDeviceToHost));
+        } else {
+            DD_TRY(copy(c, c->h_out, c->err, sizeof(int32_t), cudaMemcpyDeviceToHost));
         }
-        DD_TRY(eval(c, iw, true));
-        DD_TRY(dd::launch_keys(c->g, c->tasks, m, c->part, c->keys, c->S, c->C, c->F, c->stream));
-        c->stats.kernel_launches++;
-        std::vector<i128> hk(m);
-        std::vector<unsigned long long> hs(m), hc(m), hf(m);
-        DD_TRY(copy(c, hk.data(), c->keys, sizeof(i128) * m, cudaMemcpyDeviceToHost));
-        DD_TRY(copy(c, hs.data(), c->S, sizeof(unsigned long long) * m, cudaMemcpyDeviceToHost));
-        DD_TRY(copy(c, hc.data(), c->C, sizeof(unsigned long long) * m, cudaMemcpyDeviceToHost));
-        DD_TRY(copy(c, hf.data(), c->F, sizeof(unsigned long long) * m, cudaMemcpyDeviceToHost));
-        DD_TRY(copy(c, c->h_err, c->err, sizeof(int32_t), cudaMemcpyDeviceToHost));
-        if (iwe)
-            DD_TRY(copy(c, iwe + (size_t)j0 * M, c->iwe, sizeof(uint32_t) * (size_t)m * M, cudaMemcpyDeviceToHost));
         DD_TRY(sync(c));
-        if (c->h_err[0]) return DD_ERR_ARG;
+        if (*(const int32_t*)c->h_out) return DD_ERR_ARG;
+        const i128* hk = (const i128*)(c->h_out + at_key);
+        const unsigned long long* hs = (const unsigned long long*)(c->h_out + at_S);
         for (int32_t j = 0; j < m; j++) {
             K[j0 + j] = from_i128(hk[j]);
             if (S) S[j0 + j] = hs[j];
-            if (N) N[j0 + j] = (int64_t)(kind == dd::TASK_POINT ? hc[j] : hf[j]);
+            if (N) N[j0 + j] = (int64_t)(kind == dd::TASK_POINT ? hs[m + j] : hs[2 * m + j]);
         }
+        if (m == 0) break;
+        j0 += m;
     }
     return DD_OK;
 }
@@ -513,7 +572,7 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
         DD_TRY(cudaMalloc((void**)&c->trace, sizeof(dd::TraceRec) * trace_cap));
         c->trace_cap = trace_cap;
     }
-    int rc = ingest(c, evs, nw);
+    int rc = stage(c, evs, nw);
     if (rc) return rc;
     const int64_t M = (int64_t)c->g.W * c->g.H;
     bool model = false;
@@ -529,7 +588,8 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
         q.pad0 = q.pad1 = 0;
         model |= prm[w].warm == DD_WARM_MODEL;
     }
-    DD_TRY(copy(c, c->params, c->h_params, sizeof(dd::WinParams) * nw, cudaMemcpyHostToDevice));
+    rc = ingest(c, nw);
+    if (rc) return rc;
     if (model) {                                  // the model's guesses, on the device
         dd::MlpDev m;
         int dev = -1;
@@ -539,7 +599,6 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
         DD_TRY(dd::launch_warm(c->g, nw, c->feat_counts, c->wins, c->params, m, c->stream));
         c->stats.kernel_launches++;
     }
-    DD_TRY(cudaMemsetAsync(c->sch, 0, sizeof(dd::Sched), c->stream));
     DD_TRY(dd::launch_init(c->g, nw, c->st, c->tasks, c->max_tasks, c->part, c->wins, c->params, c->jobs,
                            c->job_stride, c->sch, c->cfg.pop_k, c->cfg.queue_capacity, c->cfg.max_rounds,
                            (int32_t)trace_cap, c->stream));
@@ -571,7 +630,7 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
         int batch = c->timing ? 1 : 2;
         for (;;) {
             for (int b = 0; b < batch; b++) {
-                DD_TRY(eval(c, nullptr, nw == 1));
+                DD_TRY(eval(c, eval_args(c, nullptr, nw == 1)));
                 DD_TRY(dd::launch_control(c->g, nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err,
                                           tr_dev, c->jobs, c->job_stride, c->sch, 0, 0, c->stream));
                 c->stats.kernel_launches++;
@@ -583,11 +642,11 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
         }
     }
     DD_TRY(copy(c, c->h_st, c->st, sizeof(dd::SolveState) * nw, cudaMemcpyDeviceToHost));
-    DD_TRY(copy(c, c->h_sch, c->sch, sizeof(dd::Sched), cudaMemcpyDeviceToHost));
+    if (graph) DD_TRY(copy(c, c->h_sch, c->sch, sizeof(dd::Sched), cudaMemcpyDeviceToHost));
     std::vector<dd::TraceRec> tr((size_t)trace_cap);
     if (trace_cap > 0) DD_TRY(copy(c, tr.data(), c->trace, sizeof(dd::TraceRec) * trace_cap, cudaMemcpyDeviceToHost));
     DD_TRY(sync(c));
-    if (search && c->h_sch->failed) {             // a wait ran out: leave the merge buffers as they must be
+    if (search && c->h_st[0].phase != dd::PH_DONE) {   // a wait ran out: leave the merge buffers as they must be
         const size_t M1 = (size_t)c->g.planes * M, tiles = (size_t)c->max_tasks * c->g.n_tiles;
         DD_TRY(cudaMemsetAsync(c->macc, 0, sizeof(uint32_t) * (size_t)c->max_tasks * M1, c->stream));
         DD_TRY(cudaMemsetAsync(c->mdone, 0, sizeof(int32_t) * tiles, c->stream));
@@ -679,34 +738,23 @@ void dd_destroy(dd_ctx* c) {
     release(c->row_count);
     release(c->row_off);
     release(c->cursor);
-    release(c->err);
-    release(c->wins);
-    release(c->params);
     release(c->st);
     release(c->queues);
     release(c->tasks);
     release(c->part);
     release(c->jobs);
-    release(c->chunk_win);
-    release(c->sch);
+    release(c->call);
     release(c->macc);
     release(c->mdone);
     release(c->msums);
-    release(c->keys);
-    release(c->S);
-    release(c->C);
-    release(c->F);
+    release(c->out);
     release(c->iwe);
     release(c->trace);
     release(c->feat_counts);
     release_host(c->h_st);
-    release_host(c->h_tasks);
-    release_host(c->h_jobs);
-    release_host(c->h_sch);
-    release_host(c->h_wins);
-    release_host(c->h_params);
-    release_host(c->h_chunks);
     release_host(c->h_err);
+    release_host(c->h_call);
+    release_host(c->h_out);
     for (cudaEvent_t e : c->t_ev) cudaEventDestroy(e);
     if (c->own) cudaStreamDestroy(c->own);
     delete c;
@@ -776,26 +824,19 @@ int dd_create(int32_t W, int32_t H, float foe_x, float foe_y, const dd_config* c
         if (rc == DD_OK && cudaMalloc(p, bytes) != cudaSuccess) rc = DD_ERR_OOM;
     };
     const size_t M = (size_t)c->g.planes * W * H;      // image cells of one task
-    A((void**)&c->sch, sizeof(dd::Sched));
     A((void**)&c->macc, sizeof(uint32_t) * (size_t)c->max_tasks * M);
     A((void**)&c->mdone, sizeof(int32_t) * (size_t)c->max_tasks * c->g.n_tiles);
     A((void**)&c->msums, sizeof(dd::Partial) * (size_t)c->max_tasks * c->g.n_tiles);
-    if (rc == DD_OK && (cudaMemset(c->macc, 0, sizeof(uint32_t) * (size_t)c->max_tasks * M) != cudaSuccess ||
-                        cudaMemset(c->mdone, 0, sizeof(int32_t) * (size_t)c->max_tasks * c->g.n_tiles) != cudaSuccess ||
-                        cudaMemset(c->msums, 0, sizeof(dd::Partial) * (size_t)c->max_tasks * c->g.n_tiles) !=
-                            cudaSuccess))
-        rc = DD_ERR_CUDA;
-    A((void**)&c->keys, sizeof(i128) * c->max_tasks);
-    A((void**)&c->S, sizeof(unsigned long long) * c->max_tasks);
-    A((void**)&c->C, sizeof(unsigned long long) * c->max_tasks);
-    A((void**)&c->F, sizeof(unsigned long long) * c->max_tasks);
-    if (rc == DD_OK && cudaMallocHost((void**)&c->h_tasks, sizeof(dd::Task) * c->max_tasks) != cudaSuccess)
-        rc = DD_ERR_OOM;
-    if (rc == DD_OK &&
-        cudaMallocHost((void**)&c->h_jobs, sizeof(dd::Job) * (size_t)c->max_tasks * c->g.max_splits) != cudaSuccess)
-        rc = DD_ERR_OOM;
-    if (rc == DD_OK && cudaMallocHost((void**)&c->h_sch, sizeof(dd::Sched)) != cudaSuccess) rc = DD_ERR_OOM;
+    const size_t out_bytes = 16 + (sizeof(i128) + 3 * sizeof(unsigned long long)) * (size_t)c->max_tasks;
+    A((void**)&c->out, out_bytes);
+    if (rc == DD_OK && cudaMallocHost((void**)&c->h_out, out_bytes) != cudaSuccess) rc = DD_ERR_OOM;
     if (rc == DD_OK && cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking) != cudaSuccess) rc = DD_ERR_CUDA;
+    const size_t tiles = (size_t)c->max_tasks * c->g.n_tiles;
+    if (rc == DD_OK &&
+        (cudaMemsetAsync(c->macc, 0, sizeof(uint32_t) * (size_t)c->max_tasks * M, c->own) != cudaSuccess ||
+         cudaMemsetAsync(c->mdone, 0, sizeof(int32_t) * tiles, c->own) != cudaSuccess ||
+         cudaMemsetAsync(c->msums, 0, sizeof(dd::Partial) * tiles, c->own) != cudaSuccess))
+        rc = DD_ERR_CUDA;
     if (rc == DD_OK && dd::eval_smem_setup(c->g) != cudaSuccess) rc = DD_ERR_CUDA;
     if (rc == DD_OK && (c->eval_blocks = dd::eval_resident_blocks(c->g, c->threads)) <= 0) rc = DD_ERR_CUDA;
     c->g.split_target = c->eval_blocks > 1 ? c->eval_blocks - 1 : c->eval_blocks;   // a search keeps one for its control
@@ -812,6 +853,7 @@ int dd_create(int32_t W, int32_t H, float foe_x, float foe_y, const dd_config* c
 
 int dd_set_stream(dd_ctx* c, void* stream) {
     if (!c) return DD_ERR_ARG;
+    if (c->stream == c->own) DD_TRY(cudaStreamSynchronize(c->own));   // dd_create's clears, before another stream's work
     c->stream = stream ? (cudaStream_t)stream : c->own;
     return DD_OK;
 }
@@ -850,13 +892,6 @@ int dd_contrast(dd_ctx* c, const dd_events* ev, const float* D, int32_t nD, dd_i
     if (rc) return rc;
     for (int32_t j = 0; j < nD; j++)
         if (!d_ok(D[j], ev->tau)) return DD_ERR_ARG;
-    rc = ingest(c, ev, 1);
-    if (rc) return rc;
-    if (nD == 0) {
-        DD_TRY(copy(c, c->h_err, c->err, sizeof(int32_t), cudaMemcpyDeviceToHost));
-        DD_TRY(sync(c));
-        return c->h_err[0] ? DD_ERR_ARG : DD_OK;
-    }
     return eval_tasks(c, ev, nD, dd::TASK_POINT, D, D, K, S, N_in, iwe);
 }
 
@@ -867,13 +902,6 @@ int dd_bound(dd_ctx* c, const dd_events* ev, const float* D_lo, const float* D_h
     if (rc) return rc;
     for (int32_t j = 0; j < n; j++)
         if (!d_ok(D_lo[j], ev->tau) || !d_ok(D_hi[j], ev->tau) || !(D_lo[j] <= D_hi[j])) return DD_ERR_ARG;
-    rc = ingest(c, ev, 1);
-    if (rc) return rc;
-    if (n == 0) {
-        DD_TRY(copy(c, c->h_err, c->err, sizeof(int32_t), cudaMemcpyDeviceToHost));
-        DD_TRY(sync(c));
-        return c->h_err[0] ? DD_ERR_ARG : DD_OK;
-    }
     return eval_tasks(c, ev, n, dd::TASK_BOUND, D_lo, D_hi, Kbar, Sbar, N_full, iwe);
 }
 
@@ -904,7 +932,9 @@ int dd_features(dd_ctx* c, const dd_events* windows, int32_t n_windows, float* f
         const int rc = check_events(&windows[w], c->g.planes);
         if (rc) return rc;
     }
-    int rc = ingest(c, windows, n_windows);
+    int rc = stage(c, windows, n_windows);
+    if (rc) return rc;
+    rc = ingest(c, n_windows);
     if (rc) return rc;
     rc = feature_counts(c, n_windows);
     if (rc) return rc;

@@ -287,10 +287,11 @@ struct EvalArgs {
     Merge mg;
 };
 
-// Kernel launches (dd_kernels.cu).  All asynchronous on `s`.
+// Kernel launches (dd_kernels.cu).  All asynchronous on `s`.  launch_ingest
+// leaves row_count zero; clear = false: it and err are zero already.
 cudaError_t launch_ingest(const Geom& g, const WinIn* wins_dev, int32_t n_windows, const int32_t* chunk_win_dev,
                           int32_t n_chunks, Ev* out, int32_t* row_count, int32_t* row_off,
-                          int32_t* cursor, int32_t* err, cudaStream_t s);
+                          int32_t* cursor, int32_t* err, cudaStream_t s, bool clear = true, int* launches = nullptr);
 cudaError_t launch_eval(const Geom& g, const EvalArgs& a, int threads, int grid_blocks, cudaStream_t s);
 int eval_resident_blocks(const Geom& g, int threads);
 // All rounds of one window's search in one cooperative launch of at most
@@ -302,7 +303,7 @@ cudaError_t launch_search(const Geom& g, const EvalArgs& a, const CtlArgs& c, in
                           cudaStream_t s);
 cudaError_t launch_keys(const Geom& g, const Task* tasks, int32_t n_tasks, Partial* part, i128* key,
                         unsigned long long* S, unsigned long long* cells, unsigned long long* full,
-                        cudaStream_t s);
+                        cudaStream_t s, const int32_t* err = nullptr, int32_t* err_out = nullptr);
 // Windows w0 .. w0 + n_windows - 1 start a search; split_ok < 0: split bound
 // tasks only when n_windows == 1.
 cudaError_t launch_init(const Geom& g, int32_t n_windows, SolveState* st, Task* tasks, int32_t task_stride,

@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(INGEST_THREADS) k_row_hist(Geom g, const WinIn
 }
 
 // Exclusive scan of one window's bin counts (at most 4096 bins), block = window.
-__global__ void __launch_bounds__(1024) k_row_scan(int bins, const int32_t* row_count, int32_t* row_off,
-                                                   int32_t* cursor) {
+// Leaves the counts zero for the next call.
+__global__ void __launch_bounds__(1024) k_row_scan(int bins, int32_t* row_count, int32_t* row_off, int32_t* cursor) {
     __shared__ int32_t wsum[32];
     const int w = blockIdx.x;
     row_count += (size_t)w * bins;
@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(1024) k_row_scan(int bins, const int32_t* row_
     for (int k = 0; k < per; k++) {
         int r = base + k;
         local[k] = r < bins ? row_count[r] : 0;
+        if (r < bins) row_count[r] = 0;
         tot += local[k];
     }
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -304,13 +305,16 @@ __global__ void __launch_bounds__(INGEST_THREADS) k_row_scatter(Geom g, const Wi
 
 cudaError_t launch_ingest(const Geom& g, const WinIn* wins_dev, int32_t n_windows, const int32_t* chunk_win_dev,
                           int32_t n_chunks, Ev* out, int32_t* row_count, int32_t* row_off,
-                          int32_t* cursor, int32_t* err, cudaStream_t s) {
+                          int32_t* cursor, int32_t* err, cudaStream_t s, bool clear, int* launches) {
     const int bins = bins_of(g);
     if (n_windows <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(row_count, 0, sizeof(int32_t) * bins * (size_t)n_windows, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(err, 0, sizeof(int32_t) * (size_t)n_windows, s);
-    if (e != cudaSuccess) return e;
+    if (clear) {
+        cudaError_t e = cudaMemsetAsync(row_count, 0, sizeof(int32_t) * bins * (size_t)n_windows, s);
+        if (e != cudaSuccess) return e;
+        e = cudaMemsetAsync(err, 0, sizeof(int32_t) * (size_t)n_windows, s);
+        if (e != cudaSuccess) return e;
+    }
+    if (launches) *launches = n_chunks > 0 ? 3 : 1;
     const unsigned blocks = (unsigned)n_chunks * INGEST_SUB;
     if (n_chunks > 0) k_row_hist<<<blocks, INGEST_THREADS, 0, s>>>(g, wins_dev, chunk_win_dev, row_count, err);
     k_row_scan<<<n_windows, 1024, 0, s>>>(bins, row_count, row_off, cursor);
@@ -1277,8 +1281,10 @@ cudaError_t launch_eval(const Geom& g, const EvalArgs& a, int threads, int grid_
 // ------------------------------------------------------------------- keys
 
 __global__ void k_keys(Geom g, const Task* tasks, int32_t n_tasks, Partial* part, i128* key,
-                       unsigned long long* S_out, unsigned long long* C_out, unsigned long long* F_out) {
+                       unsigned long long* S_out, unsigned long long* C_out, unsigned long long* F_out,
+                       const int32_t* err, int32_t* err_out) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0 && err_out) *err_out = *err;
     if (t >= n_tasks) return;
     const Partial p = part[t];
     part[t] = Partial{};                          // cleared for the next evaluation
@@ -1291,9 +1297,9 @@ __global__ void k_keys(Geom g, const Task* tasks, int32_t n_tasks, Partial* part
 
 cudaError_t launch_keys(const Geom& g, const Task* tasks, int32_t n_tasks, Partial* part, i128* key,
                         unsigned long long* S, unsigned long long* cells, unsigned long long* full,
-                        cudaStream_t s) {
+                        cudaStream_t s, const int32_t* err, int32_t* err_out) {
     if (n_tasks <= 0) return cudaSuccess;
-    k_keys<<<(n_tasks + 63) / 64, 64, 0, s>>>(g, tasks, n_tasks, part, key, S, cells, full);
+    k_keys<<<(n_tasks + 63) / 64, 64, 0, s>>>(g, tasks, n_tasks, part, key, S, cells, full, err, err_out);
     return cudaGetLastError();
 }
 
