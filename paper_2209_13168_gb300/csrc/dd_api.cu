@@ -394,6 +394,9 @@ int32_t stage_tasks(dd_ctx* c, int32_t n, int kind, const float* A, const float*
             jb.task = j;
             jb.split = s;
             jb.splits = tasks[j].splits;
+            jb.D_lo = jb.D_c = tasks[j].D_lo;
+            jb.D_hi = tasks[j].D_hi;
+            jb.kind = kind;
         }
     std::memset(c->h_sch, 0, sizeof(dd::Sched));
     c->h_sch->n_jobs[0] = nj;

@@ -48,8 +48,12 @@ struct Task {
 // evaluates the three tasks of one expanded interval together: the contrast
 // at its centre (task `task`) and the bounds of its two halves (tasks
 // `split` and `split` + 1).
-struct Job {
+// It carries its task's interval and kind, so that preparing a unit reads the
+// job and the window only.
+struct __align__(16) Job {
     int32_t win, task, split, splits;
+    float D_lo, D_hi, D_c;        // a fused job: the whole interval and its centre
+    int32_t kind;
 };
 
 // Sums of one task's IWE: per task, over all its row bands; counts per

@@ -513,13 +513,10 @@ __device__ __forceinline__ void prepare_unit(const Geom& g, const EvalArgs& a, c
     const Job jb = jobs[j];
     const WinIn* win = a.wins + jb.win;
     const int64_t ev_off = win->ev_off;
-    const float tau = win->tau;
-    const Task* wt = a.tasks + (size_t)jb.win * a.task_stride;
-    const Task tk = wt[jb.task];
+    const float tau = win->tau, Dl = jb.D_lo, Dh = jb.D_hi;
     const bool fused = jb.splits < 0;             // one expanded interval: its three tasks together
-    const float Dl = fused ? wt[jb.split].D_lo : tk.D_lo, Dh = fused ? wt[jb.split + 1].D_hi : tk.D_hi;
     const float cells = bound_cells(g, Dl, Dh, tau);
-    const int kind = fused ? UNIT_FUSED : (tk.kind == TASK_POINT ? UNIT_POINT
+    const int kind = fused ? UNIT_FUSED : (jb.kind == TASK_POINT ? UNIT_POINT
                                                                  : (cells >= DENSE_CELLS ? UNIT_DENSE : UNIT_BOUND));
     const int plane = ti >= g.plane_tiles ? 1 : 0, band = ti - plane * g.plane_tiles;
     int splits = fused ? 1 : max(1, jb.splits);
@@ -562,7 +559,7 @@ __device__ __forceinline__ void prepare_unit(const Geom& g, const EvalArgs& a, c
         un.rows = rows;
         un.D_lo = Dl;
         un.D_hi = Dh;
-        un.D_c = tk.D_lo;
+        un.D_c = jb.D_c;
         un.tau = tau;
         un.win = jb.win;
         un.task = jb.task;
@@ -1121,13 +1118,13 @@ __device__ __noinline__ void merge_split(const Geom& g, const EvalArgs& a, const
 // of its left and right halves.
 constexpr int UNIT_SUMS = 9;
 
-// One warp adds n of the warps' sums (rows 0.. of `red`) to the tasks' sums
-// k0.. (per plane).
+// Adds n of the warps' sums (rows 0.. of `red`) to the tasks' sums k0.. (per
+// plane), the warps taking one each: nine by one warp took 0.4 us.
 __device__ __forceinline__ void add_sums(const EvalArgs& a, const Unit& un, unsigned long long (*red)[MAX_WARPS],
                                          int n, int k0 = 0) {
     const int lane = threadIdx.x & 31, nw = work_warps();
     Partial* wp = a.part + (size_t)un.win * a.task_stride;
-    for (int k = k0; k < k0 + n; k++) {
+    for (int k = k0 + (int)(threadIdx.x >> 5); k < k0 + n; k += nw) {
         const unsigned long long t = warp_total(lane < nw ? red[k - k0][lane] : 0ull);
         if (lane == 0 && t) {
             Partial* q = wp + (k < 3 ? un.task : un.left + (k >= 6));
@@ -1228,7 +1225,7 @@ __device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, cons
         single_unit(g, a, un, T, k == 0 ? UNIT_POINT : kind, k == 1 ? un.D_lo : un.D_c, k == 1 ? un.D_c : un.D_hi,
                     scratch, nullptr, red, s_last);
         work_sync();
-        if (wid == 0) add_sums(a, un, red, 3, 3 * k);
+        add_sums(a, un, red, 3, 3 * k);
     }
     return 0;
 }
@@ -1307,7 +1304,7 @@ __device__ __forceinline__ void eval_round(const Geom& g, const EvalArgs& a, con
             clear_tile(tile, tile_words);
             sm.over = 0;
         }
-        if (wid == nw - 1 && sums) add_sums(a, un, sm.red, sums);
+        add_sums(a, un, sm.red, sums);
     }
 }
 
@@ -1399,6 +1396,7 @@ struct __align__(16) CtlShared {
     Node sorted_kids[2 * MAX_POP + 1];
     Node q_stage[Q_STAGE];
     Node q_head[MAX_POP];               // the merged queue's first entries, for the dequeue
+    float4 t_iv[3 * MAX_POP];           // per next-round task: its interval, and its centre (points)
     int16_t t_fuse[3 * MAX_POP];        // per next-round task: 0 own jobs, -1 part of a fused
                                         // job, k > 0 the centre of a fused job (left half k - 1)
     int8_t t_dense[3 * MAX_POP];        // per next-round task: a dense bound that may be split
@@ -1406,7 +1404,7 @@ struct __align__(16) CtlShared {
     int16_t t_at[3 * MAX_POP];          // and the place of its first one in the window's jobs
     uint4 pop_mask[2];                  // per 32 dequeued: to split, fused, dense left and right halves
     int pop_fail[2];                    // first that fails the gap test
-    int s_nk, s_stop, s_base;
+    int s_nk, s_stop, s_base, s_total;
     int q_shared;                       // resident: the queue is in the block's shared memory
 };
 
@@ -1514,6 +1512,10 @@ __global__ void k_init(Geom g, int32_t sharers, int32_t w0, SolveState* st_all, 
             j.task = t;
             j.split = s;
             j.splits = tasks[t].splits;
+            j.D_lo = tasks[t].D_lo;
+            j.D_hi = tasks[t].D_hi;
+            j.D_c = 0.0f;
+            j.kind = TASK_BOUND;
             jobs[o++] = j;
         }
     Job j;
@@ -1521,6 +1523,8 @@ __global__ void k_init(Geom g, int32_t sharers, int32_t w0, SolveState* st_all, 
     j.task = 0;
     j.split = 0;
     j.splits = 1;
+    j.D_lo = j.D_hi = j.D_c = tasks[0].D_lo;
+    j.kind = TASK_POINT;
     jobs[o] = j;
 }
 
@@ -1768,10 +1772,13 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
         // A child's rank among the children (they are distinct: popped
         // intervals are disjoint) counted by `per` threads, each over every
         // per-th child, summed within the thread group.
-        int per = 1;
-        while (nk > 8 && per < 32 && 2 * per * nk <= (int)blockDim.x) per *= 2;
+        int per = 1, lg = 0;
+        while (nk > 8 && per < 32 && 2 * per * nk <= (int)blockDim.x) {
+            per *= 2;
+            lg++;
+        }
         for (int base = 0; base < nk * per; base += blockDim.x) {
-            const int i = (base + tid) / per, p = (base + tid) % per;
+            const int i = (base + tid) >> lg, p = (base + tid) & (per - 1);
             int r = 0;
             if (i < nk)
                 for (int j = p; j < nk; j += per) r += better(sm.kids[j], sm.kids[i]);
@@ -1855,11 +1862,7 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
         p.t_point = tid;
         p.t_left = p.t_right = -1;
         p.pad = 0;
-        Task t;
-        t.D_lo = t.D_hi = p.c;
-        t.kind = TASK_POINT;
-        t.splits = 1;                             // the job builder decides (fill_splits)
-        tasks[tid] = t;
+        sm.t_iv[tid] = make_float4(p.lo, p.hi, p.c, 0.0f);
         sm.t_fuse[tid] = 0;
         sm.t_dense[tid] = 0;
         if (split) {
@@ -1870,13 +1873,8 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
             sm.t_fuse[l] = sm.t_fuse[l + 1] = fuse ? (int16_t)-1 : (int16_t)0;
             sm.t_dense[l] = dense_l;
             sm.t_dense[l + 1] = dense_r;
-            t.kind = TASK_BOUND;
-            t.D_lo = p.lo;
-            t.D_hi = p.c;
-            tasks[l] = t;
-            t.D_lo = p.c;
-            t.D_hi = p.hi;
-            tasks[l + 1] = t;
+            sm.t_iv[l] = make_float4(p.lo, p.c, 0.0f, 0.0f);
+            sm.t_iv[l + 1] = make_float4(p.c, p.hi, 0.0f, 0.0f);
         }
         s.pop[tid] = p;
     }
@@ -1937,8 +1935,9 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
             }
         }
         if (lane == 0) {
+            sm.s_total = total;
             if (c.n_windows == 1) {               // the only block: the list is its own
-                sch->n_jobs[par ^ 1] = total;
+                if (!RESIDENT) sch->n_jobs[par ^ 1] = total;
                 sm.s_base = 0;
             } else {
                 sm.s_base = atomicAdd(&sch->n_jobs[par ^ 1], total);
@@ -1949,12 +1948,18 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
     if (!done)                                    // the jobs, written by the whole block
         for (int q = tid; q < nt; q += blockDim.x) {
             const int n = sm.t_jobs[q], t = nt - 1 - q;
-            const int fz = n > 0 ? (int)sm.t_fuse[t] : 0;
+            if (n == 0) continue;
+            const int fz = (int)sm.t_fuse[t];
             Job* out = jobs + sm.s_base + sm.t_at[q];
+            Job j;
+            j.win = w;
+            j.task = t;
+            j.kind = t < np ? TASK_POINT : TASK_BOUND;
+            const float4 iv = sm.t_iv[t];         // a point's: its centre and, to be fused, its interval
+            j.D_lo = fz > 0 ? iv.x : (t < np ? iv.z : iv.x);
+            j.D_hi = fz > 0 ? iv.y : (t < np ? iv.z : iv.y);
+            j.D_c = iv.z;
             for (int k = 0; k < n; k++) {
-                Job j;
-                j.win = w;
-                j.task = t;
                 j.split = fz > 0 ? fz - 1 : k;
                 j.splits = fz > 0 ? -1 : n;
                 out[k] = j;
@@ -2006,7 +2011,11 @@ __device__ __forceinline__ int32_t load_acquire(const int32_t* p) {
     return v;
 }
 __device__ __forceinline__ void store_release(unsigned long long* p, unsigned long long v) {
+    // cumulative: the block's writes before its last barrier come with it
     asm volatile("st.release.gpu.global.u64 [%0], %1;" : : "l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ void add_release(int32_t* p, int32_t v) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" : : "l"(p), "r"(v) : "memory");
 }
 
 // Polls before a block gives up on the others: each takes about a
@@ -2027,7 +2036,7 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, Ctl
         if (threadIdx.x == 0) {
             const int32_t all = (int32_t)(round + 1) * others;
             int polls = 0;
-            while (load_acquire(&sch->ticket) != all && ++polls < SEARCH_POLLS) __nanosleep(20);
+            while (load_acquire(&sch->ticket) != all && ++polls < SEARCH_POLLS) {}
             sm.s_stop = polls >= SEARCH_POLLS;
         }
         __syncthreads();
@@ -2039,12 +2048,8 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, Ctl
         control_body<true>(g, c, 0, sm, (int)(round & 1), q_mem, q_cap);
         __syncthreads();                          // the round's tasks and jobs are written
         const bool done = sm.s.phase == PH_DONE;
-        if (threadIdx.x == 0) {
-            __threadfence();
-            store_release(&sch->go, (unsigned long long)(round + 1) << 32 |
-                                        (done ? 0u : (uint32_t)sch->n_jobs[(round & 1) ^ 1]));
-            if (done) sch->round = (int32_t)(round + 1);
-        }
+        if (threadIdx.x == 0)
+            store_release(&sch->go, (unsigned long long)(round + 1) << 32 | (done ? 0u : (uint32_t)sm.s_total));
         if (done) return;
     }
 }
@@ -2082,11 +2087,10 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
             eval_round(g, a, a.jobs + (size_t)par * a.job_stride, &sch->work[par], n_units, block, blocks, tile, sm);
         __syncthreads();                          // the block's sums are on their way; s_go has been read
         if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(&sch->ticket, 1);
+            add_release(&sch->ticket, 1);
             unsigned long long v = 0;
             int polls = 0;
-            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < SEARCH_POLLS) __nanosleep(20);
+            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < SEARCH_POLLS) {}
             if (polls >= SEARCH_POLLS) {          // never in a sound run: end the search
                 sch->failed = 1;
                 v = 0;

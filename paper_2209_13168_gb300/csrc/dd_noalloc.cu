@@ -179,6 +179,8 @@ extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_
                 h_jobs[j].task = j;
                 h_jobs[j].split = 0;
                 h_jobs[j].splits = 1;
+                h_jobs[j].D_lo = h_jobs[j].D_hi = h_jobs[j].D_c = D[j0 + j];
+                h_jobs[j].kind = dd::TASK_POINT;
             }
             std::memset(&h_sch, 0, sizeof(h_sch));
             h_sch.n_jobs[0] = m;
