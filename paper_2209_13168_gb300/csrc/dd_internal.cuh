@@ -126,12 +126,12 @@ struct __align__(16) WinParams {
     int32_t pad0, pad1;
 };
 
-// Device view of a warm-start model: bfloat16 weights transposed to
-// [in][out] (unit j of a layer reads column j), binary32 biases.
+// Device view of a warm-start model: bfloat16 weights [out][in] (a unit's
+// inputs are contiguous), binary32 biases.
 struct MlpDev {
-    const uint16_t* w1t;    // [128][128]
-    const uint16_t* w2t;    // [128][128]
-    const uint16_t* w3t;    // [128][2]
+    const uint16_t* w1;     // [128][128]
+    const uint16_t* w2;     // [128][128]
+    const uint16_t* w3;     // [2][128]
     const float* b1;
     const float* b2;
     const float* b3;

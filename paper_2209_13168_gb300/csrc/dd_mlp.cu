@@ -39,24 +39,67 @@ constexpr float LOG2E = 1.44269504f;
 
 __device__ __forceinline__ float bf(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 
-// Unit j of a dense layer with transposed bfloat16 weights wt[in][out].
-__device__ __forceinline__ float unit(const uint16_t* wt, int n_out, const float* b, const float* x, int j) {
-    float acc = b[j];
-    for (int k = 0; k < MLP_H; k++) acc = __fadd_rn(acc, __fmul_rn(bf(wt[k * n_out + j]), x[k]));
-    return acc;
+// The 128 bfloat16 weights of one unit, contiguous, in registers: sixteen
+// 16-byte loads in flight at once, so a layer waits for memory once (one
+// 2-byte load per input, 16 in flight, made a sample's pass 8 waits a layer).
+struct Row {
+    uint4 q[MLP_H / 8];
+};
+__device__ __forceinline__ Row load_row(const uint16_t* __restrict__ w) {
+    Row r;
+#pragma unroll
+    for (int k = 0; k < MLP_H / 8; k++) r.q[k] = __ldg(reinterpret_cast<const uint4*>(w) + k);
+    return r;
+}
+template <class F>
+__device__ __forceinline__ void each_weight(const Row& r, F&& f) {   // f(input, weight) for inputs 0..127 in turn
+#pragma unroll
+    for (int k = 0; k < MLP_H / 8; k++) {
+        const uint32_t w[4] = {r.q[k].x, r.q[k].y, r.q[k].z, r.q[k].w};
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            f(8 * k + 2 * i, __uint_as_float(w[i] << 16));
+            f(8 * k + 2 * i + 1, __uint_as_float(w[i] & 0xffff0000u));
+        }
+    }
 }
 
-// The forward pass of one sample by a block of 128 threads; x, h1, h2 and
-// out in shared memory.  Every thread returns after the last barrier.
-__device__ void forward(const MlpDev& m, const float* x, float* h1, float* h2, float* out) {
+// A dense layer's unit for S samples x[s][in] in shared memory: weight * input
+// for inputs 0..127 in turn onto the bias.
+template <int S>
+__device__ __forceinline__ void unit(const Row& w, float bias, const float (*x)[MLP_H], float (&acc)[S]) {
+#pragma unroll
+    for (int s = 0; s < S; s++) acc[s] = bias;
+    each_weight(w, [&](int k, float v) {
+#pragma unroll
+        for (int s = 0; s < S; s++) acc[s] = __fadd_rn(acc[s], __fmul_rn(v, x[s][k]));
+    });
+}
+
+// The forward pass of S samples by a block of 128 threads; x, h1, h2 and out
+// in shared memory.  Every thread returns after the last barrier.
+template <int S>
+__device__ __forceinline__ void forward(const MlpDev& m, const float (*x)[MLP_H], float (*h1)[MLP_H], float (*h2)[MLP_H],
+                                        float (*out)[MLP_OUT]) {
     const int j = threadIdx.x;
-    const float a1 = unit(m.w1t, MLP_H, m.b1, x, j);
-    h1[j] = a1 > 0.0f ? a1 : 0.0f;
+    float a[S];
+    const Row w1 = load_row(m.w1 + j * FEATURES);
+    const float b1 = m.b1[j], b2 = m.b2[j];
+    unit<S>(w1, b1, x, a);
+    const Row w2 = load_row(m.w2 + j * MLP_H);
+#pragma unroll
+    for (int s = 0; s < S; s++) h1[s][j] = a[s] > 0.0f ? a[s] : 0.0f;
     __syncthreads();
-    const float a2 = unit(m.w2t, MLP_H, m.b2, h1, j);
-    h2[j] = a2 > 0.0f ? a2 : 0.0f;
+    unit<S>(w2, b2, h1, a);
+#pragma unroll
+    for (int s = 0; s < S; s++) h2[s][j] = a[s] > 0.0f ? a[s] : 0.0f;
     __syncthreads();
-    if (j < MLP_OUT) out[j] = unit(m.w3t, MLP_OUT, m.b3, h2, j);
+    if (j < MLP_OUT * S) {
+        const int o = j % MLP_OUT;
+        float v[1];
+        unit<1>(load_row(m.w3 + o * MLP_H), m.b3[o], h2 + j / MLP_OUT, v);
+        out[j / MLP_OUT][o] = v[0];
+    }
     __syncthreads();
 }
 
@@ -102,21 +145,22 @@ __global__ void __launch_bounds__(FEAT_THREADS) k_features(Geom g, const WinIn* 
 // network, and the guess and half-width written into its search parameters.
 __global__ void __launch_bounds__(MLP_H) k_warm(int32_t n_windows, const int32_t* __restrict__ counts,
                                                 const WinIn* __restrict__ wins, WinParams* params, MlpDev m) {
-    __shared__ float x[FEATURES], h1[MLP_H], h2[MLP_H], out[MLP_OUT];
+    __shared__ __align__(16) float x[1][FEATURES], h1[1][MLP_H], h2[1][MLP_H];
+    __shared__ float out[1][MLP_OUT];
     const int w = blockIdx.x;
     if (w >= n_windows || params[w].warm != DD_WARM_MODEL) return;
     const int j = threadIdx.x;
     const int64_t n = wins[w].n;
-    x[j] = n > 0 ? __fdiv_rn((float)(counts[(size_t)w * FEATURES + j] * FEATURES), (float)n) : 0.0f;
+    x[0][j] = n > 0 ? __fdiv_rn((float)(counts[(size_t)w * FEATURES + j] * FEATURES), (float)n) : 0.0f;
     __syncthreads();
-    forward(m, x, h1, h2, out);
+    forward<1>(m, x, h1, h2, out);
     if (j == 0) {
         const float tau = wins[w].tau;
-        float v = __fadd_rn(__fmul_rn(out[1], LOG2E), 0.5f);
+        float v = __fadd_rn(__fmul_rn(out[0][1], LOG2E), 0.5f);
         if (!(v >= -20.0f)) v = -20.0f;
         if (v > 1.0f) v = 1.0f;
         const int e = (int)floorf(v);
-        params[w].D_warm = __fdiv_rn(out[0], tau);
+        params[w].D_warm = __fdiv_rn(out[0][0], tau);
         params[w].w_warm = __fdiv_rn(__uint_as_float((uint32_t)(e + 127) << 23), tau);
         params[w].warm = 1;
     }
@@ -133,90 +177,156 @@ __global__ void __launch_bounds__(FEATURES) k_feature_norm(const int32_t* __rest
 
 // -------------------------------------------------------------- training
 
-// Block b: forward pass of sample b, activations kept for the backward pass.
-__global__ void __launch_bounds__(MLP_H) k_fwd(MlpDev m, const float* __restrict__ X, float* h1g, float* h2g,
-                                               float* outg) {
-    __shared__ float x[FEATURES], h1[MLP_H], h2[MLP_H], out[MLP_OUT];
+// Block b: the outputs of sample b.
+__global__ void __launch_bounds__(MLP_H) k_fwd(MlpDev m, const float* __restrict__ X, float* outg) {
+    __shared__ __align__(16) float x[1][FEATURES], h1[1][MLP_H], h2[1][MLP_H];
+    __shared__ float out[1][MLP_OUT];
     const int b = blockIdx.x, j = threadIdx.x;
-    x[j] = X[(size_t)b * FEATURES + j];
+    x[0][j] = X[(size_t)b * FEATURES + j];
     __syncthreads();
-    forward(m, x, h1, h2, out);
-    h1g[(size_t)b * MLP_H + j] = h1[j];
-    h2g[(size_t)b * MLP_H + j] = h2[j];
-    if (j < MLP_OUT) outg[(size_t)b * MLP_OUT + j] = out[j];
+    forward<1>(m, x, h1, h2, out);
+    if (j < MLP_OUT) outg[(size_t)b * MLP_OUT + j] = out[0][j];
 }
 
-constexpr int LOSS_THREADS = 256;
+// What the weight gradients need of every sample, and its loss.
+struct Acts {
+    float *h1, *h2, *g1, *g2;    // [B][128]
+    float *gout;                 // [B][2]
+    float *loss;                 // [B]
+};
 
-// The loss (mean over B) and its gradient with respect to the outputs; one
-// block, summed in a fixed order.
-__global__ void __launch_bounds__(LOSS_THREADS) k_loss(int32_t B, const float* __restrict__ out,
-                                                       const float* __restrict__ u_star, float* gout, float* loss) {
-    __shared__ float part[LOSS_THREADS];
-    float acc = 0.0f;
-    const float inv = 1.0f / (float)B;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        const float u = out[2 * b], l = out[2 * b + 1];
-        const float e = u_star[b] - u;
+// Block b: forward and backward pass of samples S b .. S b + S - 1: the hidden
+// activations, the loss and its gradient with respect to the outputs and to
+// the hidden units (through the ReLUs, with the bfloat16 weights).
+// A sample's gradient depends on the others only through 1/B.  One sample a
+// block while that fits one wave of the device, else SAMPLES, which share the
+// weights' loads (1,684 samples: the four-launch form 208 us in all).
+constexpr int SAMPLES = 4;
+template <int S>
+__global__ void __launch_bounds__(MLP_H) k_sample(MlpDev m, const uint16_t* __restrict__ w2t, int32_t B,
+                                                  const float* __restrict__ X, const float* __restrict__ u_star,
+                                                  Acts a) {
+    __shared__ __align__(16) float x[S][FEATURES], h1[S][MLP_H], h2[S][MLP_H], g2[S][MLP_H];
+    __shared__ float out[S][MLP_OUT], go[S][MLP_OUT];
+    const int b0 = S * blockIdx.x, k = threadIdx.x;
+#pragma unroll
+    for (int s = 0; s < S; s++) x[s][k] = b0 + s < B ? X[(size_t)(b0 + s) * FEATURES + k] : 0.0f;
+    __syncthreads();
+    forward<S>(m, x, h1, h2, out);
+    if (k < S && b0 + k < B) {
+        const float inv = 1.0f / (float)B;
+        const float u = out[k][0], l = out[k][1];
+        const float e = u_star[b0 + k] - u;
         const float q = 9.0f * expf(-2.0f * l);
-        acc += 0.5f * q * e * e + l;
-        gout[2 * b] = -q * e * inv;
-        gout[2 * b + 1] = (1.0f - q * e * e) * inv;
+        a.loss[b0 + k] = 0.5f * q * e * e + l;
+        go[k][0] = -q * e * inv;
+        go[k][1] = (1.0f - q * e * e) * inv;
+        a.gout[2 * (size_t)(b0 + k)] = go[k][0];
+        a.gout[2 * (size_t)(b0 + k) + 1] = go[k][1];
     }
-    part[threadIdx.x] = acc;
     __syncthreads();
-    for (int o = LOSS_THREADS / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
+    const Row wk = load_row(w2t + k * MLP_H);    // of hidden unit k to each unit of the next layer
+    const float wa = bf(m.w3[k]), wb = bf(m.w3[MLP_H + k]);
+#pragma unroll
+    for (int s = 0; s < S; s++) {
+        if (b0 + s >= B) break;
+        const float v = h2[s][k] > 0.0f ? wa * go[s][0] + wb * go[s][1] : 0.0f;
+        g2[s][k] = v;
+        a.g2[(size_t)(b0 + s) * MLP_H + k] = v;
+        a.h1[(size_t)(b0 + s) * MLP_H + k] = h1[s][k];
+        a.h2[(size_t)(b0 + s) * MLP_H + k] = h2[s][k];
+    }
+    __syncthreads();
+    float acc[S][2] = {};                         // even and odd units
+    each_weight(wk, [&](int j, float v) {
+#pragma unroll
+        for (int s = 0; s < S; s++) acc[s][j & 1] = __fmaf_rn(v, g2[s][j], acc[s][j & 1]);
+    });
+#pragma unroll
+    for (int s = 0; s < S; s++)
+        if (b0 + s < B) a.g1[(size_t)(b0 + s) * MLP_H + k] = h1[s][k] > 0.0f ? acc[s][0] + acc[s][1] : 0.0f;
+}
+
+// Weight gradients of WG_CHUNK samples (blockIdx.y): blocks 0-15 and 16-31 a
+// 32 x 32 tile of the first two layers (both operands staged in shared
+// memory, four outputs a thread), block 32 the output layer, the biases and,
+// once, the mean loss.  Each chunk writes its own partial gradient; they are
+// added in order (k_wsum), so the result does not depend on the launch.  With
+// one thread per parameter over the whole batch in turn, the chain of B loads
+// and additions was most of a training step (256 samples: 45 us in all).
+constexpr int WG_CHUNK = 64, WG_TILE = 32, WG_THREADS = 256, WG_TILES = 2 * (MLP_H / WG_TILE) * (MLP_H / WG_TILE);
+__global__ void __launch_bounds__(WG_THREADS) k_wgrad(int32_t B, const float* __restrict__ X, Acts a, float* part,
+                                                      float* loss) {
+    __shared__ __align__(16) float G[WG_CHUNK][WG_TILE];
+    __shared__ float A[WG_CHUNK][WG_TILE];
+    const int t = threadIdx.x, b0 = blockIdx.y * WG_CHUNK, n = min(WG_CHUNK, B - b0);
+    float* out = part + (size_t)blockIdx.y * N_PARAMS;
+    if (blockIdx.x < WG_TILES) {
+        const int tile = blockIdx.x % (WG_TILES / 2), j0 = tile / 4 * WG_TILE, i0 = tile % 4 * WG_TILE;
+        const bool first = blockIdx.x < WG_TILES / 2;
+        const float* g = (first ? a.g1 : a.g2) + (size_t)b0 * MLP_H + j0;
+        const float* v = (first ? X : a.h1) + (size_t)b0 * MLP_H + i0;
+#pragma unroll
+        for (int q = 0; q < WG_CHUNK * WG_TILE / WG_THREADS; q++) {
+            const int r = t / WG_TILE + q * (WG_THREADS / WG_TILE), c = t % WG_TILE;
+            G[r][c] = r < n ? g[(size_t)r * MLP_H + c] : 0.0f;
+            A[r][c] = r < n ? v[(size_t)r * MLP_H + c] : 0.0f;
+        }
         __syncthreads();
+        const int i = t % WG_TILE, j = 4 * (t / WG_TILE);
+        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
+#pragma unroll 16
+        for (int r = 0; r < WG_CHUNK; r++) {
+            const float4 q = *reinterpret_cast<const float4*>(&G[r][j]);
+            const float x = A[r][i];
+            s0 = __fmaf_rn(q.x, x, s0);
+            s1 = __fmaf_rn(q.y, x, s1);
+            s2 = __fmaf_rn(q.z, x, s2);
+            s3 = __fmaf_rn(q.w, x, s3);
+        }
+        float* o = out + (first ? P_W1 : P_W2) + (size_t)(j0 + j) * MLP_H + i0 + i;
+        o[0] = s0;
+        o[MLP_H] = s1;
+        o[2 * MLP_H] = s2;
+        o[3 * MLP_H] = s3;
+        return;
     }
-    if (threadIdx.x == 0 && loss) *loss = part[0] * inv;
+    {                                             // W3 [2][128], then both hidden biases, then b3
+        const int o = t / MLP_H, i = t % MLP_H;
+        const float* gb = o ? a.g2 : a.g1;
+        float w = 0.0f, h = 0.0f, z = 0.0f;
+#pragma unroll 16
+        for (int r = 0; r < n; r++) {
+            const float g = a.gout[2 * (size_t)(b0 + r) + o];
+            w = __fmaf_rn(g, a.h2[(size_t)(b0 + r) * MLP_H + i], w);
+            h += gb[(size_t)(b0 + r) * MLP_H + i];
+            z += g;
+        }
+        out[P_W3 + t] = w;
+        out[(o ? P_B2 : P_B1) + i] = h;
+        if (i == 0) out[P_B3 + o] = z;
+    }
+    if (blockIdx.y == 0 && loss) {                // the mean loss, summed in a fixed order
+        float* sum = &A[0][0];
+        float acc = 0.0f;
+        for (int b = t; b < B; b += WG_THREADS) acc += a.loss[b];
+        sum[t] = acc;
+        __syncthreads();
+        for (int o = WG_THREADS / 2; o > 0; o >>= 1) {
+            if (t < o) sum[t] += sum[t + o];
+            __syncthreads();
+        }
+        if (t == 0) *loss = sum[0] * (1.0f / (float)B);
+    }
 }
 
-// Block b: gradients with respect to the hidden units of sample b (through
-// the ReLUs), with the [out][in] bfloat16 weights.
-__global__ void __launch_bounds__(MLP_H) k_back(const uint16_t* __restrict__ w2, const uint16_t* __restrict__ w3,
-                                                const float* __restrict__ h1g, const float* __restrict__ h2g,
-                                                const float* __restrict__ gout, float* g1g, float* g2g) {
-    __shared__ float g2[MLP_H];
-    const int b = blockIdx.x, k = threadIdx.x;
-    const float go0 = gout[2 * b], go1 = gout[2 * b + 1];
-    float a = bf(w3[k]) * go0 + bf(w3[MLP_H + k]) * go1;
-    const float v2 = h2g[(size_t)b * MLP_H + k] > 0.0f ? a : 0.0f;
-    g2[k] = v2;
-    g2g[(size_t)b * MLP_H + k] = v2;
-    __syncthreads();
-    a = 0.0f;
-    for (int j = 0; j < MLP_H; j++) a += bf(w2[j * MLP_H + k]) * g2[j];
-    g1g[(size_t)b * MLP_H + k] = h1g[(size_t)b * MLP_H + k] > 0.0f ? a : 0.0f;
-}
-
-// One thread per parameter: its gradient summed over the B samples in order.
-__global__ void __launch_bounds__(256) k_wgrad(int32_t B, const float* __restrict__ X, const float* __restrict__ h1,
-                                               const float* __restrict__ h2, const float* __restrict__ g1,
-                                               const float* __restrict__ g2, const float* __restrict__ gout,
-                                               float* grad) {
+// The chunks' partial gradients added in order.
+__global__ void __launch_bounds__(256) k_wsum(int32_t chunks, const float* __restrict__ part, float* grad) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= N_PARAMS) return;
-    const float *gv, *av;
-    int gs, as, gi, ai;
-    if (p < P_B1) {
-        gv = g1; gs = MLP_H; gi = p / FEATURES; av = X; as = FEATURES; ai = p % FEATURES;
-    } else if (p < P_W2) {
-        gv = g1; gs = MLP_H; gi = p - P_B1; av = nullptr; as = 0; ai = 0;
-    } else if (p < P_B2) {
-        gv = g2; gs = MLP_H; gi = (p - P_W2) / MLP_H; av = h1; as = MLP_H; ai = (p - P_W2) % MLP_H;
-    } else if (p < P_W3) {
-        gv = g2; gs = MLP_H; gi = p - P_B2; av = nullptr; as = 0; ai = 0;
-    } else if (p < P_B3) {
-        gv = gout; gs = MLP_OUT; gi = (p - P_W3) / MLP_H; av = h2; as = MLP_H; ai = (p - P_W3) % MLP_H;
-    } else {
-        gv = gout; gs = MLP_OUT; gi = p - P_B3; av = nullptr; as = 0; ai = 0;
-    }
     float acc = 0.0f;
-    if (av)
-        for (int b = 0; b < B; b++) acc += gv[(size_t)b * gs + gi] * av[(size_t)b * as + ai];
-    else
-        for (int b = 0; b < B; b++) acc += gv[(size_t)b * gs + gi];
+#pragma unroll 8
+    for (int c = 0; c < chunks; c++) acc += part[(size_t)c * N_PARAMS + p];
     grad[p] = acc;
 }
 
@@ -229,14 +339,14 @@ __device__ __forceinline__ bool is_weight(int p, int* layer, int* o, int* i) {
 
 struct Weights {
     uint16_t *w1, *w2, *w3;      // [out][in]
-    uint16_t *w1t, *w2t, *w3t;   // [in][out]
+    uint16_t* w2t;               // [in][out], for the backward pass
 };
 
 __device__ __forceinline__ void store_weight(const Weights& wb, int layer, int o, int i, float v) {
     const uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(v));
-    if (layer == 0) { wb.w1[o * FEATURES + i] = h; wb.w1t[i * MLP_H + o] = h; }
+    if (layer == 0) wb.w1[o * FEATURES + i] = h;
     else if (layer == 1) { wb.w2[o * MLP_H + i] = h; wb.w2t[i * MLP_H + o] = h; }
-    else { wb.w3[o * MLP_H + i] = h; wb.w3t[i * MLP_OUT + o] = h; }
+    else wb.w3[o * MLP_H + i] = h;
 }
 
 // One thread per parameter: an Adam step on the binary32 master value
@@ -309,13 +419,15 @@ struct dd_mlp {
     int64_t step = 0;
     // training activations for up to cap samples
     int32_t cap = 0;
-    float *h1 = nullptr, *h2 = nullptr, *out = nullptr, *gout = nullptr, *g1 = nullptr, *g2 = nullptr;
+    dd::Acts act{};
+    float* part = nullptr;          // partial gradients per chunk of samples
 };
 
 namespace {
 
 constexpr int NP = DD_MLP_PARAMS;
 constexpr int B_MAX = 4096;
+constexpr int ONE_SAMPLE_MAX = 608;   // samples up to which each has a block of its own (four per SM)
 
 template <class T>
 void release(T*& p) {
@@ -323,13 +435,16 @@ void release(T*& p) {
     p = nullptr;
 }
 
+int chunks_of(int32_t B) { return (B + dd::WG_CHUNK - 1) / dd::WG_CHUNK; }
+
 void free_acts(dd_mlp* m) {
-    release(m->h1);
-    release(m->h2);
-    release(m->out);
-    release(m->gout);
-    release(m->g1);
-    release(m->g2);
+    release(m->act.h1);
+    release(m->act.h2);
+    release(m->act.g1);
+    release(m->act.g2);
+    release(m->act.gout);
+    release(m->act.loss);
+    release(m->part);
     m->cap = 0;
 }
 
@@ -337,12 +452,13 @@ int ensure_acts(dd_mlp* m, int32_t B) {
     if (B <= m->cap) return DD_OK;
     free_acts(m);
     const size_t n = (size_t)B;
-    if (cudaMalloc((void**)&m->h1, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
-        cudaMalloc((void**)&m->h2, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
-        cudaMalloc((void**)&m->g1, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
-        cudaMalloc((void**)&m->g2, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
-        cudaMalloc((void**)&m->out, sizeof(float) * n * dd::MLP_OUT) != cudaSuccess ||
-        cudaMalloc((void**)&m->gout, sizeof(float) * n * dd::MLP_OUT) != cudaSuccess) {
+    if (cudaMalloc((void**)&m->act.h1, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
+        cudaMalloc((void**)&m->act.h2, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
+        cudaMalloc((void**)&m->act.g1, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
+        cudaMalloc((void**)&m->act.g2, sizeof(float) * n * dd::MLP_H) != cudaSuccess ||
+        cudaMalloc((void**)&m->act.gout, sizeof(float) * n * dd::MLP_OUT) != cudaSuccess ||
+        cudaMalloc((void**)&m->act.loss, sizeof(float) * n) != cudaSuccess ||
+        cudaMalloc((void**)&m->part, sizeof(float) * (size_t)chunks_of(B) * NP) != cudaSuccess) {
         free_acts(m);
         return DD_ERR_OOM;
     }
@@ -352,9 +468,9 @@ int ensure_acts(dd_mlp* m, int32_t B) {
 
 dd::MlpDev view(const dd_mlp* m) {
     dd::MlpDev v;
-    v.w1t = m->wb.w1t;
-    v.w2t = m->wb.w2t;
-    v.w3t = m->wb.w3t;
+    v.w1 = m->wb.w1;
+    v.w2 = m->wb.w2;
+    v.w3 = m->wb.w3;
     v.b1 = m->master + dd::P_B1;
     v.b2 = m->master + dd::P_B2;
     v.b3 = m->master + dd::P_B3;
@@ -376,9 +492,7 @@ void destroy(dd_mlp* m) {
     release(m->wb.w1);
     release(m->wb.w2);
     release(m->wb.w3);
-    release(m->wb.w1t);
     release(m->wb.w2t);
-    release(m->wb.w3t);
     free_acts(m);
     delete m;
 }
@@ -406,10 +520,15 @@ int grad_impl(dd_mlp* m, const float* X, const float* u_star, int32_t B, float* 
     int rc = ensure_acts(m, B);
     if (rc) return rc;
     const dd::MlpDev v = view(m);
-    dd::k_fwd<<<B, dd::MLP_H, 0, m->stream>>>(v, X, m->h1, m->h2, m->out);
-    dd::k_loss<<<1, dd::LOSS_THREADS, 0, m->stream>>>(B, m->out, u_star, m->gout, loss);
-    dd::k_back<<<B, dd::MLP_H, 0, m->stream>>>(m->wb.w2, m->wb.w3, m->h1, m->h2, m->gout, m->g1, m->g2);
-    dd::k_wgrad<<<(NP + 255) / 256, 256, 0, m->stream>>>(B, X, m->h1, m->h2, m->g1, m->g2, m->gout, grad);
+    if (B <= ONE_SAMPLE_MAX)
+        dd::k_sample<1><<<B, dd::MLP_H, 0, m->stream>>>(v, m->wb.w2t, B, X, u_star, m->act);
+    else
+        dd::k_sample<dd::SAMPLES><<<(B + dd::SAMPLES - 1) / dd::SAMPLES, dd::MLP_H, 0, m->stream>>>(
+            v, m->wb.w2t, B, X, u_star, m->act);
+    const int chunks = chunks_of(B);
+    float* part = chunks == 1 ? grad : m->part;
+    dd::k_wgrad<<<dim3(dd::WG_TILES + 1, chunks), dd::WG_THREADS, 0, m->stream>>>(B, X, m->act, part, loss);
+    if (chunks > 1) dd::k_wsum<<<(NP + 255) / 256, 256, 0, m->stream>>>(chunks, m->part, grad);
     return cudaGetLastError() == cudaSuccess ? DD_OK : DD_ERR_CUDA;
 }
 
@@ -443,11 +562,9 @@ int dd_mlp_create(uint64_t seed, dd_mlp** out) {
               cudaMalloc((void**)&m->exp, sizeof(float) * NP) == cudaSuccess &&
               cudaMalloc((void**)&m->loss, sizeof(float)) == cudaSuccess &&
               cudaMalloc((void**)&m->wb.w1, 2 * dd::MLP_H * dd::FEATURES) == cudaSuccess &&
-              cudaMalloc((void**)&m->wb.w1t, 2 * dd::MLP_H * dd::FEATURES) == cudaSuccess &&
               cudaMalloc((void**)&m->wb.w2, 2 * dd::MLP_H * dd::MLP_H) == cudaSuccess &&
               cudaMalloc((void**)&m->wb.w2t, 2 * dd::MLP_H * dd::MLP_H) == cudaSuccess &&
-              cudaMalloc((void**)&m->wb.w3, 2 * dd::MLP_OUT * dd::MLP_H) == cudaSuccess &&
-              cudaMalloc((void**)&m->wb.w3t, 2 * dd::MLP_OUT * dd::MLP_H) == cudaSuccess;
+              cudaMalloc((void**)&m->wb.w3, 2 * dd::MLP_OUT * dd::MLP_H) == cudaSuccess;
     if (!ok) {
         destroy(m);
         return DD_ERR_OOM;
@@ -545,9 +662,7 @@ int dd_mlp_load(dd_mlp* m, const char* path) {
 int dd_mlp_forward(dd_mlp* m, const float* X, int32_t B, float* out) {
     if (!m || B < 0 || (B > 0 && (!X || !out))) return DD_ERR_ARG;
     if (B == 0) return DD_OK;
-    int rc = ensure_acts(m, B);
-    if (rc) return rc;
-    dd::k_fwd<<<B, dd::MLP_H, 0, m->stream>>>(view(m), X, m->h1, m->h2, out);
+    dd::k_fwd<<<B, dd::MLP_H, 0, m->stream>>>(view(m), X, out);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(m->stream) != cudaSuccess) return DD_ERR_CUDA;
     return DD_OK;
 }
