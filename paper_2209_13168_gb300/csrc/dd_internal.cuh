@@ -240,6 +240,16 @@ inline int32_t jobs_per_window(const Geom& g, int32_t max_tasks) {
 // column in consecutive rows fall in different shared-memory banks.
 __host__ __device__ inline int32_t tile_pitch(const Geom& g) { return g.W | 1; }
 
+// Rows of W pixels whose tile lets `blocks` evaluation blocks of `threads`
+// working threads share an SM's 228 KB of shared memory (the kernel's own
+// shared variables and 1 KB a block that the hardware keeps: 4 KB).
+constexpr int EVAL_WARP_WORDS = 320;   // scratch words per working warp
+inline int32_t band_rows_for(int32_t W, int32_t threads, int32_t blocks) {
+    const int32_t bytes = 228 * 1024 / blocks - 4096 - 4 * EVAL_WARP_WORDS * (threads / 32);
+    const int32_t rows = bytes / (4 * (W | 1));
+    return rows < 1 ? 1 : rows;
+}
+
 // Time buckets for a sort over H rows (rows of every plane): as many as fit
 // 4096 bins, at most 8.
 inline int32_t time_buckets(int32_t H) {

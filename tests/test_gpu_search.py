@@ -62,3 +62,18 @@ def test_window_beyond_the_launch_limit():
         ctx.close()
     for k in KEYS:
         assert got[0][k] == got[1][k], k
+
+
+# one interval a round, so that bands (the default height, one row, a height
+# that the slices do not divide, the whole frame) are cut into slices of rows;
+# above 131,072 events a unit holds a share of the events and is not cut
+@pytest.mark.parametrize("n", [900, 20000, 140000])
+@pytest.mark.parametrize("band_rows", [0, 1, 13, 97])
+def test_bands_cut_into_slices(n, band_rows):
+    w = make_window(131, 97, 64.0, 50.5, n - n // 3, n // 36, n // 3, 0.35, 0.3, seed=76)
+    ctx = dd.Context(131, 97, 64.0, 50.5, pop_k=1, band_rows=band_rows)
+    got = ctx.solve(dd.Events.of(w, device="cuda"), -1.0, 1.0, 1e-3, 0.0)
+    ctx.close()
+    want = O.solve(O.Window.of(w), -1.0, 1.0, 1e-3, 0.0, 1)
+    for k in KEYS:
+        assert got[k] == want[k], (k, got[k], want[k])
