@@ -648,8 +648,8 @@ __device__ __forceinline__ uint32_t field_inc() {
 // The previous count in an atomic's answer (0 if it was not issued): into V,
 // and into top, their maximum (a field that held FIELD_MAX has run over into
 // the next one).
-template <int F>
-__device__ __forceinline__ void take(uint32_t old, unsigned long long& V, uint32_t& top) {
+template <int F, class Sum>
+__device__ __forceinline__ void take(uint32_t old, Sum& V, uint32_t& top) {
     if (F == WHOLE) {
         V += old;
     } else if (F != DENSE) {
@@ -664,8 +664,8 @@ __device__ __forceinline__ void take(uint32_t old, unsigned long long& V, uint32
 // compiled to a branch around it (measured: about five control instructions
 // per atomic, a third of a wide bound's instructions); an address that is
 // always valid takes none.
-template <int F>
-__device__ __forceinline__ void bump(const Tile& T, uint32_t at, bool here, unsigned long long& V, uint32_t& top) {
+template <int F, class Sum>
+__device__ __forceinline__ void bump(const Tile& T, uint32_t at, bool here, Sum& V, uint32_t& top) {
     const uint32_t to = here ? at : T.idle;
     if (F == DENSE) {
         asm volatile("red.shared.add.u32 [%0], 1;" : : "r"(to) : "memory");
@@ -678,8 +678,8 @@ __device__ __forceinline__ void bump(const Tile& T, uint32_t at, bool here, unsi
 
 // Adds one to the field of biased pixel c if it is in the tile (and `also`
 // holds); n counts the increments.
-template <int F>
-__device__ __forceinline__ void bump_pixel(const Tile& T, uint2 c, unsigned long long& V, uint32_t& n, uint32_t& top,
+template <int F, class Sum>
+__device__ __forceinline__ void bump_pixel(const Tile& T, uint2 c, Sum& V, uint32_t& n, uint32_t& top,
                                            bool also = true) {
     const uint32_t r = c.y - T.row0, x = c.x - CELL0, at = T.base + c.y * T.pitch + 4u * c.x;
     bool here = (r < T.rows) & (x < T.W) & also;
@@ -761,9 +761,9 @@ __device__ __forceinline__ int walk_range(const Geom& g, const Tile& T, float4 v
 // the tile's rows and the frame's columns.  dn, rm: the minor offset and the
 // major one's reciprocal.  A run has at most three cells: its s-range spans
 // 1.008 major cells and the slope is at most 1.
-template <int F>
+template <int F, class Sum>
 __device__ __forceinline__ void walk_cells(const Geom& g, const Tile& T, bool mx, uint32_t k, int n, float dn, float rm,
-                                           float sa, float sb, unsigned long long& V, uint32_t& C, uint32_t& top) {
+                                           float sa, float sb, Sum& V, uint32_t& C, uint32_t& top) {
     const float fm = mx ? g.fx : g.fy, fn = mx ? g.fy : g.fx;
     const float h = copysignf(HALF_PLUS, rm);     // so that lo is the smaller end
     const uint32_t jmin = mx ? T.row0 : CELL0, jmax = mx ? T.row0 + T.rows - 1 : CELL0 + T.W - 1;
@@ -793,9 +793,9 @@ __device__ __forceinline__ void walk_cells(const Geom& g, const Tile& T, bool mx
 }
 
 // A short segment walked by its own lane.
-template <int F>
-__device__ __forceinline__ void walk_lane(const Geom& g, const Tile& T, float4 v, const Span& s,
-                                          unsigned long long& V, uint32_t& C, uint32_t& top) {
+template <int F, class Sum>
+__device__ __forceinline__ void walk_lane(const Geom& g, const Tile& T, float4 v, const Span& s, Sum& V,
+                                          uint32_t& C, uint32_t& top) {
     const bool mx = fabsf(v.x) >= fabsf(v.y);
     uint32_t k;
     const int n = walk_range(g, T, v, s, mx, k);
@@ -1037,14 +1037,22 @@ __device__ __forceinline__ void bound_pass(const Geom& g, const Unit& un, const 
 // between them) and one barrier instead of five.  The sums of squares, 2 sum(v) + increments,
 // are those of three separate passes.  Returns false if the list or a field
 // overflowed: then the tile holds nothing of use.
+//
+// With few candidates a unit's fixed instructions count (16 windows of
+// 1280x720, 70 chunks a unit: 13,155 warp instructions), so a warp's sums stay
+// within 32 bits and take one warp reduction each: previous counts are at most
+// 1022, a warp has at most FUSED_CHUNKS chunks (2^16 x 32 x 1022 < 2^31) or
+// WARP_WORDS listed events of at most 3 x 4096 cells (320 x 12,288 x 1022 <
+// 2^32).
+constexpr int FUSED_CHUNKS = 1 << 16;             // per warp
 struct FusedSums {
-    unsigned long long V[4];                      // previous counts: stable, centre, left, right
+    uint32_t V[4];                                // previous counts: stable, centre, left, right
     uint32_t n, C[3], F[2];                       // stable increments; each task's own; the halves' N_full
 };
 
 template <int F>
 __device__ __forceinline__ void fused_half(const Geom& g, const Tile& T, float4 v, f32x2 foe, float s1, float s2,
-                                           unsigned long long& V, uint32_t& C, uint32_t& full, uint32_t& top) {
+                                           uint32_t& V, uint32_t& C, uint32_t& full, uint32_t& top) {
     const Span s = span_of(foe, pair(v.x, v.y), s1, s2, pair(WIDEN_DN, WIDEN_UP));
     full += counts_full(g, T, s);
     const bool single = s.a.x == s.b.x && s.a.y == s.b.y, two = adjacent(s);
@@ -1081,7 +1089,7 @@ __device__ __forceinline__ bool fused_pass(const Geom& g, const Unit& un, const 
             listed += __popc(m);
         }
     }
-    if (top >= FIELD_MAX || listed > WARP_WORDS) *s_over = 1;
+    if (top >= FIELD_MAX || listed > WARP_WORDS || chunks > FUSED_CHUNKS * nw) *s_over = 1;
     work_sync();
     if (*s_over) return false;
     const float c = un.D_c, gc = warp_g(c, tref);
@@ -1281,24 +1289,17 @@ __device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, cons
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     FusedSums q = {};
     if (fused_pass(g, un, T, scratch, s_over, q)) {
-        const unsigned long long S0 = 2 * q.V[0] + q.n;
-        auto put = [&](int k, unsigned long long x) {
-            x = warp_total(x);
-            if (lane == 0) red[k][wid] = x;
-        };
-        auto put32 = [&](int k, uint32_t x) {
-            x = __reduce_add_sync(0xffffffffu, x);
-            if (lane == 0) red[k][wid] = x;
-        };
-        put(0, S0 + 2 * q.V[1] + q.C[0]);
-        put32(1, q.n + q.C[0]);
-        if (lane == 0) red[2][wid] = 0;
-        put(3, S0 + 2 * q.V[2] + q.C[1]);
-        put32(4, q.n + q.C[1]);
-        put32(5, q.n + q.F[0]);
-        put(6, S0 + 2 * q.V[3] + q.C[2]);
-        put32(7, q.n + q.C[2]);
-        put32(8, q.n + q.F[1]);
+        auto total = [](uint32_t x) { return __reduce_add_sync(0xffffffffu, x); };
+        const uint32_t n = total(q.n), v0 = total(q.V[0]);
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const uint32_t v = total(q.V[k + 1]), c = total(q.C[k]), f = k ? n + total(q.F[k - 1]) : 0u;
+            if (lane == 0) {
+                red[3 * k][wid] = 2 * ((unsigned long long)v0 + v) + n + c;
+                red[3 * k + 1][wid] = n + c;
+                red[3 * k + 2][wid] = f;
+            }
+        }
         return 9;
     }
     const int kind = bound_cells(g, un.D_lo, un.D_hi, un.tau) >= DENSE_CELLS ? UNIT_DENSE : UNIT_BOUND;

@@ -97,3 +97,20 @@ def test_fused_units_with_a_full_list():
             assert got[k] == want[k], (k, got[k], want[k])
         assert got["trace"] == want["trace"]
         ctx.close()
+
+
+@pytest.mark.parametrize("n", [(1 << 21) - 512, (1 << 21) + 512])
+def test_fused_units_at_the_most_chunks(n):
+    # one warp per block and one band: 65,536 chunks are the most whose sums
+    # one warp keeps in 32 bits; a unit with more runs its tasks one by one
+    w = make_window(256, 90, 128.0, 45.0, 900, 40, 300, 0.3, 0.4, seed=77)
+    rng = np.random.default_rng(77)
+    w.x, w.y = rng.integers(0, 256, n).astype(np.int16), rng.integers(0, 90, n).astype(np.int16)
+    w.t = np.sort(rng.random(n) * 0.3).astype(np.float32)
+    w.p = np.ones(n, np.int8)
+    want = O.solve(O.Window.of(w), -1e-3, 1e-3, 5e-4, 0.0, 4)
+    ctx = dd.Context(256, 90, 128.0, 45.0, pop_k=4, threads=32, fuse_span=100, band_rows=90)
+    got = ctx.solve(dd.Events.of(w, device="cuda"), -1e-3, 1e-3, 5e-4, 0.0)
+    ctx.close()
+    for k in KEYS:
+        assert got[k] == want[k], (k, got[k], want[k])
