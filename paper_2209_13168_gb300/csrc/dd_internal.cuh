@@ -126,11 +126,12 @@ struct __align__(16) WinParams {
     int32_t pad0, pad1;
 };
 
-// Device view of a warm-start model: bfloat16 weights [out][in] (a unit's
-// inputs are contiguous), binary32 biases.
+// Device view of a warm-start model: bfloat16 weights, binary32 biases.  The
+// hidden layers' matrices in groups of eight inputs, so that neighbouring
+// units' weights lie side by side.
 struct MlpDev {
-    const uint16_t* w1;     // [128][128]
-    const uint16_t* w2;     // [128][128]
+    const uint16_t* w1;     // [128 / 8 inputs][128 units][8 inputs]
+    const uint16_t* w2;     // the same
     const uint16_t* w3;     // [2][128]
     const float* b1;
     const float* b2;

@@ -39,16 +39,27 @@ constexpr float LOG2E = 1.44269504f;
 
 __device__ __forceinline__ float bf(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 
-// The 128 bfloat16 weights of one unit, contiguous, in registers: sixteen
-// 16-byte loads in flight at once, so a layer waits for memory once (one
-// 2-byte load per input, 16 in flight, made a sample's pass 8 waits a layer).
+// The 128 bfloat16 weights of one unit in registers: sixteen 16-byte loads in
+// flight at once, so a layer waits for memory once.  The hidden layers'
+// matrices are stored in groups of eight inputs, [in / 8][unit][8], so that a
+// warp's load is 512 consecutive bytes (with contiguous rows each load touched
+// 32 lines: a gradient of 256 samples 28.6 us, now 21.6; of 2,048 43.1 and
+// 34.9).  The output layer's two rows of 128 are each contiguous (UNITS = 1).
+constexpr int IN_GROUP = 8;
+__host__ __device__ __forceinline__ int grouped(int unit, int in) {
+    return (in / IN_GROUP * MLP_H + unit) * IN_GROUP + in % IN_GROUP;
+}
 struct Row {
-    uint4 q[MLP_H / 8];
+    uint4 q[MLP_H / IN_GROUP];
 };
-__device__ __forceinline__ Row load_row(const uint16_t* __restrict__ w) {
+template <int UNITS = MLP_H>
+__device__ __forceinline__ Row load_row(const uint16_t* __restrict__ w, int unit) {
     Row r;
 #pragma unroll
-    for (int k = 0; k < MLP_H / 8; k++) r.q[k] = __ldg(reinterpret_cast<const uint4*>(w) + k);
+    for (int k = 0; k < MLP_H / IN_GROUP; k++) {
+        const uint4* q = reinterpret_cast<const uint4*>(w) + (UNITS > 1 ? k * UNITS + unit : unit * (MLP_H / IN_GROUP) + k);
+        r.q[k] = __ldg(q);
+    }
     return r;
 }
 template <class F>
@@ -77,27 +88,31 @@ __device__ __forceinline__ void unit(const Row& w, float bias, const float (*x)[
 }
 
 // The forward pass of S samples by a block of 128 threads; x, h1, h2 and out
-// in shared memory.  Every thread returns after the last barrier.
-template <int S>
+// in shared memory.  Both hidden layers' weights are loaded before the first
+// layer, the output layer's (and, `ahead` of it, what the caller needs next)
+// before the second, so that the block waits for memory once.  Every thread
+// returns after the last barrier.
+template <int S, class Ahead>
 __device__ __forceinline__ void forward(const MlpDev& m, const float (*x)[MLP_H], float (*h1)[MLP_H], float (*h2)[MLP_H],
-                                        float (*out)[MLP_OUT]) {
+                                        float (*out)[MLP_OUT], Ahead&& ahead) {
     const int j = threadIdx.x;
     float a[S];
-    const Row w1 = load_row(m.w1 + j * FEATURES);
+    const Row w1 = load_row(m.w1, j), w2 = load_row(m.w2, j);
     const float b1 = m.b1[j], b2 = m.b2[j];
     unit<S>(w1, b1, x, a);
-    const Row w2 = load_row(m.w2 + j * MLP_H);
 #pragma unroll
     for (int s = 0; s < S; s++) h1[s][j] = a[s] > 0.0f ? a[s] : 0.0f;
+    const Row w3 = load_row<1>(m.w3, j % MLP_OUT);
     __syncthreads();
     unit<S>(w2, b2, h1, a);
+    ahead();
 #pragma unroll
     for (int s = 0; s < S; s++) h2[s][j] = a[s] > 0.0f ? a[s] : 0.0f;
     __syncthreads();
     if (j < MLP_OUT * S) {
         const int o = j % MLP_OUT;
         float v[1];
-        unit<1>(load_row(m.w3 + o * MLP_H), m.b3[o], h2 + j / MLP_OUT, v);
+        unit<1>(w3, m.b3[o], h2 + j / MLP_OUT, v);
         out[j / MLP_OUT][o] = v[0];
     }
     __syncthreads();
@@ -153,7 +168,7 @@ __global__ void __launch_bounds__(MLP_H) k_warm(int32_t n_windows, const int32_t
     const int64_t n = wins[w].n;
     x[0][j] = n > 0 ? __fdiv_rn((float)(counts[(size_t)w * FEATURES + j] * FEATURES), (float)n) : 0.0f;
     __syncthreads();
-    forward<1>(m, x, h1, h2, out);
+    forward<1>(m, x, h1, h2, out, [] {});
     if (j == 0) {
         const float tau = wins[w].tau;
         float v = __fadd_rn(__fmul_rn(out[0][1], LOG2E), 0.5f);
@@ -184,7 +199,7 @@ __global__ void __launch_bounds__(MLP_H) k_fwd(MlpDev m, const float* __restrict
     const int b = blockIdx.x, j = threadIdx.x;
     x[0][j] = X[(size_t)b * FEATURES + j];
     __syncthreads();
-    forward<1>(m, x, h1, h2, out);
+    forward<1>(m, x, h1, h2, out, [] {});
     if (j < MLP_OUT) outg[(size_t)b * MLP_OUT + j] = out[0][j];
 }
 
@@ -212,7 +227,8 @@ __global__ void __launch_bounds__(MLP_H) k_sample(MlpDev m, const uint16_t* __re
 #pragma unroll
     for (int s = 0; s < S; s++) x[s][k] = b0 + s < B ? X[(size_t)(b0 + s) * FEATURES + k] : 0.0f;
     __syncthreads();
-    forward<S>(m, x, h1, h2, out);
+    Row wk;                                       // of hidden unit k to each unit of the next layer
+    forward<S>(m, x, h1, h2, out, [&] { wk = load_row(w2t, k); });
     if (k < S && b0 + k < B) {
         const float inv = 1.0f / (float)B;
         const float u = out[k][0], l = out[k][1];
@@ -225,7 +241,6 @@ __global__ void __launch_bounds__(MLP_H) k_sample(MlpDev m, const uint16_t* __re
         a.gout[2 * (size_t)(b0 + k) + 1] = go[k][1];
     }
     __syncthreads();
-    const Row wk = load_row(w2t + k * MLP_H);    // of hidden unit k to each unit of the next layer
     const float wa = bf(m.w3[k]), wb = bf(m.w3[MLP_H + k]);
 #pragma unroll
     for (int s = 0; s < S; s++) {
@@ -249,8 +264,8 @@ __global__ void __launch_bounds__(MLP_H) k_sample(MlpDev m, const uint16_t* __re
 
 // Weight gradients of WG_CHUNK samples (blockIdx.y): blocks 0-15 and 16-31 a
 // 32 x 32 tile of the first two layers (both operands staged in shared
-// memory, four outputs a thread), block 32 the output layer, the biases and,
-// once, the mean loss.  Each chunk writes its own partial gradient; they are
+// memory, four outputs a thread), block 32 the output layer and the biases,
+// block 33, once, the mean loss.  Each chunk writes its own partial gradient; they are
 // added in order (k_wsum), so the result does not depend on the launch.  With
 // one thread per parameter over the whole batch in turn, the chain of B loads
 // and additions was most of a training step (256 samples: 45 us in all).
@@ -291,22 +306,8 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad(int32_t B, const float* __
         o[3 * MLP_H] = s3;
         return;
     }
-    {                                             // W3 [2][128], then both hidden biases, then b3
-        const int o = t / MLP_H, i = t % MLP_H;
-        const float* gb = o ? a.g2 : a.g1;
-        float w = 0.0f, h = 0.0f, z = 0.0f;
-#pragma unroll 16
-        for (int r = 0; r < n; r++) {
-            const float g = a.gout[2 * (size_t)(b0 + r) + o];
-            w = __fmaf_rn(g, a.h2[(size_t)(b0 + r) * MLP_H + i], w);
-            h += gb[(size_t)(b0 + r) * MLP_H + i];
-            z += g;
-        }
-        out[P_W3 + t] = w;
-        out[(o ? P_B2 : P_B1) + i] = h;
-        if (i == 0) out[P_B3 + o] = z;
-    }
-    if (blockIdx.y == 0 && loss) {                // the mean loss, summed in a fixed order
+    if (blockIdx.x > WG_TILES) {                  // the mean loss, summed in a fixed order
+        if (blockIdx.y || !loss) return;
         float* sum = &A[0][0];
         float acc = 0.0f;
         for (int b = t; b < B; b += WG_THREADS) acc += a.loss[b];
@@ -317,7 +318,22 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad(int32_t B, const float* __
             __syncthreads();
         }
         if (t == 0) *loss = sum[0] * (1.0f / (float)B);
+        return;
     }
+    // W3 [2][128], then both hidden biases, then b3
+    const int o = t / MLP_H, i = t % MLP_H;
+    const float* gb = o ? a.g2 : a.g1;
+    float w = 0.0f, h = 0.0f, z = 0.0f;
+#pragma unroll 16
+    for (int r = 0; r < n; r++) {
+        const float g = a.gout[2 * (size_t)(b0 + r) + o];
+        w = __fmaf_rn(g, a.h2[(size_t)(b0 + r) * MLP_H + i], w);
+        h += gb[(size_t)(b0 + r) * MLP_H + i];
+        z += g;
+    }
+    out[P_W3 + t] = w;
+    out[(o ? P_B2 : P_B1) + i] = h;
+    if (i == 0) out[P_B3 + o] = z;
 }
 
 // The chunks' partial gradients added in order.
@@ -338,14 +354,14 @@ __device__ __forceinline__ bool is_weight(int p, int* layer, int* o, int* i) {
 }
 
 struct Weights {
-    uint16_t *w1, *w2, *w3;      // [out][in]
-    uint16_t* w2t;               // [in][out], for the backward pass
+    uint16_t *w1, *w2, *w3;      // w1, w2 grouped; w3 [out][in]
+    uint16_t* w2t;               // w2 transposed, grouped, for the backward pass
 };
 
 __device__ __forceinline__ void store_weight(const Weights& wb, int layer, int o, int i, float v) {
     const uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(v));
-    if (layer == 0) wb.w1[o * FEATURES + i] = h;
-    else if (layer == 1) { wb.w2[o * MLP_H + i] = h; wb.w2t[i * MLP_H + o] = h; }
+    if (layer == 0) wb.w1[grouped(o, i)] = h;
+    else if (layer == 1) { wb.w2[grouped(o, i)] = h; wb.w2t[grouped(i, o)] = h; }
     else wb.w3[o * MLP_H + i] = h;
 }
 
@@ -527,7 +543,7 @@ int grad_impl(dd_mlp* m, const float* X, const float* u_star, int32_t B, float* 
             v, m->wb.w2t, B, X, u_star, m->act);
     const int chunks = chunks_of(B);
     float* part = chunks == 1 ? grad : m->part;
-    dd::k_wgrad<<<dim3(dd::WG_TILES + 1, chunks), dd::WG_THREADS, 0, m->stream>>>(B, X, m->act, part, loss);
+    dd::k_wgrad<<<dim3(dd::WG_TILES + 2, chunks), dd::WG_THREADS, 0, m->stream>>>(B, X, m->act, part, loss);
     if (chunks > 1) dd::k_wsum<<<(NP + 255) / 256, 256, 0, m->stream>>>(chunks, m->part, grad);
     return cudaGetLastError() == cudaSuccess ? DD_OK : DD_ERR_CUDA;
 }
