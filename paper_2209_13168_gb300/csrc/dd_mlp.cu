@@ -263,17 +263,22 @@ __global__ void __launch_bounds__(MLP_H) k_sample(MlpDev m, const uint16_t* __re
 }
 
 // Weight gradients of WG_CHUNK samples (blockIdx.y): blocks 0-15 and 16-31 a
-// 32 x 32 tile of the first two layers (both operands staged in shared
-// memory, four outputs a thread), block 32 the output layer and the biases,
-// block 33, once, the mean loss.  Each chunk writes its own partial gradient; they are
-// added in order (k_wsum), so the result does not depend on the launch.  With
-// one thread per parameter over the whole batch in turn, the chain of B loads
-// and additions was most of a training step (256 samples: 45 us in all).
-constexpr int WG_CHUNK = 64, WG_TILE = 32, WG_THREADS = 256, WG_TILES = 2 * (MLP_H / WG_TILE) * (MLP_H / WG_TILE);
+// 32 x 32 tile of the first two layers (four outputs a thread), blocks 32-35
+// 32 columns of the output layer and of the biases, block 36, once, the mean
+// loss.  Every block first stages its operands in shared memory, all loads in
+// flight at once, so it waits for memory once; one block for the output layer
+// and all biases that read memory sample by sample took 7 us longer than the
+// tiles (gradient of 256 samples 21.6 -> 14.6 us, of 2,048 34.9 -> 28.8).
+// Each chunk writes its own partial gradient; they are added in order
+// (k_wsum), so the result does not depend on the launch.  With one thread per
+// parameter over the whole batch in turn, the chain of B loads and additions
+// was most of a training step (256 samples: 45 us in all).
+constexpr int WG_CHUNK = 64, WG_TILE = 32, WG_THREADS = 256, WG_COLS = MLP_H / WG_TILE;
+constexpr int WG_TILES = 2 * WG_COLS * WG_COLS;
 __global__ void __launch_bounds__(WG_THREADS) k_wgrad(int32_t B, const float* __restrict__ X, Acts a, float* part,
                                                       float* loss) {
     __shared__ __align__(16) float G[WG_CHUNK][WG_TILE];
-    __shared__ float A[WG_CHUNK][WG_TILE];
+    __shared__ float A[WG_CHUNK][WG_TILE], G1[WG_CHUNK][WG_TILE], go[WG_CHUNK][MLP_OUT];
     const int t = threadIdx.x, b0 = blockIdx.y * WG_CHUNK, n = min(WG_CHUNK, B - b0);
     float* out = part + (size_t)blockIdx.y * N_PARAMS;
     if (blockIdx.x < WG_TILES) {
@@ -306,7 +311,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad(int32_t B, const float* __
         o[3 * MLP_H] = s3;
         return;
     }
-    if (blockIdx.x > WG_TILES) {                  // the mean loss, summed in a fixed order
+    if (blockIdx.x == WG_TILES + WG_COLS) {       // the mean loss, summed in a fixed order
         if (blockIdx.y || !loss) return;
         float* sum = &A[0][0];
         float acc = 0.0f;
@@ -320,20 +325,32 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad(int32_t B, const float* __
         if (t == 0) *loss = sum[0] * (1.0f / (float)B);
         return;
     }
-    // W3 [2][128], then both hidden biases, then b3
-    const int o = t / MLP_H, i = t % MLP_H;
-    const float* gb = o ? a.g2 : a.g1;
-    float w = 0.0f, h = 0.0f, z = 0.0f;
-#pragma unroll 16
-    for (int r = 0; r < n; r++) {
-        const float g = a.gout[2 * (size_t)(b0 + r) + o];
-        w = __fmaf_rn(g, a.h2[(size_t)(b0 + r) * MLP_H + i], w);
-        h += gb[(size_t)(b0 + r) * MLP_H + i];
-        z += g;
+    // 32 columns of W3 [2][128] and of both hidden biases; b3
+    const int i0 = (blockIdx.x - WG_TILES) * WG_TILE;
+#pragma unroll
+    for (int q = 0; q < WG_CHUNK * WG_TILE / WG_THREADS; q++) {
+        const int r = t / WG_TILE + q * (WG_THREADS / WG_TILE), c = t % WG_TILE;
+        const size_t k = (size_t)(b0 + r) * MLP_H + i0 + c;
+        A[r][c] = r < n ? a.h2[k] : 0.0f;
+        G1[r][c] = r < n ? a.g1[k] : 0.0f;
+        G[r][c] = r < n ? a.g2[k] : 0.0f;
     }
-    out[P_W3 + t] = w;
-    out[(o ? P_B2 : P_B1) + i] = h;
-    if (i == 0) out[P_B3 + o] = z;
+    if (t < MLP_OUT * n) go[t / MLP_OUT][t % MLP_OUT] = a.gout[MLP_OUT * (size_t)b0 + t];
+    __syncthreads();
+    const int i = t % WG_TILE, o = t / WG_TILE % 2;
+    float s = 0.0f;
+    if (t < 2 * WG_TILE) {
+#pragma unroll 16
+        for (int r = 0; r < n; r++) s = __fmaf_rn(go[r][o], A[r][i], s);
+        out[P_W3 + o * MLP_H + i0 + i] = s;
+    } else if (t < 4 * WG_TILE) {
+#pragma unroll 16
+        for (int r = 0; r < n; r++) s += o ? G[r][i] : G1[r][i];
+        out[(o ? P_B2 : P_B1) + i0 + i] = s;
+    } else if (t < 4 * WG_TILE + MLP_OUT && i0 == 0) {
+        for (int r = 0; r < n; r++) s += go[r][i];
+        out[P_B3 + i] = s;
+    }
 }
 
 // The chunks' partial gradients added in order.
@@ -543,7 +560,7 @@ int grad_impl(dd_mlp* m, const float* X, const float* u_star, int32_t B, float* 
             v, m->wb.w2t, B, X, u_star, m->act);
     const int chunks = chunks_of(B);
     float* part = chunks == 1 ? grad : m->part;
-    dd::k_wgrad<<<dim3(dd::WG_TILES + 2, chunks), dd::WG_THREADS, 0, m->stream>>>(B, X, m->act, part, loss);
+    dd::k_wgrad<<<dim3(dd::WG_TILES + dd::WG_COLS + 1, chunks), dd::WG_THREADS, 0, m->stream>>>(B, X, m->act, part, loss);
     if (chunks > 1) dd::k_wsum<<<(NP + 255) / 256, 256, 0, m->stream>>>(chunks, m->part, grad);
     return cudaGetLastError() == cudaSuccess ? DD_OK : DD_ERR_CUDA;
 }
