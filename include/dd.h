@@ -77,12 +77,13 @@ typedef struct { uint64_t lo; int64_t hi; } dd_i128;
 typedef struct {
     int32_t pop_k;          /* intervals dequeued per BnB round (default 1 = Algorithm 1) */
     int32_t queue_capacity; /* BnB queue entries per window (default 8192)               */
-    int32_t band_rows;      /* rows of the shared-memory IWE tile (default: from W)      */
+    int32_t band_rows;      /* rows of the shared-memory IWE tile (default: from W and H) */
     int32_t threads;        /* threads per block of the IWE kernels, a multiple of 32    */
                             /* up to 512 (default 512; above 480 a block works with 480)  */
     int32_t max_rounds;     /* BnB round limit, DD_ERR_TIMEOUT beyond (default 1<<20)    */
-    int32_t host_loop;      /* 0: each solve's rounds run as one CUDA graph with a       */
-                            /*    conditional loop (no host round trips); 1: the host    */
+    int32_t host_loop;      /* 0: no host round trips: a single window's rounds run in   */
+                            /*    one cooperative launch (up to 4,194,304 events), else  */
+                            /*    as one CUDA graph with a conditional loop; 1: the host */
                             /*    launches the rounds in batches and polls for the end   */
     int32_t max_splits;     /* most blocks that share one row band of a bound (default 16) */
     int32_t warp_to_start;  /* 0: events warped to the window's end (Eq. 11, the paper's  */
