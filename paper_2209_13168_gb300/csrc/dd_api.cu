@@ -607,16 +607,19 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
                            (int32_t)trace_cap, c->stream));
     c->stats.kernel_launches++;
     dd::TraceRec* tr_dev = trace_cap > 0 ? c->trace : nullptr;
-    // One window: all rounds in one cooperative launch.  Several: one graph
+    // A few windows: all rounds in one cooperative launch.  More: one graph
     // launch, whose control step runs one block per window at once.
     const bool device = !c->cfg.host_loop && !c->timing;
-    const bool search = device && nw == 1 && c->search_blocks > 1 && evs[0].n <= dd::SEARCH_MAX_EVENTS;
+    int64_t all_events = 0;
+    for (int w = 0; w < nw; w++) all_events += evs[w].n;
+    const bool search = device && nw <= dd::SEARCH_WINDOWS && c->search_blocks > 2 * nw - 1 &&
+                        all_events <= dd::SEARCH_MAX_EVENTS;
     const bool graph = device && !search;
     dd::NvtxRange rounds("dd rounds");
     if (search) {
-        const dd::CtlArgs ctl = dd::control_args(1, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err, tr_dev,
+        const dd::CtlArgs ctl = dd::control_args(nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err, tr_dev,
                                                  c->jobs, c->job_stride, c->sch, 0, 0, 1, nullptr);
-        DD_TRY(dd::launch_search(c->g, eval_args(c, nullptr, true), ctl, c->threads, c->search_blocks, c->stream));
+        DD_TRY(dd::launch_search(c->g, eval_args(c, nullptr, nw == 1), ctl, c->threads, c->search_blocks, c->stream));
         c->stats.kernel_launches++;
         c->stats.eval_launches++;
     } else if (graph) {
@@ -649,7 +652,9 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
     std::vector<dd::TraceRec> tr((size_t)trace_cap);
     if (trace_cap > 0) DD_TRY(copy(c, tr.data(), c->trace, sizeof(dd::TraceRec) * trace_cap, cudaMemcpyDeviceToHost));
     DD_TRY(sync(c));
-    if (search && c->h_st[0].phase != dd::PH_DONE) {   // a wait ran out: leave the merge buffers as they must be
+    bool ended = true;
+    for (int w = 0; w < nw; w++) ended &= c->h_st[w].phase == dd::PH_DONE;
+    if (search && !ended) {                       // a wait ran out: leave the merge buffers as they must be
         const size_t M1 = (size_t)c->g.planes * M, tiles = (size_t)c->max_tasks * c->g.n_tiles;
         DD_TRY(cudaMemsetAsync(c->macc, 0, sizeof(uint32_t) * (size_t)c->max_tasks * M1, c->stream));
         DD_TRY(cudaMemsetAsync(c->mdone, 0, sizeof(int32_t) * tiles, c->stream));

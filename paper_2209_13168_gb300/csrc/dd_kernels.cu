@@ -1685,7 +1685,7 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
     unsigned long long* cells = sm.cells;
     Sched* sch = c.sch;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = (int)blockDim.x >> 5;
-    const int running = RESIDENT ? 1 : sch->running;   // searches still running after the last round
+    const int running = RESIDENT ? __ldcg(&sch->running) : sch->running;   // searches still running after the last round
     SolveState* st = c.st_all + w;
     Task* tasks = c.tasks_all + (size_t)w * c.task_stride;
     Partial* part = c.part_all + (size_t)w * c.task_stride;
@@ -2108,16 +2108,19 @@ __device__ __forceinline__ void add_release(int32_t* p, int32_t v) {
 // fraction of a second.
 constexpr int SEARCH_POLLS = 1 << 23;
 
-// The control block of k_search: waits for the `others` evaluating blocks,
-// runs the control step and announces the next round.
-__device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, CtlShared& sm, Node* q_mem, int q_cap,
+// Window w's control block of k_search: waits for the `others` evaluating
+// blocks and runs the window's control step; the last window's block to finish
+// announces the next round (or, with no search left, the end).
+__device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int w, CtlShared& sm, Node* q_mem, int q_cap,
                                             int others) {
     Sched* sch = c.sch;
+    const int nw = c.n_windows;
     for (int i = threadIdx.x; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
-        reinterpret_cast<int4*>(&sm.s)[i] = reinterpret_cast<const int4*>(c.st_all)[i];
+        reinterpret_cast<int4*>(&sm.s)[i] = reinterpret_cast<const int4*>(c.st_all + w)[i];
     if (threadIdx.x == 0) sm.q_shared = 1;        // empty
     __syncthreads();
     for (uint32_t round = 0;; round++) {
+        const int par = (int)(round & 1);
         if (threadIdx.x == 0) {
             const int32_t all = (int32_t)(round + 1) * others;
             int polls = 0;
@@ -2130,17 +2133,43 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, Ctl
             return;
         }
         __syncthreads();
-        control_body<true>(g, c, 0, sm, (int)(round & 1), q_mem, q_cap);
+        control_body<true>(g, c, w, sm, par, q_mem, q_cap);
         __syncthreads();                          // the round's tasks and jobs are written
         const bool done = sm.s.phase == PH_DONE;
-        if (threadIdx.x == 0)
-            store_release(&sch->go, (unsigned long long)(round + 1) << 32 | (done ? 0u : (uint32_t)sm.s_total));
-        if (done) return;
+        const unsigned long long next = (unsigned long long)(round + 1) << 32;
+        if (nw == 1) {
+            if (threadIdx.x == 0) store_release(&sch->go, next | (done ? 0u : (uint32_t)sm.s_total));
+            if (done) return;
+            continue;
+        }
+        if (threadIdx.x == 0) {
+            __threadfence();
+            if (!done) atomicAdd(&sch->active, 1);
+            if (atomicAdd(&sch->controls, 1) == (int32_t)(round + 1) * nw - 1) {   // the last window of the round
+                __threadfence();
+                const int active = atomicExch(&sch->active, 0);
+                const int jobs = atomicAdd(&sch->n_jobs[par ^ 1], 0);
+                sch->running = active;
+                sch->n_jobs[par] = 0;             // every block has read its round's count
+                store_release(&sch->go, next | (active ? (uint32_t)jobs : 0u));
+            }
+            unsigned long long v = 0;
+            int polls = 0;
+            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < SEARCH_POLLS) {}
+            if (polls >= SEARCH_POLLS) {          // never in a sound run
+                sch->failed = 1;
+                v = 0;
+            }
+            sm.s_stop = (uint32_t)v == 0;         // every search has ended
+        }
+        __syncthreads();
+        if (sm.s_stop) return;
+        __syncthreads();
     }
 }
 
-// All rounds of one window's search in one cooperative launch.  Block 0 runs
-// the control steps, with the search's state and queue in its shared memory;
+// All rounds of a few windows' searches in one cooperative launch.  Block w runs
+// window w's control steps, with its state and queue in shared memory;
 // the others evaluate a round's units as k_eval does, count themselves in
 // sch->ticket and poll sch->go for the next round.  A search of few events is
 // bound by the latency of its rounds, and a round of two graph nodes, the
@@ -2153,9 +2182,10 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
     __shared__ EvalShared sm;
     __shared__ unsigned long long s_go;
     Sched* sch = a.sch;
-    if (blockIdx.x == 0) {
+    const int nw = c.n_windows;
+    if ((int)blockIdx.x < nw) {
         CtlShared& ctl = *reinterpret_cast<CtlShared*>(tile);
-        control_rounds(g, c, ctl, reinterpret_cast<Node*>(&ctl + 1), q_cap, (int)gridDim.x - 1);
+        control_rounds(g, c, blockIdx.x, ctl, reinterpret_cast<Node*>(&ctl + 1), q_cap, (int)gridDim.x - nw);
         return;
     }
     if (threadIdx.x == 0) {
@@ -2164,7 +2194,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
         s_go = (unsigned long long)(uint32_t)sch->n_jobs[0];
     }
     __syncthreads();
-    const int block = (int)blockIdx.x - 1, blocks = (int)gridDim.x - 1;
+    const int block = (int)blockIdx.x - nw, blocks = (int)gridDim.x - nw;
     for (uint32_t round = 0;; round++) {
         const int par = round & 1, n_jobs = (int)(uint32_t)s_go;
         const int slices = round_slices(g, n_jobs), n_units = n_jobs * g.n_tiles * slices;
@@ -2246,7 +2276,7 @@ int search_resident_blocks(const Geom& g, int threads) {
 
 cudaError_t launch_search(const Geom& g, const EvalArgs& a, const CtlArgs& c, int threads, int grid_blocks,
                           cudaStream_t s) {
-    if (grid_blocks < 2) return cudaErrorInvalidValue;            // block 0 evaluates nothing
+    if (grid_blocks <= c.n_windows) return cudaErrorInvalidValue; // no block would evaluate
     int q_cap = search_queue(g, threads);
     void* args[] = {const_cast<Geom*>(&g), const_cast<EvalArgs*>(&a), const_cast<CtlArgs*>(&c), &q_cap};
     return cudaLaunchCooperativeKernel((const void*)k_search, dim3(grid_blocks), dim3(threads + 32), args,

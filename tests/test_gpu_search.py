@@ -1,5 +1,5 @@
-"""One window's search in one cooperative launch: a control block with the
-queue in its shared memory while it fits, evaluating blocks that poll for the
+"""One window's or a few windows' searches in one cooperative launch: a control
+block each with the queue in its shared memory while it fits, evaluating blocks that poll for the
 next round.  Results, counts and traces are the oracle's whatever the queue's
 place (never, sometimes or always in shared memory), and windows beyond the
 launch's size limit go through the graph with the same result.
@@ -77,3 +77,34 @@ def test_bands_cut_into_slices(n, band_rows):
     want = O.solve(O.Window.of(w), -1.0, 1.0, 1e-3, 0.0, 1)
     for k in KEYS:
         assert got[k] == want[k], (k, got[k], want[k])
+
+
+# up to 16 windows share one launch, 17 go through the graph; they end in
+# different rounds, one has a single event
+@pytest.mark.parametrize("windows", [2, 3, 16, 17])
+@pytest.mark.parametrize("pop_k,threads", [(1, 480), (16, 480), (16, 32)])
+def test_a_few_windows_in_one_launch(windows, pop_k, threads):
+    ws = [make_window(96, 64, 48.0, 32.0, 300 + 170 * i, 30, 100 + 40 * i, 0.2 + 0.02 * i, 0.3, seed=80 + i)
+          for i in range(windows)]
+    ws[1].x, ws[1].y, ws[1].t, ws[1].p = ws[1].x[:1], ws[1].y[:1], ws[1].t[:1], ws[1].p[:1]
+    evs = [dd.Events.of(w, device="cuda") for w in ws]
+    got = {}
+    for host_loop in (0, 1):
+        ctx = dd.Context(96, 64, 48.0, 32.0, pop_k=pop_k, threads=threads, host_loop=host_loop)
+        rc, got[host_loop] = ctx.solve_batch(evs, [(-1.0, 1.0, 1e-3, 0.0)] * windows)
+        assert rc == dd.DD_OK
+        ctx.close()
+    for i, w in enumerate(ws):
+        want = O.solve(O.Window.of(w), -1.0, 1.0, 1e-3, 0.0, pop_k)
+        for k in KEYS:
+            assert got[0][i][k] == got[1][i][k] == want[k], (i, k)
+
+
+def test_a_few_windows_with_limits():
+    ws = [make_window(96, 64, 48.0, 32.0, 900, 40, 300, 0.3, 0.4, seed=90 + i) for i in range(3)]
+    evs = [dd.Events.of(w, device="cuda") for w in ws]
+    for kw, status in (({"max_rounds": 5}, dd.DD_ERR_TIMEOUT), ({"queue_capacity": 3}, dd.DD_ERR_QUEUE_OVERFLOW)):
+        ctx = dd.Context(96, 64, 48.0, 32.0, pop_k=4, **kw)
+        rc, out = ctx.solve_batch(evs)
+        assert rc == status and all(r["status"] == status for r in out)
+        ctx.close()
