@@ -81,10 +81,11 @@ typedef struct {
     int32_t threads;        /* threads per block of the IWE kernels, a multiple of 32    */
                             /* up to 512 (default 512; above 480 a block works with 480)  */
     int32_t max_rounds;     /* BnB round limit, DD_ERR_TIMEOUT beyond (default 1<<20)    */
-    int32_t host_loop;      /* 0: no host round trips: a single window's rounds run in   */
-                            /*    one cooperative launch (up to 4,194,304 events), else  */
-                            /*    as one CUDA graph with a conditional loop; 1: the host */
-                            /*    launches the rounds in batches and polls for the end   */
+    int32_t host_loop;      /* 0: no host round trips: the rounds of up to 16 windows    */
+                            /*    with at most 4,194,304 events run in one cooperative   */
+                            /*    launch, others as one CUDA graph with a conditional    */
+                            /*    loop; 1: the host launches the rounds in batches and   */
+                            /*    polls for the end                                      */
     int32_t max_splits;     /* most blocks that share one row band of a bound (default 16) */
     int32_t warp_to_start;  /* 0: events warped to the window's end (Eq. 11, the paper's  */
                             /*    reference time tau); 1: to its start (reference time 0: */
@@ -215,8 +216,8 @@ int dd_solve(dd_ctx* ctx, const dd_events* ev, float D_lo, float D_hi, float tol
  * context's frame geometry): every round evaluates the pending intervals of
  * all windows in one launch and runs one control block per window; each
  * window keeps its own device-resident queue and incumbent, and a window that
- * has finished simply stops contributing work.  The rounds run as one CUDA
- * graph (or host-driven batches with dd_config.host_loop).  windows[w] and
+ * has finished simply stops contributing work.  The rounds run without
+ * host round trips (or in host-driven batches with dd_config.host_loop).  windows[w] and
  * params[w] (host arrays) describe window w; out[w] receives its result,
  * identical to dd_solve on that window alone with the same pop_k.
  * Returns DD_OK when every window succeeded; otherwise the first failing
