@@ -1676,8 +1676,9 @@ __device__ __forceinline__ i128 warp_max_i128(i128 v, bool valid, unsigned& at) 
 // RESIDENT (the control block of k_search): the state stays in `sm` from round
 // to round, and so does the queue while it has at most q_cap entries (two
 // buffers of q_cap at q_mem); the state reaches global memory when the search
-// ends, the queue when it grows beyond that.
-template <bool RESIDENT>
+// ends, the queue when it grows beyond that.  FEW: its launch has several
+// windows.
+template <bool RESIDENT, bool FEW = false>
 __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, int w, CtlShared& sm, int par,
                                              Node* q_mem = nullptr, int q_cap = 0) {
     SolveState& s = sm.s;
@@ -1685,7 +1686,8 @@ __device__ __forceinline__ void control_body(const Geom& g, const CtlArgs& c, in
     unsigned long long* cells = sm.cells;
     Sched* sch = c.sch;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = (int)blockDim.x >> 5;
-    const int running = RESIDENT ? __ldcg(&sch->running) : sch->running;   // searches still running after the last round
+    // searches still running after the last round
+    const int running = !RESIDENT ? sch->running : (FEW ? __ldcg(&sch->running) : 1);
     SolveState* st = c.st_all + w;
     Task* tasks = c.tasks_all + (size_t)w * c.task_stride;
     Partial* part = c.part_all + (size_t)w * c.task_stride;
@@ -2111,10 +2113,11 @@ constexpr int SEARCH_POLLS = 1 << 23;
 // Window w's control block of k_search: waits for the `others` evaluating
 // blocks and runs the window's control step; the last window's block to finish
 // announces the next round (or, with no search left, the end).
-__device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int w, CtlShared& sm, Node* q_mem, int q_cap,
+template <bool FEW>
+__device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int window, CtlShared& sm, Node* q_mem, int q_cap,
                                             int others) {
     Sched* sch = c.sch;
-    const int nw = c.n_windows;
+    const int w = FEW ? window : 0, nw = FEW ? c.n_windows : 1;
     for (int i = threadIdx.x; i < (int)(sizeof(SolveState) / 16); i += blockDim.x)
         reinterpret_cast<int4*>(&sm.s)[i] = reinterpret_cast<const int4*>(c.st_all + w)[i];
     if (threadIdx.x == 0) sm.q_shared = 1;        // empty
@@ -2133,11 +2136,11 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int
             return;
         }
         __syncthreads();
-        control_body<true>(g, c, w, sm, par, q_mem, q_cap);
+        control_body<true, FEW>(g, c, w, sm, par, q_mem, q_cap);
         __syncthreads();                          // the round's tasks and jobs are written
         const bool done = sm.s.phase == PH_DONE;
         const unsigned long long next = (unsigned long long)(round + 1) << 32;
-        if (nw == 1) {
+        if (!FEW) {
             if (threadIdx.x == 0) store_release(&sch->go, next | (done ? 0u : (uint32_t)sm.s_total));
             if (done) return;
             continue;
@@ -2174,7 +2177,10 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int
 // sch->ticket and poll sch->go for the next round.  A search of few events is
 // bound by the latency of its rounds, and a round of two graph nodes, the
 // loop's condition and a control step that reads and writes its state in L2
-// costs about 10 us beside the evaluation.
+// costs about 10 us beside the evaluation.  A kernel of its own for one window
+// (FEW false): with the window and their number read at run time its searches
+// took 1-5% longer (30,000 events, one interval a round: 3.34 / 3.50 ms).
+template <bool FEW>
 __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_constant__ Geom g,
                                                                  const __grid_constant__ EvalArgs a,
                                                                  const __grid_constant__ CtlArgs c, int q_cap) {
@@ -2182,10 +2188,10 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
     __shared__ EvalShared sm;
     __shared__ unsigned long long s_go;
     Sched* sch = a.sch;
-    const int nw = c.n_windows;
+    const int nw = FEW ? c.n_windows : 1;
     if ((int)blockIdx.x < nw) {
         CtlShared& ctl = *reinterpret_cast<CtlShared*>(tile);
-        control_rounds(g, c, blockIdx.x, ctl, reinterpret_cast<Node*>(&ctl + 1), q_cap, (int)gridDim.x - nw);
+        control_rounds<FEW>(g, c, blockIdx.x, ctl, reinterpret_cast<Node*>(&ctl + 1), q_cap, (int)gridDim.x - nw);
         return;
     }
     if (threadIdx.x == 0) {
@@ -2267,9 +2273,12 @@ int search_resident_blocks(const Geom& g, int threads) {
     int per_sm = 0, dev = 0, sms = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_search, threads + 32, search_smem_bytes(g, threads)) !=
-        cudaSuccess)
+    int one = 0;
+    const size_t bytes = search_smem_bytes(g, threads);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&one, k_search<false>, threads + 32, bytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_search<true>, threads + 32, bytes) != cudaSuccess)
         return 0;
+    if (one < per_sm) per_sm = one;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     return per_sm * sms;
 }
@@ -2279,8 +2288,9 @@ cudaError_t launch_search(const Geom& g, const EvalArgs& a, const CtlArgs& c, in
     if (grid_blocks <= c.n_windows) return cudaErrorInvalidValue; // no block would evaluate
     int q_cap = search_queue(g, threads);
     void* args[] = {const_cast<Geom*>(&g), const_cast<EvalArgs*>(&a), const_cast<CtlArgs*>(&c), &q_cap};
-    return cudaLaunchCooperativeKernel((const void*)k_search, dim3(grid_blocks), dim3(threads + 32), args,
-                                       search_smem_bytes(g, threads), s);
+    const void* kernel = c.n_windows == 1 ? (const void*)k_search<false> : (const void*)k_search<true>;
+    return cudaLaunchCooperativeKernel(kernel, dim3(grid_blocks), dim3(threads + 32), args, search_smem_bytes(g, threads),
+                                       s);
 }
 
 // Function attributes are per device: the carveout and the dynamic
@@ -2302,7 +2312,8 @@ cudaError_t eval_smem_setup(const Geom& g) {
         // One shared-memory carveout for every kernel of the library, so that
         // consecutive launches never wait for an L1 / shared reconfiguration.
         const void* fns[] = {(const void*)k_eval, (const void*)k_control, (const void*)k_init,
-                             (const void*)k_keys, (const void*)k_search, (const void*)k_ingest_small, (const void*)k_row_hist, (const void*)k_row_scan,
+                             (const void*)k_keys, (const void*)k_search<false>, (const void*)k_search<true>,
+                             (const void*)k_ingest_small, (const void*)k_row_hist, (const void*)k_row_scan,
                              (const void*)k_row_scatter};
         for (const void* f : fns) {
             e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -2314,7 +2325,8 @@ cudaError_t eval_smem_setup(const Geom& g) {
     const int bytes = (int)search_smem_bytes(g, EVAL_THREADS);   // any block size
     if (bytes <= g_smem_bytes[dev]) return cudaSuccess;
     e = cudaFuncSetAttribute(k_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_search, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_search<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_search<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) g_smem_bytes[dev] = bytes;
     return e;
 }
