@@ -86,6 +86,27 @@ def test_fused_units_with_a_hot_pixel(hot, threads):
     ctx.close()
 
 
+def test_fused_units_whose_listed_events_overflow():
+    # every band holds a pixel of 1,200 events that moves over a border in most
+    # intervals: its events are listed (80 a warp) and a field overflows only
+    # in the second part of the unit, which the warps reach one by one
+    w = make_window(96, 64, 48.0, 32.0, 900, 40, 300, 0.3, 0.4, seed=78)
+    rows, hot = np.arange(2, 64, 4), 1200
+    x = np.concatenate([w.x, np.full(rows.size * hot, 70, np.int16)])
+    y = np.concatenate([w.y, np.repeat(rows, hot).astype(np.int16)])
+    t = np.concatenate([w.t, np.full(rows.size * hot, 0.1, np.float32)])
+    w.x, w.y, w.t, w.p = x, y, t, np.ones(x.size, np.int8)
+    want = O.solve(O.Window.of(w), -1.0, 1.0, 1e-3, 0.0, 16, trace_cap=4096)
+    ev = dd.Events.of(w, device="cuda")
+    ctx = dd.Context(96, 64, 48.0, 32.0, pop_k=16, band_rows=4, fuse_span=1_000_000)
+    for _ in range(20):
+        got = ctx.solve(ev, -1.0, 1.0, 1e-3, 0.0, trace_cap=4096)
+        for k in KEYS:
+            assert got[k] == want[k], (k, got[k], want[k])
+        assert got["trace"] == want["trace"]
+    ctx.close()
+
+
 def test_fused_units_with_a_full_list():
     # one warp per block: bands with more than 320 unstable events
     w = make_window(160, 90, 80.0, 45.0, 9000, 250, 3000, 0.35, 0.3, seed=74)
