@@ -85,7 +85,9 @@ typedef struct {
                             /*    with at most 4,194,304 events run in one cooperative   */
                             /*    launch, others as one CUDA graph with a conditional    */
                             /*    loop; 1: the host launches the rounds in batches and   */
-                            /*    polls for the end                                      */
+                            /*    polls for the end.  The cooperative launch starts once */
+                            /*    all its blocks (two per SM) fit beside other work on   */
+                            /*    the device; 1 runs on whatever part of it is free      */
     int32_t max_splits;     /* most blocks that share one row band of a bound (default 16) */
     int32_t warp_to_start;  /* 0: events warped to the window's end (Eq. 11, the paper's  */
                             /*    reference time tau); 1: to its start (reference time 0: */
@@ -315,6 +317,13 @@ int dd_reset_stats(dd_ctx* ctx);
  * behaviour without the batching), so every timed launch evaluates work:
  * launch k of a solve is its round k. */
 int dd_set_timing(dd_ctx* ctx, int32_t enable);
+
+/* Limit of the waits inside the one launch that runs up to 16 windows'
+ * searches (dd_config.host_loop): a block polls at most `polls` times for the
+ * others (0: the default, about 1.6 s).  When a wait runs out the launch ends
+ * and the call runs the same searches again through the CUDA graph, with the
+ * same results; only the time differs.  Errors: DD_ERR_ARG (polls < 0). */
+int dd_set_wait_limit(dd_ctx* ctx, int32_t polls);
 
 /* Telemetry: the device durations (ms) of the timed IWE launches since the
  * last dd_reset_stats, in launch order, the first DD_MAX_LAUNCH_TIMES of

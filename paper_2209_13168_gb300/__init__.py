@@ -7,7 +7,7 @@ missing or fails to load, every entry point raises.
 
 The functions keep the C names (dd_create, dd_contrast, dd_bound, dd_solve,
 dd_solve_trace, dd_solve_window, dd_solve_batch, dd_features, dd_set_warm_model,
-dd_set_stream, dd_get_stats, dd_reset_stats, dd_set_timing, dd_destroy,
+dd_set_stream, dd_get_stats, dd_reset_stats, dd_set_timing, dd_set_wait_limit, dd_destroy,
 dd_strerror, dd_resample, dd_resample_foe, dd_time_span, dd_stream_solve,
 dd_probe_peaks, the dd_serve_* and dd_mlp_* families); ``Context``, ``Server``
 and ``Mlp`` wrap them for numpy arrays (host events) and torch CUDA tensors
@@ -153,6 +153,7 @@ SIGNATURES = {
     "dd_get_stats": (ctypes.c_int, [_VP, _P(dd_stats)]),
     "dd_reset_stats": (ctypes.c_int, [_VP]),
     "dd_set_timing": (ctypes.c_int, [_VP, ctypes.c_int32]),
+    "dd_set_wait_limit": (ctypes.c_int, [_VP, ctypes.c_int32]),
     "dd_get_launch_times": (ctypes.c_int, [_VP, _VP, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]),
     "dd_contrast_noalloc": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32, ctypes.c_float, ctypes.c_float,
                                            _P(dd_events), _VP, ctypes.c_int32, _VP, _VP]),
@@ -229,6 +230,10 @@ def dd_reset_stats(h):
 
 def dd_set_timing(h, enable):
     _check(load().dd_set_timing(h, 1 if enable else 0), "dd_set_timing")
+
+
+def dd_set_wait_limit(h, polls):
+    _check(load().dd_set_wait_limit(h, polls), "dd_set_wait_limit")
 
 
 def dd_get_launch_times(h):
@@ -706,6 +711,9 @@ class Context:
 
     def set_timing(self, enable):
         dd_set_timing(self.h, enable)
+
+    def set_wait_limit(self, polls):
+        dd_set_wait_limit(self.h, polls)
 
     def launch_times(self):
         return dd_get_launch_times(self.h)

@@ -21,6 +21,7 @@ struct dd_ctx {
     int max_tasks = 0;            // task slots per window
     int eval_blocks = 0;          // resident blocks of the evaluation grid
     int search_blocks = 0;        // resident blocks of a one-launch search (0: not available)
+    int search_polls = dd::SEARCH_POLLS;   // its waits' limit (dd_set_wait_limit)
     cudaStream_t own = nullptr, stream = nullptr;
 
     // events: sorted, for all windows of a call
@@ -602,69 +603,75 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
         DD_TRY(dd::launch_warm(c->g, nw, c->feat_counts, c->wins, c->params, m, c->stream));
         c->stats.kernel_launches++;
     }
-    DD_TRY(dd::launch_init(c->g, nw, c->st, c->tasks, c->max_tasks, c->part, c->wins, c->params, c->jobs,
-                           c->job_stride, c->sch, c->cfg.pop_k, c->cfg.queue_capacity, c->cfg.max_rounds,
-                           (int32_t)trace_cap, c->stream));
-    c->stats.kernel_launches++;
     dd::TraceRec* tr_dev = trace_cap > 0 ? c->trace : nullptr;
+    std::vector<dd::TraceRec> tr((size_t)trace_cap);
     // A few windows: all rounds in one cooperative launch.  More: one graph
     // launch, whose control step runs one block per window at once.
     const bool device = !c->cfg.host_loop && !c->timing;
     int64_t all_events = 0;
     for (int w = 0; w < nw; w++) all_events += evs[w].n;
-    const bool search = device && nw <= dd::SEARCH_WINDOWS && c->search_blocks > 2 * nw - 1 &&
-                        all_events <= dd::SEARCH_MAX_EVENTS;
-    const bool graph = device && !search;
+    bool search = device && nw <= dd::SEARCH_WINDOWS && c->search_blocks > 2 * nw - 1 &&
+                  all_events <= dd::SEARCH_MAX_EVENTS;
     dd::NvtxRange rounds("dd rounds");
-    if (search) {
-        const dd::CtlArgs ctl = dd::control_args(nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err, tr_dev,
-                                                 c->jobs, c->job_stride, c->sch, 0, 0, 1, nullptr);
-        DD_TRY(dd::launch_search(c->g, eval_args(c, nullptr, nw == 1), ctl, c->threads, c->search_blocks, c->stream));
+    for (;; search = false) {
+        DD_TRY(dd::launch_init(c->g, nw, c->st, c->tasks, c->max_tasks, c->part, c->wins, c->params, c->jobs,
+                               c->job_stride, c->sch, c->cfg.pop_k, c->cfg.queue_capacity, c->cfg.max_rounds,
+                               (int32_t)trace_cap, c->stream));
         c->stats.kernel_launches++;
-        c->stats.eval_launches++;
-    } else if (graph) {
-        // One graph launch runs every round on the device.
-        if (!c->gexec || c->g_nw != nw || c->g_key[0] != (const void*)c->ev || c->g_key[1] != (const void*)tr_dev ||
-            c->g_key[2] != (const void*)c->st) {
-            rc = build_graph(c, nw, tr_dev);
-            if (rc) return rc;
-        }
-        DD_TRY(cudaGraphLaunch(c->gexec, c->stream));
-    } else {
-        // Host-driven rounds: launch batches, poll for the end.  With timing
-        // on, one round per poll, so that every timed launch has work.
-        int batch = c->timing ? 1 : 2;
-        for (;;) {
-            for (int b = 0; b < batch; b++) {
-                DD_TRY(eval(c, eval_args(c, nullptr, nw == 1)));
-                DD_TRY(dd::launch_control(c->g, nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err,
-                                          tr_dev, c->jobs, c->job_stride, c->sch, 0, 0, c->stream));
-                c->stats.kernel_launches++;
+        const bool graph = device && !search;
+        if (search) {
+            dd::CtlArgs ctl = dd::control_args(nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err, tr_dev,
+                                               c->jobs, c->job_stride, c->sch, 0, 0, 1, nullptr);
+            ctl.polls = c->search_polls;
+            DD_TRY(dd::launch_search(c->g, eval_args(c, nullptr, nw == 1), ctl, c->threads, c->search_blocks,
+                                     c->stream));
+            c->stats.kernel_launches++;
+            c->stats.eval_launches++;
+        } else if (graph) {
+            // One graph launch runs every round on the device.
+            if (!c->gexec || c->g_nw != nw || c->g_key[0] != (const void*)c->ev || c->g_key[1] != (const void*)tr_dev ||
+                c->g_key[2] != (const void*)c->st) {
+                rc = build_graph(c, nw, tr_dev);
+                if (rc) return rc;
             }
-            DD_TRY(copy(c, c->h_sch, c->sch, sizeof(dd::Sched), cudaMemcpyDeviceToHost));
-            DD_TRY(sync(c));
-            if (c->h_sch->running == 0) break;
-            if (batch < 64 && !c->timing) batch *= 2;
+            DD_TRY(cudaGraphLaunch(c->gexec, c->stream));
+        } else {
+            // Host-driven rounds: launch batches, poll for the end.  With timing
+            // on, one round per poll, so that every timed launch has work.
+            int batch = c->timing ? 1 : 2;
+            for (;;) {
+                for (int b = 0; b < batch; b++) {
+                    DD_TRY(eval(c, eval_args(c, nullptr, nw == 1)));
+                    DD_TRY(dd::launch_control(c->g, nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err,
+                                              tr_dev, c->jobs, c->job_stride, c->sch, 0, 0, c->stream));
+                    c->stats.kernel_launches++;
+                }
+                DD_TRY(copy(c, c->h_sch, c->sch, sizeof(dd::Sched), cudaMemcpyDeviceToHost));
+                DD_TRY(sync(c));
+                if (c->h_sch->running == 0) break;
+                if (batch < 64 && !c->timing) batch *= 2;
+            }
         }
-    }
-    DD_TRY(copy(c, c->h_st, c->st, sizeof(dd::SolveState) * nw, cudaMemcpyDeviceToHost));
-    if (graph) DD_TRY(copy(c, c->h_sch, c->sch, sizeof(dd::Sched), cudaMemcpyDeviceToHost));
-    std::vector<dd::TraceRec> tr((size_t)trace_cap);
-    if (trace_cap > 0) DD_TRY(copy(c, tr.data(), c->trace, sizeof(dd::TraceRec) * trace_cap, cudaMemcpyDeviceToHost));
-    DD_TRY(sync(c));
-    bool ended = true;
-    for (int w = 0; w < nw; w++) ended &= c->h_st[w].phase == dd::PH_DONE;
-    if (search && !ended) {                       // a wait ran out: leave the merge buffers as they must be
+        DD_TRY(copy(c, c->h_st, c->st, sizeof(dd::SolveState) * nw, cudaMemcpyDeviceToHost));
+        if (graph) DD_TRY(copy(c, c->h_sch, c->sch, sizeof(dd::Sched), cudaMemcpyDeviceToHost));
+        if (trace_cap > 0)
+            DD_TRY(copy(c, tr.data(), c->trace, sizeof(dd::TraceRec) * trace_cap, cudaMemcpyDeviceToHost));
+        DD_TRY(sync(c));
+        if (graph) {                              // every round ran one evaluation and one control launch
+            c->stats.kernel_launches += 2 * (int64_t)c->h_sch->round;
+            c->stats.eval_launches += c->h_sch->round;
+        }
+        bool ended = true;
+        for (int w = 0; w < nw; w++) ended &= c->h_st[w].phase == dd::PH_DONE;
+        if (!search || ended) break;
+        // A wait of the one launch ran out: the same searches from their start
+        // through the graph, with every sum zero as it must be between uses
+        // (launch_init clears the tasks').
         const size_t M1 = (size_t)c->g.planes * M, tiles = (size_t)c->max_tasks * c->g.n_tiles;
         DD_TRY(cudaMemsetAsync(c->macc, 0, sizeof(uint32_t) * (size_t)c->max_tasks * M1, c->stream));
         DD_TRY(cudaMemsetAsync(c->mdone, 0, sizeof(int32_t) * tiles, c->stream));
         DD_TRY(cudaMemsetAsync(c->msums, 0, sizeof(dd::Partial) * tiles, c->stream));
-        DD_TRY(sync(c));
-        return DD_ERR_CUDA;
-    }
-    if (graph) {                                  // every round ran one evaluation and one control launch
-        c->stats.kernel_launches += 2 * (int64_t)c->h_sch->round;
-        c->stats.eval_launches += c->h_sch->round;
+        DD_TRY(cudaMemsetAsync(c->sch, 0, sizeof(dd::Sched), c->stream));
     }
     int status = DD_OK;
     for (int w = 0; w < nw; w++)
@@ -897,6 +904,12 @@ int dd_get_launch_times(dd_ctx* c, float* ms, int32_t cap, int32_t* n) {
 int dd_set_timing(dd_ctx* c, int32_t enable) {
     if (!c) return DD_ERR_ARG;
     c->timing = enable != 0;
+    return DD_OK;
+}
+
+int dd_set_wait_limit(dd_ctx* c, int32_t polls) {
+    if (!c || polls < 0) return DD_ERR_ARG;
+    c->search_polls = polls ? polls : dd::SEARCH_POLLS;
     return DD_OK;
 }
 

@@ -160,7 +160,6 @@ struct Sched {
     int32_t n_jobs[2];
     int32_t work[2];
     int32_t ticket, active, running;
-    int32_t failed;                // k_search: a block gave up waiting for the others
     int32_t controls;              // k_search: control steps run, over all windows and rounds
     unsigned long long go;         // k_search: (next round) << 32 | its jobs
 };
@@ -284,6 +283,7 @@ struct CtlArgs {
     cudaGraphConditionalHandle loop;
     int32_t use_loop, split_ok;
     int32_t* phase_out;
+    int32_t polls;                 // k_search: polls before a block gives up waiting for the others
 };
 
 // Everything an evaluation launch reads or writes.
@@ -312,11 +312,21 @@ cudaError_t launch_eval(const Geom& g, const EvalArgs& a, int threads, int grid_
 int eval_resident_blocks(const Geom& g, int threads);
 // All rounds of a few windows' searches in one cooperative launch of at most
 // search_resident_blocks blocks, for at most SEARCH_MAX_EVENTS events in all
-// (a round's waits are bounded) and SEARCH_WINDOWS windows: each keeps one
+// (a round stays short beside the limit of its waits) and SEARCH_WINDOWS
+// windows: each keeps one
 // block for its control steps, and beyond that the blocks missing from the
 // evaluation cost what the shorter rounds save (graph -> one launch: 2 windows
 // of 346x260 475 -> 405 us, 7 of a stream 840 -> 780, 6 of 511x389 1,136 ->
 // 1,040; 19 to 64 windows between 6% faster and 9% slower).
+//
+// Every wait of one block for the others ends after c.polls polls (by default
+// SEARCH_POLLS: 1.6 s at 0.19 us a poll).  A block that gives up returns, so
+// the others' waits run out as well, the launch ends and the windows' states
+// in memory are not all PH_DONE: the caller then clears the sums (the merge
+// buffers and the tasks') and runs the searches another way.  A sound round
+// can outlast the limit: its work is events times the cells of their segments
+// times tasks, and the events of one row all go to one block.
+constexpr int SEARCH_POLLS = 1 << 23;
 constexpr int64_t SEARCH_MAX_EVENTS = 1 << 22;
 constexpr int SEARCH_WINDOWS = 16;
 int search_resident_blocks(const Geom& g, int threads);

@@ -2110,11 +2110,6 @@ __device__ __forceinline__ void add_release(int32_t* p, int32_t v) {
     asm volatile("red.release.gpu.global.add.s32 [%0], %1;" : : "l"(p), "r"(v) : "memory");
 }
 
-// Polls before a block gives up on the others: each takes about a
-// microsecond, and rounds of at most SEARCH_MAX_EVENTS events end within a
-// fraction of a second.
-constexpr int SEARCH_POLLS = 1 << 23;
-
 // Window w's control block of k_search: waits for the `others` evaluating
 // blocks and runs the window's control step; the last window's block to finish
 // announces the next round (or, with no search left, the end).
@@ -2132,14 +2127,11 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int
         if (threadIdx.x == 0) {
             const int32_t all = (int32_t)(round + 1) * others;
             int polls = 0;
-            while (load_acquire(&sch->ticket) != all && ++polls < SEARCH_POLLS) {}
-            sm.s_stop = polls >= SEARCH_POLLS;
+            while (load_acquire(&sch->ticket) != all && ++polls < c.polls) {}
+            sm.s_stop = polls >= c.polls;
         }
         __syncthreads();
-        if (sm.s_stop) {                          // never in a sound run
-            if (threadIdx.x == 0) sch->failed = 1;
-            return;
-        }
+        if (sm.s_stop) return;                    // given up: the search stays unfinished
         __syncthreads();
         control_body<true, FEW>(g, c, w, sm, par, q_mem, q_cap);
         __syncthreads();                          // the round's tasks and jobs are written
@@ -2163,12 +2155,8 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int
             }
             unsigned long long v = 0;
             int polls = 0;
-            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < SEARCH_POLLS) {}
-            if (polls >= SEARCH_POLLS) {          // never in a sound run
-                sch->failed = 1;
-                v = 0;
-            }
-            sm.s_stop = (uint32_t)v == 0;         // every search has ended
+            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < c.polls) {}
+            sm.s_stop = polls >= c.polls || (uint32_t)v == 0;     // given up, or every search has ended
         }
         __syncthreads();
         if (sm.s_stop) return;
@@ -2217,12 +2205,8 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
             add_release(&sch->ticket, 1);
             unsigned long long v = 0;
             int polls = 0;
-            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < SEARCH_POLLS) {}
-            if (polls >= SEARCH_POLLS) {          // never in a sound run: end the search
-                sch->failed = 1;
-                v = 0;
-            }
-            s_go = v;
+            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < c.polls) {}
+            s_go = polls >= c.polls ? 0 : v;      // given up: no more jobs
         }
         __syncthreads();
         if ((uint32_t)s_go == 0) return;
@@ -2232,7 +2216,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
 CtlArgs control_args(int32_t n_windows, SolveState* st, Node* queues, Task* tasks, int32_t task_stride, Partial* part,
                      const int32_t* err, TraceRec* trace, Job* jobs, int32_t job_stride, Sched* sch,
                      cudaGraphConditionalHandle loop, int32_t use_loop, int32_t split_ok, int32_t* phase_out) {
-    CtlArgs c;
+    CtlArgs c{};
     c.n_windows = n_windows;
     c.st_all = st;
     c.queues = queues;

@@ -38,6 +38,74 @@ def test_queue_in_and_out_of_shared_memory(threads, band_rows, pop_k):
     ctx.close()
 
 
+# A wait that runs out ends the launch, and the same searches run through the
+# graph: at the first round (one poll) or wherever a round outlasts the polls.
+# What the unfinished round left in the sums (of tasks, and of bands split by
+# events: 140,000 of them on a wide frame) must not reach the rerun or what
+# the context evaluates next.
+@pytest.mark.parametrize("polls", [1, 16, 64])
+@pytest.mark.parametrize("windows,n", [(1, 3000), (1, 140000), (3, 3000)])
+def test_a_wait_that_runs_out(polls, windows, n):
+    ws = [make_window(640, 480, 320.0, 240.0, n - n // 4, n // 36, n // 4, 0.35, 0.3, seed=60 + i)
+          for i in range(windows)]
+    evs = [dd.Events.of(w, device="cuda") for w in ws]
+    ctx = dd.Context(640, 480, 320.0, 240.0, pop_k=16)
+    ctx.set_wait_limit(polls)
+    for _ in range(2):
+        ctx.reset_stats()
+        rc, got = ctx.solve_batch(evs, [(-1.0, 1.0, 2e-2, 0.0)] * windows)
+        assert rc == dd.DD_OK
+        if polls == 1:
+            assert ctx.stats()["eval_launches"] == 1 + max(r["rounds"] for r in got) + 1   # the root's round too
+        for w, r in zip(ws, got):
+            want = O.solve(O.Window.of(w), -1.0, 1.0, 2e-2, 0.0, 16)
+            for k in KEYS:
+                assert r[k] == want[k], (k, r[k], want[k])
+        win = O.Window.of(ws[0])
+        assert ctx.contrast(evs[0], [0.1, 0.35])[0] == [O.contrast(win, D)[0] for D in (0.1, 0.35)]
+        assert ctx.bound(evs[0], [-1.0, 0.3], [1.0, 0.4])[0] == [O.bound(win, a, b)[0] for a, b in ((-1.0, 1.0), (0.3, 0.4))]
+    ctx.set_wait_limit(0)
+    trace = ctx.solve(evs[0], -1.0, 1.0, 2e-2, 0.0, trace_cap=4096)["trace"]
+    ctx.set_wait_limit(polls)
+    assert ctx.solve(evs[0], -1.0, 1.0, 2e-2, 0.0, trace_cap=4096)["trace"] == trace
+    with pytest.raises(dd.DDError):
+        ctx.set_wait_limit(-1)
+    ctx.close()
+
+
+# The one launch takes every SM: searches of two contexts on their own threads
+# and streams take turns, and a search takes turns with a server's rounds.
+def test_searches_beside_other_work():
+    import threading
+    ws = [make_window(160, 90, 80.0, 45.0, 4000 + 900 * i, 110, 1300, 0.35, 0.3, seed=75 + i) for i in range(2)]
+    want = [O.solve(O.Window.of(w), -1.0, 1.0, 1e-3, 0.0, 8) for w in ws]
+    evs = [dd.Events.of(w, device="cuda") for w in ws]
+    ctxs = [dd.Context(160, 90, 80.0, 45.0, pop_k=8) for _ in range(3)]
+    srv = dd.Server(ctxs[2], max_slots=4, max_events=1 << 13)
+    got = [[], [], []]
+
+    def search(i):
+        for _ in range(30):
+            got[i].append(ctxs[i].solve(evs[i], -1.0, 1.0, 1e-3, 0.0))
+
+    threads = [threading.Thread(target=search, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for _ in range(5):
+        tickets = [srv.submit(evs[k % 2], (-1.0, 1.0, 1e-3, 0.0)) for k in range(8)]
+        got[2] += [srv.wait(k) for k in tickets]
+    for t in threads:
+        t.join()
+    srv.stop()
+    assert [len(g) for g in got] == [30, 30, 40]
+    for i in range(3):
+        for j, r in enumerate(got[i]):
+            for k in KEYS:
+                assert r[k] == want[i if i < 2 else j % 2][k], (i, j, k)
+    for c in ctxs:
+        c.close()
+
+
 def test_round_and_queue_limits():
     w = make_window(160, 90, 80.0, 45.0, 4000, 110, 1300, 0.35, 0.3, seed=75)
     ev = dd.Events.of(w, device="cuda")
