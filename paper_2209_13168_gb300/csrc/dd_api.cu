@@ -535,9 +535,6 @@ void fill_result(const dd::SolveState& s, const dd_events& ev, int64_t M, dd_res
 int feature_counts(dd_ctx* c, int nw) {
     if (nw > c->feat_cap) {
         release(c->feat_counts);
-    release(c->rs_counts);
-    release(c->rs_offsets);
-    release(c->rs_err);
         c->feat_cap = 0;
         DD_TRY(cudaMalloc((void**)&c->feat_counts, sizeof(int32_t) * dd::FEATURES * (size_t)nw));
         c->feat_cap = nw;
@@ -766,6 +763,9 @@ void dd_destroy(dd_ctx* c) {
     release(c->iwe);
     release(c->trace);
     release(c->feat_counts);
+    release(c->rs_counts);
+    release(c->rs_offsets);
+    release(c->rs_err);
     release_host(c->h_st);
     release_host(c->h_err);
     release_host(c->h_call);

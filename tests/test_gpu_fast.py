@@ -55,6 +55,22 @@ def test_resample_rejects_events_outside_the_frame():
     ctx.close()
 
 
+def test_resample_between_feature_calls():
+    # the two share a context, each with scratch of its own: features of more
+    # windows than before must leave the resampling's alone
+    w = window_config1()
+    want = O.resample(O.Window.of(w), 80, 60, 0.5, 3)
+    ctx = dd.Context(w.W, w.H, w.foe_x, w.foe_y)
+    ev = dd.Events.of(w, device="cuda")
+    for windows in (1, 5, 40):
+        feats = ctx.features([ev] * windows).cpu().numpy()
+        assert all(np.array_equal(f, O.features(O.Window.of(w))[0]) for f in feats)
+        x, y, t = dd.dd_resample(ctx.h, ev, w.W, w.H, 80, 60, 0.5, 3)
+        assert np.array_equal(x.cpu().numpy(), want.x) and np.array_equal(y.cpu().numpy(), want.y)
+        assert np.array_equal(t.cpu().numpy(), want.t)
+    ctx.close()
+
+
 @pytest.mark.parametrize("pop_k", [1, 16])
 def test_fast_solve_matches_oracle(pop_k):
     w = window_config2()
