@@ -809,16 +809,7 @@ int dd_create(int32_t W, int32_t H, float foe_x, float foe_y, const dd_config* c
     c->g.H = H;
     c->g.fx = foe_x;
     c->g.fy = foe_y;
-    // Default band: the tallest whose tile leaves room for two evaluation
-    // blocks per SM, the frame's rows divided evenly among as many bands: a
-    // unit's fixed cost is shared by more events (against bands of 40 KB: 43
-    // windows of a 511x389 stream 5.8 -> 4.1 ms, 55 of a 346x260 one 4.8 ->
-    // 4.0 ms; a search with few jobs a round slices its bands).
-    int rows = k.band_rows;
-    if (!rows) {
-        const int most = dd::band_rows_for(W, c->threads, 2), bands = (H + most - 1) / most;
-        rows = (H + bands - 1) / bands;
-    }
+    int rows = k.band_rows ? k.band_rows : dd::default_band_rows(W, H, c->threads);
     if (rows < 1) rows = 1;
     if (rows > H) rows = H;
     if ((size_t)rows * (W | 1) * 4 > 200 * 1024) rows = (int)(200 * 1024 / (4 * (W | 1)));

@@ -250,6 +250,15 @@ inline int32_t band_rows_for(int32_t W, int32_t threads, int32_t blocks) {
     const int32_t rows = bytes / (4 * (W | 1));
     return rows < 1 ? 1 : rows;
 }
+// The default band: the tallest whose tile leaves room for two evaluation
+// blocks per SM, the frame's rows divided evenly among as many bands: a unit's
+// fixed cost is shared by more events (against bands of 40 KB: 43 windows of a
+// 511x389 stream 5.8 -> 4.1 ms, 55 of a 346x260 one 4.8 -> 4.0 ms; a search
+// with few jobs a round slices its bands).
+inline int32_t default_band_rows(int32_t W, int32_t H, int32_t threads) {
+    const int32_t most = band_rows_for(W, threads, 2), bands = (H + most - 1) / most;
+    return (H + bands - 1) / bands;
+}
 
 // Time buckets for a sort over H rows (rows of every plane): as many as fit
 // 4096 bins, at most 8.
@@ -393,6 +402,9 @@ void ctx_info(const struct ::dd_ctx* c, Geom* g, int32_t* threads, int32_t* eval
 const struct ::dd_mlp* ctx_warm_model(const struct ::dd_ctx* c);
 cudaStream_t ctx_stream(const struct ::dd_ctx* c);
 cudaError_t eval_smem_setup(const Geom& g);
+
+// The geometry that dd_contrast_noalloc evaluates a frame with (dd_noalloc.cu).
+Geom noalloc_geom(int32_t W, int32_t H, float foe_x, float foe_y);
 
 // Host checks shared by the entry points (dd_api.cu): a window descriptor
 // (DD_OK or DD_ERR_ARG; with two polarity planes the events must carry p),

@@ -14,7 +14,7 @@ namespace {
 constexpr int64_t NA_MAX_EVENTS = DD_NOALLOC_MAX_EVENTS;
 constexpr int NA_MAX_ROWS = 4096;   // sort bins: time buckets x rows
 constexpr int NA_MAX_TASKS = 64;     // hypotheses per kernel launch (calls are chunked)
-constexpr int NA_MAX_TILES = 1024;   // row bands of one frame (at most 683 for 4096 x 4096)
+constexpr int NA_MAX_TILES = 1024;   // row bands of one frame (at most 820 for 4096 x 4096)
 
 // Byte offsets of the sub-buffers inside the static array (each 256-aligned).
 constexpr size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
@@ -64,8 +64,32 @@ int scratch_base(int dev, unsigned char** out) {
     return DD_OK;
 }
 
-
 }  // namespace
+
+namespace dd {
+// Bands of dd_create's default height.  Bands of 96 KB of counts, as here
+// before a block's warps had scratch of their own beside the tile, leave one
+// block per SM (640x480, 129 hypotheses, 100,000 events: 214 us, with two
+// blocks 197; 600,000 events 377 and 317; 1280x720, eight hypotheses, 98 and
+// 106: 320 units on 304 blocks).  The keys are exact sums and do not depend on
+// the band.
+Geom noalloc_geom(int32_t W, int32_t H, float foe_x, float foe_y) {
+    Geom g{};
+    g.W = W;
+    g.H = H;
+    g.fx = foe_x;
+    g.fy = foe_y;
+    g.band_rows = default_band_rows(W, H, EVAL_THREADS);
+    g.n_tiles = (H + g.band_rows - 1) / g.band_rows;
+    g.n_tb = time_buckets(H);
+    g.max_splits = 1;
+    g.split_target = 0;
+    g.ref0 = 0;
+    g.planes = 1;                                 // polarity unused (Eq. 12 as the paper writes it)
+    g.plane_tiles = g.n_tiles;
+    return g;
+}
+}  // namespace dd
 
 extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_y, const dd_events* ev,
                                    const float* D, int32_t nD, dd_i128* K, void* stream) {
@@ -86,26 +110,7 @@ extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_
     int rc = scratch_base(dev, &base);
     if (rc) return rc;
 
-    dd::Geom g{};
-    g.W = W;
-    g.H = H;
-    g.fx = foe_x;
-    g.fy = foe_y;
-    // Bands of about 96 KB of counts: taller than dd_create's default of
-    // 40 KB, because a contrast-only call has no bound tasks to split over
-    // several blocks, so fewer, taller units mean fewer candidate-run set-ups
-    // per hypothesis.  The keys are exact sums and do not depend on the band.
-    int rows = (int)(96 * 1024 / (4 * W));
-    if (rows < 1) rows = 1;
-    if (rows > H) rows = H;
-    g.band_rows = rows;
-    g.n_tiles = (H + rows - 1) / rows;
-    g.n_tb = dd::time_buckets(H);
-    g.max_splits = 1;
-    g.split_target = 0;
-    g.ref0 = 0;
-    g.planes = 1;                                 // polarity unused (Eq. 12 as the paper writes it)
-    g.plane_tiles = g.n_tiles;
+    const dd::Geom g = dd::noalloc_geom(W, H, foe_x, foe_y);
     if (g.n_tiles > NA_MAX_TILES) return DD_ERR_CAPACITY;
     if (dd::eval_smem_setup(g) != cudaSuccess) return DD_ERR_CUDA;
 

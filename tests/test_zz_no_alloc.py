@@ -76,7 +76,7 @@ def test_noalloc_leaves_free_device_memory_unchanged():
 @pytest.mark.parametrize("W,H,fx,fy,seed", [(4096, 4096, 4096.0, 0.0, 77), (1, 4096, 0.0, 4096.0, 78),
                                             (4096, 1, 0.0, 1.0, 79)])
 def test_noalloc_largest_and_degenerate_frames(W, H, fx, fy, seed):
-    # The largest frame (683 row bands, 4096 sort bins) and one-pixel-wide or
+    # The largest frame (820 row bands, 4096 sort bins) and one-pixel-wide or
     # -high frames, FOE on a corner, a few thousand events.
     w = make_window(W, H, fx, fy, 2000, 60, 500, 0.25, 0.3, seed)
     ev = dd.Events.of(w, device="cuda")
@@ -84,6 +84,35 @@ def test_noalloc_largest_and_degenerate_frames(W, H, fx, fy, seed):
     got = dd.dd_contrast_noalloc(W, H, fx, fy, ev, Ds)
     assert got == reference_keys(w, ev, Ds)
     assert got == oracle_keys(w, Ds)
+
+
+def test_noalloc_runs_two_blocks_per_sm(tmp_path):
+    # its bands leave room for two resident evaluation blocks on every SM, as
+    # the kernel is built for, at the narrowest and widest frames too
+    import os
+    import subprocess
+    from paper_2209_13168_gb300 import _build
+    probe = tmp_path / "probe.cu"
+    probe.write_text("""#include <cstdio>
+#include "dd_internal.cuh"
+int main() {
+    const int frames[][2] = {{346, 260}, {640, 480}, {1280, 720}, {333, 251}, {511, 389}, {1, 4096}, {4096, 1}, {4096, 4096}};
+    cudaDeviceProp p;
+    if (cudaGetDeviceProperties(&p, 0) != cudaSuccess) return 1;
+    for (auto f : frames) {
+        const dd::Geom g = dd::noalloc_geom(f[0], f[1], 0.0f, 0.0f);
+        if (dd::eval_smem_setup(g) != cudaSuccess) return 1;
+        printf("%d %d %d\\n", f[0], f[1], dd::eval_resident_blocks(g, dd::EVAL_THREADS) / p.multiProcessorCount);
+    }
+    return 0;
+}
+""")
+    exe, lib = tmp_path / "probe", os.path.dirname(_build.LIB)
+    subprocess.check_call([_build.nvcc(), *_build.ARCH, "-std=c++17", "-I", _build.CSRC, "-I", _build.INCLUDE, str(probe),
+                           "-o", str(exe), "-L", lib, "-l:libdd.so", "-Xlinker", "-rpath," + lib])
+    for line in subprocess.check_output([str(exe)], text=True).splitlines():
+        W, H, blocks = map(int, line.split())
+        assert blocks == 2, (W, H, blocks)
 
 
 def test_noalloc_rejects_what_dd_contrast_rejects():
