@@ -957,7 +957,7 @@ __device__ __forceinline__ void bound_pass(const Geom& g, const Unit& un, const 
     const float tref = warp_tref(g, un.tau);
     const f32x2 foe = pair(g.fx, g.fy), minus_D = pair(-Dl, -Dh), gg = pair(warp_g(Dl, tref), warp_g(Dh, tref));
     const f32x2 widen = pair(WIDEN_DN, WIDEN_UP);
-    uint32_t one = 0, more = 0, full = 0, top = 0;
+    uint32_t one = 0, full = 0, top = 0;
     int head = 0, tail = 0;
     RunRing runs = {scratch, 0, 0};
     auto span = [&](float4 v) {
@@ -972,9 +972,11 @@ __device__ __forceinline__ void bound_pass(const Geom& g, const Unit& un, const 
         const Span s = span(v);
         full += (uint32_t)(valid & counts_full(g, T, s));
         const bool two = adjacent(s);
+        uint32_t more = 0;
         bump_pixel<WHOLE>(T, s.a, V, more, top, two);
         bump_pixel<WHOLE>(T, s.b, V, more, top, two);
         walk_warp<WHOLE>(g, T, v, s, valid & !two & meets(T, s), scratch + RING, V, more, top);
+        C += more;
     };
     Cursor cur(un);
     for (int ch = (int)(threadIdx.x >> 5); ch < chunks; ch += U * nw) {
@@ -997,6 +999,7 @@ __device__ __forceinline__ void bound_pass(const Geom& g, const Unit& un, const 
                 bool walk = !single;
                 const bool two = adjacent(s);
                 if (__popc(__ballot_sync(0xffffffffu, two)) >= 2) {
+                    uint32_t more = 0;            // not used: counted from the tile
                     bump_pixel<DENSE>(T, s.a, V, more, top, two);
                     bump_pixel<DENSE>(T, s.b, V, more, top, two);
                     walk = walk && !two;
@@ -1017,7 +1020,7 @@ __device__ __forceinline__ void bound_pass(const Geom& g, const Unit& un, const 
     }
     if (IS_DENSE) runs.flush(g, T);
     else queued(lane < tail - head);
-    C += (unsigned long long)one + more;
+    C += one;
     F += (unsigned long long)one + full;
 }
 
@@ -1232,7 +1235,13 @@ __device__ __forceinline__ void add_sums(const EvalArgs& a, const Unit& un, unsi
 
 // The pass of a point or bound unit and its warps' sums.  Images and dense
 // sums are read from the finished tile.  Ends before the barrier after which
-// the sums may be read and the tile cleared.
+// the sums may be read and the tile cleared.  A window has at most 2^30
+// events, so a warp's points and full events add up in 32 bits; a sparse
+// bound's cells do in units of at most SPARSE_CHUNKS chunks: an event covers at
+// most three cells in each of 4096 columns or rows (its estimate is well below
+// that, but no bound on it: far from the reference time it falls short).
+constexpr int SPARSE_CHUNKS = 1 << 13;
+static_assert(SPARSE_CHUNKS * 32ull * 3 * 4096 <= 0xffffffffull, "a sparse unit's cells fit 32 bits");
 __device__ __forceinline__ void single_unit(const Geom& g, const EvalArgs& a, const Unit& un, const Tile& T, int kind,
                                             float Dl, float Dh, uint32_t* scratch, uint32_t* out,
                                             unsigned long long (*red)[MAX_WARPS], int* s_last) {
@@ -1275,7 +1284,8 @@ __device__ __forceinline__ void single_unit(const Geom& g, const EvalArgs& a, co
         }
     }
     S = warp_total(S);
-    C = kind == UNIT_DENSE || un.chunks > (1 << 20) ? warp_total(C) : __reduce_add_sync(0xffffffffu, (uint32_t)C);
+    const bool wide = kind == UNIT_DENSE || (kind == UNIT_BOUND && un.chunks > SPARSE_CHUNKS);
+    C = wide ? warp_total(C) : __reduce_add_sync(0xffffffffu, (uint32_t)C);
     if (kind != UNIT_POINT) F = __reduce_add_sync(0xffffffffu, (uint32_t)F);
     if (lane == 0) {
         red[0][wid] = S;

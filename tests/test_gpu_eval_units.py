@@ -68,6 +68,25 @@ def test_domain_ends_far_outside_the_frame(to_start):
     ctx.close()
 
 
+def test_more_than_32_bits_of_increments_in_one_warp():
+    # n copies of one event whose segment is long although the bound counts as
+    # sparse (far from the reference time, at the domain's end), all walked by
+    # the one warp of one block: counts grow with n, keys with its square
+    n, tau = 21_000_000, 0.5
+    x, y, t = np.array([60], np.int16), np.array([0], np.int16), np.array([tau], np.float32)
+    one = O.solve(O.Window(4096, 1, 0.0, 0.0, x, y, t, 0.0, tau, t_ref=0.0), -128.0, -121.0, 10.0, 0.0, 1)
+    assert one["nodes_expanded"] == 1 and n * one["bound_increments"] > 1 << 32
+    ev = dd.Events(*(torch.from_numpy(a).cuda().repeat(n) for a in (x, y, t)), 0.0, tau)
+    torch.cuda.synchronize()
+    ctx = dd.Context(4096, 1, 0.0, 0.0, threads=32, warp_to_start=1)
+    got = ctx.solve(ev, -128.0, -121.0, 10.0, 0.0)
+    ctx.close()
+    for k in ("bound_increments", "cell_increments"):
+        assert got[k] == n * one[k], (k, got[k], n * one[k])
+    for k in ("K_hat", "gap_K"):
+        assert got[k] == n * n * one[k], k
+
+
 @pytest.mark.parametrize("hot", [1022, 1023, 1024, 2500])
 @pytest.mark.parametrize("threads", [32, 480])
 def test_fused_units_with_a_hot_pixel(hot, threads):
