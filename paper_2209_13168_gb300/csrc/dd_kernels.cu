@@ -1039,11 +1039,12 @@ __device__ __forceinline__ void bound_pass(const Geom& g, const Unit& un, const 
 // one pass instead of five (with the increments of two tasks taken back
 // between them) and one barrier instead of five.  The sums of squares, 2 sum(v) +
 // increments, are those of three separate passes.  Returns false if the list
-// or a field overflowed: then the tile holds nothing of use.  over[0] is set
-// before the first barrier and read after it, over[1] likewise at the second:
-// with one word, a warp that still reads it after the first barrier could see
-// another warp's overflow of the listed events, leave early and stay a barrier
-// ahead of its block.
+// or a field overflowed: then the tile holds nothing of use.  *s_over is 1
+// after an overflow before the first barrier and 2 after one between the two:
+// a warp that reads it late after the first barrier must not take another
+// warp's overflow of the listed events for one of the first part, leave early
+// and stay a barrier ahead of its block (two words instead of two values: 256
+// uneven windows 49.1 -> 51.2 ms, a 1280x720 stream 56.2 -> 59.2 ms).
 //
 // With few candidates a unit's fixed instructions count (16 windows of
 // 1280x720, 70 chunks a unit: 13,155 warp instructions), so a warp's sums stay
@@ -1069,7 +1070,7 @@ __device__ __forceinline__ void fused_half(const Geom& g, const Tile& T, float4 
 }
 
 __device__ __forceinline__ bool fused_pass(const Geom& g, const Unit& un, const Tile& T, uint32_t* list,
-                                           int* over, FusedSums& q) {
+                                           int* s_over, FusedSums& q) {
     constexpr int U = 2;
     const int lane = threadIdx.x & 31, nw = work_warps(), chunks = un.chunks;
     const float4* ev = reinterpret_cast<const float4*>(un.ev);
@@ -1096,9 +1097,9 @@ __device__ __forceinline__ bool fused_pass(const Geom& g, const Unit& un, const 
             listed += __popc(m);
         }
     }
-    if (top >= FIELD_MAX || listed > WARP_WORDS || chunks > FUSED_CHUNKS * nw) over[0] = 1;
+    if (top >= FIELD_MAX || listed > WARP_WORDS || chunks > FUSED_CHUNKS * nw) *s_over = 1;
     work_sync();
-    if (over[0]) return false;
+    if (*s_over == 1) return false;
     const float c = un.D_c, gc = warp_g(c, tref);
     for (int k = lane; k < listed; k += 32) {
         const float4 v = load_event(ev, (int)list[k]);
@@ -1108,9 +1109,9 @@ __device__ __forceinline__ bool fused_pass(const Geom& g, const Unit& un, const 
         fused_half<FIELD_L>(g, T, v, foe, lo_of(s2), sc, q.V[2], q.C[1], q.F[0], top);
         fused_half<FIELD_R>(g, T, v, foe, sc, hi_of(s2), q.V[3], q.C[2], q.F[1], top);
     }
-    if (top >= FIELD_MAX) over[1] = 1;
+    if (top >= FIELD_MAX) *s_over = 2;
     work_sync();
-    return !over[1];
+    return !*s_over;
 }
 
 // ------------------------------------------------------------------- units
@@ -1299,10 +1300,10 @@ __device__ __forceinline__ void single_unit(const Geom& g, const EvalArgs& a, co
 // number of sums left in `red`.
 __device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, const Unit& un, const Tile& T,
                                           int tile_words, uint32_t* scratch, unsigned long long (*red)[MAX_WARPS],
-                                          int* over, int* s_last) {
+                                          int* s_over, int* s_last) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     FusedSums q = {};
-    if (fused_pass(g, un, T, scratch, over, q)) {
+    if (fused_pass(g, un, T, scratch, s_over, q)) {
         auto total = [](uint32_t x) { return __reduce_add_sync(0xffffffffu, x); };
         const uint32_t n = total(q.n), v0 = total(q.V[0]);
 #pragma unroll
@@ -1357,7 +1358,7 @@ struct EvalShared {
     unsigned long long red[UNIT_SUMS][MAX_WARPS];
     uint32_t idle[32];
     int last;
-    int over[2];              // a fused unit's overflows: stable events and lists, listed events
+    int over;                // a fused unit's overflow (fused_pass)
 };
 
 // The share of block `block` of `blocks` in a round of n_units units.  The tile arrives clear and
@@ -1392,7 +1393,7 @@ __device__ __forceinline__ void eval_round(const Geom& g, const EvalArgs& a, con
         T.W = (uint32_t)g.W;
         int sums = 3;
         if (un.kind == UNIT_FUSED) {
-            sums = fused_unit(g, a, un, T, tile_words, scratch, sm.red, sm.over, &sm.last);
+            sums = fused_unit(g, a, un, T, tile_words, scratch, sm.red, &sm.over, &sm.last);
         } else {
             uint32_t* out = a.iwe_out ? a.iwe_out + ((size_t)un.task * g.planes + un.plane) * g.W * g.H + (size_t)un.y0 * g.W
                                       : nullptr;
@@ -1402,7 +1403,7 @@ __device__ __forceinline__ void eval_round(const Geom& g, const EvalArgs& a, con
         work_sync();                              // the pass is done
         if (threadIdx.x == 0) {
             clear_tile(tile, tile_words);
-            sm.over[0] = sm.over[1] = 0;
+            sm.over = 0;
         }
         add_sums(a, un, sm.red, sums);
     }
@@ -1422,7 +1423,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_eval(const __grid_cons
     if ((int)blockIdx.x >= n_units) return;
     if (threadIdx.x == 0) {
         clear_tile(tile, eval_tile_words(g));
-        sm.over[0] = sm.over[1] = 0;
+        sm.over = 0;
     }
     eval_round(g, a, a.jobs + (size_t)par * a.job_stride, &sch->work[par], n_units, 1, blockIdx.x, gridDim.x, tile, sm);
 }
@@ -2199,7 +2200,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
     }
     if (threadIdx.x == 0) {
         clear_tile(tile, eval_tile_words(g));
-        sm.over[0] = sm.over[1] = 0;
+        sm.over = 0;
         s_go = (unsigned long long)(uint32_t)sch->n_jobs[0];
     }
     __syncthreads();
