@@ -575,6 +575,7 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
     }
     int rc = stage(c, evs, nw);
     if (rc) return rc;
+    c->h_sch->polls = c->search_polls;
     const int64_t M = (int64_t)c->g.W * c->g.H;
     bool model = false;
     for (int w = 0; w < nw; w++) {
@@ -617,9 +618,8 @@ int solve_impl(dd_ctx* c, const dd_events* evs, int nw, const dd_window_params* 
         c->stats.kernel_launches++;
         const bool graph = device && !search;
         if (search) {
-            dd::CtlArgs ctl = dd::control_args(nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err, tr_dev,
-                                               c->jobs, c->job_stride, c->sch, 0, 0, 1, nullptr);
-            ctl.polls = c->search_polls;
+            const dd::CtlArgs ctl = dd::control_args(nw, c->st, c->queues, c->tasks, c->max_tasks, c->part, c->err,
+                                                     tr_dev, c->jobs, c->job_stride, c->sch, 0, 0, 1, nullptr);
             DD_TRY(dd::launch_search(c->g, eval_args(c, nullptr, nw == 1), ctl, c->threads, c->search_blocks,
                                      c->stream));
             c->stats.kernel_launches++;

@@ -160,6 +160,7 @@ struct Sched {
     int32_t n_jobs[2];
     int32_t work[2];
     int32_t ticket, active, running;
+    int32_t polls;                 // k_search: polls before a block gives up waiting for the others
     int32_t controls;              // k_search: control steps run, over all windows and rounds
     unsigned long long go;         // k_search: (next round) << 32 | its jobs
 };
@@ -292,7 +293,6 @@ struct CtlArgs {
     cudaGraphConditionalHandle loop;
     int32_t use_loop, split_ok;
     int32_t* phase_out;
-    int32_t polls;                 // k_search: polls before a block gives up waiting for the others
 };
 
 // Everything an evaluation launch reads or writes.
@@ -328,8 +328,9 @@ int eval_resident_blocks(const Geom& g, int threads);
 // of 346x260 475 -> 405 us, 7 of a stream 840 -> 780, 6 of 511x389 1,136 ->
 // 1,040; 19 to 64 windows between 6% faster and 9% slower).
 //
-// Every wait of one block for the others ends after c.polls polls (by default
-// SEARCH_POLLS: 1.6 s at 0.19 us a poll).  A block that gives up returns, so
+// Every wait of one block for the others ends after Sched::polls polls (by
+// default SEARCH_POLLS: 1.6 s at 0.19 us a poll; in memory: as an argument of
+// the kernel it cost a search of 232 rounds 1%).  A block that gives up returns, so
 // the others' waits run out as well, the launch ends and the windows' states
 // in memory are not all PH_DONE: the caller then clears the sums (the merge
 // buffers and the tasks') and runs the searches another way.  A sound round

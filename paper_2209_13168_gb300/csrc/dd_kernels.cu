@@ -2121,6 +2121,20 @@ __device__ __forceinline__ void add_release(int32_t* p, int32_t v) {
     asm volatile("red.release.gpu.global.add.s32 [%0], %1;" : : "l"(p), "r"(v) : "memory");
 }
 
+// Polls for the announcement of `round`, and for the reports of `all` blocks;
+// 0 (no jobs) or false after `limit` polls.
+__device__ __forceinline__ unsigned long long wait_go(const unsigned long long* go, uint32_t round, int limit) {
+    unsigned long long v;
+    while ((uint32_t)((v = load_acquire(go)) >> 32) != round)
+        if (--limit <= 0) return 0;
+    return v;
+}
+__device__ __forceinline__ bool wait_all(const int32_t* ticket, int32_t all, int limit) {
+    while (load_acquire(ticket) != all)
+        if (--limit <= 0) return false;
+    return true;
+}
+
 // Window w's control block of k_search: waits for the `others` evaluating
 // blocks and runs the window's control step; the last window's block to finish
 // announces the next round (or, with no search left, the end).
@@ -2136,10 +2150,8 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int
     for (uint32_t round = 0;; round++) {
         const int par = (int)(round & 1);
         if (threadIdx.x == 0) {
-            const int32_t all = (int32_t)(round + 1) * others;
-            int polls = 0;
-            while (load_acquire(&sch->ticket) != all && ++polls < c.polls) {}
-            sm.s_stop = polls >= c.polls;
+            const int32_t all = (int32_t)((round + 1) * (uint32_t)others);   // wraps as the count does
+            sm.s_stop = !wait_all(&sch->ticket, all, __ldcg(&sch->polls));
         }
         __syncthreads();
         if (sm.s_stop) return;                    // given up: the search stays unfinished
@@ -2156,7 +2168,7 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int
         if (threadIdx.x == 0) {
             __threadfence();
             if (!done) atomicAdd(&sch->active, 1);
-            if (atomicAdd(&sch->controls, 1) == (int32_t)(round + 1) * nw - 1) {   // the last window of the round
+            if (atomicAdd(&sch->controls, 1) == (int32_t)((round + 1) * (uint32_t)nw - 1)) {   // the round's last window
                 __threadfence();
                 const int active = atomicExch(&sch->active, 0);
                 const int jobs = atomicAdd(&sch->n_jobs[par ^ 1], 0);
@@ -2164,10 +2176,7 @@ __device__ __noinline__ void control_rounds(const Geom& g, const CtlArgs& c, int
                 sch->n_jobs[par] = 0;             // every block has read its round's count
                 store_release(&sch->go, next | (active ? (uint32_t)jobs : 0u));
             }
-            unsigned long long v = 0;
-            int polls = 0;
-            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < c.polls) {}
-            sm.s_stop = polls >= c.polls || (uint32_t)v == 0;     // given up, or every search has ended
+            sm.s_stop = (uint32_t)wait_go(&sch->go, round + 1, __ldcg(&sch->polls)) == 0;  // given up, or all have ended
         }
         __syncthreads();
         if (sm.s_stop) return;
@@ -2191,6 +2200,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
     extern __shared__ __align__(16) uint32_t tile[];
     __shared__ EvalShared sm;
     __shared__ unsigned long long s_go;
+    __shared__ int s_polls;
     Sched* sch = a.sch;
     const int nw = FEW ? c.n_windows : 1;
     if ((int)blockIdx.x < nw) {
@@ -2202,6 +2212,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
         clear_tile(tile, eval_tile_words(g));
         sm.over = 0;
         s_go = (unsigned long long)(uint32_t)sch->n_jobs[0];
+        s_polls = sch->polls;
     }
     __syncthreads();
     const int block = (int)blockIdx.x - nw, blocks = (int)gridDim.x - nw;
@@ -2214,10 +2225,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
         __syncthreads();                          // the block's sums are on their way; s_go has been read
         if (threadIdx.x == 0) {
             add_release(&sch->ticket, 1);
-            unsigned long long v = 0;
-            int polls = 0;
-            while ((uint32_t)((v = load_acquire(&sch->go)) >> 32) != round + 1 && ++polls < c.polls) {}
-            s_go = polls >= c.polls ? 0 : v;      // given up: no more jobs
+            s_go = wait_go(&sch->go, round + 1, s_polls);     // 0 if given up: no more jobs
         }
         __syncthreads();
         if ((uint32_t)s_go == 0) return;
@@ -2227,7 +2235,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_search(const __grid_co
 CtlArgs control_args(int32_t n_windows, SolveState* st, Node* queues, Task* tasks, int32_t task_stride, Partial* part,
                      const int32_t* err, TraceRec* trace, Job* jobs, int32_t job_stride, Sched* sch,
                      cudaGraphConditionalHandle loop, int32_t use_loop, int32_t split_ok, int32_t* phase_out) {
-    CtlArgs c{};
+    CtlArgs c;
     c.n_windows = n_windows;
     c.st_all = st;
     c.queues = queues;
