@@ -404,6 +404,11 @@ int32_t stage_tasks(dd_ctx* c, int32_t n, int kind, const float* A, const float*
     a->tasks = (dd::Task*)(c->call + at_tasks);
     a->jobs = (dd::Job*)(c->call + at_jobs);
     c->call_used = at_jobs + sizeof(dd::Job) * (size_t)nj;
+    // Few points or short bounds: bands in slices (a call on 600,000 events of
+    // 346x260: one bound of width 1/100 277 us without, 88 with, one contrast 127
+    // and 65).  Dense bounds are divided by their splits already: slices of them
+    // as well took 240 us where none take 189.
+    a->slices = n_dense ? 1 : dd::round_slices(c->g, nj);
     return m;
 }
 

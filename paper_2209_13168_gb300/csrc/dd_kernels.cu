@@ -499,19 +499,6 @@ struct Cursor {
     }
 };
 
-// Slices of rows (at least SLICE_ROWS each) that every band of a search's
-// round of `n_jobs` jobs is divided into, so that a round with few jobs (one
-// interval's, or its fused job alone) still fills the grid though the bands
-// are tall.  One interval a round, slices against none: 640x480 with 30,000
-// events 3.39 / 3.67 ms, 333x251 with 10,000 2.96 / 3.17 ms.
-constexpr int SLICE_ROWS = 4;
-__device__ __forceinline__ int round_slices(const Geom& g, int n_jobs) {
-    const int units = n_jobs * g.n_tiles;
-    return units > 0 && 2 * units <= g.split_target
-               ? min(g.split_target / units, (g.band_rows + SLICE_ROWS - 1) / SLICE_ROWS)
-               : 1;
-}
-
 // Prepares unit `id` (job id / (n_tiles slices), band, slice of it) in `un`:
 // one warp, one time bucket per lane.  The jobs' rows or events are divided
 // here, so no other thread divides.
@@ -1415,7 +1402,7 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_eval(const __grid_cons
     __shared__ EvalShared sm;
     Sched* sch = a.sch;
     const int par = sch->round & 1;
-    const int n_units = sch->n_jobs[par] * g.n_tiles;
+    const int n_units = sch->n_jobs[par] * g.n_tiles * a.slices;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sch->n_jobs[par ^ 1] = 0;
         sch->work[par ^ 1] = 0;
@@ -1425,7 +1412,8 @@ __global__ void __launch_bounds__(EVAL_THREADS + 32, 2) k_eval(const __grid_cons
         clear_tile(tile, eval_tile_words(g));
         sm.over = 0;
     }
-    eval_round(g, a, a.jobs + (size_t)par * a.job_stride, &sch->work[par], n_units, 1, blockIdx.x, gridDim.x, tile, sm);
+    eval_round(g, a, a.jobs + (size_t)par * a.job_stride, &sch->work[par], n_units, a.slices, blockIdx.x, gridDim.x, tile,
+               sm);
 }
 
 // The checked-build error word (always 0 in other builds); reset clears it.

@@ -47,6 +47,28 @@ def test_chunk_edges(n, threads):
         ctx.close()
 
 
+# a call of few points or short bounds divides its bands (the default height,
+# one row, a height that the slices do not divide, the whole frame)
+@pytest.mark.parametrize("band_rows", [0, 1, 13, 97])
+@pytest.mark.parametrize("polarity", [0, 1])
+def test_few_tasks_in_slices(band_rows, polarity):
+    w = make_window(131, 97, 64.0, 50.5, 6000, 170, 2000, 0.35, 0.3, seed=79)
+    ctx = dd.Context(131, 97, 64.0, 50.5, band_rows=band_rows, polarity=polarity)
+    win, ev = O.Window.of(w, polarity=bool(polarity)), dd.Events.of(w, device="cuda", polarity=bool(polarity))
+    for Ds in ([0.35], [-0.9, 0.0, 0.9]):
+        K, S, N, img = ctx.contrast(ev, Ds, want_iwe=True)
+        for j, D in enumerate(Ds):
+            k, s, n, im = O.contrast(win, D, want_iwe=True)
+            assert (K[j], int(S[j]), int(N[j])) == (k, s, n) and np.array_equal(img[j], im), D
+    for lo, hi in (([0.35], [0.36]), ([-0.5, 0.3], [-0.49, 0.32])):
+        lo, hi = np.asarray(lo, np.float32), np.asarray(hi, np.float32)
+        K, S, N, img = ctx.bound(ev, lo, hi, want_iwe=True)
+        for j in range(len(lo)):
+            k, s, n, im = O.bound(win, float(lo[j]), float(hi[j]), want_iwe=True)
+            assert (K[j], int(S[j]), int(N[j])) == (k, s, n) and np.array_equal(img[j], im), (lo[j], hi[j])
+    ctx.close()
+
+
 @pytest.mark.parametrize("foe", [(0.0, 0.0), (160.0, 60.0), (320.0, 119.75)])
 def test_segments_of_run_lengths(foe):
     # intervals whose longest segments cover 1, 6-8, 13-15 and over 100 major cells
