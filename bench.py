@@ -521,7 +521,7 @@ def run_ours(args):
     # the scatter's other two ceilings, from the library's own probes
     atom_peak, l2_peak = dd.dd_probe_peaks(stream.cuda_stream)
     incr = rr["cell_increments"]
-    ev_bytes = 8 * N * (pe + be)                  # one 8-byte event record per event-warp
+    ev_bytes = 8 * N * (pe + be)                  # an event's 8 input bytes per event-warp
     roofline_atomics = {"bound": "shared_atomics", "achieved": incr / (eval_ms_per_solve / 1e3) / 1e9,
                         "peak": atom_peak / 1e9, "unit": "G increments/s",
                         "frac": incr / (eval_ms_per_solve / 1e3) / atom_peak,

@@ -162,7 +162,6 @@ dd::EvalArgs eval_args(dd_ctx* c, uint32_t* iwe_out, bool single) {
     a.ev = c->ev;
     a.row_off = c->row_off;
     a.wins = c->wins;
-    a.tasks = c->tasks;
     a.task_stride = c->max_tasks;
     a.jobs = c->jobs;
     a.job_stride = c->job_stride;
@@ -371,7 +370,8 @@ dd_i128 from_i128(i128 v) {
 
 // Stage up to max_tasks tasks (point or bound) of one window, and their jobs,
 // at call_used; returns the number of tasks and sets their places.
-int32_t stage_tasks(dd_ctx* c, int32_t n, int kind, const float* A, const float* B, float tau, dd::EvalArgs* a) {
+int32_t stage_tasks(dd_ctx* c, int32_t n, int kind, const float* A, const float* B, float tau, dd::EvalArgs* a,
+                    const dd::Task** tasks_dev) {
     const int32_t m = n < c->max_tasks ? n : c->max_tasks;
     const size_t at_tasks = c->call_used, at_jobs = at_tasks + align64(sizeof(dd::Task) * (size_t)m);
     dd::Task* tasks = (dd::Task*)(c->h_call + at_tasks);
@@ -401,7 +401,7 @@ int32_t stage_tasks(dd_ctx* c, int32_t n, int kind, const float* A, const float*
         }
     std::memset(c->h_sch, 0, sizeof(dd::Sched));
     c->h_sch->n_jobs[0] = nj;
-    a->tasks = (dd::Task*)(c->call + at_tasks);
+    *tasks_dev = (const dd::Task*)(c->call + at_tasks);
     a->jobs = (dd::Job*)(c->call + at_jobs);
     c->call_used = at_jobs + sizeof(dd::Job) * (size_t)nj;
     // Few points or short bounds: bands in slices (a call on 600,000 events of
@@ -427,7 +427,8 @@ int eval_tasks(dd_ctx* c, const dd_events* ev, int32_t n, int kind, const float*
         dd::EvalArgs a = eval_args(c, nullptr, true);
         int32_t m = 0;
         c->call_used = tail;
-        if (n > 0) m = stage_tasks(c, n - j0, kind, A + j0, B + j0, ev->tau, &a);
+        const dd::Task* tasks = nullptr;
+        if (n > 0) m = stage_tasks(c, n - j0, kind, A + j0, B + j0, ev->tau, &a, &tasks);
         if (j0 == 0) {
             rc = ingest(c, 1);
             if (rc) return rc;
@@ -449,7 +450,7 @@ int eval_tasks(dd_ctx* c, const dd_events* ev, int32_t n, int kind, const float*
                 a.iwe_out = c->iwe;
             }
             DD_TRY(eval(c, a));
-            DD_TRY(dd::launch_keys(c->g, a.tasks, m, c->part, (i128*)(c->out + at_key),
+            DD_TRY(dd::launch_keys(c->g, tasks, m, c->part, (i128*)(c->out + at_key),
                                    (unsigned long long*)(c->out + at_S), (unsigned long long*)(c->out + at_S + w),
                                    (unsigned long long*)(c->out + at_S + 2 * w), c->stream, c->err, (int32_t*)c->out));
             c->stats.kernel_launches++;

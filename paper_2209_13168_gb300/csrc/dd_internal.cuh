@@ -313,8 +313,7 @@ struct EvalArgs {
     const Ev* ev;
     const int32_t* row_off;        // per window: bins_of(g) + 1 entries
     const WinIn* wins;
-    const Task* tasks;             // per window: task_stride entries
-    int32_t task_stride;
+    int32_t task_stride;           // per window: task slots in part
     const Job* jobs;               // two lists of job_stride entries
     int32_t job_stride;
     Sched* sch;

@@ -33,12 +33,6 @@ __device__ __forceinline__ float warp_g(float D, float tau) {
 __device__ __forceinline__ float warp_s(float D, float t, float g) {
     return __fmul_rn(__fsub_rn(1.0f, __fmul_rn(D, t)), g);
 }
-// Eq. (12), pixel u covers [u - 1/2, u + 1/2).
-__device__ __forceinline__ int cell_of(float foe, float d, float s) {
-    return __float2int_rd(__fadd_rn(__fadd_rn(foe, __fmul_rn(d, s)), 0.5f));
-}
-__device__ __forceinline__ float fmin_t(float a, float b) { return a < b ? a : b; }
-__device__ __forceinline__ float fmax_t(float a, float b) { return a < b ? b : a; }
 
 // --------------------------------------------------- paired binary32 arithmetic
 
@@ -82,7 +76,8 @@ __device__ __forceinline__ f32x2 floor2(f32x2 v) {
     asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(v), "l"(pair(CELL0_F, CELL0_F)));
     return r;
 }
-// Eq. (12): floor((foe + d s) + 1/2), biased, of one coordinate and of a pair.
+// Eq. (12), pixel u covers [u - 1/2, u + 1/2): floor((foe + d s) + 1/2), biased,
+// of one coordinate and of a pair.
 __device__ __forceinline__ uint32_t cell1(float foe, float d, float s) {
     return __float_as_uint(__fadd_rd(__fadd_rn(__fadd_rn(foe, __fmul_rn(d, s)), 0.5f), CELL0_F));
 }
@@ -120,11 +115,6 @@ __device__ __forceinline__ bool dd_in(long long i, long long n, unsigned bit) {
 #else
 #define DD_IN(i, n, bit) true
 #endif
-
-__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // Warp sum of 64-bit values as three 32-bit warp reductions (20, 20 and 24
 // bits per part: 32 of each add up within 32 bits).
@@ -468,8 +458,8 @@ struct __align__(16) Run {
 };
 constexpr Run NO_RUN = {0, INT32_MIN, INT32_MAX, 0};   // after the last run: chunks without events
 
-// One unit -- a job's row band -- as warp 0 prepares it in shared memory for
-// the block: everything that is the same for all threads is worked out once.
+// One unit -- a job's row band -- as the block's last warp prepares it in
+// shared memory for the others: everything that is the same for all threads is worked out once.
 enum UnitKind : int { UNIT_NONE = 0, UNIT_POINT, UNIT_BOUND, UNIT_DENSE, UNIT_FUSED };
 
 struct __align__(16) Unit {
@@ -1320,7 +1310,7 @@ __device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, cons
 // IWE evaluation of the round's job list.  A grid of resident blocks takes
 // units (job, row band).  The last warp of a block only prepares units, one
 // ahead of the others: a unit's preparation is a chain of dependent L2 loads
-// (its number, job, task, bin offsets) that takes longer than a small unit's
+// (its number, job, window, bin offsets) that takes longer than a small unit's
 // pass over its events.  Per unit there is one barrier of the whole block
 // (the unit is prepared, the tile is clear) and one of the working warps (the
 // pass is done), after which the sums go to the tasks and the tile is cleared
@@ -1333,7 +1323,7 @@ __device__ __forceinline__ int fused_unit(const Geom& g, const EvalArgs& a, cons
 // few instructions per event and cell; with few units, the latency of a unit
 // (its preparation 2.7 us, two barriers, one L2 round trip per four chunks).
 // Two blocks of 480 + 32 threads per SM with 64 registers a thread and tiles
-// of up to 96 KB: three of 256 + 32 with smaller tiles are 4% faster on
+// of up to 91 KB: three of 256 + 32 with smaller tiles are 4% faster on
 // 640-pixel frames in late rounds but 29% slower on 1280-pixel ones, where
 // the lower tile re-reads more events.  Against one thread deciding each
 // unit's split, candidates and sums in every warp (512 threads, 3 blocks of 40

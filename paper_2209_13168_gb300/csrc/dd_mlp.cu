@@ -6,7 +6,7 @@
 // trained on windows solved exactly, proposes a guess and a half-width
 // instead (include/dd.h states the contract).  Everything here is small next
 // to the search: the features are one pass over the window's sorted events
-// (8 bytes per event), the network 66k multiply-adds per window.  It runs
+// (16 bytes per event), the network 66k multiply-adds per window.  It runs
 // on CUDA cores in binary32 with a fixed summation order (each unit adds
 // weight * input for inputs 0..127 in turn onto its bias), so a window's
 // guess is reproducible bit for bit.
@@ -39,12 +39,15 @@ constexpr float LOG2E = 1.44269504f;
 
 __device__ __forceinline__ float bf(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 
-// The 128 bfloat16 weights of one unit in registers: sixteen 16-byte loads in
-// flight at once, so a layer waits for memory once.  The hidden layers'
-// matrices are stored in groups of eight inputs, [in / 8][unit][8], so that a
-// warp's load is 512 consecutive bytes (with contiguous rows each load touched
-// 32 lines: a gradient of 256 samples 28.6 us, now 21.6; of 2,048 43.1 and
-// 34.9).  The output layer's two rows of 128 are each contiguous (UNITS = 1).
+// The 128 bfloat16 weights of one unit as sixteen 16-byte loads, independent of
+// one another.  How many are in flight is the compiler's choice: a row is 64
+// registers, and the kernels have 98 (k_sample, one sample), 102 (four) and 36
+// (k_fwd, k_warm): about one layer's loads, and not half of one's in the last
+// two.  The hidden layers' matrices are stored in groups of
+// eight inputs, [in / 8][unit][8], so that a warp's load is 512 consecutive
+// bytes (with contiguous rows each load touched 32 lines: a gradient of 256
+// samples 28.6 us, then 21.6; of 2,048 43.1 and 34.9).  The output layer's two
+// rows of 128 are each contiguous (UNITS = 1).
 constexpr int IN_GROUP = 8;
 __host__ __device__ __forceinline__ int grouped(int unit, int in) {
     return (in / IN_GROUP * MLP_H + unit) * IN_GROUP + in % IN_GROUP;
@@ -88,10 +91,10 @@ __device__ __forceinline__ void unit(const Row& w, float bias, const float (*x)[
 }
 
 // The forward pass of S samples by a block of 128 threads; x, h1, h2 and out
-// in shared memory.  Both hidden layers' weights are loaded before the first
+// in shared memory.  Both hidden layers' weights are asked for before the first
 // layer, the output layer's (and, `ahead` of it, what the caller needs next)
-// before the second, so that the block waits for memory once.  Every thread
-// returns after the last barrier.
+// before the second, so that loads may run ahead of the layer that uses them.
+// Every thread returns after the last barrier.
 template <int S, class Ahead>
 __device__ __forceinline__ void forward(const MlpDev& m, const float (*x)[MLP_H], float (*h1)[MLP_H], float (*h2)[MLP_H],
                                         float (*out)[MLP_OUT], Ahead&& ahead) {

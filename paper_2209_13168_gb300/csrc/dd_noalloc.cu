@@ -159,7 +159,6 @@ extern "C" int dd_contrast_noalloc(int32_t W, int32_t H, float foe_x, float foe_
     a.ev = ev_sorted;
     a.row_off = row_off;
     a.wins = win;
-    a.tasks = tasks;
     a.task_stride = NA_MAX_TASKS;
     a.jobs = jobs;
     a.job_stride = NA_MAX_TASKS;

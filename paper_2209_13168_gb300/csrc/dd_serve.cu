@@ -377,7 +377,6 @@ void loop(dd_server* s) {
     a.ev = s->ev;
     a.row_off = s->row_off;
     a.wins = s->wins;
-    a.tasks = s->tasks;
     a.task_stride = s->max_tasks;
     a.jobs = s->jobs;
     a.job_stride = s->job_stride;

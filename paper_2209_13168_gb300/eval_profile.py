@@ -29,7 +29,7 @@ def window(name):
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--window", default="config2", choices=["config2", "descent"])
-    ap.add_argument("--warmup", type=int, default=0, help="untimed graph solves first (not seen as rounds)")
+    ap.add_argument("--warmup", type=int, default=0, help="untimed solves first, in one launch (not seen as rounds)")
     ap.add_argument("--fuse-span", type=int, default=None, help="dd_config.fuse_span (default: the tuned value)")
     for k in ("band-rows", "threads", "pop-k", "max-splits"):
         ap.add_argument("--" + k, type=int, default=None, help="override the tuned " + k.replace("-", "_"))
