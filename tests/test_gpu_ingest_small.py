@@ -41,10 +41,14 @@ def test_malformed_events_are_reported(field, value):
     a = getattr(w, field).copy()
     a[1777] = value
     setattr(w, field, a)
-    ctx = dd.Context(330, 250, 165.0, 125.0, pop_k=8)
-    for call in (lambda e: ctx.contrast(e, [0.1]), lambda e: ctx.solve(e, -1.0, 1.0, 1e-2)):
+    ctx, fresh = (dd.Context(330, 250, 165.0, 125.0, pop_k=8) for _ in range(2))
+    calls = (lambda c, e: c.contrast(e, [0.1])[0], lambda c, e: c.bound(e, [0.1], [0.4])[0],
+             lambda c, e: c.solve(e, -1.0, 1.0, 1e-2))
+    want = [call(fresh, good) for call in calls]
+    for bad in calls:
         with pytest.raises(dd.DDError) as e:
-            call(dd.Events.of(w, device="cuda"))
+            bad(ctx, dd.Events.of(w, device="cuda"))
         assert e.value.status == dd.DD_ERR_ARG
-        call(good)                                # the next call on the context is unaffected
+        assert [call(ctx, good) for call in calls] == want        # the next calls on the context are unaffected
+    fresh.close()
     ctx.close()

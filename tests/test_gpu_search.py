@@ -4,6 +4,8 @@ next round.  Results, counts and traces are the oracle's whatever the queue's
 place (never, sometimes or always in shared memory), and windows beyond the
 launch's size limit go through the graph with the same result.
 """
+import functools
+
 import pytest
 
 import oracle as O
@@ -134,17 +136,23 @@ def test_window_beyond_the_launch_limit():
 
 # one interval a round, so that bands (the default height, one row, a height
 # that the slices do not divide, the whole frame) are cut into slices of rows;
-# above 131,072 events a unit holds a share of the events and is not cut
-@pytest.mark.parametrize("n", [900, 20000, 140000])
+# above 131,072 events a long bound's unit (64 cells; the root of the longest
+# window here has 157) holds a share of the events and is not cut
+@pytest.mark.parametrize("n,tau", [(900, 0.3), (20000, 0.3), (140000, 0.3), (140000, 0.7)])
 @pytest.mark.parametrize("band_rows", [0, 1, 13, 97])
-def test_bands_cut_into_slices(n, band_rows):
-    w = make_window(131, 97, 64.0, 50.5, n - n // 3, n // 36, n // 3, 0.35, 0.3, seed=76)
+def test_bands_cut_into_slices(n, tau, band_rows):
+    w, want = _window_to_slice(n, tau)
     ctx = dd.Context(131, 97, 64.0, 50.5, pop_k=1, band_rows=band_rows)
     got = ctx.solve(dd.Events.of(w, device="cuda"), -1.0, 1.0, 1e-3, 0.0)
     ctx.close()
-    want = O.solve(O.Window.of(w), -1.0, 1.0, 1e-3, 0.0, 1)
     for k in KEYS:
         assert got[k] == want[k], (k, got[k], want[k])
+
+
+@functools.lru_cache(maxsize=None)
+def _window_to_slice(n, tau):
+    w = make_window(131, 97, 64.0, 50.5, n - n // 3, n // 36, n // 3, 0.35, tau, seed=76)
+    return w, O.solve(O.Window.of(w), -1.0, 1.0, 1e-3, 0.0, 1)
 
 
 # up to 16 windows share one launch, 17 go through the graph; they end in

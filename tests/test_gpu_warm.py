@@ -134,6 +134,31 @@ def test_gradient_against_binary64(B):
     m.close()
 
 
+# Chunks of 64 samples with one missing and one over; the last size with a
+# block per sample (608), and the first ones with four (whole, one and three
+# short); the largest.  A unit's chain of 128 additions is off by 128 x 2^-24 =
+# 8e-6 at most relative to its terms, which also turns a ReLU over now and then
+# (3e-5 of the gradient the most seen in 36 draws): 1e-4.  One sample left out
+# is 1/4096 = 2.4e-4 and more.
+@pytest.mark.parametrize("B", [63, 65, 608, 609, 611, 612, 4093, 4096])
+def test_gradient_at_the_edges_of_its_launches(B):
+    m = dd.Mlp()
+    p = random_params(20 + B)
+    m.set_params(p)
+    rng = np.random.default_rng(B)
+    X = (rng.random((B, 128)) * 2).astype(np.float32)
+    u = rng.uniform(0.0, 0.35, B).astype(np.float32)
+    g, loss = m.grad(torch.from_numpy(X).cuda(), torch.from_numpy(u).cuda())
+    g = g.cpu().numpy().astype(np.float64)
+    want_loss, want = O.mlp_loss_f64(evaluated(p).astype(np.float64), X.astype(np.float64), u.astype(np.float64))
+    assert abs(float(loss.item()) - want_loss) <= 1e-5 * abs(want_loss)
+    o = O.OFFSETS
+    for a, b in (("W1", "b1"), ("b1", "W2"), ("W2", "b2"), ("b2", "W3"), ("W3", "b3"), ("b3", None)):
+        sl = slice(o[a], o[b] if b else None)
+        assert np.linalg.norm(g[sl] - want[sl]) <= 1e-4 * np.linalg.norm(want[sl]), a
+    m.close()
+
+
 def test_training_lowers_the_loss_and_checkpoints(tmp_path):
     rng = np.random.default_rng(6)
     X = torch.from_numpy((rng.random((256, 128)) * 2).astype(np.float32)).cuda()
