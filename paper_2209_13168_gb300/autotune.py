@@ -11,6 +11,8 @@ results are identical for every candidate (the table stores times, and the
 tuner checks that every candidate returned the same keys).
 
     python -m paper_2209_13168_gb300.autotune --out tuned.json
+
+--measure times the table's own knobs again and changes the times only.
 """
 import argparse
 import itertools
@@ -24,13 +26,13 @@ import paper_2209_13168_gb300 as dd
 DEFAULT_TABLE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned_gb300.json")
 
 CANDIDATES = {
-    "band_rows": [8, 10, 12, 16, 18, 20, 24, 38],
+    "band_rows": [8, 12, 16, 18, 20, 24, 32, 35, 44, 48],
     "threads": [128, 256, 512],
     "pop_k": [16, 32, 64],
     "max_splits": [4, 8, 16],
 }
 # second stage: dd_config.fuse_span (-1: never fuse, one task per unit)
-FUSE_CANDIDATES = [-1, 10, 25, 40, 70]
+FUSE_CANDIDATES = [-1, 10, 25, 40, 70, 150, 300, 600]
 KNOBS = ("band_rows", "threads", "pop_k", "max_splits", "fuse_span")
 
 
@@ -59,13 +61,24 @@ def _time(fn, reps):
     return (time.perf_counter() - t0) / reps, out
 
 
+def measure(windows, evs, knobs, mode, reps):
+    """Seconds per window with these knobs, and the windows' keys."""
+    w0 = windows[0]
+    ctx = dd.Context(w0.W, w0.H, w0.foe_x, w0.foe_y, **knobs)
+    if mode == "single":
+        dt, out = _time(lambda: [ctx.solve(e) for e in evs], reps)
+    else:
+        dt, (_, out) = _time(lambda: ctx.solve_batch(evs), reps)
+    ctx.close()
+    return dt / len(evs), [r["K_hat"] for r in out]
+
+
 def tune(windows, mode="single", candidates=None, reps=3, log=print):
     """Best knobs for windows of one geometry (synth.Window objects)."""
     import torch
     cand = dict(CANDIDATES)
     if candidates:
         cand.update(candidates)
-    w0 = windows[0]
     evs = [dd.Events.of(w, device="cuda") for w in windows]
     best, ref = None, None
     grid = list(itertools.product(cand["band_rows"], cand["threads"], cand["pop_k"],
@@ -74,17 +87,7 @@ def tune(windows, mode="single", candidates=None, reps=3, log=print):
     stage2 = False
     while grid:
         rows, thr, k, ms, fz = grid.pop(0)
-        ctx = dd.Context(w0.W, w0.H, w0.foe_x, w0.foe_y, pop_k=k, band_rows=rows, threads=thr, max_splits=ms,
-                         fuse_span=fz)
-        if mode == "single":
-            dt, out = _time(lambda: [ctx.solve(e) for e in evs], reps)
-            keys = [r["K_hat"] for r in out]
-            dt /= len(evs)
-        else:
-            dt, out = _time(lambda: ctx.solve_batch(evs), reps)
-            keys = [r["K_hat"] for r in out[1]]
-            dt /= len(evs)
-        ctx.close()
+        dt, keys = measure(windows, evs, dict(zip(KNOBS, (rows, thr, k, ms, fz))), mode, reps)
         if ref is None:
             ref = keys
         assert keys == ref, "a schedule knob changed a result"
@@ -149,25 +152,10 @@ def fast_mode_windows(W2=160, H2=90, keep=0.25, step=20):
     return out
 
 
-def main():
-    ap = argparse.ArgumentParser()
-    ap.add_argument("--out", default=DEFAULT_TABLE)
-    ap.add_argument("--quick", action="store_true",
-                    help="fewer candidates: the band heights, block sizes, pop widths and split caps that won on this GPU")
-    ap.add_argument("--reps", type=int, default=3, help="timed repetitions per candidate (single windows)")
-    ap.add_argument("--only", default=None, help="tune only the jobs whose name contains this (e.g. 1280x720)")
-    args = ap.parse_args()
-    import torch
+def workloads():
+    """(mode, windows) of every entry of the table."""
     from synth import window_config1, window_config2
-    from synth.descent import batch_params3, batch_window3
-    torch.cuda.set_device(0)
-    name = gpu_name()
-    table = load_table(args.out)
-    cand = None
-    if args.quick:
-        cand = {"band_rows": [12, 16, 20, 24], "threads": [256, 512], "pop_k": [16, 32, 64], "max_splits": [8, 16],
-                "fuse_span": [-1, 15, 25, 40, 70]}
-    from synth.descent import serve_config5
+    from synth.descent import batch_params3, batch_window3, serve_config5
     jobs = [("single", [window_config1()]), ("single", [window_config2()])]
     params = batch_params3()
     jobs.append(("batch", [batch_window3(i, params) for i in range(256)]))
@@ -176,15 +164,43 @@ def main():
     jobs.append(("single", [serve_config5(0, k) for k in (20, 60, 100, 140, 180)]))
     jobs.append(("batch", [serve_config5(0, k, n_scale=0.5) for k in range(0, 189, 3)]))
     jobs.append(("single", fast_mode_windows()))
-    for mode, ws in jobs:
+    return jobs
+
+
+def main():
+    ap = argparse.ArgumentParser()
+    ap.add_argument("--out", default=DEFAULT_TABLE)
+    ap.add_argument("--quick", action="store_true",
+                    help="fewer candidates: the band heights, block sizes, pop widths and split caps that won on this GPU")
+    ap.add_argument("--measure", action="store_true", help="keep every entry's knobs and time them again")
+    ap.add_argument("--reps", type=int, default=3, help="timed repetitions per candidate (single windows)")
+    ap.add_argument("--only", default=None, help="tune only the jobs whose name contains this (e.g. 1280x720)")
+    args = ap.parse_args()
+    import torch
+    torch.cuda.set_device(0)
+    name = gpu_name()
+    table = load_table(args.out)
+    cand = None
+    if args.quick:
+        cand = {"band_rows": [16, 18, 24, 32, 35, 44], "threads": [512], "pop_k": [16, 64], "max_splits": [16],
+                "fuse_span": [25, 40, 70, 300, 600]}
+    for mode, ws in workloads():
         if args.only and args.only not in "%s %dx%d" % (mode, ws[0].W, ws[0].H):
             continue
         n = int(sum(w.n for w in ws) / len(ws))
+        k = key(ws[0].W, ws[0].H, n, mode, name)
+        if args.measure:                          # the entry's own knobs, timed again
+            if k in table:
+                evs = [dd.Events.of(w, device="cuda") for w in ws]
+                dt, _ = measure(ws, evs, {knob: table[k][knob] for knob in KNOBS}, mode, 10)
+                table[k]["ms_per_window"] = dt * 1e3
+                print("%s: %.4f ms per window" % (k, dt * 1e3), flush=True)
+            continue
         print("tuning %s %dx%d, %d windows of ~%d events" % (mode, ws[0].W, ws[0].H, len(ws), n), flush=True)
         best = tune(ws, mode, cand, reps=args.reps if mode == "single" else 3)
         best["windows"] = len(ws)
         best["events_per_window"] = n
-        table[key(ws[0].W, ws[0].H, n, mode, name)] = best
+        table[k] = best
         print("  best:", best, flush=True)
     with open(args.out + ".tmp", "w") as f:
         json.dump(table, f, indent=1, sort_keys=True)
